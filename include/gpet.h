@@ -152,12 +152,13 @@ typedef struct {
 /* Launch options; pass NULL for defaults. */
 typedef struct {
     int32_t keep_hits;       /* 1: also store every crystal interaction (tests, DOI studies) */
-    int32_t block_size;      /* threads per CTA of the transport kernel (0 = 256; kernel 3: 128, 256 or 512) */
+    int32_t block_size;      /* threads per CTA of the transport kernel (0 = the kernel's own: 256, and 448
+                                for kernel 3, which otherwise takes 128, 256 or 512)      */
     int32_t blocks_per_sm;   /* resident CTAs per SM (0 = tuned default)                   */
     int32_t kernel;          /* 0 = tuned, else 3; 1 = per-lane event loop, 2 = per-warp
-                                wavefront, 3 = wavefront with one phase per CTA            */
-    int32_t compact_every;   /* wavefront regrouping interval in events (0 = default)      */
-    int32_t pool_depth;      /* wavefront histories per lane in shared memory, 2..4 (0 = 2)  */
+                                wavefront, 3 = slot pool shared by a CTA's warps           */
+    int32_t compact_every;   /* kernel 2: regrouping interval in events (0 = default)      */
+    int32_t pool_depth;      /* kernel 2: histories per lane in shared memory, 2..4 (0 = 2)  */
     void *stream;            /* cudaStream_t */
     uint64_t h_begin, h_end; /* run only histories [h_begin, h_end) of the n_decays run (a shard);
                                 h_end = 0 means n_decays.  Decay times keep the whole run's span,
@@ -235,9 +236,10 @@ typedef struct {
     uint64_t screened_flights;            /* flights decided by the axial screen (no panel test) */
     uint64_t singles_formed;              /* singles before the energy window */
     double latency_ms;      /* served requests: submission to result ready (0 otherwise) */
-    /* events run per history phase by the CTA-synchronous kernel (kernel 3; zero for the others):
+    /* events run per history phase by the slot-pool kernel (kernel 3; zero for the others):
        [1] decay, [2] phantom step, [3] flight from the decay or phantom, [4] detector step,
-       [5] finish (digitizer of a history), [6] flight after a panel exit; [0] unused */
+       [5] finish (digitizer of a history), [6] flight after a panel exit (one that left through the
+       panel's back counts too, although its event is skipped); [0] unused */
     uint64_t phase_events[7];
 } gpet_counts;
 int gpet_result_counts(const gpet_result *r, gpet_counts *out);
@@ -424,10 +426,8 @@ int gpet_sort_times_noalloc(const uint64_t *d_t_in, uint64_t n, uint64_t *d_t_ou
 /* Library infrastructure with no counterpart in the paper: a launch-form
  * choice for the transport of Sec. 2.1.
  * Time the candidate launch forms of the transport kernel -- the per-lane
- * event loop, the per-warp wavefront, the CTA-synchronous wavefront at 128,
- * 256 or 512 threads, pool depth 2 or 3 and compaction interval 1, 2 or 4
- * (gpet_options.compact_every: detector or phantom steps a lane runs between
- * regroupings) -- on a pilot run (pilot_decays >= 1000, seed)
+ * event loop, the per-warp wavefront, the slot-pool kernel in its own shape
+ * and at 128, 256 or 512 threads -- on a pilot run (pilot_decays >= 1000, seed)
  * of the caller's workload, and return the fastest in *best (its transport
  * time in *best_ms, may be NULL).  The choice is remembered for the scanner's
  * design class (panels, layers, phantom) on this device's SM count; later

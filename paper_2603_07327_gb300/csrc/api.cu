@@ -350,6 +350,19 @@ int gpet_build_geometry(const gpet_scanner_desc *d, GeomDev &g, int64_t &n_cryst
     g.phi0 = (float)phi0;
     g.dphi = (float)(2.0 * M_PI / d->n_panels);
     g.inv_dphi = (float)(d->n_panels / (2.0 * M_PI));
+    // The depth beyond which nothing of the other panels lies, in a panel's own
+    // frame (the largest w of their corners), with a margin far above the FP32
+    // rounding of a ray's position and of the slab test.
+    g.w_clear = 3.0e38f;
+    if (!posed && d->n_panels > 2) {
+        double wmax = -1e300;
+        for (int k = 1; k < d->n_panels; ++k) {
+            const double a = 2.0 * M_PI * k / d->n_panels;
+            for (double r : {d->inner_radius_mm, d->inner_radius_mm + w})
+                wmax = std::max(wmax, r * std::cos(a) + 0.5 * U * std::fabs(std::sin(a)) - d->inner_radius_mm);
+        }
+        g.w_clear = (float)(wmax + 1e-2 + 1e-5 * (d->inner_radius_mm + w));
+    }
     if (posed) {
         std::vector<float> tab;
         const int st = build_poses(d, w, U, V, tab);

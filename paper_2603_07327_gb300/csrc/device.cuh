@@ -77,6 +77,11 @@ struct __align__(128) GeomDev {
     // ring culling: every panel box lies in the annulus R^2 <= r^2 <= rout2 and
     // inside its angular sector |phi - phi_k| <= beta (phi_k = phi0 + k dphi)
     float R2, rout2, beta, phi0, dphi, inv_dphi;
+    // depth from which a photon moving outward has left the ring: every other
+    // panel lies wholly in front of the plane w = w_clear of this panel's frame
+    // (3e38 where the panels' arrangement does not allow it)
+    float w_clear;
+    float pad_ring[3];
     // non-repetition mode (posed = 1): per panel 4 float4 in global memory --
     // (w axis, w.o), (u axis, u.o), (v axis, v.o), (o, 0) with o the centre of
     // the inner face; the ring fields above are then unused
@@ -141,9 +146,11 @@ __device__ __forceinline__ uint4 draw(uint64_t seed, uint64_t h, uint32_t tag, u
                          make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
 }
 
-// uniform (k + 1/2) 2^-23 in (0,1) from the top 23 bits (exact in FP32)
+// Uniform (k + 1/2) 2^-23 in (0,1) from the top 23 bits k, exact in FP32: the
+// bits of 1 + k 2^-23 come from one funnel shift, and subtracting 1 - 2^-24
+// leaves (2 k + 1) 2^-24, which FP32 holds exactly (no int-to-float conversion).
 __device__ __forceinline__ float u01(uint32_t w) {
-    return ((float)(w >> 9) + 0.5f) * 1.1920928955078125e-07f;
+    return __uint_as_float(__funnelshift_r(w, 0x7Fu, 9)) - 0.999999940395355224609375f;
 }
 
 // ---------------------------------------------------------------------------
@@ -219,20 +226,20 @@ __device__ __forceinline__ int kahn_sample(uint64_t seed, uint64_t h, uint32_t t
 }
 
 // rotate (a, b, c) [third component = scanner axis] by polar (cos ct, 1-cos omc) and
-// azimuth 2 pi u; frame-equivariant under rotations about the axis
-__device__ __forceinline__ void rotate_dir(float &a, float &b, float &c, float omc, float u_phi) {
+// azimuth (sine sp, cosine cp); frame-equivariant under rotations about the axis
+__device__ __forceinline__ void rotate_dir(float &a, float &b, float &c, float omc, float sp, float cp) {
     const float ct = 1.0f - omc;
     const float st = sqrtf(fmaxf(omc * (2.0f - omc), 0.0f));
-    float sp, cp;
-    sincospif(2.0f * u_phi, &sp, &cp);
     if (fabsf(c) < 0.99999f) {
         // transverse norm from the transverse components (= sqrt(1 - c^2) for a
         // unit vector, without the cancellation of 1 - c^2 near the axis)
         const float q = sqrtf(fmaf(a, a, b * b));
         const float iq = 1.0f / q;
-        const float na = a * ct + st * (a * c * cp - b * sp) * iq;
-        const float nb = b * ct + st * (b * c * cp + a * sp) * iq;
-        const float nc = c * ct - st * q * cp;
+        // (the fused operations are spelled out: left to the compiler, each place
+        // that inlines this would round a scattered direction its own way)
+        const float na = fmaf(a, ct, st * fmaf(a * c, cp, -(b * sp)) * iq);
+        const float nb = fmaf(b, ct, st * fmaf(a, sp, b * c * cp) * iq);
+        const float nc = fmaf(c, ct, -(st * q * cp));
         a = na; b = nb; c = nc;
     } else {
         const float sg = c > 0.0f ? 1.0f : -1.0f;
@@ -255,6 +262,7 @@ __device__ __forceinline__ Loc locate(const GeomDev &g, int k, float w, float u,
     L.layer = -1; L.module = -1; L.crystal = -1;
     // layer-selection step: the layer whose depth range holds w
     int l = -1, owner = g.n_layers - 1;
+#pragma unroll 1
     for (int j = 0; j < g.n_layers; ++j) {
         if (w < g.layers[j].w0) { owner = j; break; }
         if (w < g.layers[j].w1) { l = j; break; }
@@ -283,11 +291,13 @@ __device__ __forceinline__ Loc locate(const GeomDev &g, int k, float w, float u,
 }
 
 // distance along (dw, du, dv) from an inside point to the panel box exit
+// (the face that the ray moves toward is selected first, so that a warp's lanes
+// share one division per axis)
 __device__ __forceinline__ float panel_exit(const GeomDev &g, float w, float u, float v, float dw, float du, float dv) {
     float t = 3.0e38f;
-    if (dw > 0.0f) t = fminf(t, (g.W - w) / dw); else if (dw < 0.0f) t = fminf(t, -w / dw);
-    if (du > 0.0f) t = fminf(t, (g.half_u - u) / du); else if (du < 0.0f) t = fminf(t, (-g.half_u - u) / du);
-    if (dv > 0.0f) t = fminf(t, (g.half_v - v) / dv); else if (dv < 0.0f) t = fminf(t, (-g.half_v - v) / dv);
+    if (dw != 0.0f) t = fminf(t, (dw > 0.0f ? g.W - w : -w) / dw);
+    if (du != 0.0f) t = fminf(t, ((du > 0.0f ? g.half_u : -g.half_u) - u) / du);
+    if (dv != 0.0f) t = fminf(t, ((dv > 0.0f ? g.half_v : -g.half_v) - v) / dv);
     return fmaxf(t, 0.0f);
 }
 
@@ -393,15 +403,14 @@ __device__ __forceinline__ float atan2_as(float y, float x) {
 
 constexpr int kFlightScreened = -2;  // flight() result: no panel, decided without slab tests
 
-// Slab-test the panels whose angular sector can meet the azimuths the ray
-// sweeps between t = ta and t = tb (a stretch inside the annulus that holds
-// all panel boxes; along a line the azimuth is monotonic and the sweep is
-// shorter than pi).  Panel k can be entered there only if its centre angle
-// k*dphi lies within beta of the swept interval; 1e-3 rad of margin covers
-// FP32 rounding.
-__device__ __forceinline__ void flight_sector(const GeomDev &g, float x, float y, float z, float dx, float dy,
-                                              float dz, float ta, float tb, int skip, int &best, float &bi,
-                                              float &bo) {
+// Panels whose angular sector can meet the azimuths the ray sweeps between
+// t = ta and t = tb (a stretch inside the annulus that holds all panel boxes;
+// along a line the azimuth is monotonic and the sweep is shorter than pi): n
+// panels from index k on, modulo the ring.  Panel k can be entered there only
+// if its centre angle k*dphi lies within beta of the swept interval; 1e-3 rad
+// of margin covers FP32 rounding.
+__device__ __forceinline__ void flight_sector(const GeomDev &g, float x, float y, float dx, float dy, float ta,
+                                              float tb, int &k, int &n) {
     const float p1 = atan2_as(fmaf(ta, dy, y), fmaf(ta, dx, x)) - g.phi0;
     float p2 = atan2_as(fmaf(tb, dy, y), fmaf(tb, dx, x)) - g.phi0;
     // unwrap p2 next to p1
@@ -411,13 +420,9 @@ __device__ __forceinline__ void flight_sector(const GeomDev &g, float x, float y
     const int jlo = (int)ceilf(lo * g.inv_dphi), jhi = (int)floorf(hi * g.inv_dphi);
     // jlo mod n by a float floor: (jlo + 1/2) / n lies at least 1/(2n) from an
     // integer, far beyond the rounding of the quotient for the |jlo| < 4n that
-    // phi0 in [0, 2 pi) allows; then step through the panels with a wrap
-    const int n = g.n_panels;
-    int k = jlo - n * (int)floorf(((float)jlo + 0.5f) * __frcp_rn((float)n));
-    for (int j = jlo; j <= jhi && j < jlo + n; ++j) {
-        if (k != skip) panel_slab(g, k, x, y, z, dx, dy, dz, best, bi, bo);
-        k = k + 1 == n ? 0 : k + 1;
-    }
+    // phi0 in [0, 2 pi) allows
+    k = jlo - g.n_panels * (int)floorf(((float)jlo + 0.5f) * __frcp_rn((float)g.n_panels));
+    n = min(max(jhi - jlo + 1, 0), g.n_panels);
 }
 
 // Axial screen of a ray that starts inside the ring (c0 = x^2 + y^2 below
@@ -436,14 +441,23 @@ __device__ __forceinline__ bool inside_screened(const GeomDev &g, float z, float
 
 // The screen flight() applies first to a ray from (x, d): the same test,
 // for deciding at a photon's start that its flight cannot reach a panel.
+template <bool kPosed = true>
 __device__ __forceinline__ bool start_screened(const GeomDev &g, float x, float y, float z, float dx, float dy,
                                                float dz) {
-    if (g.posed || g.n_panels <= 2) return false;
+    if ((kPosed && g.posed) || g.n_panels <= 2) return false;
     const float c0 = fmaf(x, x, y * y);
     if (!(c0 < g.R2 * 0.9999f)) return false;
     const float a = fmaf(dx, dx, dy * dy), b = fmaf(x, dx, y * dy);
     float t1;
     return inside_screened(g, z, dz, a, b, c0, t1);
+}
+
+// Start outside the inner circle (c0 >= 0.9999 R^2): true when the ray is
+// beyond the outer circle and never comes back inside it (the circle is widened
+// by 1e-4 in r^2 so that rounding can only add candidates)
+__device__ __forceinline__ bool outside_screened(const GeomDev &g, float a, float b, float c0) {
+    const float cA = c0 - g.rout2 * 1.0001f;
+    return cA > 0.0f && (b >= 0.0f || fmaf(b, b, -a * cA) <= 0.0f);
 }
 
 // Line-plane flight (Sec. 2.1): nearest panel entered along (x, d), skipping
@@ -453,71 +467,81 @@ __device__ __forceinline__ bool start_screened(const GeomDev &g, float x, float 
 // for a ray that starts inside R, at most two (before and after it passes
 // inside R) for one that starts in or beyond the annulus.  Only panels whose
 // sector meets the azimuths of those stretches are slab-tested, which gives
-// the same result as testing all panels.
+// the same result as testing all panels.  All cases choose their candidates
+// first and share one slab-test loop, so that a warp's lanes test together and
+// the test's code is there once.  kPosed = false: no geometry of the launch
+// has panel poses.
+template <bool kPosed = true>
 __device__ __forceinline__ int flight(const GeomDev &g, float x, float y, float z, float dx, float dy, float dz,
                                       int skip, float &t_in, float &t_out) {
     int best = -1;
     float bi = 3.0e38f, bo = 0.0f;
-    const float c0 = fmaf(x, x, y * y);
-    const float a = fmaf(dx, dx, dy * dy);
-    const float b = fmaf(x, dx, y * dy);
-    if (g.posed) {
+    if (kPosed && g.posed) {
         // panels placed one by one: no ring symmetry to cull with
+#pragma unroll 1
         for (int k = 0; k < g.n_panels; ++k) {
             if (k == skip) continue;
             panel_slab_posed(g, k, x, y, z, dx, dy, dz, best, bi, bo);
         }
-    } else if (g.n_panels <= 2) {
-        for (int k = 0; k < g.n_panels; ++k) {
-            if (k == skip) continue;
-            panel_slab(g, k, x, y, z, dx, dy, dz, best, bi, bo);
-        }
-    } else if (c0 < g.R2 * 0.9999f) {
-        // parallel to the axis, or axially beyond the panels when it reaches
-        // the annulus: screened; else t1 = exit distance of the circle R
-        float t1 = 0.0f;
-        if (inside_screened(g, z, dz, a, b, c0, t1)) {
-            t_in = bi;
-            t_out = bo;
-            return kFlightScreened;
-        }
-        // exit distance of the circle R_out (stable root, c0 < R^2)
-        const float d2 = g.rout2 - c0;
-        const float s2 = sqrtf(fmaf(b, b, a * d2));
-        const float t2 = b > 0.0f ? __fdividef(d2, b + s2) : __fdividef(s2 - b, a);
-        flight_sector(g, x, y, z, dx, dy, dz, t1, t2, skip, best, bi, bo);
-    } else if (a > 0.0f) {
-        // start in or beyond the annulus; its circles are widened by 1e-4 in
-        // r^2 so that rounding can only add candidates
-        const float ro2 = g.rout2 * 1.0001f, ri2 = g.R2 * 0.9999f;
-        const float cA = c0 - ro2;
-        const float DA = fmaf(b, b, -a * cA);
-        if (cA > 0.0f && (b >= 0.0f || DA <= 0.0f)) {
-            t_in = bi;
-            t_out = bo;
-            return kFlightScreened;  // beyond the outer circle and never coming back inside it
-        }
-        const float sA = sqrtf(fmaxf(DA, 0.0f));
-        // roots tA <= tB of the outer circle (stable forms)
-        const float tB = b > 0.0f ? __fdividef(-cA, b + sA) : __fdividef(sA - b, a);
-        const float tA = b > 0.0f ? __fdividef(-(b + sA), a) : __fdividef(cA, sA - b);
-        const float t0 = fmaxf(tA, 0.0f);
-        const float cR = c0 - ri2;
-        const float DR = fmaf(b, b, -a * cR);
-        if (b < 0.0f && DR > 0.0f) {
-            // passes inside the inner circle between tC and tD
-            const float sR = sqrtf(DR);
-            const float tC = __fdividef(cR, sR - b), tD = __fdividef(sR - b, a);
-            flight_sector(g, x, y, z, dx, dy, dz, t0, tC, skip, best, bi, bo);
-            flight_sector(g, x, y, z, dx, dy, dz, tD, tB, skip, best, bi, bo);
+        t_in = bi;
+        t_out = bo;
+        return best;
+    }
+    t_in = bi;
+    t_out = bo;
+    const float c0 = fmaf(x, x, y * y);
+    const float a = fmaf(dx, dx, dy * dy);
+    const float b = fmaf(x, dx, y * dy);
+    float ta = 0.0f, tb = 0.0f;       // the stretch nearest in time, and the second one when there is one
+    float tc = 0.0f, td = 0.0f;
+    bool two = false;
+    const bool all = g.n_panels <= 2 || !(c0 < g.R2 * 0.9999f || a > 0.0f);
+    if (!all) {
+        if (c0 < g.R2 * 0.9999f) {
+            // parallel to the axis, or axially beyond the panels when it reaches
+            // the annulus: screened; else ta = exit distance of the circle R
+            if (inside_screened(g, z, dz, a, b, c0, ta)) return kFlightScreened;
+            // exit distance of the circle R_out (stable root, c0 < R^2)
+            const float d2 = g.rout2 - c0;
+            const float s2 = sqrtf(fmaf(b, b, a * d2));
+            tb = b > 0.0f ? __fdividef(d2, b + s2) : __fdividef(s2 - b, a);
         } else {
-            flight_sector(g, x, y, z, dx, dy, dz, t0, tB, skip, best, bi, bo);
+            // start in or beyond the annulus; its circles are widened by 1e-4 in
+            // r^2 so that rounding can only add candidates
+            const float ro2 = g.rout2 * 1.0001f, ri2 = g.R2 * 0.9999f;
+            const float cA = c0 - ro2;
+            const float DA = fmaf(b, b, -a * cA);
+            if (outside_screened(g, a, b, c0)) return kFlightScreened;
+            const float sA = sqrtf(fmaxf(DA, 0.0f));
+            // roots tA <= tB of the outer circle (stable forms)
+            tb = b > 0.0f ? __fdividef(-cA, b + sA) : __fdividef(sA - b, a);
+            const float tA = b > 0.0f ? __fdividef(-(b + sA), a) : __fdividef(cA, sA - b);
+            ta = fmaxf(tA, 0.0f);
+            const float cR = c0 - ri2;
+            const float DR = fmaf(b, b, -a * cR);
+            if (b < 0.0f && DR > 0.0f) {
+                // passes inside the inner circle between the end of the first
+                // stretch and the start of the second
+                const float sR = sqrtf(DR);
+                td = tb;
+                tb = __fdividef(cR, sR - b);
+                tc = __fdividef(sR - b, a);
+                two = true;
+            }
         }
-    } else {
-        for (int k = 0; k < g.n_panels; ++k) {
-            if (k == skip) continue;
-            panel_slab(g, k, x, y, z, dx, dy, dz, best, bi, bo);
+    }
+    for (;;) {
+        int k = 0, n = g.n_panels;
+        if (!all) flight_sector(g, x, y, dx, dy, ta, tb, k, n);
+#pragma unroll 1
+        for (; n > 0; --n) {
+            if (k != skip) panel_slab(g, k, x, y, z, dx, dy, dz, best, bi, bo);
+            k = k + 1 == g.n_panels ? 0 : k + 1;
         }
+        if (!two) break;
+        two = false;
+        ta = tc;
+        tb = td;
     }
     t_in = bi;
     t_out = bo;

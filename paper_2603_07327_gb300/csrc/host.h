@@ -62,8 +62,9 @@ struct RunCaps {
 struct RunHeader {
     // det_steps, flights, trials, entered, phantom_steps, hits, wavefront iterations,
     // wavefront lanes, screened flights, singles formed
-    // ... singles formed, then (CTA-synchronous kernel) the events run per phase in slots 10 + phase
-    unsigned long long counters[20];
+    // ... singles formed, then (slot-pool kernel) the events run per phase in slots 10 + phase
+    // [17, 20): a live launch's stalled wait; from kCtaCounters: the CTA kernel's own counts
+    unsigned long long counters[kCtaCounters + kCtaCounterSlots];
     unsigned long long n_singles, n_hits, n_ovf, n_sorted, n_coinc, next_chunk;
     int status;
     int pad[3];

@@ -18,6 +18,9 @@ struct LaunchCfg {
     int max_smem_geoms;  // geometry descriptors staged in shared memory
     int compact_every;   // wavefront regrouping interval (events)
     int pool_depth;      // wavefront slots per lane (pool = 32 x depth histories per warp)
+    bool phantom;        // a job of the launch has a phantom, or one may be appended
+    bool posed;          // a geometry of the launch has panel poses, or one may be appended
+    bool live;           // a live launch
 };
 
 // radix sort working set (keys ping-pong between two buffers)
@@ -135,7 +138,12 @@ cudaError_t launch_transport_cta(const WorkDev &W, const OutDev &O, const Launch
 // warps resident at once in the transport launch that cfg selects (sizes the work chunks)
 cudaError_t transport_resident_warps(int n_geoms, const LaunchCfg &cfg, long long *warps);
 cudaError_t wave_resident_warps(int n_geoms, const LaunchCfg &cfg, long long *warps);
+constexpr int kCtaThreads = 448;   // threads per CTA of the CTA kernel's default shape
 cudaError_t cta_resident_warps(int n_geoms, const LaunchCfg &cfg, long long *warps);
+// the CTA kernel's own counts (raw, kCtaCounterSlots of them behind the launch's first kCtaCounters) added to
+// the launch's counters (host)
+constexpr int kCtaCounters = 20, kCtaCounterSlots = 16;
+void cta_counters(unsigned long long *counters, const unsigned long long *raw);
 cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const CoincDev &C, int sm_count,
                               cudaStream_t st);
 cudaError_t launch_radix_passes(const SortDev &S, int sm_count, cudaStream_t st);

@@ -78,11 +78,11 @@ int run_default_cfg(Run &R, const gpet_options *opt_in, const gpet_scanner *sc) 
     R.cfg.kernel = (opt && opt->kernel > 0) ? opt->kernel : kKernelCta;
     if (R.cfg.kernel != kKernelLoop && R.cfg.kernel != kKernelWave && R.cfg.kernel != kKernelCta)
         return gpet_fail(GPET_ERR_INVALID_ARG, "kernel %d not in {1, 2, 3}", R.cfg.kernel);
-    // CTA-synchronous kernel: CTAs of 128, 256 or 512 threads; others <= 256
-    R.cfg.block_size = (opt && opt->block_size > 0) ? opt->block_size : 256;
-    if (R.cfg.kernel == kKernelCta
-            ? (R.cfg.block_size != 128 && R.cfg.block_size != 256 && R.cfg.block_size != 512)
-            : (R.cfg.block_size % 32 || R.cfg.block_size > 256))
+    // CTA kernel: CTAs of 128, 256 or 512 threads, or its default shape; others <= 256
+    R.cfg.block_size = (opt && opt->block_size > 0) ? opt->block_size : R.cfg.kernel == kKernelCta ? kCtaThreads : 256;
+    if (R.cfg.kernel == kKernelCta ? (opt && opt->block_size > 0 && R.cfg.block_size != 128 && R.cfg.block_size != 256 &&
+                                      R.cfg.block_size != 512)
+                                   : (R.cfg.block_size % 32 || R.cfg.block_size > 256))
         return gpet_fail(GPET_ERR_INVALID_ARG, "block_size %d not valid for kernel %d", R.cfg.block_size,
                          R.cfg.kernel);
     const int bps = (opt && opt->blocks_per_sm > 0) ? opt->blocks_per_sm : 4;
@@ -122,7 +122,13 @@ int run_plan(Run &R) {
     const int64_t tcc = R.live ? std::max<int64_t>(tc, R.live_cap.crystals) : tc;
     R.live_tally_used = tc;
     uint64_t total = 0;
-    for (auto &J : R.jobs) total += J.n_hist;
+    R.cfg.live = R.live;
+    R.cfg.phantom = R.cfg.posed = R.live;
+    for (const GeomDev &g : R.geoms) R.cfg.posed = R.cfg.posed || g.posed;
+    for (auto &J : R.jobs) {
+        total += J.n_hist;
+        R.cfg.phantom = R.cfg.phantom || J.has_phantom || J.src_kind == GPET_SOURCE_PHANTOM;
+    }
     uint64_t cs = R.live_cap.chunk;
     if (!R.live && !R.digitize_only) {
         // chunks: about 48 per resident warp, so that warps run out of work
@@ -426,6 +432,7 @@ int run_collect(Run &R) {
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(rs);
     if (e != cudaSuccess) return gpet_cuda_fail(e, "run read-back");
+    cta_counters(R.h_hdr.counters, R.h_hdr.counters + kCtaCounters);
     if (R.ev[0] && cudaEventElapsedTime(&R.transport_ms, R.ev[0], R.ev[1]) != cudaSuccess) {
         R.transport_ms = -1.f;
         cudaGetLastError();  // a missing stage time is not an error of the run: clear it
@@ -508,7 +515,8 @@ int run_with_retry(Run &R) {
             R.caps.guess = false;
             R.caps.singles = std::max<uint64_t>(R.caps.singles, R.h_hdr.n_singles + 1024);
             R.caps.hits = std::max<uint64_t>(R.caps.hits, R.h_hdr.n_hits + 1024);
-            R.caps.ovf = std::max<uint64_t>(R.caps.ovf, R.h_hdr.n_ovf + 1024);
+            // (which lists overflow can depend on the launch's schedule: with room to spare)
+            R.caps.ovf = std::max<uint64_t>(R.caps.ovf, R.h_hdr.n_ovf + R.h_hdr.n_ovf / 4 + 4096);
             run_release(R);
             continue;
         }

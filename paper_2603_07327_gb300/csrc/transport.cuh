@@ -1,6 +1,6 @@
 // transport.cuh -- per-history photon-pair transport as a set of events that
 // advance one history by one step.  Every transport kernel (the per-lane event
-// loop, the per-warp wavefront, the CTA-synchronous wavefront and the overflow
+// loop, the per-warp wavefront, the slot-pool kernel and the overflow
 // re-simulation) runs these same events, so they produce identical histories.
 //
 // Paper anchors (arxiv 2603.07327): Sec. 2.1 (flight by line-plane
@@ -167,6 +167,7 @@ __device__ __forceinline__ void warp_refill(const WorkDev &W, uint32_t need, Ref
     const int lane = threadIdx.x & 31;
     got = false;
     R.waiting = false;
+#pragma unroll 1
     while (need && !R.exhausted) {
         const uint64_t avail = R.end - R.next;
         if (avail == 0) {
@@ -187,6 +188,7 @@ __device__ __forceinline__ void warp_refill(const WorkDev &W, uint32_t need, Ref
                 // fixed launch bisects the whole table (cached in L1; measured
                 // faster there).
                 int lo = kLive ? R.job : 0, hi = W.n_jobs - 1, step = 1;
+#pragma unroll 1
                 while (kLive && lo < hi) {
                     const int probe = min(lo + step, hi);
                     if (table_load<kLive>(W.chunk_start + probe) <= c) {
@@ -197,6 +199,7 @@ __device__ __forceinline__ void warp_refill(const WorkDev &W, uint32_t need, Ref
                         break;
                     }
                 }
+#pragma unroll 1
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
                     if (table_load<kLive>(W.chunk_start + mid) <= c) lo = mid; else hi = mid - 1;
@@ -285,8 +288,9 @@ struct Counters {
     uint32_t src, fl_ev, fl_out, fin;
 };
 
+template <bool kPosed = true>
 __device__ __forceinline__ void to_global(const GeomDev &g, PState &s) {
-    if (g.posed) {
+    if (kPosed && g.posed) {
         const float4 aw = __ldg(g.pose + 4 * s.panel), au = __ldg(g.pose + 4 * s.panel + 1);
         const float4 av = __ldg(g.pose + 4 * s.panel + 2), o = __ldg(g.pose + 4 * s.panel + 3);
         const float w = s.x, u = s.y, v = s.z, dw = s.dx, du = s.dy, dv = s.dz;
@@ -359,6 +363,7 @@ __device__ __forceinline__ int64_t pick_voxel(const JobDev &J, double target) {
         lo = __ldg(J.ph_guide + b);
         if (b + 1 < J.ph_buckets) hi = min(hi, (int64_t)__ldg(J.ph_guide + b + 1));
     }
+#pragma unroll 1
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
         if (__ldg(J.ph_cdf + mid) > target) hi = mid; else lo = mid + 1;
@@ -366,15 +371,20 @@ __device__ __forceinline__ int64_t pick_voxel(const JobDev &J, double target) {
     return lo;
 }
 
-// decay of history h (Sec. 2.3): time, annihilation point, photon-0 direction
-__device__ __forceinline__ void ev_source(const JobDev &J, const GeomDev &g, PState &s, Counters &cnt) {
-    cnt.src++;
-    const uint4 r = draw(J.seed, s.h, kTagSource, 0u, 0u, 0u);
-    const uint64_t r64 = ((uint64_t)r.x << 32) | r.y;
-    s.t0 = __umul64hi(J.t_span_ps, r64);
-    if (J.src_kind == 1) {
-        const uint4 q = draw(J.seed, s.h, kTagSource, 0u, 0u, 1u);
-        const uint4 zq = draw(J.seed, s.h, kTagSource, 0u, 0u, 2u);
+// decay time (ps) of history h, from the first draw of its decay
+__device__ __forceinline__ uint64_t decay_time(const JobDev &J, const uint4 r) {
+    return __umul64hi(J.t_span_ps, ((uint64_t)r.x << 32) | r.y);
+}
+
+// decay of history h (Sec. 2.3) from its first draw r and its azimuth (sine
+// sp, cosine cp of 2 pi u01(r.w)): annihilation point (x0, y0, z0), photon-0
+// direction (ox, oy, oz).  kMap: an activity map may be the source.
+template <bool kMap = true>
+__device__ __forceinline__ void sample_decay(const JobDev &J, uint64_t h, const uint4 r, float sp, float cp, float &x0,
+                                             float &y0, float &z0, float &ox, float &oy, float &oz) {
+    if (kMap && J.src_kind == 1) {
+        const uint4 q = draw(J.seed, h, kTagSource, 0u, 0u, 1u);
+        const uint4 zq = draw(J.seed, h, kTagSource, 0u, 0u, 2u);
         const uint64_t r53 = ((uint64_t)q.x << 21) | (q.y >> 11);
         const double target = (double)r53 * 0x1p-53 * J.ph_total;
         const int64_t vi = pick_voxel(J, target);
@@ -386,42 +396,50 @@ __device__ __forceinline__ void ev_source(const JobDev &J, const GeomDev &g, PSt
         } else {
             ix = vi % J.ph_nx; iy = (vi / J.ph_nx) % J.ph_ny; iz = vi / ((int64_t)J.ph_nx * J.ph_ny);
         }
-        s.x0 = fmaf((float)ix + u01(q.z), J.ph_voxel[0], J.ph_origin[0]);
-        s.y0 = fmaf((float)iy + u01(q.w), J.ph_voxel[1], J.ph_origin[1]);
-        s.z0 = fmaf((float)iz + u01(zq.x), J.ph_voxel[2], J.ph_origin[2]);
+        x0 = fmaf((float)ix + u01(q.z), J.ph_voxel[0], J.ph_origin[0]);
+        y0 = fmaf((float)iy + u01(q.w), J.ph_voxel[1], J.ph_origin[1]);
+        z0 = fmaf((float)iz + u01(zq.x), J.ph_voxel[2], J.ph_origin[2]);
     } else {
-        s.x0 = J.src_pos[0]; s.y0 = J.src_pos[1]; s.z0 = J.src_pos[2];
+        x0 = J.src_pos[0]; y0 = J.src_pos[1]; z0 = J.src_pos[2];
     }
     if (J.src_kind == 2) {
-        s.ox = J.src_dir[0]; s.oy = J.src_dir[1]; s.oz = J.src_dir[2];
+        ox = J.src_dir[0]; oy = J.src_dir[1]; oz = J.src_dir[2];
     } else {
         const float ct = 2.0f * u01(r.z) - 1.0f;
         const float st = sqrtf((1.0f - ct) * (1.0f + ct));
-        float sp, cp;
-        sincospif(2.0f * u01(r.w), &sp, &cp);
-        s.ox = st * cp; s.oy = st * sp; s.oz = ct;
+        ox = st * cp; oy = st * sp; oz = ct;
     }
+}
+
+__device__ __forceinline__ void ev_source(const JobDev &J, const GeomDev &g, PState &s, Counters &cnt) {
+    cnt.src++;
+    const uint4 r = draw(J.seed, s.h, kTagSource, 0u, 0u, 0u);
+    s.t0 = decay_time(J, r);
+    float sp, cp;
+    sincospif(2.0f * u01(r.w), &sp, &cp);
+    sample_decay(J, s.h, r, sp, cp, s.x0, s.y0, s.z0, s.ox, s.oy, s.oz);
     s.gamma = 0;
     s.nsing = 0;
     s.ovf = 0;
     start_photon(J, g, s, cnt);
 }
 
-// one Woodcock step in the voxel phantom
-__device__ __forceinline__ int ev_phantom(const JobDev &J, const GeomDev &g, const WorkDev &W, PState &s,
-                                          Counters &cnt) {
-    if (s.sph >= (uint32_t)kMaxSteps) return kStatusTimeout;
-    const uint4 r = draw(J.seed, s.h, kTagPhantom, s.gamma, s.sph, 0u);
-    const uint32_t step_id = s.sph++;
-    cnt.ph_steps++;
+// outcome of a Woodcock step: left the region, a virtual collision, a
+// photoelectric absorption or a Compton scatter
+enum : int { kStepExit = 0, kStepVirtual = 1, kStepPhoto = 2, kStepCompton = 3 };
+
+// one Woodcock step in the voxel phantom with draw r: moves the photon
+// (x, path) to its collision point or to the grid's exit
+__device__ __forceinline__ int phantom_step(const JobDev &J, const WorkDev &W, const uint4 r, PState &s) {
     // distance to the grid box exit
     float t_out = 3.0e38f;
-    if (s.dx > 0.f) t_out = fminf(t_out, (J.ph_hi[0] - s.x) / s.dx); else if (s.dx < 0.f) t_out = fminf(t_out, (J.ph_origin[0] - s.x) / s.dx);
-    if (s.dy > 0.f) t_out = fminf(t_out, (J.ph_hi[1] - s.y) / s.dy); else if (s.dy < 0.f) t_out = fminf(t_out, (J.ph_origin[1] - s.y) / s.dy);
-    if (s.dz > 0.f) t_out = fminf(t_out, (J.ph_hi[2] - s.z) / s.dz); else if (s.dz < 0.f) t_out = fminf(t_out, (J.ph_origin[2] - s.z) / s.dz);
+    if (s.dx != 0.f) t_out = fminf(t_out, ((s.dx > 0.f ? J.ph_hi[0] : J.ph_origin[0]) - s.x) / s.dx);
+    if (s.dy != 0.f) t_out = fminf(t_out, ((s.dy > 0.f ? J.ph_hi[1] : J.ph_origin[1]) - s.y) / s.dy);
+    if (s.dz != 0.f) t_out = fminf(t_out, ((s.dz > 0.f ? J.ph_hi[2] : J.ph_origin[2]) - s.z) / s.dz);
     t_out = fmaxf(t_out, 0.0f);
     const Xs xs = xs_at(s.E, W.gtab, W.ln_emin, W.inv_h);
     float mu_maj = 0.0f;
+#pragma unroll 1
     for (int m = 0; m < J.ph_nmat; ++m) mu_maj = fmaxf(mu_maj, mu_total(J.ph_mu_c511[m], J.ph_mu_pe511[m], xs));
     // free path -ln(u) / mu: the fast log's absolute error (< 4e-7) moves a
     // step by < 5e-5 mm even in water, far below the position tolerance
@@ -429,8 +447,7 @@ __device__ __forceinline__ int ev_phantom(const JobDev &J, const GeomDev &g, con
     if (step >= t_out) {
         s.x = fmaf(t_out, s.dx, s.x); s.y = fmaf(t_out, s.dy, s.y); s.z = fmaf(t_out, s.dz, s.z);
         s.path += t_out;
-        s.phase = kPhFlight;
-        return kStatusOk;
+        return kStepExit;
     }
     s.x = fmaf(step, s.dx, s.x); s.y = fmaf(step, s.dy, s.y); s.z = fmaf(step, s.dz, s.z);
     s.path += step;
@@ -441,36 +458,41 @@ __device__ __forceinline__ int ev_phantom(const JobDev &J, const GeomDev &g, con
     const int m = __ldg(J.ph_mat + ((int64_t)iz * J.ph_ny + iy) * J.ph_nx + ix);
     const float pe = J.ph_mu_pe511[m] * xs.r3;
     const float mu_m = fmaf(J.ph_mu_c511[m], xs.g, pe);
-    if (u01(r.y) * mu_maj >= mu_m) return kStatusOk;          // virtual
-    if (u01(r.z) * mu_m < pe) { photon_done(J, g, s, cnt); return kStatusOk; }   // photoelectric
+    if (u01(r.y) * mu_maj >= mu_m) return kStepVirtual;
+    return u01(r.z) * mu_m < pe ? kStepPhoto : kStepCompton;
+}
+
+__device__ __forceinline__ int ev_phantom(const JobDev &J, const GeomDev &g, const WorkDev &W, PState &s,
+                                          Counters &cnt) {
+    if (s.sph >= (uint32_t)kMaxSteps) return kStatusTimeout;
+    const uint4 r = draw(J.seed, s.h, kTagPhantom, s.gamma, s.sph, 0u);
+    const uint32_t step_id = s.sph++;
+    cnt.ph_steps++;
+    const int what = phantom_step(J, W, r, s);
+    if (what == kStepExit) { s.phase = kPhFlight; return kStatusOk; }
+    if (what == kStepVirtual) return kStatusOk;
+    if (what == kStepPhoto) { photon_done(J, g, s, cnt); return kStatusOk; }
     float xm1;                                                   // Compton (Klein-Nishina)
     const int nt = kahn_sample(J.seed, s.h, kTagPhantom, s.gamma, step_id, s.E, xm1);
     if (nt < 0) return kStatusTimeout;
     cnt.trials += (uint32_t)nt;
     const float omc = xm1 / (s.E * kInvMec2);
-    rotate_dir(s.dx, s.dy, s.dz, omc, u01(r.w));
+    float sp, cp;
+    sincospif(2.0f * u01(r.w), &sp, &cp);
+    rotate_dir(s.dx, s.dy, s.dz, omc, sp, cp);
     const float Ep = s.E / (1.0f + xm1);
     if (Ep < J.e_cut) { photon_done(J, g, s, cnt); return kStatusOk; }
     s.E = Ep;
     return kStatusOk;
 }
 
-// flight to the next panel by line-plane intersection
-__device__ __forceinline__ void ev_flight(const JobDev &J, const GeomDev &g, PState &s, Counters &cnt) {
-    cnt.flights++;
-    cnt.fl_ev++;
-    float t_in, t_out;
-    const int k = flight(g, s.x, s.y, s.z, s.dx, s.dy, s.dz, s.last, t_in, t_out);
-    if (k < 0) {
-        if (k == kFlightScreened) cnt.screened++;
-        photon_done(J, g, s, cnt);
-        return;
-    }
-    cnt.entered++;
-    // entry point, then the panel-local frame (w, u, v)
+// the photon at panel k's box, t_in along its ray, in the panel-local frame
+// (w, u, v)
+template <bool kPosed = true>
+__device__ __forceinline__ void enter_panel(const GeomDev &g, int k, float t_in, PState &s) {
     const float ex = fmaf(t_in, s.dx, s.x), ey = fmaf(t_in, s.dy, s.y), ez = fmaf(t_in, s.dz, s.z);
     s.path += t_in;
-    if (g.posed) {
+    if (kPosed && g.posed) {
         const float4 aw = __ldg(g.pose + 4 * k), au = __ldg(g.pose + 4 * k + 1), av = __ldg(g.pose + 4 * k + 2);
         const float dw = fmaf(s.dx, aw.x, fmaf(s.dy, aw.y, s.dz * aw.z));
         const float du = fmaf(s.dx, au.x, fmaf(s.dy, au.y, s.dz * au.z));
@@ -487,6 +509,21 @@ __device__ __forceinline__ void ev_flight(const JobDev &J, const GeomDev &g, PSt
         s.x = w; s.y = u; s.z = ez;
         s.dx = dw; s.dy = du;
     }
+}
+
+// flight to the next panel by line-plane intersection
+__device__ __forceinline__ void ev_flight(const JobDev &J, const GeomDev &g, PState &s, Counters &cnt) {
+    cnt.flights++;
+    cnt.fl_ev++;
+    float t_in, t_out;
+    const int k = flight(g, s.x, s.y, s.z, s.dx, s.dy, s.dz, s.last, t_in, t_out);
+    if (k < 0) {
+        if (k == kFlightScreened) cnt.screened++;
+        photon_done(J, g, s, cnt);
+        return;
+    }
+    cnt.entered++;
+    enter_panel(g, k, t_in, s);
     s.trem = t_out - t_in;
     s.panel = k;
     s.phase = kPhPanel;
@@ -518,6 +555,23 @@ __device__ __forceinline__ void add_single(const GeomDev &g, PState &s, const Si
     }
 }
 
+// one crystal interaction of s into the optional hit list
+__device__ __forceinline__ void store_hit(const OutDev &O, const PState &s, int crystal, int layer, uint32_t step_id,
+                                          float dep, uint32_t dtp) {
+    const unsigned long long slot = atomicAdd(O.n_hits, 1ull);
+    if (slot >= O.hit_cap) return;
+    O.hit_h[slot] = s.h;
+    O.hit_t[slot] = s.t0 + dtp;
+    O.hit_gstep[slot] = (int32_t)((s.gamma << 24) | step_id);
+    O.hit_crystal[slot] = crystal;
+    O.hit_layer[slot] = layer;
+    O.hit_job[slot] = s.job;
+    O.hit_wuv[3 * slot] = s.x;
+    O.hit_wuv[3 * slot + 1] = s.y;
+    O.hit_wuv[3 * slot + 2] = s.z;
+    O.hit_e[slot] = dep;
+}
+
 // a crystal interaction: tallies, optional hit list, singles list of the history
 template <bool kTallies>
 __device__ __forceinline__ void record_hit(const JobDev &J, const GeomDev &g, const OutDev &O, PState &s,
@@ -528,23 +582,39 @@ __device__ __forceinline__ void record_hit(const JobDev &J, const GeomDev &g, co
     if (kTallies) {
         atomicAdd(J.tally_count + crystal, 1ull);
         atomicAdd(J.tally_efx + crystal, (unsigned long long)__float2ull_rn(dep * kEfxScale));
-        if (O.hit_cap) {
-            const unsigned long long slot = atomicAdd(O.n_hits, 1ull);
-            if (slot < O.hit_cap) {
-                O.hit_h[slot] = s.h;
-                O.hit_t[slot] = s.t0 + dtp;
-                O.hit_gstep[slot] = (int32_t)((s.gamma << 24) | step_id);
-                O.hit_crystal[slot] = crystal;
-                O.hit_layer[slot] = layer;
-                O.hit_job[slot] = s.job;
-                O.hit_wuv[3 * slot] = s.x;
-                O.hit_wuv[3 * slot + 1] = s.y;
-                O.hit_wuv[3 * slot + 2] = s.z;
-                O.hit_e[slot] = dep;
-            }
-        }
+        if (O.hit_cap) store_hit(O, s, crystal, layer, step_id, dep, dtp);
     }
     add_single(g, s, SL, max_entries, crystal, module, dep, dtp, s.x);
+}
+
+// one Woodcock step inside the current panel with draw r: moves the photon
+// (x, path) to its collision point L or to the panel's exit
+// (left_ring: the photon left it through the back and can meet no other panel)
+template <bool kPosed = true>
+__device__ __forceinline__ int panel_step(const GeomDev &g, const WorkDev &W, const uint4 r, PState &s, Loc &L,
+                                          bool &left_ring) {
+    const Xs xs = xs_at(s.E, W.gtab, W.ln_emin, W.inv_h);
+    float mu_maj = 0.0f;
+#pragma unroll 1
+    for (int m = 0; m < g.n_materials; ++m) mu_maj = fmaxf(mu_maj, mu_total(g.mu_c511[m], g.mu_pe511[m], xs));
+    // free path -ln(u) / mu: the fast log's absolute error (< 4e-7) moves a
+    // step by < 5e-5 mm even in water, far below the position tolerance
+    const float step = mu_maj > 0.0f ? -__logf(u01(r.x)) * (10.0f / mu_maj) : 3.0e38f;
+    if (step >= s.trem) {                      // leaves the panel: back to flight
+        s.x = fmaf(s.trem, s.dx, s.x); s.y = fmaf(s.trem, s.dy, s.y); s.z = fmaf(s.trem, s.dz, s.z);
+        s.path += s.trem;
+        left_ring = s.x >= g.w_clear && s.dx >= 0.0f;
+        to_global<kPosed>(g, s);
+        return kStepExit;
+    }
+    s.x = fmaf(step, s.dx, s.x); s.y = fmaf(step, s.dy, s.y); s.z = fmaf(step, s.dz, s.z);
+    s.path += step;
+    s.trem -= step;
+    L = locate(g, s.panel, s.x, s.y, s.z);
+    const float pe = g.mu_pe511[L.mat] * xs.r3;
+    const float mu_m = fmaf(g.mu_c511[L.mat], xs.g, pe);
+    if (u01(r.y) * mu_maj >= mu_m) return kStepVirtual;
+    return u01(r.z) * mu_m < pe ? kStepPhoto : kStepCompton;
 }
 
 // one Woodcock step inside the current panel (layer selection, interaction, hit)
@@ -555,31 +625,19 @@ __device__ __forceinline__ int ev_panel(const JobDev &J, const GeomDev &g, const
     const uint4 r = draw(J.seed, s.h, kTagDetector, s.gamma, s.sdet, 0u);
     const uint32_t step_id = s.sdet++;
     cnt.det_steps++;
-    const Xs xs = xs_at(s.E, W.gtab, W.ln_emin, W.inv_h);
-    float mu_maj = 0.0f;
-    for (int m = 0; m < g.n_materials; ++m) mu_maj = fmaxf(mu_maj, mu_total(g.mu_c511[m], g.mu_pe511[m], xs));
-    // free path -ln(u) / mu: the fast log's absolute error (< 4e-7) moves a
-    // step by < 5e-5 mm even in water, far below the position tolerance
-    const float step = mu_maj > 0.0f ? -__logf(u01(r.x)) * (10.0f / mu_maj) : 3.0e38f;
-    if (step >= s.trem) {                      // leaves the panel: back to flight
-        s.x = fmaf(s.trem, s.dx, s.x); s.y = fmaf(s.trem, s.dy, s.y); s.z = fmaf(s.trem, s.dz, s.z);
-        s.path += s.trem;
-        to_global(g, s);
+    Loc L;
+    bool left_ring;
+    const int what = panel_step(g, W, r, s, L, left_ring);
+    if (what == kStepExit) {
         s.last = s.panel;
         s.panel = -1;
         s.phase = kPhFlightOut;
         return kStatusOk;
     }
-    s.x = fmaf(step, s.dx, s.x); s.y = fmaf(step, s.dy, s.y); s.z = fmaf(step, s.dz, s.z);
-    s.path += step;
-    s.trem -= step;
-    const Loc L = locate(g, s.panel, s.x, s.y, s.z);
-    const float pe = g.mu_pe511[L.mat] * xs.r3;
-    const float mu_m = fmaf(g.mu_c511[L.mat], xs.g, pe);
-    if (u01(r.y) * mu_maj >= mu_m) return kStatusOk;   // virtual
+    if (what == kStepVirtual) return kStatusOk;
     float dep;
     bool dead = false;
-    if (u01(r.z) * mu_m < pe) {                        // photoelectric
+    if (what == kStepPhoto) {
         dep = s.E;
         dead = true;
     } else {                                           // Compton (Klein-Nishina)
@@ -591,7 +649,9 @@ __device__ __forceinline__ int ev_panel(const JobDev &J, const GeomDev &g, const
         // rotation in the panel frame with v as polar reference: for the ring
         // (w, u, v) is a rotation of (x, y, z) about the axis, so this equals the
         // global rotation; a posed panel takes its own v axis
-        rotate_dir(s.dx, s.dy, s.dz, omc, u01(r.w));
+        float sp, cp;
+        sincospif(2.0f * u01(r.w), &sp, &cp);
+        rotate_dir(s.dx, s.dy, s.dz, omc, sp, cp);
         const float Ep = s.E / (1.0f + xm1);
         if (Ep < J.e_cut) {
             dep = s.E;
@@ -608,101 +668,145 @@ __device__ __forceinline__ int ev_panel(const JobDev &J, const GeomDev &g, const
     return kStatusOk;
 }
 
-// digitizer for one finished history: blur, window, warp-aggregated append
-// (call with the lanes of `mask` converged; `active` lanes own a history).
+// one single of a finished history: readout unit, raw and blurred energy,
+// blurred depth, earliest time offset, and whether the energy window keeps it
+struct SingleOut {
+    bool keep;
+    uint32_t unit, dt;
+    float e, eb, db;
+};
+
+// draw of the blur of history h's single in readout unit `unit`
+__device__ __forceinline__ uint4 draw_blur(const JobDev &J, uint64_t h, uint32_t unit) {
+    return philox4x32_10(make_uint4((uint32_t)h, (uint32_t)(h >> 32), kTagDigi << 28, unit),
+                         make_uint2((uint32_t)J.seed, (uint32_t)(J.seed >> 32)));
+}
+
+// digitizer of one single: energy e deposited in `unit`, energy x depth ew,
+// with its draw q and (sp, cp) = sine and cosine of 2 pi u01(q.y).
+// One Box-Muller pair: the cosine normal blurs the energy, the sine one the depth.
+__device__ __forceinline__ void blur_single(const JobDev &J, const uint4 q, float sp, float cp, uint32_t unit, float e,
+                                            uint32_t dt, float ew, SingleOut &o) {
+    o.unit = unit;
+    o.e = e;
+    o.dt = dt;
+    // the accurate log here: near u = 1 the radius is small and an
+    // absolute log error would become a large relative error of the blur
+    const float rad = sqrtf(-2.0f * logf(u01(q.x)));
+    const float sigma = J.sig_k * sqrtf(kE0 * e);
+    o.eb = fmaf(sigma, rad * cp, e);
+    o.db = fmaf(J.sig_doi, rad * sp, ew / e);
+    o.keep = o.eb >= J.e_lo && o.eb <= J.e_hi;
+}
+
+// a kept single's record
+__device__ __forceinline__ void write_single(const GeomDev &g, RawSingle *dst, int job, uint64_t h, uint64_t t,
+                                             const SingleOut &o) {
+    // units per panel: 1, its modules, or its crystals
+    const uint32_t per = g.readout_level == 0 ? 1u : (uint32_t)(g.modules_u * g.modules_v) *
+                                                         (g.readout_level == 1 ? 1u : (uint32_t)g.crystals_per_module);
+    const int panel = (int)(o.unit / per);
+    uint4 *r = reinterpret_cast<uint4 *>(dst);
+    r[0] = make_uint4((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)h, (uint32_t)(h >> 32));
+    r[1] = make_uint4(o.unit, (uint32_t)panel, (uint32_t)job, __float_as_uint(o.eb));
+    r[2] = make_uint4(__float_as_uint(o.e), __float_as_uint(o.db), 0u, 0u);
+}
+
+// a kept single at slot `slot` of the launch's buffer: record and sort key
+__device__ __forceinline__ void store_single(const GeomDev *__restrict__ geoms, const OutDev &O, const JobDev &J, int job,
+                                             uint64_t h, uint64_t t, const SingleOut &o, unsigned long long slot) {
+    if (slot >= O.s_cap) return;
+    O.s_keys[slot] = O.key_shift < 64 ? ((uint64_t)job << O.key_shift) | t : t;
+    write_single(geoms[J.geom], O.s_raw + slot, job, h, t, o);
+}
+
+// Append the kept singles of a warp (call with the lanes of `mask` converged):
+// warp-aggregated slots, one record and one sort key each.
 // kJobDest = false: no job of the launch has a singles buffer of its own
 // (every fixed launch), and the singles go to the launch's buffer alone.
+// kDrawTime: the decay time is drawn again here (t0 ignored).
+template <bool kJobDest, bool kDrawTime>
+__device__ __forceinline__ void append_single(const GeomDev *__restrict__ geoms, const OutDev &O, const JobDev &J,
+                                              int job, uint64_t h, uint64_t t0, const SingleOut &o, uint32_t mask) {
+    const int lane = threadIdx.x & 31;
+    const bool keep = o.keep;
+    const uint32_t b = __ballot_sync(mask, keep);
+    if (!b) return;
+    // destination: the launch's singles buffer, or the job's own
+    RawSingle *dst = O.s_raw;
+    unsigned long long *dst_n = O.n_singles, dst_cap = O.s_cap;
+    if (kJobDest && keep && J.s_raw) {
+        dst = J.s_raw;
+        dst_n = J.n_singles;
+        dst_cap = J.s_cap;
+    }
+    unsigned long long slot = 0;
+    if (!kJobDest || __all_sync(mask, dst_n == O.n_singles)) {
+        // one counter for the warp (every fixed launch)
+        unsigned long long base = 0;
+        const int leader = __ffs(b) - 1;
+        if (lane == leader) base = atomicAdd(O.n_singles, (unsigned long long)__popc(b));
+        base = __shfl_sync(mask, base, leader);
+        slot = base + __popc(b & lanemask_lt());
+    } else if (keep) {
+        // lanes grouped by destination, one atomic per group
+        const uint32_t grp = __match_any_sync(b, reinterpret_cast<unsigned long long>(dst_n));
+        const int leader = __ffs(grp) - 1;
+        unsigned long long base = 0;
+        if (lane == leader) base = atomicAdd(dst_n, (unsigned long long)__popc(grp));
+        base = __shfl_sync(grp, base, leader);
+        slot = base + __popc(grp & lanemask_lt());
+    }
+    if (!keep || slot >= dst_cap) return;
+    if (kDrawTime) t0 = decay_time(J, draw(J.seed, h, kTagSource, 0u, 0u, 0u));
+    const uint64_t t = t0 + o.dt;
+    if (kJobDest && J.s_raw) {
+        // a job with its own buffer is job 0 of the one-job run that buffer belongs to
+        J.s_keys[slot] = t;
+        write_single(geoms[J.geom], dst + slot, 0, h, t, o);
+    } else {
+        store_single(geoms, O, J, job, h, t, o, slot);
+    }
+}
+
+// histories whose singles list overflowed go to the list of the re-simulation
+// kernel (call with the lanes of `mask` converged)
+__device__ __forceinline__ void append_overflow(const OutDev &O, bool ovf, uint64_t h, int job, uint32_t mask) {
+    const uint32_t b = __ballot_sync(mask, ovf);
+    if (!b) return;
+    unsigned long long base = 0;
+    const int leader = __ffs(b) - 1;
+    if ((int)(threadIdx.x & 31) == leader) base = atomicAdd(O.n_ovf, (unsigned long long)__popc(b));
+    base = __shfl_sync(mask, base, leader);
+    if (ovf) {
+        const unsigned long long slot = base + __popc(b & lanemask_lt());
+        if (slot < O.ovf_cap) { O.ovf_h[slot] = h; O.ovf_job[slot] = job; }
+    }
+}
+
+// digitizer for one finished history: every single of its list (call with the
+// lanes of `mask` converged; `active` lanes own a history)
 template <bool kJobDest = true>
 __device__ __forceinline__ void ev_finish(const JobDev *__restrict__ jobs, const GeomDev *__restrict__ geoms,
                                           const OutDev &O, const PState &s, bool active, const SinglesList &SL,
                                           uint32_t mask, Counters &cnt) {
-    const int lane = threadIdx.x & 31;
-    const JobDev *J = active ? &jobs[s.job] : nullptr;
+    const JobDev &J = jobs[active ? s.job : 0];
     const bool ovf = active && s.ovf;
     const uint32_t n = (active && !ovf) ? s.nsing : 0u;
     cnt.singles += n;
-    // histories whose list overflowed go to the fallback list instead
-    {
-        const uint32_t b = __ballot_sync(mask, ovf);
-        if (b) {
-            unsigned long long base = 0;
-            const int leader = __ffs(b) - 1;
-            if (lane == leader) base = atomicAdd(O.n_ovf, (unsigned long long)__popc(b));
-            base = __shfl_sync(mask, base, leader);
-            if (ovf) {
-                const unsigned long long slot = base + __popc(b & lanemask_lt());
-                if (slot < O.ovf_cap) { O.ovf_h[slot] = s.h; O.ovf_job[slot] = s.job; }
-            }
-        }
-    }
+    append_overflow(O, ovf, s.h, s.job, mask);
     const uint32_t nmax = __reduce_max_sync(mask, n);
     for (uint32_t j = 0; j < nmax; ++j) {
-        bool keep = false;
-        float e = 0.f, eb = 0.f, db = 0.f;
-        uint32_t unit = 0, dt = 0;
+        SingleOut o;
+        o.keep = false;
         if (j < n) {
-            unit = SL.unit[j * SL.stride];
-            e = SL.e[j * SL.stride];
-            dt = SL.dt[j * SL.stride];
-            const uint4 q = philox4x32_10(make_uint4((uint32_t)s.h, (uint32_t)(s.h >> 32), kTagDigi << 28, unit),
-                                          make_uint2((uint32_t)J->seed, (uint32_t)(J->seed >> 32)));
-            // one Box-Muller pair: the cosine normal blurs the energy, the sine one the depth
+            const uint32_t unit = SL.unit[j * SL.stride];
+            const uint4 q = draw_blur(J, s.h, unit);
             float sp, cp;
             sincospif(2.0f * u01(q.y), &sp, &cp);
-            // the accurate log here: near u = 1 the radius is small and an
-            // absolute log error would become a large relative error of the blur
-            const float rad = sqrtf(-2.0f * logf(u01(q.x)));
-            const float sigma = J->sig_k * sqrtf(kE0 * e);
-            eb = fmaf(sigma, rad * cp, e);
-            db = fmaf(J->sig_doi, rad * sp, SL.ew[j * SL.stride] / e);
-            keep = eb >= J->e_lo && eb <= J->e_hi;
+            blur_single(J, q, sp, cp, unit, SL.e[j * SL.stride], SL.dt[j * SL.stride], SL.ew[j * SL.stride], o);
         }
-        const uint32_t b = __ballot_sync(mask, keep);
-        if (!b) continue;
-        // destination: the launch's singles buffer, or the job's own
-        RawSingle *dst = O.s_raw;
-        unsigned long long *dst_n = O.n_singles, dst_cap = O.s_cap;
-        if (kJobDest && keep && J->s_raw) {
-            dst = J->s_raw;
-            dst_n = J->n_singles;
-            dst_cap = J->s_cap;
-        }
-        unsigned long long slot = 0;
-        if (!kJobDest || __all_sync(mask, dst_n == O.n_singles)) {
-            // one counter for the warp (every fixed launch)
-            unsigned long long base = 0;
-            const int leader = __ffs(b) - 1;
-            if (lane == leader) base = atomicAdd(O.n_singles, (unsigned long long)__popc(b));
-            base = __shfl_sync(mask, base, leader);
-            slot = base + __popc(b & lanemask_lt());
-        } else if (keep) {
-            // lanes grouped by destination, one atomic per group
-            const uint32_t grp = __match_any_sync(b, reinterpret_cast<unsigned long long>(dst_n));
-            const int leader = __ffs(grp) - 1;
-            unsigned long long base = 0;
-            if (lane == leader) base = atomicAdd(dst_n, (unsigned long long)__popc(grp));
-            base = __shfl_sync(grp, base, leader);
-            slot = base + __popc(grp & lanemask_lt());
-        }
-        if (keep) {
-            if (slot < dst_cap) {
-                const GeomDev &g = geoms[J->geom];
-                int panel;
-                if (g.readout_level == 0) panel = (int)unit;
-                else if (g.readout_level == 1) panel = (int)(unit / (uint32_t)(g.modules_u * g.modules_v));
-                else panel = (int)(unit / (uint32_t)(g.crystals_per_module * g.modules_u * g.modules_v));
-                const uint64_t t = s.t0 + dt;
-                // the sort key: a job with its own buffer is the one job of its run
-                if (kJobDest && J->s_raw) J->s_keys[slot] = t;
-                else O.s_keys[slot] = O.key_shift < 64 ? ((uint64_t)s.job << O.key_shift) | t : t;
-                uint4 *r = reinterpret_cast<uint4 *>(dst + slot);
-                r[0] = make_uint4((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)s.h, (uint32_t)(s.h >> 32));
-                // a job with its own buffer is job 0 of the run that buffer belongs to
-                r[1] = make_uint4(unit, (uint32_t)panel, kJobDest && J->s_raw ? 0u : (uint32_t)s.job,
-                                  __float_as_uint(eb));
-                r[2] = make_uint4(__float_as_uint(e), __float_as_uint(db), 0u, 0u);
-            }
-        }
+        append_single<kJobDest, false>(geoms, O, J, s.job, s.h, s.t0, o, mask);
     }
 }
 

@@ -1,14 +1,40 @@
-// transport_cta.cu -- CTA-synchronous wavefront transport kernel.
+// transport_cta.cu -- warp-autonomous wavefront transport kernel over a pool
+// of history slots that a CTA shares.
 //
-// Same per-warp pools of history slots as the wavefront kernel, but the phase
-// is chosen for the whole CTA: every iteration each warp posts the phase
-// census of its pool to shared memory, one barrier later all warps read the
-// CTA totals and agree on the most populated phase, and every warp of the CTA
-// runs that same event.  All of a CTA's warps then execute one event's code
-// at a time, which keeps the instruction cache warm (an SM holds one or two
-// such CTAs); warps with no slot in the chosen phase wait for the next
-// iteration.  The events are those of transport.cuh, so the results equal the
-// other kernels' bit for bit.
+// A CTA keeps its history slots in shared memory and one 32-bit mask per
+// (phase, lane class): bit i of mask[p][l] says that slot i of lane class l
+// waits in phase p.  A slot stays with its lane class (slot i of class l is
+// always served by lane l of some warp), so every state access is free of bank
+// conflicts.  Each warp, on its own, takes the phase in which most of its lanes
+// have a slot, claims one slot per lane (an atomic AND on the mask), runs that
+// phase's event, and hands each slot on to its next phase (an atomic OR).  There
+// is no barrier: a warp that waits for memory or for its slowest lane delays no
+// other.
+//
+// What bounds it is instruction issue: no DRAM traffic to speak of, and the
+// state never leaves the SM.  Three things make that work:
+//   - Events are cut where their lanes would diverge.  A Woodcock step only
+//     finds the collision; sampling it (one Kahn trial, rotation, record) is an
+//     event of its own with its lanes packed, and a rejected trial waits for the
+//     next one.  The finish event digitizes one single per lane, where a loop
+//     over a history's singles waits for the warp's longest list.
+//   - The code of all events together is small (45 KB, the hot part less), since
+//     the warps of an SM are in different phases at once: one flight routine with
+//     one slab-test loop for every kind of flight, one Philox draw and one sine
+//     and cosine for all events that need them, cold paths out of line.  At 74 KB
+//     the same scheme lost half of its issue slots to instruction fetch (7.6 of
+//     14 warp-cycles per issue; now 1.9 of 9), and events that a whole CTA runs
+//     together behind a barrier lost them to the barrier (6.0 of 13.5).
+//   - First flights of a pair's two photons are one event (the same ray in both
+//     directions), which keeps photon 1's panel and distances in the slot until
+//     its turn; a photon that leaves through a panel's back, where no other panel
+//     can be, ends without a flight event.
+// Photons of a pair run one after the other, and events are those of
+// transport.cuh, so the histories equal the other kernels' bit for bit.
+//
+// Measured on a GB300, transport of one sweep position of 1e7 pairs: 2.52 ms
+// with the phase chosen per CTA behind a barrier and per-warp pools, 1.28 ms
+// here.
 #include "internal.h"
 #include "transport.cuh"
 
@@ -16,379 +42,690 @@ namespace gpet {
 
 namespace {
 
-constexpr int kCtaS = 6;     // singles-list entries per history (overflow -> redo kernel)
-constexpr int kCtaWords = 23;
-constexpr int kNumPh = 7;    // phases 0..6
+// one more phase here than in transport.cuh: a collision to be sampled
+constexpr uint32_t kPhInteract = 7;
+constexpr int kPhCount = 8;
+constexpr int kCtaS = 6;      // singles of one history (more -> redo kernel)
+constexpr int kEntries = 48;  // singles entries of a lane class, for all of its slots
 
-enum : int {
-    kCh0 = 0, kCh1, kCt0, kCt1, kCx, kCy, kCz, kCdx, kCdy, kCdz, kCx0, kCy0, kCz0, kCox, kCoy, kCoz, kCE, kCpath,
-    kCtrem, kCjob, kCpack, kCsteps
-};
+// state words of a slot; the last four only where a job has a phantom
+enum : int { kSh0 = 0, kSh1,
+             kSjob,             // job; [16:23) photon 1's first panel + 1 (0: it enters none); [23:29) sixth entry
+             kSox, kSoy, kSoz,
+             kSx, kSy, kSz, kSdx, kSdy, kSdz, kSE,
+             kSpath,            // path; distance to the panel of a photon 0 that has not entered it yet
+             kStrem,            // distance to the panel's exit; crystal id of a collision to be sampled
+             kSin1, kSrem1,     // photon 1's distance to its first panel, and through it
+             kSrw,              // azimuth word (top 23 bits) of a collision and its Kahn trials (low 9 bits);
+                                // distance to the next panel of a photon between panels
+             kSpk,
+             kSlist,            // the history's singles: six bits each, entries of the lane class
+             kSx0, kSy0, kSz0, kSph };
+constexpr int kWordsPlain = kSx0, kWordsPhantom = kSph + 1;
+constexpr int kJobPanel1 = 16, kJobEntry = 23;
 
-template <int SPL>
+// packed word: [0:7) panel + 1 (finish event: next single), [7:14) last panel + 1
+// (in a panel: not 0 where the photon has still to enter it; a collision: bit 7
+// counts 512 Kahn trials), [14] photon, [15:18) singles in the list, [18] list
+// overflowed, [19] photon 1 starts in the phantom, [20] photon not in its first
+// panel yet (its state is the decay's), [21:31) detector steps, [31]
+// photoelectric absorption
+constexpr int kPkLast = 7, kPkSing = 15, kPkStep = 21;
+constexpr uint32_t kPkPanel = 0x7Fu, kPkLastMask = 0x7Fu << kPkLast, kPkGamma = 1u << 14, kPkSingMask = 7u << kPkSing,
+                   kPkOvf = 1u << 18, kPkPhantom1 = 1u << 19, kPkFresh = 1u << 20, kPkStepMask = 0x3FFu << kPkStep,
+                   kPkPhoto = 1u << 31;
+static_assert(kMaxSteps < 1024 && kMaxPanels < 127 && kCtaS <= 6 && kMaxTrials <= 1024, "packed word fields");
+
+// event counters: slots 0..7 count the events of each phase (decays in 0,
+// lanes fed in 1); lane i of a warp keeps counter i
+enum : int { kNLanes = 1, kNScrStart = 8, kNScrFlight, kNEntered, kNHits, kNTrials, kNSingles, kNFin, kNIter, kNCount };
+constexpr int kSticky = 22;    // lanes with a slot in a warp's last phase for which it stays with that phase
+constexpr uint32_t kMaxSpins = 1u << 24;  // waits for a slot (over a second) before a warp gives up
+constexpr unsigned kFlushEvery = 1u << 20;  // events; below 2^32 counts in as many of any kind
+
+template <int SLOTS, bool PH>
 struct CtaPool {
-    static constexpr int kPool = 32 * SPL;
-    uint32_t st[kCtaWords][kPool];
-    uint32_t sl_unit[kCtaS * kPool];
-    float sl_e[kCtaS * kPool];
-    uint32_t sl_dt[kCtaS * kPool];
-    float sl_ew[kCtaS * kPool];
+    static constexpr int kWords = PH ? kWordsPhantom : kWordsPlain;
+    static constexpr int kN = SLOTS * 32;
+    uint32_t st[kWords * kN];
+    uint32_t e_unit[kEntries * 32];
+    float e_e[kEntries * 32];
+    uint32_t e_dt[kEntries * 32];
+    float e_ew[kEntries * 32];
 };
 
-template <class Pool>
-__device__ __forceinline__ uint32_t cphase(const Pool &P, int q) { return (P.st[kCpack][q] >> 16) & 7u; }
-
-template <class Pool>
-__device__ __forceinline__ void cload(const Pool &P, int q, PState &s) {
-    s.h = ((uint64_t)P.st[kCh1][q] << 32) | P.st[kCh0][q];
-    s.t0 = ((uint64_t)P.st[kCt1][q] << 32) | P.st[kCt0][q];
-    s.x = __uint_as_float(P.st[kCx][q]);
-    s.y = __uint_as_float(P.st[kCy][q]);
-    s.z = __uint_as_float(P.st[kCz][q]);
-    s.dx = __uint_as_float(P.st[kCdx][q]);
-    s.dy = __uint_as_float(P.st[kCdy][q]);
-    s.dz = __uint_as_float(P.st[kCdz][q]);
-    s.x0 = __uint_as_float(P.st[kCx0][q]);
-    s.y0 = __uint_as_float(P.st[kCy0][q]);
-    s.z0 = __uint_as_float(P.st[kCz0][q]);
-    s.ox = __uint_as_float(P.st[kCox][q]);
-    s.oy = __uint_as_float(P.st[kCoy][q]);
-    s.oz = __uint_as_float(P.st[kCoz][q]);
-    s.E = __uint_as_float(P.st[kCE][q]);
-    s.path = __uint_as_float(P.st[kCpath][q]);
-    s.trem = __uint_as_float(P.st[kCtrem][q]);
-    s.job = (int32_t)P.st[kCjob][q];
-    const uint32_t pk = P.st[kCpack][q];
-    s.panel = (int32_t)(pk & 0x7Fu) - 1;
-    s.last = (int32_t)((pk >> 7) & 0x7Fu) - 1;
-    s.gamma = (pk >> 14) & 1u;
-    s.phase = (pk >> 16) & 7u;
-    s.nsing = (pk >> 19) & 31u;
-    s.ovf = (pk >> 24) & 1u;
-    const uint32_t sw = P.st[kCsteps][q];
-    s.sph = sw & 0xFFFFu;
-    s.sdet = sw >> 16;
+// entries of a history's list, and the free entries of a lane class
+__device__ __forceinline__ uint32_t list_entry(uint32_t list, uint32_t jobw, uint32_t i) {
+    return i < 5u ? (list >> (6 * i)) & 63u : (jobw >> kJobEntry) & 63u;
 }
-
-template <class Pool>
-__device__ __forceinline__ void cstore(Pool &P, int q, const PState &s, bool all) {
-    if (all) {
-        P.st[kCh0][q] = (uint32_t)s.h;
-        P.st[kCh1][q] = (uint32_t)(s.h >> 32);
-        P.st[kCt0][q] = (uint32_t)s.t0;
-        P.st[kCt1][q] = (uint32_t)(s.t0 >> 32);
-        P.st[kCx0][q] = __float_as_uint(s.x0);
-        P.st[kCy0][q] = __float_as_uint(s.y0);
-        P.st[kCz0][q] = __float_as_uint(s.z0);
-        P.st[kCox][q] = __float_as_uint(s.ox);
-        P.st[kCoy][q] = __float_as_uint(s.oy);
-        P.st[kCoz][q] = __float_as_uint(s.oz);
-        P.st[kCjob][q] = (uint32_t)s.job;
+__device__ __forceinline__ void free_entry(uint32_t (*efree)[32], int lane, uint32_t e) {
+    atomicOr(&efree[e >> 5][lane], 1u << (e & 31u));
+}
+// a free entry, or kEntries
+__device__ __forceinline__ uint32_t take_entry(uint32_t (*efree)[32], int lane) {
+#pragma unroll 1
+    for (int w = 0; w < 2; ++w) {
+        uint32_t f = *reinterpret_cast<volatile uint32_t *>(&efree[w][lane]);
+#pragma unroll 1
+        while (f) {
+            const uint32_t b = f & (0u - f);
+            const uint32_t old = atomicAnd(&efree[w][lane], ~b);
+            if (old & b) return (uint32_t)(32 * w) + 31u - (uint32_t)__clz((int)b);
+            f = old & ~b;
+        }
     }
-    P.st[kCx][q] = __float_as_uint(s.x);
-    P.st[kCy][q] = __float_as_uint(s.y);
-    P.st[kCz][q] = __float_as_uint(s.z);
-    P.st[kCdx][q] = __float_as_uint(s.dx);
-    P.st[kCdy][q] = __float_as_uint(s.dy);
-    P.st[kCdz][q] = __float_as_uint(s.dz);
-    P.st[kCE][q] = __float_as_uint(s.E);
-    P.st[kCpath][q] = __float_as_uint(s.path);
-    P.st[kCtrem][q] = __float_as_uint(s.trem);
-    P.st[kCpack][q] = (uint32_t)(s.panel + 1) | ((uint32_t)(s.last + 1) << 7) | (s.gamma << 14) | (s.phase << 16) |
-                      (s.nsing << 19) | (s.ovf << 24);
-    P.st[kCsteps][q] = (s.sph & 0xFFFFu) | (s.sdet << 16);
+    return (uint32_t)kEntries;
 }
 
-// one event of phase p for a lane's history
-__device__ __forceinline__ int run_event(int p, const JobDev &J, const GeomDev &g, const WorkDev &W, const OutDev &O,
-                                         PState &s, const SinglesList &SL, Counters &cnt) {
-    int st = kStatusOk;
-    switch (p) {
-        case kPhSource: ev_source(J, g, s, cnt); break;
-        case kPhPhantom: st = ev_phantom(J, g, W, s, cnt); break;
-        case kPhFlight: case kPhFlightOut:
-            cnt.fl_out += p == kPhFlightOut ? 1u : 0u;
-            ev_flight(J, g, s, cnt);
-            break;
-        case kPhPanel: st = ev_panel<true>(J, g, W, O, s, SL, kCtaS, cnt); break;
-        default: st = kStatusBadPhase; break;
+// Photon of packed word pk is done: the slot's next phase.  Photon 0 hands
+// over to photon 1, which starts in the phantom, at the panel its first flight
+// found (panel1 = panel + 1), or not at all (0); a history without singles has
+// nothing to digitize, its slot is free.
+__device__ __forceinline__ uint32_t photon_end(uint32_t &pk, uint32_t panel1) {
+    const bool first = !(pk & kPkGamma), ph1 = pk & kPkPhantom1;
+    pk &= kPkSingMask | kPkOvf;
+    if (first && (ph1 || panel1)) {
+        pk |= kPkGamma | (ph1 ? 0u : kPkFresh | panel1);
+        return ph1 ? kPhPhantom : kPhPanel;
     }
-    return st;
+    return pk ? kPhFinish : kPhIdle;
 }
 
-// Launch modes, one instantiation each, so that a fixed launch carries none
-// of the other modes' instructions:
-//   kModeFixed  : a fixed work table, one event per slot and phase choice;
-//   kModeRepeat : the compaction interval -- a slot repeats its event up to
-//                 `repeat` times while it stays in the chosen phase (steps of
-//                 the phantom and of the detector repeat);
-//   kModeLive   : a live launch (chunks the host appends while the kernel
-//                 runs, bounded idle waits, per-job singles buffers).
-enum : int { kModeFixed = 0, kModeRepeat = 1, kModeLive = 2 };
+// n more of event counter i, kept by lane i (a function, so that every lane evaluates n)
+__device__ __forceinline__ void count(uint32_t &acc, int i, uint32_t n) {
+    if ((int)(threadIdx.x & 31) == i) acc += n;
+}
+
+// a crystal interaction into the optional hit list (tests, depth studies)
+__device__ __noinline__ void keep_hit(const OutDev &O, const JobDev &J, const GeomDev &g, uint64_t h, int job,
+                                      uint32_t gamma, uint32_t step, int crystal, float dep, uint32_t dtp, float x,
+                                      float y, float z) {
+    PState s;
+    s.h = h;
+    s.t0 = decay_time(J, draw(J.seed, h, kTagSource, 0u, 0u, 0u));
+    s.gamma = gamma;
+    s.job = job;
+    s.x = x; s.y = y; s.z = z;
+    const int c = crystal % g.crystals_per_module;   // the layer, from the id within the module
+    int layer = 0;
+    while (layer + 1 < g.n_layers && c >= g.layers[layer + 1].loff) ++layer;
+    store_hit(O, s, crystal, layer, step, dep, dtp);
+}
 
 }  // namespace
 
-// at most 128 registers a thread: 16 warps of the kernel stay resident per SM
-template <int SPL, int WARPS, int MODE>
-__global__ void __launch_bounds__(WARPS * 32, (16 / WARPS > 1 ? 16 / WARPS : 1)) k_transport_cta(WorkDev W, OutDev O, int ng_smem,
-                                                                                                 int repeat) {
-    constexpr bool kLive = MODE == kModeLive;
-    using Pool = CtaPool<SPL>;
-    constexpr int kPool = Pool::kPool;
+// kPhantom: jobs with a phantom may occur; kPosed: geometries with panel poses
+// may.  kLive: a live launch (chunks the host appends while the kernel runs,
+// bounded idle waits, per-job singles buffers).  Separate instantiations, so
+// that a fixed launch without them carries none of their instructions,
+// registers and state words.
+template <int WARPS, int SLOTS, int CTAS, bool kPhantom, bool kPosed, bool kLive>
+__global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(WorkDev W, OutDev O, int ng_smem) {
+    static_assert(SLOTS <= 32, "one mask bit per slot");
+    using Pool = CtaPool<SLOTS, kPhantom>;
+    constexpr int kN = Pool::kN;
     extern __shared__ __align__(16) uint8_t smem[];
     GeomDev *sgeom = reinterpret_cast<GeomDev *>(smem);
-    Pool *pools = reinterpret_cast<Pool *>(sgeom + ng_smem);
-    // CTA-wide phase totals, triple-buffered: iteration i adds into buffer
-    // i % 3 before its barrier and reads it after; the buffer of iteration
-    // i - 1 is cleared after the barrier of iteration i, which every read of
-    // it precedes and every add of iteration i + 2 follows.
-    __shared__ int census[3][8];
-    __shared__ uint8_t assign[WARPS][32];  // slot of each lane in the chosen phase
+    Pool &P = *reinterpret_cast<Pool *>(sgeom + ng_smem);
+    __shared__ uint32_t mask[kPhCount][32];
+    __shared__ uint32_t efree[2][32];
+    __shared__ Refill refills[WARPS];
     stage_geometry(W, sgeom, ng_smem);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    Pool &P = pools[wid];
+    if (threadIdx.x < 32) {
 #pragma unroll
-    for (int g = 0; g < SPL; ++g) P.st[kCpack][g * 32 + lane] = 0;
-    if (threadIdx.x < 24) (&census[0][0])[threadIdx.x] = 0;
+        for (int p = 0; p < kPhCount; ++p) mask[p][lane] = p == kPhIdle ? 0xFFFFFFFFu >> (32 - SLOTS) : 0u;
+        efree[0][lane] = 0xFFFFFFFFu;
+        efree[1][lane] = 0xFFFFFFFFu >> (64 - kEntries);
+    }
+    if (lane == 0) refill_init(refills[wid]);
     __syncthreads();
-
-    Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
-    Refill rf;
-    refill_init(rf);
-    int status = kStatusOk;
     LiveIdle idle;
     live_idle_reset(idle);
-    unsigned long long iters = 0, lanes_used = 0;
-    int buf = 0;
-    // slots turn idle only in the finish event (or on an error); a warp whose
-    // next chunk a live launch has not published yet retries every iteration
-    bool may_idle = true;
+    uint32_t *const st = P.st;
+    bool done = false;    // no histories to come for this warp
+    uint32_t acc = 0;     // lane i: event counter i
+    uint32_t ph = kPhIdle, spins = 0;
+    bool waiting = false, alone = false;   // live: the next chunk is not published; no slot in any other phase
+#define ST(w) st[(w) * kN + q]
+#define STF(w) __uint_as_float(st[(w) * kN + q])
+#define STORE3(w, a, b, c) (ST(w) = __float_as_uint(a), ST((w) + 1) = __float_as_uint(b), ST((w) + 2) = __float_as_uint(c))
 
-    for (;;) {
-        // 1. refill the warp's idle slots
+    for (unsigned it = 1;; ++it) {
+        // 1. the phase: the last one again while most lanes have a slot in it,
+        // else the one with the most lanes (ties to the later one, so that
+        // histories end before others begin)
+        uint32_t m = *reinterpret_cast<volatile uint32_t *>(&mask[ph][lane]);
+        if ((ph == kPhIdle && (done || (kLive && waiting))) || __popc(__ballot_sync(kFullMask, m != 0)) < kSticky) {
+            uint32_t best = 0;
+            alone = true;
 #pragma unroll
-        for (int g = 0; g < SPL; ++g) {
-            if (!may_idle || rf.exhausted) break;
-            const int q = g * 32 + lane;
-            const uint32_t need = __ballot_sync(kFullMask, cphase(P, q) == kPhIdle);
-            if (need) {
-                bool got;
-                uint64_t h = 0;
-                int job = 0;
-                warp_refill<kLive>(W, need, rf, got, h, job);
-                if (got) {
-                    P.st[kCh0][q] = (uint32_t)h;
-                    P.st[kCh1][q] = (uint32_t)(h >> 32);
-                    P.st[kCjob][q] = (uint32_t)job;
-                    P.st[kCpack][q] = (uint32_t)kPhSource << 16;
+            for (int p = 0; p < kPhCount; ++p) {
+                if (p == 1 || (p == 2 && !kPhantom)) continue;
+                const uint32_t v = *reinterpret_cast<volatile uint32_t *>(&mask[p][lane]);
+                uint32_t n = (p == kPhIdle && done) ? 0u : (uint32_t)__popc(__ballot_sync(kFullMask, v != 0));
+                // a live launch's warp whose next chunk is not published yet asks for
+                // it every eighth time, or when there is nothing else to do
+                if (kLive && p == kPhIdle && waiting && (it & 7u)) n = min(n, 1u);
+                if (kLive && p != kPhIdle && n) alone = false;
+                best = max(best, n ? (n << 3) | (uint32_t)p : 0u);
+            }
+            if (best == 0) {
+                // every slot that this warp could take is in other warps' hands,
+                // which hand it on or, with no histories to come, see to its end
+                if (done) break;
+                if (++spins > kMaxSpins) {
+                    if (lane == 0) atomicOr(O.status, kStatusBadPhase);
+                    break;
                 }
-                if (kLive && rf.waiting) break;
+                __nanosleep(64);
+                continue;
             }
+            spins = 0;
+            ph = best & 7u;
+            m = *reinterpret_cast<volatile uint32_t *>(&mask[ph][lane]);
         }
-        may_idle = kLive && rf.waiting && !rf.exhausted;
-        __syncwarp();
-        // 2. the warp's census: lane p adds the warp's count of phase p
-        uint32_t ph[SPL];
-#pragma unroll
-        for (int g = 0; g < SPL; ++g) ph[g] = cphase(P, g * 32 + lane);
-        uint32_t mask_p[kNumPh][SPL];
-        int my_n = 0;
-#pragma unroll
-        for (int p = 1; p < kNumPh; ++p) {
-            int n = 0;
-#pragma unroll
-            for (int g = 0; g < SPL; ++g) {
-                mask_p[p][g] = __ballot_sync(kFullMask, ph[g] == (uint32_t)p);
-                n += __popc(mask_p[p][g]);
+        // 2. claim one slot of the phase per lane (each warp from another bit on)
+        const uint32_t rot = (uint32_t)(wid * 5) & 31u;
+        uint32_t bit = 0;
+        bool active = false;
+#pragma unroll 1
+        for (int t = 0; t < 2; ++t) {   // (a lane whose bit went to another warp tries once more)
+            if (!active && m) {
+                const uint32_t mr = __funnelshift_r(m, m, rot);
+                const uint32_t low = mr & (0u - mr);
+                bit = __funnelshift_l(low, low, rot);
+                const uint32_t old = atomicAnd(&mask[ph][lane], ~bit);
+                active = old & bit;
+                m = old & ~bit;
             }
-            if (lane == p) my_n = n;
+            if (!__any_sync(kFullMask, !active && m)) break;
         }
-        if (my_n) atomicAdd(&census[buf][lane], my_n);
-        int any_waiting = 0;
-        if constexpr (kLive) any_waiting = __syncthreads_or(rf.waiting && !rf.exhausted);
-        else __syncthreads();
-        // 3. every warp reads the same totals: the most populated phase wins
-        //    (ties to the later phase, which finishes histories sooner)
-        const uint32_t key = (lane >= 1 && lane < kNumPh) ? ((uint32_t)census[buf][lane] << 3) | (uint32_t)lane : 0u;
-        const uint32_t best = __reduce_max_sync(kFullMask, key);
-        if (threadIdx.x < 8) census[buf == 0 ? 2 : buf - 1][threadIdx.x] = 0;
-        buf = buf == 2 ? 0 : buf + 1;
-        const int best_p = (int)(best & 7u);
-        if ((best >> 3) == 0) {
-            // every slot of every warp idle after refills: done, unless a warp
-            // of a live launch waits for a chunk the host has not published yet
-            if (!kLive || !any_waiting) break;
-            // one decision for the whole CTA: its threads leave the loop together
-            if (__syncthreads_or(live_idle_wait(idle, status, W, O))) {
-                status |= kStatusLiveStall;
-                break;
-            }
-            continue;
+        const uint32_t am = __ballot_sync(kFullMask, active);
+        if (am == 0) continue;
+        __threadfence_block();
+        const int q = active ? (31 - __clz((int)bit)) * 32 + lane : lane;
+        count(acc, kNIter, 1);
+        count(acc, kNLanes, __popc(am));
+        if (it % kFlushEvery == 0) {   // (32-bit counts never wrap: see kFlushEvery)
+            if (lane < kNCount && acc) atomicAdd(O.counters + kCtaCounters + lane, (unsigned long long)acc);
+            acc = 0;
         }
-        if (kLive) live_idle_reset(idle);
-        // 4. lanes onto this warp's slots of the chosen phase: the slot of
-        //    rank r (in slot order) goes to lane r
-        int mine = 0;
-#pragma unroll
-        for (int g = 0; g < SPL; ++g) {
-            uint32_t m = 0;
-#pragma unroll
-            for (int p = 1; p < kNumPh; ++p) m = p == best_p ? mask_p[p][g] : m;
-            const int r = mine + __popc(m & lanemask_lt());
-            if (ph[g] == (uint32_t)best_p && r < 32) assign[wid][r] = (uint8_t)(g * 32 + lane);
-            mine += __popc(m);
-        }
-        __syncwarp();
-        const bool active = lane < mine;
-        const int q = active ? assign[wid][lane] : 0;
-        if (mine == 0) continue;  // nothing of this phase here: wait for the next choice
-        ++iters;
-        lanes_used += (unsigned long long)min(mine, 32);
-        PState s;
-        s.phase = kPhIdle;
-        s.job = 0;
-        const SinglesList SL{P.sl_unit + q, P.sl_e + q, P.sl_dt + q, P.sl_ew + q, kPool};
-        if (best_p == kPhFinish) {
-            if (active) cload(P, q, s);
+        // 3. the event
+        uint32_t jobw = 0, pk = 0, to = kPhIdle;
+        uint64_t h = 0;
+        bool run = active;   // lanes with a history
+        if (ph == kPhIdle) {
+            Refill rf = refills[wid];
             __syncwarp();
-            cnt.fin += active ? 1u : 0u;
-            ev_finish<kLive>(W.jobs, W.geoms, O, s, active, SL, kFullMask, cnt);
-            if (active) P.st[kCpack][q] = 0;
-            may_idle = true;
+            int job = 0;
+            warp_refill<kLive>(W, am, rf, run, h, job);
+            if (lane == 0) refills[wid] = rf;
             __syncwarp();
-            continue;
+            done = rf.exhausted;
+            waiting = rf.waiting;
+            jobw = (uint32_t)job;
+        } else if (active) {
+            jobw = ST(kSjob);
+            pk = ST(kSpk);
+            h = ((uint64_t)ST(kSh1) << 32) | ST(kSh0);
         }
-        int n_ev = 0;
-        if (active) {
-            cload(P, q, s);
-            const JobDev &J = W.jobs[s.job];
-            const GeomDev &g = J.geom < ng_smem ? sgeom[J.geom] : W.geoms[J.geom];
-            int st = kStatusOk;
-            if constexpr (MODE == kModeRepeat) {
-                // the chosen event, then again while the slot stays in its
-                // phase, up to `repeat` events in all
-                do {
-                    ++n_ev;
-                    st = run_event(best_p, J, g, W, O, s, SL, cnt);
-                } while (st == kStatusOk && n_ev < repeat && s.phase == (uint32_t)best_p);
+        const JobDev &J = W.jobs[jobw & 0xFFFFu];
+        const GeomDev &g = J.geom < ng_smem ? sgeom[J.geom] : W.geoms[J.geom];
+        const uint32_t gamma = (pk & kPkGamma) ? 1u : 0u;
+        if (ph == kPhFlight || ph == kPhFlightOut) {
+            // Flights to the next panel: the first ones of both photons from the
+            // decay point (but one that the axial screen ended), or of one photon
+            // out of a panel or the phantom.
+            uint32_t n_fl = 0, n_in = 0, n_scr = 0;
+            if (run) {
+                const bool out = ph == kPhFlightOut;
+                const bool pair = !out && (!kPhantom || ST(kSph) == 0);
+                float x, y, z, dx, dy, dz;
+                if (pair) {
+                    x = kPhantom ? STF(kSx0) : J.src_pos[0];
+                    y = kPhantom ? STF(kSy0) : J.src_pos[1];
+                    z = kPhantom ? STF(kSz0) : J.src_pos[2];
+                    const float sg = gamma ? -1.0f : 1.0f;
+                    dx = sg * STF(kSox); dy = sg * STF(kSoy); dz = sg * STF(kSoz);
+                } else {
+                    x = STF(kSx); y = STF(kSy); z = STF(kSz);
+                    dx = STF(kSdx); dy = STF(kSdy); dz = STF(kSdz);
+                }
+                const int skip = out ? (int)((pk & kPkLastMask) >> kPkLast) - 1 : -1;
+                uint32_t p0 = 0, p1 = 0, second = gamma;
+#pragma unroll 1
+                for (;;) {
+                    float t_in, t_out;
+                    const int k = flight<kPosed>(g, x, y, z, dx, dy, dz, skip, t_in, t_out);
+                    n_fl++;
+                    n_scr += k == kFlightScreened ? 1u : 0u;
+                    if (k >= 0) {
+                        n_in++;
+                        (second ? p1 : p0) = (uint32_t)(k + 1);
+                        const int wi = !pair ? kSrw : second ? kSin1 : kSpath, wr = pair && second ? kSrem1 : kStrem;
+                        st[wi * kN + q] = __float_as_uint(t_in);
+                        st[wr * kN + q] = __float_as_uint(t_out - t_in);
+                    }
+                    // photon 1 of a pair next (pk's fresh flag: the screen ended it)
+                    if (!pair || second || (pk & kPkFresh)) break;
+                    second = 1;
+                    dx = -dx; dy = -dy; dz = -dz;
+                }
+                if (pair) {
+                    ST(kSjob) = jobw | (p1 << kJobPanel1);
+                    pk = p0 ? kPkFresh | p0 : (p1 ? kPkFresh | kPkGamma | p1 : 0u);
+                    to = pk ? kPhPanel : kPhIdle;
+                } else {
+                    if (kPhantom) ST(kSph) = 0;
+                    const uint32_t k1 = p0 | p1;
+                    if (k1) {
+                        pk = (pk & ~kPkPanel) | kPkLastMask | k1;   // enters it at its next step
+                        to = kPhPanel;
+                    } else {
+                        to = photon_end(pk, (jobw >> kJobPanel1) & 0x7Fu);
+                    }
+                }
+                ST(kSpk) = pk;
+            }
+            // (at most two a lane)
+            const uint32_t n = __reduce_add_sync(kFullMask, n_fl | (n_in << 8) | (n_scr << 16));
+            count(acc, ph, n & 0xFFu);
+            count(acc, kNEntered, (n >> 8) & 0xFFu);
+            count(acc, kNScrFlight, n >> 16);
+        } else {
+            // The other events begin with a draw, made here for all of them.
+            const bool in_panel = !kPhantom || (pk & kPkPanel);
+            uint32_t c2 = kTagSource << 28, c3 = 0, rw = 0, list = 0, e = 0, unit = 0;
+            const uint32_t step = (pk & kPkStepMask) >> kPkStep;
+            if (ph == kPhPanel) {
+                c2 = (kTagDetector << 28) | (gamma << 27) | step;
+            } else if (kPhantom && ph == kPhPhantom) {
+                c2 = (kTagPhantom << 28) | (gamma << 27) | (run ? ST(kSph) : 0u);
+            } else if (ph == kPhInteract) {
+                rw = ST(kSrw);
+                c2 = (in_panel ? (kTagDetector << 28) | (step - 1u) : (kTagPhantom << 28) | (ST(kSph) - 1u)) | (gamma << 27);
+                c3 = 1u + (rw & 511u) + ((pk >> kPkLast) & 1u) * 512u;
+            } else if (ph == kPhFinish) {
+                list = ST(kSlist);
+                e = list_entry(list, jobw, pk & kPkPanel) & 63u;
+                unit = P.e_unit[(run ? e : 0u) * 32 + lane];
+                c2 = kTagDigi << 28;
+                c3 = unit;
+            }
+            const uint4 r = philox4x32_10(make_uint4((uint32_t)h, (uint32_t)(h >> 32), c2, c3),
+                                          make_uint2((uint32_t)J.seed, (uint32_t)(J.seed >> 32)));
+            if (ph == kPhPanel || (kPhantom && ph == kPhPhantom)) {
+                // one Woodcock step in the panel or the phantom
+                bool late = false;
+                uint32_t n_left = 0;
+                if (run) {
+                    PState s;
+                    s.panel = (int)(pk & kPkPanel) - 1;
+                    const uint32_t sph = kPhantom ? ST(kSph) : 0u;
+                    const bool fresh = ph == kPhPanel ? (pk & kPkFresh) != 0 : sph == 0;
+                    if (fresh) {   // starts at its decay point
+                        s.x = kPhantom ? STF(kSx0) : J.src_pos[0];
+                        s.y = kPhantom ? STF(kSy0) : J.src_pos[1];
+                        s.z = kPhantom ? STF(kSz0) : J.src_pos[2];
+                        const float sg = gamma ? -1.0f : 1.0f;
+                        s.dx = sg * STF(kSox); s.dy = sg * STF(kSoy); s.dz = sg * STF(kSoz);
+                        s.E = kE0;
+                        s.path = 0.0f;
+                        ST(kSE) = __float_as_uint(kE0);
+                    } else {
+                        s.x = STF(kSx); s.y = STF(kSy); s.z = STF(kSz);
+                        s.dx = STF(kSdx); s.dy = STF(kSdy); s.dz = STF(kSdz);
+                        s.E = STF(kSE);
+                        s.path = STF(kSpath);
+                    }
+                    to = ph;
+                    if (!kPhantom || ph == kPhPanel) {
+                        const bool enter = pk & (kPkFresh | kPkLastMask);
+                        s.trem = __uint_as_float(st[(fresh && gamma ? kSrem1 : kStrem) * kN + q]);
+                        if (enter) {
+                            const int wi = !fresh ? kSrw : gamma ? kSin1 : kSpath;
+                            enter_panel<kPosed>(g, s.panel, __uint_as_float(st[wi * kN + q]), s);
+                            pk &= ~(kPkFresh | kPkLastMask);
+                        }
+                        late = step >= (uint32_t)kMaxSteps;
+                        Loc L;
+                        bool left_ring = false;
+                        const int what = panel_step<kPosed>(g, W, r, s, L, left_ring);
+                        pk += late ? 0u : 1u << kPkStep;
+                        ST(kStrem) = what >= kStepPhoto ? (uint32_t)L.crystal : __float_as_uint(s.trem);
+                        if (enter || what == kStepExit) STORE3(kSdx, s.dx, s.dy, s.dz);
+                        if (what == kStepExit) {
+                            if (left_ring) {
+                                // its flight would end it: counted as one, without the event
+                                n_left = 1;
+                                const float c0 = fmaf(s.x, s.x, s.y * s.y), a = fmaf(s.dx, s.dx, s.dy * s.dy);
+                                if (a > 0.0f && !(c0 < g.R2 * 0.9999f) && outside_screened(g, a, fmaf(s.x, s.dx, s.y * s.dy), c0))
+                                    n_left = 1u | 1u << 16;
+                                to = photon_end(pk, (jobw >> kJobPanel1) & 0x7Fu);
+                            } else {
+                                pk = (pk & ~kPkPanel) | ((pk & kPkPanel) << kPkLast);
+                                to = kPhFlightOut;
+                            }
+                        } else if (what != kStepVirtual) {
+                            ST(kSrw) = r.w & ~511u;
+                            pk = (pk & ~kPkPhoto) | (what == kStepPhoto ? kPkPhoto : 0u);
+                            to = kPhInteract;
+                        }
+                    } else {
+                        if (fresh) STORE3(kSdx, s.dx, s.dy, s.dz);
+                        late = sph >= (uint32_t)kMaxSteps;
+                        const int what = phantom_step(J, W, r, s);
+                        ST(kSph) = sph + 1u;
+                        if (what == kStepExit) {
+                            to = kPhFlight;
+                        } else if (what == kStepPhoto) {
+                            to = photon_end(pk, 0);
+                            ST(kSph) = 0;
+                        } else if (what == kStepCompton) {
+                            ST(kSrw) = r.w & ~511u;
+                            to = kPhInteract;   // panel field 0: in the phantom
+                        }
+                    }
+                    STORE3(kSx, s.x, s.y, s.z);
+                    ST(kSpath) = __float_as_uint(s.path);
+                    ST(kSpk) = pk;
+                    if (late) {   // step cap hit: abandon the history, flag the run
+                        atomicOr(O.status, kStatusTimeout);
+                        to = kPhIdle;
+                    }
+                }
+                count(acc, ph, __popc(am));
+                n_left = __reduce_add_sync(kFullMask, n_left);
+                count(acc, kPhFlightOut, n_left & 0xFFFFu);
+                count(acc, kNScrFlight, n_left >> 16);
             } else {
-                st = run_event(best_p, J, g, W, O, s, SL, cnt);
+                // decay, collision and finish take one azimuth
+                float sp, cp;
+                sincospif(2.0f * u01(ph == kPhInteract ? rw : ph == kPhFinish ? r.y : r.w), &sp, &cp);
+                if (ph == kPhInteract) {
+                    // the collision found by a step: one Kahn trial an event, a photon
+                    // whose trial is rejected stays
+                    uint32_t n_hits = 0, n_trials = 0;
+                    if (run) {
+                        const bool photo = (pk & kPkPhoto) && in_panel;
+                        const float E = STF(kSE);
+                        float xm1 = 0.f;
+                        bool accept = true;
+                        if (!photo) {
+                            const float k = E * kInvMec2;
+                            accept = kahn_try(r, k, 1.0f + 2.0f * k, 9.0f + 2.0f * k, xm1);
+                            n_trials = accept ? c3 : 0u;
+                        }
+                        to = kPhInteract;
+                        if (!accept) {
+                            if (c3 >= (uint32_t)kMaxTrials) {
+                                atomicOr(O.status, kStatusTimeout);
+                                to = kPhIdle;
+                            }
+                            ST(kSrw) = (rw & ~511u) | (c3 & 511u);
+                            pk = (pk & ~kPkLastMask) | ((c3 >> 9) << kPkLast);
+                        } else {
+                            const float x = STF(kSx), y = STF(kSy), z = STF(kSz);
+                            const float Ep = E / (1.0f + xm1);
+                            const bool dead = photo || Ep < J.e_cut;
+                            const float dep = dead ? E : E * xm1 / (1.0f + xm1);
+                            const int crystal = in_panel ? (int)ST(kStrem) : -1;
+                            bool held = false;
+                            if (crystal >= 0) {
+                                // a crystal interaction: the history's singles, tallies, optional hit list
+                                const uint32_t dtp = (uint32_t)floorf(STF(kSpath) * kInvCmmPerPs);
+                                unit = (uint32_t)crystal;
+                                if (g.readout_level == 0) unit = (pk & kPkPanel) - 1u;
+                                else if (g.readout_level == 1) unit = (uint32_t)crystal / (uint32_t)g.crystals_per_module;
+                                const uint32_t n = (pk & kPkSingMask) >> kPkSing;
+                                list = n ? ST(kSlist) : 0u;
+                                uint32_t ei = kEntries * 32;
+#pragma unroll 1
+                                for (uint32_t i = 0; i < n; ++i) {
+                                    const uint32_t ej = list_entry(list, jobw, i) * 32 + lane;
+                                    if (P.e_unit[ej] == unit) ei = ej;
+                                }
+                                if (ei < kEntries * 32) {
+                                    P.e_e[ei] += dep;
+                                    P.e_ew[ei] += dep * x;
+                                    P.e_dt[ei] = min(P.e_dt[ei], dtp);
+                                } else {
+                                    e = n < (uint32_t)kCtaS ? take_entry(efree, lane) : (uint32_t)kEntries;
+                                    if (e < (uint32_t)kEntries) {
+                                        ei = e * 32 + lane;
+                                        P.e_unit[ei] = unit;
+                                        P.e_e[ei] = dep;
+                                        P.e_ew[ei] = dep * x;
+                                        P.e_dt[ei] = dtp;
+                                        if (n < 5u) ST(kSlist) = list | (e << (6 * n));
+                                        else ST(kSjob) = jobw | (e << kJobEntry);
+                                        pk += 1u << kPkSing;
+                                    } else if (n < (uint32_t)kCtaS && *reinterpret_cast<volatile uint32_t *>(&mask[kPhFinish][lane])) {
+                                        held = true;     // entries come free: the same trial again then
+                                    } else {
+                                        pk |= kPkOvf;    // simulated again by the redo kernel
+                                    }
+                                }
+                                if (!held) {
+                                    n_hits = 1;
+                                    atomicAdd(J.tally_count + crystal, 1ull);
+                                    atomicAdd(J.tally_efx + crystal, (unsigned long long)__float2ull_rn(dep * kEfxScale));
+                                    if (O.hit_cap)
+                                        keep_hit(O, J, g, h, (int)(jobw & 0xFFFFu), gamma, step - 1u, crystal, dep, dtp, x, y, z);
+                                }
+                            }
+                            if (held) {
+                                n_trials = 0;
+                            } else {
+                                pk &= ~kPkLastMask;
+                                if (dead) {
+                                    to = photon_end(pk, (jobw >> kJobPanel1) & 0x7Fu);
+                                    if (kPhantom) ST(kSph) = 0;
+                                } else {
+                                    // rotation in the panel frame with v as polar reference: for the ring
+                                    // (w, u, v) is a rotation of (x, y, z) about the axis, so this equals the
+                                    // global rotation; a posed panel takes its own v axis
+                                    float dx = STF(kSdx), dy = STF(kSdy), dz = STF(kSdz);
+                                    rotate_dir(dx, dy, dz, xm1 / (E * kInvMec2), sp, cp);
+                                    STORE3(kSdx, dx, dy, dz);
+                                    ST(kSE) = __float_as_uint(Ep);
+                                    if (in_panel) ST(kStrem) = __float_as_uint(panel_exit(g, x, y, z, dx, dy, dz));
+                                    to = in_panel ? kPhPanel : kPhPhantom;
+                                }
+                            }
+                        }
+                        ST(kSpk) = pk;
+                    }
+                    count(acc, kNHits, __popc(__ballot_sync(kFullMask, n_hits)));
+                    count(acc, kNTrials, __reduce_add_sync(kFullMask, n_trials));
+                } else if (ph == kPhIdle) {
+                    // decay: the pair's direction, and what its photons do first
+                    uint32_t n_scr = 0;
+                    if (run) {
+                        float x0, y0, z0, ox, oy, oz;
+                        sample_decay<kPhantom>(J, h, r, sp, cp, x0, y0, z0, ox, oy, oz);
+                        to = kPhFlight;
+                        if (kPhantom && J.has_phantom && in_phantom(J, x0, y0, z0)) {
+                            to = kPhPhantom;
+                            pk = kPkPhantom1;
+                        } else {
+                            if (start_screened<kPosed>(g, x0, y0, z0, ox, oy, oz)) {
+                                n_scr = 1;
+                                pk = kPkGamma;     // (for the flight event: photon 1's flight only)
+                            }
+                            if (start_screened<kPosed>(g, x0, y0, z0, -ox, -oy, -oz)) {
+                                pk |= kPkFresh;    // (photon 0's flight only)
+                                if (++n_scr == 2) to = kPhIdle;
+                            }
+                        }
+                        ST(kSh0) = (uint32_t)h;
+                        ST(kSh1) = (uint32_t)(h >> 32);
+                        ST(kSjob) = jobw;
+                        STORE3(kSox, ox, oy, oz);
+                        ST(kSpk) = pk;
+                        if (kPhantom) {
+                            STORE3(kSx0, x0, y0, z0);
+                            ST(kSph) = 0;
+                        }
+                    }
+                    const uint32_t got = __popc(__ballot_sync(kFullMask, run));
+                    count(acc, kPhIdle, got);
+                    count(acc, kNScrStart, __reduce_add_sync(kFullMask, n_scr));
+                    if (kLive) {
+                        if (got || !alone) {
+                            live_idle_reset(idle);
+                        } else if (!done) {
+                            // no chunk published: the launch's host has nothing yet
+                            int status = kStatusOk;
+                            if (__any_sync(kFullMask, live_idle_wait(idle, status, W, O))) {
+                                if (lane == 0) atomicOr(O.status, kStatusLiveStall);
+                                done = true;
+                            }
+                        }
+                    }
+                } else {
+                    // digitizer: one single of the history's list, in list order
+                    const uint32_t n = (pk & kPkSingMask) >> kPkSing, j = pk & kPkPanel;
+                    const bool ovf = run && (pk & kPkOvf), one = run && !ovf;
+                    append_overflow(O, ovf, h, (int)(jobw & 0xFFFFu), kFullMask);
+                    SingleOut so;
+                    so.keep = false;
+                    if (one) {
+                        const uint32_t ei = e * 32 + lane;
+                        blur_single(J, r, sp, cp, unit, P.e_e[ei], P.e_dt[ei], P.e_ew[ei], so);
+                        free_entry(efree, lane, e);
+                    }
+                    append_single<kLive, true>(W.geoms, O, J, (int)(jobw & 0xFFFFu), h, 0, so, kFullMask);
+                    if (ovf)
+#pragma unroll 1
+                        for (uint32_t i = 0; i < n; ++i) free_entry(efree, lane, list_entry(list, jobw, i));
+                    const bool last = ovf || j + 1u >= n;
+                    if (run && !last) ST(kSpk) = pk + 1u;
+                    to = last ? kPhIdle : kPhFinish;
+                    count(acc, kNFin, __popc(__ballot_sync(kFullMask, run && last)));
+                    count(acc, kNSingles, __popc(__ballot_sync(kFullMask, one)));
+                }
             }
-            if (st != kStatusOk) {
-                status |= st;
-                s.phase = kPhIdle;
-            }
-            cstore(P, q, s, best_p == kPhSource);
         }
-        may_idle = may_idle || __any_sync(kFullMask, active && s.phase == kPhIdle);
+        // 4. hand the slots on to their next phases, their state first
+        __threadfence_block();
+        if (active) atomicOr(&mask[to][lane], bit);
         __syncwarp();
     }
-    // totals, then the events per phase (slots 10 + phase: decay, phantom
-    // step, flight, detector step, finish, flight after a panel exit)
-    const uint32_t v[14] = {cnt.det_steps, cnt.flights, cnt.trials, cnt.entered, cnt.ph_steps, cnt.hits,
-                            cnt.screened, cnt.singles, cnt.src, cnt.ph_steps, cnt.fl_ev - cnt.fl_out,
-                            cnt.det_steps, cnt.fin, cnt.fl_out};
-    const int slot[14] = {0, 1, 2, 3, 4, 5, 8, 9, 11, 12, 13, 14, 15, 16};
-#pragma unroll
-    for (int i = 0; i < 14; ++i) {
-        const uint32_t x = __reduce_add_sync(kFullMask, v[i]);
-        if (lane == 0 && x) atomicAdd(O.counters + slot[i], (unsigned long long)x);
-    }
-    if (lane == 0) {
-        atomicAdd(O.counters + 6, iters);
-        atomicAdd(O.counters + 7, lanes_used);
-    }
-    if (status) atomicOr(O.status, status);
+#undef ST
+#undef STF
+#undef STORE3
+    if (lane < kNCount && acc) atomicAdd(O.counters + kCtaCounters + lane, (unsigned long long)acc);
 }
 
-// dynamic shared memory and resident CTAs of one shape (the same in every
-// mode: the launch bounds cap each mode's registers alike)
-template <int SPL, int WARPS>
-static cudaError_t cta_shape(int n_geoms, const LaunchCfg &cfg, size_t *smem, int *ctas, int *ng) {
+// The launch shapes: 448 threads by default, or 128, 256 or 512
+// (gpet_options.block_size); slots of a lane class without and with the
+// phantom's state words, and CTAs an SM.  Measured on a sweep position (1e7
+// pairs, transport ms) and on the hot-rod phantom (5e6 pairs): 12 warps 1.31 and
+// 1.97, 14 warps 1.28 and 1.89, 15 warps 1.27 and 1.88 (two CTAs an SM each);
+// 8 warps 1.66 (two CTAs) and 1.57 (three); 20 warps (one CTA) 1.68.
+template <int WARPS>
+struct Shape;
+template <> struct Shape<4> { static constexpr int kPlain = 12, kPhantom = 10, kCtas = 4; };
+template <> struct Shape<8> { static constexpr int kPlain = 18, kPhantom = 16, kCtas = 3; };
+template <> struct Shape<14> { static constexpr int kPlain = 32, kPhantom = 28, kCtas = 2; };
+template <> struct Shape<16> { static constexpr int kPlain = 32, kPhantom = 28, kCtas = 2; };
+
+using CtaKernel = void (*)(WorkDev, OutDev, int);
+
+template <int WARPS>
+static CtaKernel cta_kernel(const LaunchCfg &cfg, size_t *pool) {
+    using S = Shape<WARPS>;
+    *pool = cfg.phantom ? sizeof(CtaPool<S::kPhantom, true>) : sizeof(CtaPool<S::kPlain, false>);
+    if (cfg.live) return k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, true>;
+    if (cfg.phantom)
+        return cfg.posed ? k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, false>
+                         : k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, false, false>;
+    return cfg.posed ? k_transport_cta<WARPS, S::kPlain, S::kCtas, false, true, false>
+                     : k_transport_cta<WARPS, S::kPlain, S::kCtas, false, false, false>;
+}
+
+static CtaKernel cta_kernel(const LaunchCfg &cfg, int *threads, size_t *pool) {
+    switch (cfg.block_size) {
+        case 128: *threads = 128; return cta_kernel<4>(cfg, pool);
+        case 256: *threads = 256; return cta_kernel<8>(cfg, pool);
+        case 512: *threads = 512; return cta_kernel<16>(cfg, pool);
+        default: *threads = kCtaThreads; return cta_kernel<kCtaThreads / 32>(cfg, pool);
+    }
+}
+
+// kernel, threads, dynamic shared memory and resident CTAs of the launch that cfg selects
+static cudaError_t cta_shape(int n_geoms, const LaunchCfg &cfg, CtaKernel *k, int *threads, size_t *smem, int *ctas,
+                             int *ng) {
+    size_t pool = 0;
     int occ = 0;
-    cudaError_t e = staged_geometry(k_transport_cta<SPL, WARPS, kModeFixed>, WARPS * 32, sizeof(CtaPool<SPL>) * WARPS,
-                                    n_geoms, cfg.max_smem_geoms, ng, smem, &occ);
+    *k = cta_kernel(cfg, threads, &pool);
+    cudaError_t e = staged_geometry(*k, *threads, pool, n_geoms, cfg.max_smem_geoms, ng, smem, &occ);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
     *ctas = cfg.sm_count * occ;
     return cudaSuccess;
 }
 
-template <int SPL, int WARPS>
-static cudaError_t launch_cta(const WorkDev &W, const OutDev &O, const LaunchCfg &cfg, cudaStream_t st) {
-    size_t smem = 0;
-    int ctas = 0, ng = 0;
-    cudaError_t e = cta_shape<SPL, WARPS>(W.n_geoms, cfg, &smem, &ctas, &ng);
-    if (e != cudaSuccess) return e;
-    // a live launch runs one event per choice (its compaction interval is 1)
-    const int repeat = max(1, cfg.compact_every);
-    if (W.live_tail) k_transport_cta<SPL, WARPS, kModeLive><<<ctas, WARPS * 32, smem, st>>>(W, O, ng, 1);
-    else if (repeat > 1) k_transport_cta<SPL, WARPS, kModeRepeat><<<ctas, WARPS * 32, smem, st>>>(W, O, ng, repeat);
-    else k_transport_cta<SPL, WARPS, kModeFixed><<<ctas, WARPS * 32, smem, st>>>(W, O, ng, 1);
-    return cudaGetLastError();
-}
-
-template <int SPL, int WARPS>
-static cudaError_t warps_cta(int n_geoms, const LaunchCfg &cfg, long long *warps) {
-    size_t smem = 0;
-    int ctas = 0, ng = 0;
-    cudaError_t e = cta_shape<SPL, WARPS>(n_geoms, cfg, &smem, &ctas, &ng);
-    *warps = (long long)ctas * WARPS;
-    return e;
-}
-
 // resident warps of the launch that launch_transport_cta makes
 cudaError_t cta_resident_warps(int n_geoms, const LaunchCfg &cfg, long long *warps) {
-    if (cfg.pool_depth == 3) {
-        switch (cfg.block_size) {
-            case 128: return warps_cta<3, 4>(n_geoms, cfg, warps);
-            case 512: return warps_cta<3, 16>(n_geoms, cfg, warps);
-            default: return warps_cta<3, 8>(n_geoms, cfg, warps);
-        }
-    }
-    switch (cfg.block_size) {
-        case 128: return warps_cta<2, 4>(n_geoms, cfg, warps);
-        case 512: return warps_cta<2, 16>(n_geoms, cfg, warps);
-        default: return warps_cta<2, 8>(n_geoms, cfg, warps);
-    }
+    CtaKernel k;
+    size_t smem = 0;
+    int threads = 0, ctas = 0, ng = 0;
+    cudaError_t e = cta_shape(n_geoms, cfg, &k, &threads, &smem, &ctas, &ng);
+    *warps = (long long)ctas * (threads / 32);
+    return e;
 }
 
 cudaError_t launch_transport_cta(const WorkDev &W, const OutDev &O, const LaunchCfg &cfg, cudaStream_t st) {
-    // block_size selects the CTA width; pool_depth 3 deepens the per-warp pools
-    if (cfg.pool_depth == 3) {
-        switch (cfg.block_size) {
-            case 128: return launch_cta<3, 4>(W, O, cfg, st);
-            case 512: return launch_cta<3, 16>(W, O, cfg, st);
-            default: return launch_cta<3, 8>(W, O, cfg, st);
-        }
-    }
-    switch (cfg.block_size) {
-        case 128: return launch_cta<2, 4>(W, O, cfg, st);
-        case 512: return launch_cta<2, 16>(W, O, cfg, st);
-        default: return launch_cta<2, 8>(W, O, cfg, st);
-    }
+    CtaKernel k;
+    size_t smem = 0;
+    int threads = 0, ctas = 0, ng = 0;
+    cudaError_t e = cta_shape(W.n_geoms, cfg, &k, &threads, &smem, &ctas, &ng);
+    if (e != cudaSuccess) return e;
+    k<<<ctas, threads, smem, st>>>(W, O, ng);
+    return cudaGetLastError();
 }
 
-template <int SPL, int WARPS>
-static cudaError_t preload_cta() {
-    const size_t bytes = sizeof(CtaPool<SPL>) * WARPS + (size_t)kMaxStagedGeoms * sizeof(GeomDev);
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void *>(k_transport_cta<SPL, WARPS, kModeFixed>), bytes);
-    if (e == cudaSuccess)
-        e = ensure_dynamic_smem(reinterpret_cast<const void *>(k_transport_cta<SPL, WARPS, kModeRepeat>), bytes);
-    if (e == cudaSuccess)
-        e = ensure_dynamic_smem(reinterpret_cast<const void *>(k_transport_cta<SPL, WARPS, kModeLive>), bytes);
-    return e;
+void cta_counters(unsigned long long *c, const unsigned long long *raw) {
+    static_assert((int)kNCount == kCtaCounterSlots, "one raw slot per count");
+    c[0] += raw[kPhPanel];
+    c[1] += raw[kPhFlight] + raw[kPhFlightOut] + raw[kNScrStart];
+    c[2] += raw[kNTrials];
+    c[3] += raw[kNEntered];
+    c[4] += raw[kPhPhantom];
+    c[5] += raw[kNHits];
+    c[6] += raw[kNIter];
+    c[7] += raw[kNLanes];
+    c[8] += raw[kNScrStart] + raw[kNScrFlight];
+    c[9] += raw[kNSingles];
+    // events per phase: slots 10 + phase
+    c[10 + kPhSource] += raw[kPhIdle];
+    c[10 + kPhPhantom] += raw[kPhPhantom];
+    c[10 + kPhFlight] += raw[kPhFlight];
+    c[10 + kPhPanel] += raw[kPhPanel];
+    c[10 + kPhFinish] += raw[kNFin];
+    c[10 + kPhFlightOut] += raw[kPhFlightOut];
 }
 
 // load every instantiation and set its shared-memory limit (internal.h)
 cudaError_t preload_cta_kernels() {
-    cudaError_t e = preload_cta<2, 4>();
-    if (e == cudaSuccess) e = preload_cta<2, 8>();
-    if (e == cudaSuccess) e = preload_cta<2, 16>();
-    if (e == cudaSuccess) e = preload_cta<3, 4>();
-    if (e == cudaSuccess) e = preload_cta<3, 8>();
-    if (e == cudaSuccess) e = preload_cta<3, 16>();
-    return e;
+    LaunchCfg cfg{};
+    for (int block : {128, 256, kCtaThreads, 512})
+        for (int form = 0; form < 5; ++form) {
+            cfg.block_size = block;
+            cfg.phantom = form >= 2;
+            cfg.posed = form == 1 || form >= 3;
+            cfg.live = form == 4;
+            int threads = 0;
+            size_t pool = 0;
+            CtaKernel k = cta_kernel(cfg, &threads, &pool);
+            cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void *>(k),
+                                                pool + (size_t)kMaxStagedGeoms * sizeof(GeomDev));
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 }  // namespace gpet
