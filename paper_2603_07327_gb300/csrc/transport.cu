@@ -106,10 +106,17 @@ __global__ void __launch_bounds__(128) k_transport_redo(WorkDev W, OutDev O) {
     const unsigned long long n = min(*O.n_ovf, O.ovf_cap);
     Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
     int status = kStatusOk;
+    // The list is short (about 1e-4 of the histories) and its histories take
+    // different branches at every event: they are dealt to the warps one by one,
+    // so that lanes of a warp share one only once every warp has a history.
+    // (Dealt to consecutive threads, the 130 or 1300 histories of runs of 1e6
+    // and 1e7 pairs took 100 us; this way 38 and 30 us.)
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    const unsigned long long base0 = (unsigned long long)blockIdx.x * blockDim.x;
-    for (unsigned long long base = base0; base < n; base += stride) {
-        const unsigned long long i = base + threadIdx.x;
+    const unsigned long long warps = stride / 32;
+    const unsigned long long mine = (unsigned long long)(threadIdx.x & 31) * warps +
+                                    ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+    for (unsigned long long base = 0; base < n; base += stride) {
+        const unsigned long long i = base + mine;
         PState s;
         s.phase = kPhIdle;
         s.job = 0;
