@@ -45,10 +45,12 @@ enum : uint32_t { kTagSource = 1u, kTagPhantom = 2u, kTagDetector = 3u, kTagDigi
 // kStatusSortStall: a radix-sort tile copy or look-back did not complete
 // within the wait limit, or a pass computed an offset past its keys; the sort
 // stops (or skips the write) and its output is invalid (an internal error).
+// kStatusBuckets: a time bucket of the sort held more singles than one pass
+// sorts; the run is repeated with the radix passes.
 // kStatusLiveStall: a live launch found no new work and no end of the work
 // queue for the whole idle-wait limit; its CTAs stop (an internal error).
 enum : int { kStatusOk = 0, kStatusTimeout = 1, kStatusOverflow = 2, kStatusBadPhase = 4, kStatusSortStall = 8,
-             kStatusLiveStall = 16 };
+             kStatusLiveStall = 16, kStatusBuckets = 32 };
 
 // ---------------------------------------------------------------------------
 // geometry descriptor (FP32, one per scanner design)

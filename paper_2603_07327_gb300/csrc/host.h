@@ -83,6 +83,9 @@ struct Run {
     std::vector<unsigned long long> chunk_start;
     unsigned int chunk_size = 2048;
     RunCaps caps;
+    bool radix_only = false;             // the time sort takes the radix passes (a bucket overflowed)
+    std::vector<BucketJob> buckets;      // per job; empty: radix passes
+    BucketJob *d_buckets = nullptr;
     bool keep_hits = false;
     LaunchCfg cfg{};
     // arena

@@ -23,7 +23,13 @@ struct LaunchCfg {
     bool live;           // a live launch
 };
 
-// radix sort working set (keys ping-pong between two buffers)
+// one job's time buckets: a time t falls in bucket first + min(hi64(t * scale), n - 1)
+struct BucketJob {
+    uint64_t scale;
+    uint32_t first, n;
+};
+
+// working set of the time sort (the radix passes ping-pong between two buffers)
 struct SortDev {
     uint64_t *keys[2];
     uint32_t *vals[2];
@@ -41,7 +47,20 @@ struct SortDev {
     // tile counter per pass; NULL where the passes run through tile_hist
     unsigned long long *lb[2] = {nullptr, nullptr};
     unsigned int *tile_ctr = nullptr;
+    // time buckets (n_buckets = 0: none, radix passes): per-job tables, the
+    // counts of the buckets (then their first positions, n_buckets + 1 of them),
+    // the scan's look-back words and tile counter
+    const BucketJob *bjobs = nullptr;
+    uint32_t *bstart = nullptr;
+    unsigned long long *bscan = nullptr;
+    uint32_t n_buckets = 0;
 };
+
+// singles per time bucket at one single per history, most singles of one
+// bucket, and the narrowest bucket (ps): see sort.cu
+constexpr uint32_t kBucketHistories = 32, kBucketMax = 1024;
+constexpr uint64_t kBucketMinPs = 10000;
+constexpr uint32_t kBucketScanTile = 4096;
 
 // Bit position of the job index in the 64-bit sort keys of a launch of n_jobs
 // jobs: the job takes the fewest high bits that number the jobs, the time stamp
@@ -74,6 +93,8 @@ struct CoincDev {
 
 struct JobStatsDev {
     int n_jobs;
+    const BucketJob *bjobs;              // time buckets of the sort, or NULL: first positions of the jobs' singles
+    const uint32_t *bstart;
     unsigned long long *s_off, *c_off;   // [n_jobs + 1]
     unsigned long long *hits;            // [n_jobs]
     const unsigned long long *tally_count;

@@ -147,6 +147,28 @@ int run_plan(Run &R) {
         R.chunk_start[j + 1] = R.chunk_start[j] + (R.jobs[j].n_hist + cs - 1) / cs;
     R.live_tail = R.chunk_start[nj];
 
+    // Time buckets of the sort (see sort.cu), where the run's jobs allow them: a
+    // bucket for every kBucketHistories histories of a job, none narrower than
+    // kBucketMinPs (a photon's flight time then hardly moves a single to the
+    // next one, so that singles spread over the buckets as the decay times do).
+    // Live launches (their jobs come later) and digitize-only runs sort by radix.
+    uint64_t n_buckets = 0;
+    R.buckets.clear();
+    if (!R.live && !R.digitize_only && !R.radix_only) {
+        for (const JobDev &J : R.jobs) {
+            const uint64_t span = J.t_span_ps;
+            const uint64_t nb = std::min<uint64_t>(J.n_hist / kBucketHistories, span / kBucketMinPs);
+            if (span == 0 || J.n_hist / std::max<uint64_t>(nb, 1) > kBucketMax / 2 || n_buckets + nb > 0x3FFFFFFFu) {
+                R.buckets.clear();
+                n_buckets = 0;
+                break;
+            }
+            const uint32_t n = (uint32_t)std::max<uint64_t>(nb, 1);
+            R.buckets.push_back({n == 1 ? 0 : (uint64_t)(((unsigned __int128)n << 64) / span), (uint32_t)n_buckets, n});
+            n_buckets += n;
+        }
+    }
+
     // The first guess of the singles capacity (0.6 per history) may exceed what
     // a long run needs by far (a narrow energy window keeps few singles): it
     // takes at most a quarter of the free device memory.  The device counts
@@ -176,6 +198,10 @@ int run_plan(Run &R) {
     cv.take(R.d_tally_efx, (size_t)tcc);
     const size_t nwin = R.win_lo.size();
     if (nwin) cv.take(R.d_win_counts, (size_t)njc * nwin);
+    if (n_buckets) {
+        cv.take(R.S.bstart, n_buckets + 1);
+        cv.take(R.S.bscan, n_buckets / kBucketScanTile + 3);
+    }
     R.zero_bytes = align_up(cv.off, 256);
     cv.take(R.d_live, 3);
     cv.take(R.d_jobs, njc);
@@ -194,6 +220,7 @@ int run_plan(Run &R) {
     if (pfc) cv.take(R.d_pose, pfc);
     cv.take(R.d_chunk_start, njc + 1);
     cv.take(R.d_window, njc);
+    if (n_buckets) cv.take(R.d_buckets, njc);
     // raw singles
     OutDev &O = R.O;
     cv.take(O.s_raw, cap);
@@ -242,6 +269,17 @@ int run_plan(Run &R) {
     rebase(R.d_tally_count, base);
     rebase(R.d_tally_efx, base);
     if (nwin) rebase(R.d_win_counts, base); else R.d_win_counts = nullptr;
+    if (n_buckets) {
+        rebase(S.bstart, base);
+        rebase(S.bscan, base);
+        rebase(R.d_buckets, base);
+    } else {
+        S.bstart = nullptr;
+        S.bscan = nullptr;
+        R.d_buckets = nullptr;
+    }
+    S.n_buckets = (uint32_t)n_buckets;
+    S.bjobs = R.d_buckets;
     rebase(R.d_live, base);
     rebase(R.d_jobs, base); rebase(R.d_geoms, base); rebase(R.d_chunk_start, base); rebase(R.d_window, base);
     if (pfc) rebase(R.d_pose, base);
@@ -265,6 +303,8 @@ int run_plan(Run &R) {
     rebase(JS.s_off, base); rebase(JS.c_off, base); rebase(JS.hits, base); rebase(R.d_toff, base);
     rebase(R.d_tn, base);
     JS.n_jobs = nj;
+    JS.bjobs = S.bjobs;
+    JS.bstart = S.bstart;
     JS.tally_count = R.d_tally_count;
     JS.tally_off = R.d_toff;
     JS.tally_n = R.d_tn;
@@ -323,6 +363,8 @@ int run_plan(Run &R) {
                             cudaMemcpyHostToDevice, up);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(R.d_window, R.windows.data(), sizeof(uint64_t) * nj, cudaMemcpyHostToDevice, up);
+    if (e == cudaSuccess && n_buckets)
+        e = cudaMemcpyAsync(R.d_buckets, R.buckets.data(), sizeof(BucketJob) * nj, cudaMemcpyHostToDevice, up);
     std::vector<long long> toff(R.tally_off.begin(), R.tally_off.end()), tn(R.job_crystals.begin(), R.job_crystals.end());
     if (e == cudaSuccess) e = cudaMemcpyAsync(R.d_toff, toff.data(), sizeof(long long) * nj, cudaMemcpyHostToDevice, up);
     if (e == cudaSuccess) e = cudaMemcpyAsync(R.d_tn, tn.data(), sizeof(long long) * nj, cudaMemcpyHostToDevice, up);
@@ -449,6 +491,8 @@ int run_collect(Run &R) {
                          H.n_singles, R.O.s_cap, H.n_hits, R.O.hit_cap, H.n_ovf, R.O.ovf_cap);
     if (H.status & kStatusBadPhase)
         return gpet_fail(GPET_ERR_CUDA, "internal error: a history reached a phase no event handles");
+    if (H.status & kStatusBuckets)
+        return gpet_fail(GPET_ERR_OVERFLOW, "a time bucket of the sort holds more than %u singles", kBucketMax);
     if (H.status & kStatusLiveStall)
         return gpet_fail(GPET_ERR_CUDA,
                          "internal error: a live launch waited %.3f s for work or its end (it last saw %llu "
@@ -501,7 +545,8 @@ size_t run_footprint(uint64_t total_decays, int64_t total_crystals, int n_jobs, 
 
 int run_with_retry(Run &R) {
     int st = GPET_OK;
-    for (int attempt = 0; attempt < 2; ++attempt) {
+    bool resized = false;
+    for (int attempt = 0; attempt < 3; ++attempt) {
         st = run_plan(R);
         if (st == GPET_OK) st = run_enqueue(R);
         if (st == GPET_OK) st = run_collect(R);
@@ -510,7 +555,14 @@ int run_with_retry(Run &R) {
                            R.h_hdr.n_singles, (unsigned long long)kMaxSinglesPerLaunch);
             break;
         }
-        if (st == GPET_ERR_OVERFLOW && attempt == 0 && !(R.h_hdr.status & kStatusOverflow)) {
+        if (st == GPET_ERR_OVERFLOW && (R.h_hdr.status & kStatusBuckets) && !R.radix_only) {
+            // (the decay times are not spread as their model says: sort without buckets)
+            R.radix_only = true;
+            run_release(R);
+            continue;
+        }
+        if (st == GPET_ERR_OVERFLOW && !resized && !(R.h_hdr.status & kStatusOverflow)) {
+            resized = true;
             // the device counters kept counting past the capacities: re-run with exact sizes
             R.caps.guess = false;
             R.caps.singles = std::max<uint64_t>(R.caps.singles, R.h_hdr.n_singles + 1024);

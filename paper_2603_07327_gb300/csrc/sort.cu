@@ -593,23 +593,196 @@ static cudaError_t scatter_smem_attr() {
     return ensure_dynamic_smem(reinterpret_cast<const void *>(k_onesweep), kScatterSmemStaged);
 }
 
-// singles into time order
-__global__ void k_gather(SortDev S, SinglesDev out) {
+// ---------------------------------------------------------------------------
+// Time buckets.  Decay times are uniform over a run's span (their model), so a
+// linear map of the time spreads a job's singles evenly over its buckets, and
+// the sort is four passes whatever the key's length, where the radix sort takes
+// one per varying byte: count the buckets (each single keeps its rank of
+// arrival there), turn the counts into first positions, place each single's
+// index, and order each bucket by comparing its few singles with one another
+// while they are gathered into the time-ordered arrays.  Keys order by time,
+// then by arrival (the single's index), as the stable radix sort orders them.
+// A bucket covers kBucketHistories histories' share of the span: up to about
+// that many singles, 5 on average in a sweep ring.  More than kBucketMax in one
+// (times that are not uniform after all) sets kStatusBuckets, and the run is
+// repeated with the radix passes.
+// What bounds the passes is latency at 1e5 singles and the random accesses to
+// counters and records beyond: 150 B of DRAM per single against the radix
+// sort's 330.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t bucket_of(const SortDev &S, uint64_t key) {
+    const int job = S.job_shift < 64 ? (int)(key >> S.job_shift) : 0;
+    const uint64_t t = S.job_shift < 64 ? key & ((1ull << S.job_shift) - 1ull) : key;
+    const uint64_t scale = __ldg(reinterpret_cast<const unsigned long long *>(&S.bjobs[job].scale));
+    const uint2 fn = __ldg(reinterpret_cast<const uint2 *>(&S.bjobs[job].first));
+    return fn.x + (uint32_t)min(__umul64hi(t, scale), (unsigned long long)(fn.y - 1u));
+}
+
+__global__ void __launch_bounds__(256) k_bucket_count(SortDev S) {
+    const unsigned long long n = sort_n(S), step = (unsigned long long)gridDim.x * blockDim.x;
+    for (unsigned long long i0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * step) {
+        uint32_t r[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {   // (four counters in flight per thread)
+            const unsigned long long i = i0 + j * step;
+            if (i < n) r[j] = atomicAdd(S.bstart + bucket_of(S, __ldg(S.keys[0] + i)), 1u);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned long long i = i0 + j * step;
+            if (i < n) S.vals[0][i] = r[j];
+        }
+    }
+}
+
+// Sum of the totals of the tiles before `tile`, by its first warp: its own
+// total is published, then the words of earlier tiles are read, 32 a round trip
+// and newest first, to an inclusive sum; the tile's own inclusive sum follows.
+// Tiles are claimed in order and wait only for earlier ones, so the waits end;
+// false when a word did not come within the wait limit.
+__device__ __forceinline__ bool warp_lookback(unsigned long long *words, uint32_t tile, uint32_t total, uint32_t &base) {
+    const uint32_t lane = threadIdx.x & 31;
+    if (lane == 0) lb_store(words + tile, (tile == 0 ? kLbIncl : kLbAgg) | total);
+    base = 0;
+    bool ok = true;
+    for (uint32_t j = tile; j > 0 && ok;) {
+        unsigned long long w = kLbIncl;   // (before tile 0: nothing)
+        if (lane < j) {
+            const unsigned long long *p = words + (j - 1 - lane);
+            w = lb_load(p);
+            for (int polls = 0; (w >> 62) == 0 && polls < kLookbackPolls; ++polls) {
+                if (polls > 64) __nanosleep(64);
+                w = lb_load(p);
+            }
+        }
+        ok = !__any_sync(kFullMask, (w >> 62) == 0);
+        const uint32_t incl = __ballot_sync(kFullMask, (w >> 62) == 2);
+        const uint32_t last = incl ? (uint32_t)__ffs(incl) - 1u : 31u;
+        base += __reduce_add_sync(kFullMask, lane <= last ? (uint32_t)(w & kLbCount) : 0u);
+        j = incl ? 0u : j - 32u;
+    }
+    if (lane == 0 && tile > 0) lb_store(words + tile, kLbIncl | (unsigned long long)(base + total));
+    return ok;
+}
+
+// bucket counts to first positions, in place (n_buckets + 1 of them): one pass,
+// tiles in the order of a ticket, each tile's base by looking back
+__global__ void __launch_bounds__(1024) k_bucket_scan(SortDev S) {
+    __shared__ uint32_t sw[32];
+    __shared__ uint32_t tile_sh, base_sh;
+    __shared__ int fail_sh;
+    if (threadIdx.x == 0) tile_sh = (uint32_t)atomicAdd(S.bscan, 1ull);
+    __syncthreads();
+    const uint32_t tile = tile_sh, m = S.n_buckets + 1u;
+    const uint64_t b = (uint64_t)tile * kBucketScanTile + 4u * threadIdx.x;
+    uint32_t v[4], sum = 0, most = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        v[j] = b + j < m ? S.bstart[b + j] : 0u;
+        sum += v[j];
+        most = max(most, v[j]);
+    }
+    if (__syncthreads_or(most > kBucketMax) && threadIdx.x == 0) atomicOr(S.status, kStatusBuckets);
+    uint32_t tot;
+    uint32_t x = block_exscan(sum, tot, sw);
+    if (threadIdx.x < 32) {
+        uint32_t base = 0;
+        const bool ok = warp_lookback(S.bscan + 1, tile, tot, base);
+        if (threadIdx.x == 0) {
+            if (!ok) atomicOr(S.status, kStatusSortStall);
+            base_sh = base;
+            fail_sh = !ok;
+        }
+    }
+    __syncthreads();
+    if (fail_sh) return;
+    x += base_sh;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (b + j < m) S.bstart[b + j] = x;
+        x += v[j];
+    }
+}
+
+// each single's index to its bucket's next place, in order of arrival
+__global__ void __launch_bounds__(256) k_bucket_place(SortDev S) {
+    const unsigned long long n = sort_n(S);
+    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (unsigned long long)gridDim.x * blockDim.x) {
+        const uint32_t pos = S.bstart[bucket_of(S, __ldg(S.keys[0] + i))] + S.vals[0][i];
+        if (pos < n) S.vals[1][pos] = (uint32_t)i;   // (always, unless the scan gave up)
+    }
+}
+
+constexpr int kBucketCta = 1024;   // singles a CTA orders: the buckets that start in its stretch of positions
+constexpr int kBucketRoom = kBucketCta + (int)kBucketMax;
+
+// a single's record from the transport to place i of the time-ordered arrays
+__device__ __forceinline__ void gather_one(const RawSingle *src, const SinglesDev &out, const CoincDev &C,
+                                           unsigned long long i) {
+    const uint4 *r = reinterpret_cast<const uint4 *>(src);
+    const uint4 a = __ldg(r), b = __ldg(r + 1), c = __ldg(r + 2);
+    out.t[i] = ((uint64_t)a.y << 32) | a.x;
+    out.h[i] = ((uint64_t)a.w << 32) | a.z;
+    out.unit[i] = (int32_t)b.x;
+    out.panel[i] = (int32_t)b.y;
+    out.job[i] = (int32_t)b.z;
+    out.e[i] = __uint_as_float(b.w);
+    out.eraw[i] = __uint_as_float(c.x);
+    out.doi[i] = __uint_as_float(c.y);
+    C.flag[i] = 0;   // the coincidence pass sets flags anywhere
+}
+
+// first place at or after x where a bucket starts
+__device__ __forceinline__ uint32_t bucket_edge(const SortDev &S, unsigned long long x, unsigned long long n) {
+    if (x >= n) return (uint32_t)n;
+    const uint32_t b = bucket_of(S, __ldg(S.keys[0] + S.vals[1][x]));
+    const uint32_t s = S.bstart[b];
+    return s == (uint32_t)x ? s : S.bstart[b + 1];
+}
+
+__global__ void __launch_bounds__(256) k_bucket_sort(SortDev S, SinglesDev out, CoincDev C) {
+    __shared__ uint64_t key[kBucketRoom];
+    __shared__ uint32_t idx[kBucketRoom];
+    __shared__ uint32_t edge[2];
+    const unsigned long long n = sort_n(S);
+    // (a failed run hands nothing on: its arrays are not written)
+    const bool failed = *reinterpret_cast<volatile int *>(S.status) & (kStatusBuckets | kStatusSortStall);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *out.n = failed ? 0ull : n;
+    if (failed) return;
+    for (unsigned long long x = (unsigned long long)blockIdx.x * kBucketCta; x < n; x += (unsigned long long)gridDim.x * kBucketCta) {
+        if (threadIdx.x < 2) edge[threadIdx.x] = bucket_edge(S, x + threadIdx.x * kBucketCta, n);
+        __syncthreads();
+        const uint32_t p0 = edge[0], m = min(edge[1] - p0, (uint32_t)kBucketRoom);
+        for (uint32_t i = threadIdx.x; i < m; i += 256) {
+            const uint32_t v = S.vals[1][p0 + i];
+            idx[i] = v;
+            key[i] = __ldg(S.keys[0] + v);
+        }
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < m; i += 256) {
+            const uint64_t k = key[i];
+            const uint32_t v = idx[i], b = bucket_of(S, k);
+            const uint32_t s = S.bstart[b] - p0, e = min(S.bstart[b + 1] - p0, m);
+            uint32_t at = s;
+            for (uint32_t j = s; j < e; ++j) {
+                const uint64_t kj = key[j];
+                at += kj < k || (kj == k && idx[j] < v);
+            }
+            gather_one(S.in_raw + v, out, C, p0 + at);
+        }
+        __syncthreads();
+    }
+}
+
+// singles into time order, after the radix passes
+__global__ void k_gather(SortDev S, SinglesDev out, CoincDev C) {
     const unsigned long long n = sort_n(S);
     const int fin = S.plan[2 * kPasses];
     const uint32_t *perm = fin ? S.vals[1] : S.vals[0];
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
-        const uint4 *r = reinterpret_cast<const uint4 *>(S.in_raw + perm[i]);
-        const uint4 a = __ldg(r), b = __ldg(r + 1), c = __ldg(r + 2);
-        out.t[i] = ((uint64_t)a.y << 32) | a.x;
-        out.h[i] = ((uint64_t)a.w << 32) | a.z;
-        out.unit[i] = (int32_t)b.x;
-        out.panel[i] = (int32_t)b.y;
-        out.job[i] = (int32_t)b.z;
-        out.e[i] = __uint_as_float(b.w);
-        out.eraw[i] = __uint_as_float(c.x);
-        out.doi[i] = __uint_as_float(c.y);
+        gather_one(S.in_raw + perm[i], out, C, i);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) *out.n = n;
 }
@@ -698,34 +871,46 @@ __global__ void __launch_bounds__(1024) k_coinc_write(SinglesDev s, CoincDev C) 
 // Per-job statistics of a (batched) run: start of each job's segment in the
 // time-sorted singles and in the coincidences (both are ordered by job, the
 // high bits of the sort key), and the job's hit count from its tallies.
-__global__ void __launch_bounds__(256) k_job_stats(SinglesDev s, CoincDev C, JobStatsDev J) {
+// One warp searches each of the two (32 probes a round: 4 dependent loads for
+// 1e6 singles where a bisection by one thread takes 20) while the others sum.
+template <class JobOf>
+__device__ __forceinline__ unsigned long long warp_lower_bound(unsigned long long n, int j, JobOf job_of) {
+    unsigned long long lo = 0, hi = n;   // first i with job_of(i) >= j lies in [lo, hi]
+    while (lo < hi) {
+        const unsigned long long step = (hi - lo + 32) / 33;
+        const unsigned long long p = lo + step * ((threadIdx.x & 31) + 1) - 1;
+        const uint32_t below = __popc(__ballot_sync(kFullMask, p < hi && job_of(p) < j));
+        const unsigned long long l = lo + step * below, h = l + step - 1;
+        hi = below == 32 || h > hi ? hi : h;
+        lo = l < hi ? l : hi;
+    }
+    return lo;
+}
+
+__global__ void __launch_bounds__(512) k_job_stats(SinglesDev s, CoincDev C, JobStatsDev J) {
     const int j = blockIdx.x;
     const unsigned long long ns = *s.n, nc = *C.n;
-    if (threadIdx.x == 0) {
-        unsigned long long lo = 0, hi = ns;  // first single with job >= j
-        while (lo < hi) {
-            const unsigned long long mid = (lo + hi) >> 1;
-            if (s.job[mid] < j) lo = mid + 1; else hi = mid;
-        }
-        J.s_off[j] = lo;
-        lo = 0;
-        hi = nc;                             // first coincidence whose first single has job >= j
-        while (lo < hi) {
-            const unsigned long long mid = (lo + hi) >> 1;
-            if (s.job[C.a[mid]] < j) lo = mid + 1; else hi = mid;
-        }
-        J.c_off[j] = lo;
-        if (j == J.n_jobs - 1) {
-            J.s_off[J.n_jobs] = ns;
-            J.c_off[J.n_jobs] = nc;
-        }
+    const int wid = threadIdx.x >> 5;
+    if (wid == 0) {   // first coincidence whose first single has job >= j
+        const unsigned long long lo = j == 0 ? 0 : warp_lower_bound(nc, j, [&](unsigned long long i) { return s.job[C.a[i]]; });
+        if (threadIdx.x == 0) J.c_off[j] = lo;
+    } else if (wid == 1) {   // first single with job >= j
+        const unsigned long long lo = j == 0 ? 0
+                                      : J.bjobs ? J.bstart[J.bjobs[j].first]
+                                                : warp_lower_bound(ns, j, [&](unsigned long long i) { return s.job[i]; });
+        if (threadIdx.x == 32) J.s_off[j] = lo;
+    }
+    if (threadIdx.x == 0 && j == J.n_jobs - 1) {
+        J.s_off[J.n_jobs] = ns;
+        J.c_off[J.n_jobs] = nc;
     }
     // hits of job j = sum of its per-crystal counts
     unsigned long long acc = 0;
     const unsigned long long *t = J.tally_count + J.tally_off[j];
     const long long nt = J.tally_n[j];
-    for (long long i = threadIdx.x; i < nt; i += blockDim.x) acc += t[i];
-    __shared__ unsigned long long red[8];
+#pragma unroll 8
+    for (long long i = threadIdx.x; i < nt; i += 512) acc += t[i];
+    __shared__ unsigned long long red[16];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFullMask, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
@@ -737,7 +922,7 @@ __global__ void __launch_bounds__(256) k_job_stats(SinglesDev s, CoincDev C, Job
 }
 
 cudaError_t launch_job_stats(const SinglesDev &s, const CoincDev &C, const JobStatsDev &J, cudaStream_t st) {
-    k_job_stats<<<J.n_jobs, 256, 0, st>>>(s, C, J);
+    k_job_stats<<<J.n_jobs, 512, 0, st>>>(s, C, J);
     return cudaGetLastError();
 }
 
@@ -764,20 +949,27 @@ cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const Coi
     if (!S.status || !S.lb[0] || !S.lb[1] || !S.tile_ctr) return cudaErrorInvalidValue;
     cudaError_t e = scatter_smem_attr();
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(S.ghist, 0, sizeof(uint32_t) * kPasses * 256, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(S.tile_ctr, 0, sizeof(unsigned int) * kPasses, st);
-    if (e != cudaSuccess) return e;
-    k_make_keys<<<sm_count * 4, kSortThreads, 0, st>>>(S);
-    k_plan<<<1, kPasses * 32, 0, st>>>(S);
-    // two CTAs per SM are resident; more would only claim tiles later
-    const int tg = (int)(S.max_tiles < (unsigned long long)sm_count * 2 ? (S.max_tiles ? S.max_tiles : 1)
-                                                                        : (unsigned long long)sm_count * 2);
-    for (int p = 0; p < kPasses; ++p) k_onesweep<<<tg, kSortThreads, kScatterSmemStaged, st>>>(S, p);
     const int grid = sm_count * 4;
-    k_gather<<<grid, 256, 0, st>>>(S, out);
-    // a cluster's flags are written by the thread at its start, possibly past
-    // its own grid-stride range: clear them all before the flag kernel
-    e = cudaMemsetAsync(C.flag, 0, S.cap ? S.cap : 1, st);
+    if (S.n_buckets) {
+        const unsigned long long want = (S.cap + kBucketCta - 1) / kBucketCta;
+        const int bg = (int)(want < (unsigned long long)sm_count * 8 ? want : (unsigned long long)sm_count * 8);
+        k_bucket_count<<<bg, 256, 0, st>>>(S);
+        k_bucket_scan<<<(S.n_buckets + kBucketScanTile) / kBucketScanTile, 1024, 0, st>>>(S);
+        k_bucket_place<<<bg, 256, 0, st>>>(S);
+        k_bucket_sort<<<bg, 256, 0, st>>>(S, out, C);
+    } else {
+        e = cudaMemsetAsync(S.ghist, 0, sizeof(uint32_t) * kPasses * 256, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(S.tile_ctr, 0, sizeof(unsigned int) * kPasses, st);
+        if (e != cudaSuccess) return e;
+        k_make_keys<<<sm_count * 4, kSortThreads, 0, st>>>(S);
+        k_plan<<<1, kPasses * 32, 0, st>>>(S);
+        // two CTAs per SM are resident; more would only claim tiles later
+        const int tg = (int)(S.max_tiles < (unsigned long long)sm_count * 2 ? (S.max_tiles ? S.max_tiles : 1)
+                                                                            : (unsigned long long)sm_count * 2);
+        for (int p = 0; p < kPasses; ++p) k_onesweep<<<tg, kSortThreads, kScatterSmemStaged, st>>>(S, p);
+        k_gather<<<grid, 256, 0, st>>>(S, out, C);
+    }
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_coinc_flags<<<grid, 256, 0, st>>>(out, C);
     const int cg = (int)(S.max_tiles < (unsigned long long)sm_count * 4 ? S.max_tiles : (unsigned long long)sm_count * 4);
@@ -791,7 +983,9 @@ cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const Coi
 cudaError_t preload_sort_kernels() {
     const void *fns[] = {reinterpret_cast<const void *>(k_make_keys), reinterpret_cast<const void *>(k_plan),
                          reinterpret_cast<const void *>(k_tile_hist), reinterpret_cast<const void *>(k_digit_scan),
-                         reinterpret_cast<const void *>(k_onesweep),
+                         reinterpret_cast<const void *>(k_onesweep), reinterpret_cast<const void *>(k_bucket_count),
+                         reinterpret_cast<const void *>(k_bucket_scan), reinterpret_cast<const void *>(k_bucket_place),
+                         reinterpret_cast<const void *>(k_bucket_sort),
                          reinterpret_cast<const void *>(k_gather), reinterpret_cast<const void *>(k_coinc_flags),
                          reinterpret_cast<const void *>(k_coinc_count), reinterpret_cast<const void *>(k_coinc_scan),
                          reinterpret_cast<const void *>(k_coinc_write), reinterpret_cast<const void *>(k_job_stats)};
