@@ -60,7 +60,7 @@ struct SortDev {
 // bucket, and the narrowest bucket (ps): see sort.cu
 constexpr uint32_t kBucketHistories = 32, kBucketMax = 1024;
 constexpr uint64_t kBucketMinPs = 10000;
-constexpr uint32_t kBucketScanTile = 4096;
+constexpr uint32_t kBucketScanTile = 4096, kCoincScanTile = 1024;
 
 // Bit position of the job index in the 64-bit sort keys of a launch of n_jobs
 // jobs: the job takes the fewest high bits that number the jobs, the time stamp
@@ -84,8 +84,7 @@ struct SinglesDev {
 };
 
 struct CoincDev {
-    uint8_t *flag;
-    uint32_t *tile_cnt;
+    unsigned long long *scan;        // tile ticket, then a look-back word per tile
     int32_t *a, *b;
     unsigned long long *n;
     const uint64_t *window_ps;       // per job

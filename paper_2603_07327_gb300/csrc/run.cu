@@ -178,8 +178,8 @@ int run_plan(Run &R) {
         size_t free_b = 0, total_b = 0;
         if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
             // arena bytes per single of capacity: raw record, two key and index
-            // buffers, the time-ordered arrays, coincidence flag and pair slots
-            const uint64_t per_single = sizeof(RawSingle) + 2 * 8 + 2 * 4 + 8 + 8 + 6 * 4 + 1 + 4;
+            // buffers, the time-ordered arrays, coincidence pair slots
+            const uint64_t per_single = sizeof(RawSingle) + 2 * 8 + 2 * 4 + 8 + 8 + 6 * 4 + 4;
             R.caps.singles = std::min<uint64_t>(R.caps.singles, std::max<uint64_t>(65536, free_b / 4 / per_single));
         } else {
             cudaGetLastError();
@@ -198,6 +198,7 @@ int run_plan(Run &R) {
     cv.take(R.d_tally_efx, (size_t)tcc);
     const size_t nwin = R.win_lo.size();
     if (nwin) cv.take(R.d_win_counts, (size_t)njc * nwin);
+    cv.take(R.C.scan, cap / kCoincScanTile + 2);
     if (n_buckets) {
         cv.take(R.S.bstart, n_buckets + 1);
         cv.take(R.S.bscan, n_buckets / kBucketScanTile + 3);
@@ -245,8 +246,6 @@ int run_plan(Run &R) {
     cv.take(SD.e, cap); cv.take(SD.eraw, cap); cv.take(SD.doi, cap);
     // coincidences
     CoincDev &C = R.C;
-    cv.take(C.flag, cap);
-    cv.take(C.tile_cnt, tiles);
     cv.take(C.a, cap / 2 + 1); cv.take(C.b, cap / 2 + 1);
     // per-job statistics
     JobStatsDev &JS = R.JS;
@@ -299,7 +298,7 @@ int run_plan(Run &R) {
     rebase(S.plan, base); rebase(S.lb[0], base); rebase(S.lb[1], base); rebase(S.tile_ctr, base);
     rebase(SD.t, base); rebase(SD.h, base); rebase(SD.unit, base); rebase(SD.panel, base); rebase(SD.job, base);
     rebase(SD.e, base); rebase(SD.eraw, base); rebase(SD.doi, base);
-    rebase(C.flag, base); rebase(C.tile_cnt, base); rebase(C.a, base); rebase(C.b, base);
+    rebase(C.scan, base); rebase(C.a, base); rebase(C.b, base);
     rebase(JS.s_off, base); rebase(JS.c_off, base); rebase(JS.hits, base); rebase(R.d_toff, base);
     rebase(R.d_tn, base);
     JS.n_jobs = nj;
@@ -538,7 +537,7 @@ size_t run_footprint(uint64_t total_decays, int64_t total_crystals, int n_jobs, 
     b += ocap * 12;                              // overflow list
     b += cap * (2 * 8 + 2 * 4) + 2 * 256 * 8 * tiles + 8 * 4 + 128;  // sort (look-back words, tile counters)
     b += cap * (8 + 8 + 4 * 6);                  // sorted singles
-    b += cap + 4 * tiles + 2 * 4 * (cap / 2 + 1); // coincidences
+    b += 8 * (cap / kCoincScanTile + 2) + 2 * 4 * (cap / 2 + 1); // coincidences
     b += 8 * (n_jobs + 1) * 2 + 8 * n_jobs * 3;  // per-job statistics
     return b + 64 * 256;                         // alignment slack
 }

@@ -714,12 +714,14 @@ __global__ void __launch_bounds__(256) k_bucket_place(SortDev S) {
     }
 }
 
-constexpr int kBucketCta = 1024;   // singles a CTA orders: the buckets that start in its stretch of positions
+// Singles a CTA orders: the buckets that start in its stretch of positions.  Two
+// a thread: the pass is a chain of dependent loads (index, key, bucket, record),
+// so it wants many CTAs with few singles each.
+constexpr int kBucketCta = 512;
 constexpr int kBucketRoom = kBucketCta + (int)kBucketMax;
 
 // a single's record from the transport to place i of the time-ordered arrays
-__device__ __forceinline__ void gather_one(const RawSingle *src, const SinglesDev &out, const CoincDev &C,
-                                           unsigned long long i) {
+__device__ __forceinline__ void gather_one(const RawSingle *src, const SinglesDev &out, unsigned long long i) {
     const uint4 *r = reinterpret_cast<const uint4 *>(src);
     const uint4 a = __ldg(r), b = __ldg(r + 1), c = __ldg(r + 2);
     out.t[i] = ((uint64_t)a.y << 32) | a.x;
@@ -730,7 +732,6 @@ __device__ __forceinline__ void gather_one(const RawSingle *src, const SinglesDe
     out.e[i] = __uint_as_float(b.w);
     out.eraw[i] = __uint_as_float(c.x);
     out.doi[i] = __uint_as_float(c.y);
-    C.flag[i] = 0;   // the coincidence pass sets flags anywhere
 }
 
 // first place at or after x where a bucket starts
@@ -741,7 +742,7 @@ __device__ __forceinline__ uint32_t bucket_edge(const SortDev &S, unsigned long 
     return s == (uint32_t)x ? s : S.bstart[b + 1];
 }
 
-__global__ void __launch_bounds__(256) k_bucket_sort(SortDev S, SinglesDev out, CoincDev C) {
+__global__ void __launch_bounds__(256) k_bucket_sort(SortDev S, SinglesDev out) {
     __shared__ uint64_t key[kBucketRoom];
     __shared__ uint32_t idx[kBucketRoom];
     __shared__ uint32_t edge[2];
@@ -754,116 +755,139 @@ __global__ void __launch_bounds__(256) k_bucket_sort(SortDev S, SinglesDev out, 
         if (threadIdx.x < 2) edge[threadIdx.x] = bucket_edge(S, x + threadIdx.x * kBucketCta, n);
         __syncthreads();
         const uint32_t p0 = edge[0], m = min(edge[1] - p0, (uint32_t)kBucketRoom);
-        for (uint32_t i = threadIdx.x; i < m; i += 256) {
-            const uint32_t v = S.vals[1][p0 + i];
-            idx[i] = v;
-            key[i] = __ldg(S.keys[0] + v);
+        for (uint32_t i0 = threadIdx.x; i0 < m; i0 += 512) {
+            const uint32_t i1 = i0 + 256;
+            const uint32_t v0 = S.vals[1][p0 + i0], v1 = i1 < m ? S.vals[1][p0 + i1] : v0;
+            const uint64_t k0 = __ldg(S.keys[0] + v0), k1 = __ldg(S.keys[0] + v1);
+            idx[i0] = v0;
+            key[i0] = k0;
+            if (i1 < m) {
+                idx[i1] = v1;
+                key[i1] = k1;
+            }
         }
         __syncthreads();
-        for (uint32_t i = threadIdx.x; i < m; i += 256) {
-            const uint64_t k = key[i];
-            const uint32_t v = idx[i], b = bucket_of(S, k);
-            const uint32_t s = S.bstart[b] - p0, e = min(S.bstart[b + 1] - p0, m);
-            uint32_t at = s;
-            for (uint32_t j = s; j < e; ++j) {
-                const uint64_t kj = key[j];
-                at += kj < k || (kj == k && idx[j] < v);
+        for (uint32_t i0 = threadIdx.x; i0 < m; i0 += 512) {
+            uint32_t lo[2], hi[2], v[2];
+            uint64_t k[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint32_t i = i0 + 256 * q < m ? i0 + 256 * q : i0;
+                k[q] = key[i];
+                v[q] = idx[i];
+                const uint32_t b = bucket_of(S, k[q]);
+                lo[q] = S.bstart[b] - p0;
+                hi[q] = min(S.bstart[b + 1] - p0, m);
             }
-            gather_one(S.in_raw + v, out, C, p0 + at);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint32_t at = lo[q];
+                for (uint32_t j = lo[q]; j < hi[q]; ++j) {
+                    const uint64_t kj = key[j];
+                    at += kj < k[q] || (kj == k[q] && idx[j] < v[q]);
+                }
+                lo[q] = at;
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (i0 + 256 * q < m) gather_one(S.in_raw + v[q], out, p0 + lo[q]);
         }
         __syncthreads();
     }
 }
 
 // singles into time order, after the radix passes
-__global__ void k_gather(SortDev S, SinglesDev out, CoincDev C) {
+__global__ void k_gather(SortDev S, SinglesDev out) {
     const unsigned long long n = sort_n(S);
     const int fin = S.plan[2 * kPasses];
     const uint32_t *perm = fin ? S.vals[1] : S.vals[0];
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
-        gather_one(S.in_raw + perm[i], out, C, i);
+        gather_one(S.in_raw + perm[i], out, i);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) *out.n = n;
 }
 
 // Coincidence sorting.  A cluster is a maximal run of time-sorted singles of
 // one job whose consecutive gaps are <= window; windows never cross cluster
-// ends, so each cluster is processed alone by the thread at its start: the
-// earliest unconsumed single opens [t0, t0 + window]; exactly two singles in
-// different panels make a coincidence; all singles in the window are consumed.
-__global__ void k_coinc_flags(SinglesDev s, CoincDev C) {
-    const unsigned long long n = *s.n;
-    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (unsigned long long)gridDim.x * blockDim.x) {
-        const uint64_t ti = s.t[i];
-        const int ji = s.job[i];
-        const uint64_t W = C.window_ps[ji];
-        const bool start = i == 0 || s.job[i - 1] != ji || ti - s.t[i - 1] > W;
-        if (!start) continue;
-        unsigned long long a = i;
-        for (;;) {
-            unsigned long long b = a;
-            const uint64_t ta = s.t[a];
-            while (b + 1 < n && s.job[b + 1] == ji && s.t[b + 1] - ta <= W) ++b;
-            if (b == a + 1 && s.panel[a] != s.panel[b]) C.flag[a] = 1;
-            // the cluster ends where the next gap exceeds the window
-            if (b + 1 >= n || s.job[b + 1] != ji || s.t[b + 1] - s.t[b] > W) break;
-            a = b + 1;
+// ends, so each cluster is processed alone: the earliest unconsumed single opens
+// [t0, t0 + window]; exactly two singles in different panels make a coincidence;
+// all singles in the window are consumed.
+// One pass over tiles of singles: the thread at a cluster's start replays it,
+// and the one at the tile's first single also the cluster that began before the
+// tile (walking back to its start), each up to the tile's end; the pairs found
+// in the tile are written after those of the tiles before it, whose number comes
+// by look-back.  (Flags, counts, a scan and the writes as kernels of their own
+// took 41 us for 1.6e6 singles and 18 us for any small number.)
+constexpr int kCoincThreads = 256, kCoincPer = 4, kCoincTile = kCoincThreads * kCoincPer;
+static_assert(kCoincTile == (int)kCoincScanTile, "look-back words are allocated per tile");
+
+__global__ void __launch_bounds__(kCoincThreads) k_coinc(SinglesDev s, CoincDev C, int *status) {
+    __shared__ uint64_t st[kCoincTile + 2];   // times and jobs of the tile, one single more at either end
+    __shared__ int32_t sj[kCoincTile + 2];
+    __shared__ uint32_t flag[kCoincTile / 32];
+    __shared__ uint32_t sw[32], tile_sh, base_sh;
+    __shared__ int fail_sh;
+    const unsigned long long n = *s.n, tiles = (n + kCoincTile - 1) / kCoincTile;
+    for (;;) {
+        if (threadIdx.x == 0) tile_sh = (uint32_t)atomicAdd(C.scan, 1ull);
+        if (threadIdx.x < kCoincTile / 32) flag[threadIdx.x] = 0;
+        __syncthreads();
+        const uint32_t tile = tile_sh;
+        if (tile >= tiles) break;
+        const unsigned long long lo = (unsigned long long)tile * kCoincTile;
+        const unsigned long long hi = lo + kCoincTile < n ? lo + kCoincTile : n;
+        for (int k = threadIdx.x; k < kCoincTile + 2; k += kCoincThreads) {
+            const unsigned long long i = lo + k - 1;   // (wraps below 0: not < n)
+            st[k] = i < n ? s.t[i] : 0ull;
+            sj[k] = i < n ? s.job[i] : -1;
         }
-    }
-}
-
-// compaction of flagged indices, in index order: counts per tile, one
-// scan block, writes
-__global__ void __launch_bounds__(1024) k_coinc_count(SinglesDev s, CoincDev C) {
-    __shared__ uint32_t sw[32];
-    const unsigned long long n = *s.n;
-    const unsigned long long tiles = (n + 4095) / 4096;
-    for (unsigned long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        uint32_t c = 0;
-        for (int j = 0; j < 4; ++j) {
-            const unsigned long long i = t * 4096 + (unsigned long long)j * 1024 + threadIdx.x;
-            if (i < n) c += C.flag[i];
-        }
-        uint32_t tot;
-        block_exscan(c, tot, sw);
-        if (threadIdx.x == 0) C.tile_cnt[t] = tot;
-    }
-}
-
-__global__ void __launch_bounds__(1024) k_coinc_scan(SinglesDev s, CoincDev C) {
-    __shared__ uint32_t sw[32];
-    const unsigned long long n = *s.n;
-    const unsigned long long tiles = (n + 4095) / 4096;
-    uint32_t base = 0;
-    for (unsigned long long c = 0; c < tiles; c += blockDim.x) {
-        const unsigned long long t = c + threadIdx.x;
-        const uint32_t v = t < tiles ? C.tile_cnt[t] : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_exscan(v, tot, sw);
-        if (t < tiles) C.tile_cnt[t] = base + ex;
-        base += tot;
-    }
-    if (threadIdx.x == 0) *C.n = base;
-}
-
-__global__ void __launch_bounds__(1024) k_coinc_write(SinglesDev s, CoincDev C) {
-    __shared__ uint32_t sw[32];
-    const unsigned long long n = *s.n;
-    const unsigned long long tiles = (n + 4095) / 4096;
-    for (unsigned long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        uint32_t base = C.tile_cnt[t];
-        for (int j = 0; j < 4; ++j) {
-            const unsigned long long i = t * 4096 + (unsigned long long)j * 1024 + threadIdx.x;
-            const uint32_t f = i < n ? C.flag[i] : 0u;
-            uint32_t tot;
-            const uint32_t ex = block_exscan(f, tot, sw);
-            if (f) {
-                C.a[base + ex] = (int32_t)i;
-                C.b[base + ex] = (int32_t)(i + 1);
+        __syncthreads();
+        auto T = [&](unsigned long long i) { return i + 1 - lo < kCoincTile + 2 ? st[i + 1 - lo] : s.t[i]; };
+        auto JOB = [&](unsigned long long i) { return i + 1 - lo < kCoincTile + 2 ? sj[i + 1 - lo] : s.job[i]; };
+#pragma unroll 1
+        for (int q = 0; q < kCoincPer; ++q) {
+            const unsigned long long i = lo + q * kCoincThreads + threadIdx.x;
+            if (i >= hi) break;
+            const int ji = JOB(i);
+            const uint64_t W = C.window_ps[ji];
+            unsigned long long a = i;
+            if (i > 0 && JOB(i - 1) == ji && T(i) - T(i - 1) <= W) {
+                if (i != lo) continue;   // inside a cluster
+                do --a; while (a > 0 && JOB(a - 1) == ji && T(a) - T(a - 1) <= W);
             }
-            base += tot;
+            while (a < hi) {
+                unsigned long long b = a;
+                const uint64_t ta = T(a);
+                while (b + 1 < n && JOB(b + 1) == ji && T(b + 1) - ta <= W) ++b;
+                if (b == a + 1 && a >= lo && s.panel[a] != s.panel[b])
+                    atomicOr(&flag[(a - lo) >> 5], 1u << ((a - lo) & 31));
+                // the cluster ends where the next gap exceeds the window
+                if (b + 1 >= n || JOB(b + 1) != ji || T(b + 1) - T(b) > W) break;
+                a = b + 1;
+            }
+        }
+        __syncthreads();
+        uint32_t f = (flag[threadIdx.x * kCoincPer >> 5] >> (threadIdx.x * kCoincPer & 31)) & ((1u << kCoincPer) - 1u);
+        uint32_t tot;
+        uint32_t at = block_exscan(__popc(f), tot, sw);
+        if (threadIdx.x < 32) {
+            uint32_t base = 0;
+            const bool ok = warp_lookback(C.scan + 1, tile, tot, base);
+            if (threadIdx.x == 0) {
+                if (!ok) atomicOr(status, kStatusSortStall);
+                if (ok && hi == n) *C.n = base + tot;
+                base_sh = base;
+                fail_sh = !ok;
+            }
+        }
+        __syncthreads();
+        if (fail_sh) break;
+        at += base_sh;
+        for (; f; f &= f - 1) {
+            const int32_t a = (int32_t)(lo + threadIdx.x * kCoincPer + __ffs(f) - 1);
+            C.a[at] = a;
+            C.b[at++] = a + 1;
         }
     }
 }
@@ -887,7 +911,7 @@ __device__ __forceinline__ unsigned long long warp_lower_bound(unsigned long lon
     return lo;
 }
 
-__global__ void __launch_bounds__(512) k_job_stats(SinglesDev s, CoincDev C, JobStatsDev J) {
+__global__ void __launch_bounds__(1024) k_job_stats(SinglesDev s, CoincDev C, JobStatsDev J) {
     const int j = blockIdx.x;
     const unsigned long long ns = *s.n, nc = *C.n;
     const int wid = threadIdx.x >> 5;
@@ -908,9 +932,9 @@ __global__ void __launch_bounds__(512) k_job_stats(SinglesDev s, CoincDev C, Job
     unsigned long long acc = 0;
     const unsigned long long *t = J.tally_count + J.tally_off[j];
     const long long nt = J.tally_n[j];
-#pragma unroll 8
-    for (long long i = threadIdx.x; i < nt; i += 512) acc += t[i];
-    __shared__ unsigned long long red[16];
+#pragma unroll 16
+    for (long long i = threadIdx.x; i < nt; i += 1024) acc += t[i];
+    __shared__ unsigned long long red[32];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFullMask, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
@@ -922,7 +946,7 @@ __global__ void __launch_bounds__(512) k_job_stats(SinglesDev s, CoincDev C, Job
 }
 
 cudaError_t launch_job_stats(const SinglesDev &s, const CoincDev &C, const JobStatsDev &J, cudaStream_t st) {
-    k_job_stats<<<J.n_jobs, 512, 0, st>>>(s, C, J);
+    k_job_stats<<<J.n_jobs, 1024, 0, st>>>(s, C, J);
     return cudaGetLastError();
 }
 
@@ -956,7 +980,7 @@ cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const Coi
         k_bucket_count<<<bg, 256, 0, st>>>(S);
         k_bucket_scan<<<(S.n_buckets + kBucketScanTile) / kBucketScanTile, 1024, 0, st>>>(S);
         k_bucket_place<<<bg, 256, 0, st>>>(S);
-        k_bucket_sort<<<bg, 256, 0, st>>>(S, out, C);
+        k_bucket_sort<<<bg, 256, 0, st>>>(S, out);
     } else {
         e = cudaMemsetAsync(S.ghist, 0, sizeof(uint32_t) * kPasses * 256, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(S.tile_ctr, 0, sizeof(unsigned int) * kPasses, st);
@@ -967,15 +991,13 @@ cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const Coi
         const int tg = (int)(S.max_tiles < (unsigned long long)sm_count * 2 ? (S.max_tiles ? S.max_tiles : 1)
                                                                             : (unsigned long long)sm_count * 2);
         for (int p = 0; p < kPasses; ++p) k_onesweep<<<tg, kSortThreads, kScatterSmemStaged, st>>>(S, p);
-        k_gather<<<grid, 256, 0, st>>>(S, out, C);
+        k_gather<<<grid, 256, 0, st>>>(S, out);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_coinc_flags<<<grid, 256, 0, st>>>(out, C);
-    const int cg = (int)(S.max_tiles < (unsigned long long)sm_count * 4 ? S.max_tiles : (unsigned long long)sm_count * 4);
-    k_coinc_count<<<cg, 1024, 0, st>>>(out, C);
-    k_coinc_scan<<<1, 1024, 0, st>>>(out, C);
-    k_coinc_write<<<cg, 1024, 0, st>>>(out, C);
+    const unsigned long long ct = (S.cap + kCoincTile - 1) / kCoincTile;
+    const int cg = (int)(ct < (unsigned long long)sm_count * 8 ? ct : (unsigned long long)sm_count * 8);
+    k_coinc<<<cg, kCoincThreads, 0, st>>>(out, C, S.status);
     return cudaGetLastError();
 }
 
@@ -986,9 +1008,8 @@ cudaError_t preload_sort_kernels() {
                          reinterpret_cast<const void *>(k_onesweep), reinterpret_cast<const void *>(k_bucket_count),
                          reinterpret_cast<const void *>(k_bucket_scan), reinterpret_cast<const void *>(k_bucket_place),
                          reinterpret_cast<const void *>(k_bucket_sort),
-                         reinterpret_cast<const void *>(k_gather), reinterpret_cast<const void *>(k_coinc_flags),
-                         reinterpret_cast<const void *>(k_coinc_count), reinterpret_cast<const void *>(k_coinc_scan),
-                         reinterpret_cast<const void *>(k_coinc_write), reinterpret_cast<const void *>(k_job_stats)};
+                         reinterpret_cast<const void *>(k_gather), reinterpret_cast<const void *>(k_coinc),
+                         reinterpret_cast<const void *>(k_job_stats)};
     cudaFuncAttributes fa;
     for (const void *f : fns) {
         const cudaError_t e = cudaFuncGetAttributes(&fa, f);
