@@ -35,16 +35,16 @@ struct SortDev {
     uint32_t *vals[2];
     uint32_t *ghist;                 // [8][256]
     int *plan;                       // [8] active, [8] source buffer, [1] final buffer
-    uint32_t *tile_hist;             // [256][max_tiles]
+    uint32_t *tile_words;            // allocation-free sort: look-back words [tiles][256]
     unsigned long long max_tiles;
     unsigned long long cap;
     const unsigned long long *n_in;  // device count of unsorted singles
     const RawSingle *in_raw;         // unsorted singles
-    int *status;                     // run status word (kStatusSortStall), or NULL: unstaged passes
+    int *status;                     // run status word (kStatusSortStall)
     int job_shift;                   // sort key = (job << job_shift) | t_ps; 64: the key is t_ps alone
     // one-sweep passes (the simulation path): decoupled look-back words, two
     // buffers of [tiles][256] that alternate between active passes, and a
-    // tile counter per pass; NULL where the passes run through tile_hist
+    // tile counter per pass
     unsigned long long *lb[2] = {nullptr, nullptr};
     unsigned int *tile_ctr = nullptr;
     // time buckets (n_buckets = 0: none, radix passes): per-job tables, the
@@ -166,7 +166,29 @@ constexpr int kCtaCounters = 20, kCtaCounterSlots = 16;
 void cta_counters(unsigned long long *counters, const unsigned long long *raw);
 cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const CoincDev &C, int sm_count,
                               cudaStream_t st);
-cudaError_t launch_radix_passes(const SortDev &S, int sm_count, cudaStream_t st);
+cudaError_t launch_noalloc_passes(const SortDev &S, unsigned tiles, cudaStream_t st);
+
+// Pass plan of a radix sort from the digit histograms S.ghist, by a block of
+// eight warps: which passes run, and which buffer each one reads.
+__device__ __forceinline__ void plan_passes(const SortDev &S, unsigned long long n) {
+    constexpr int kP = 8;
+    __shared__ int active[kP];
+    const int p = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t mx = 0;
+    for (int d = lane; d < 256; d += 32) mx = max(mx, __ldcg(S.ghist + p * 256 + d));
+    mx = __reduce_max_sync(kFullMask, mx);
+    if (lane == 0) active[p] = (n > 1 && (unsigned long long)mx < n) ? 1 : 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int cur = 0;
+        for (int q = 0; q < kP; ++q) {
+            S.plan[q] = active[q];
+            S.plan[kP + q] = cur;
+            if (active[q]) cur ^= 1;
+        }
+        S.plan[2 * kP] = cur;  // buffer holding the sorted result
+    }
+}
 
 // energy windows of one pass over the time-sorted singles
 constexpr int kMaxWindows = 16;

@@ -1,24 +1,24 @@
-// sort.cu -- digitizer back end: LSD radix sort of singles by 64-bit time key,
-// gather into time order, coincidence sorting (Sec. 2.3 timing window).
+// sort.cu -- digitizer back end: time sort of singles by 64-bit key, gather
+// into time order, coincidence sorting (Sec. 2.3 timing window).
 //
 // Keys are (job << shift) | t_ps, with the job in the fewest high bits that
 // number the launch's jobs (none for one job), so a batch of jobs sorts as
 // independent segments and a single run sorts on the whole 64-bit time.  The
-// transport writes them beside the records.  The
-// sort is a least-significant-digit radix sort with 8-bit
-// digits: one fused pass builds the eight digit histograms, a plan kernel
-// drops the passes whose digit is the same for every key (high time bytes,
-// unused job bits), and in the simulation path every remaining pass is one
-// kernel (k_onesweep: tiles claimed in order, each tile's digit offsets from
-// the global histogram and a decoupled look-back over the tiles before it).
-// The allocation-free sort runs each pass as tile histogram -> per-digit scan
-// -> stable scatter.  Stable ranks inside a tile come from the lanes of
-// a warp with the same digit (the intersection of bit-plane ballots), in input
-// order.  In the simulation path the scatter's input tiles are streamed into
-// shared memory by the bulk-copy engine (cp.async.bulk completing on an
-// mbarrier), one tile ahead of the tile being ranked.  The element count is
-// read on the device, so the whole chain is enqueued without a host round
-// trip.
+// transport writes them beside the records.  Runs whose decay times spread
+// over buckets of at least kBucketMinPs sort by time buckets (below).  The rest
+// -- very high activities, live launches, digitize-only runs -- take a
+// least-significant-digit radix sort with 8-bit digits: one fused pass builds
+// the eight digit histograms, a plan kernel drops the passes whose digit is the
+// same for every key (high time bytes, unused job bits), and every remaining
+// pass is one kernel (k_onesweep: tiles claimed in order, each tile's digit
+// offsets from the global histogram and a decoupled look-back over the tiles
+// before it).  Stable ranks inside a tile come from the lanes of a warp with the
+// same digit (the intersection of bit-plane ballots), in input order.  A pass's
+// input tiles are streamed into shared memory by the bulk-copy engine
+// (cp.async.bulk completing on an mbarrier), one tile ahead of the tile being
+// ranked.  The allocation-free sort has passes of its own (k_noalloc_pass).  The
+// element count is read on the device, so the whole chain is enqueued without a
+// host round trip.
 #include "internal.h"
 
 namespace gpet {
@@ -27,7 +27,7 @@ constexpr int kSortThreads = 256;
 constexpr int kSortItems = 16;
 constexpr int kTile = kSortThreads * kSortItems;  // 4096 keys per tile
 constexpr int kPasses = 8;
-static_assert(kSortThreads == 256, "one thread per 8-bit digit in the scatter's prefix step");
+static_assert(kSortThreads == 256, "one thread per 8-bit digit in the pass's prefix step");
 
 __device__ __forceinline__ uint32_t lane_lt() {
     uint32_t m;
@@ -70,54 +70,7 @@ __global__ void __launch_bounds__(kSortThreads) k_make_keys(SortDev S) {
 }
 
 // which passes run, and which buffer each one reads (one warp per pass)
-__global__ void __launch_bounds__(kPasses * 32) k_plan(SortDev S) {
-    __shared__ int active[kPasses];
-    const int p = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned long long n = sort_n(S);
-    uint32_t mx = 0;
-    for (int d = lane; d < 256; d += 32) mx = max(mx, S.ghist[p * 256 + d]);
-    mx = __reduce_max_sync(kFullMask, mx);
-    if (lane == 0) active[p] = (n > 1 && (unsigned long long)mx < n) ? 1 : 0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int cur = 0;
-        for (int q = 0; q < kPasses; ++q) {
-            S.plan[q] = active[q];
-            S.plan[kPasses + q] = cur;
-            if (active[q]) cur ^= 1;
-        }
-        S.plan[2 * kPasses] = cur;  // buffer holding the sorted result
-    }
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_tile_hist(SortDev S, int p) {
-    if (!S.plan[p]) return;
-    const int src = S.plan[kPasses + p];
-    const unsigned long long n = sort_n(S);
-    const unsigned long long tiles = (n + kTile - 1) / kTile;
-    __shared__ uint32_t h[256];
-    const uint64_t *keys = src ? S.keys[1] : S.keys[0];
-    for (unsigned long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
-        __syncthreads();
-        const unsigned long long b = t * kTile;
-        // all of the tile's loads are issued before the first shared atomic
-        uint64_t k[kSortItems];
-#pragma unroll
-        for (int j = 0; j < kSortItems; ++j) {
-            const unsigned long long i = b + (unsigned long long)j * kSortThreads + threadIdx.x;
-            k[j] = i < n ? __ldg(keys + i) : 0ull;
-        }
-#pragma unroll
-        for (int j = 0; j < kSortItems; ++j) {
-            const unsigned long long i = b + (unsigned long long)j * kSortThreads + threadIdx.x;
-            if (i < n) atomicAdd(&h[(k[j] >> (8 * p)) & 0xFF], 1u);
-        }
-        __syncthreads();
-        for (int d = threadIdx.x; d < 256; d += blockDim.x) S.tile_hist[(size_t)d * S.max_tiles + t] = h[d];
-        __syncthreads();
-    }
-}
+__global__ void __launch_bounds__(kPasses * 32) k_plan(SortDev S) { plan_passes(S, sort_n(S)); }
 
 // block-wide exclusive scan of one value per thread (blockDim a multiple of 32, at most 1024)
 __device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t &total, uint32_t *sw) {
@@ -146,27 +99,7 @@ __device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t &total, ui
     return warp_base + x - v;
 }
 
-// per digit: base of the digit + exclusive scan over tiles -> scatter offsets
-__global__ void __launch_bounds__(1024) k_digit_scan(SortDev S, int p) {
-    if (!S.plan[p]) return;
-    __shared__ uint32_t sw[32];
-    const int d = blockIdx.x;
-    const unsigned long long n = sort_n(S);
-    const unsigned long long tiles = (n + kTile - 1) / kTile;
-    uint32_t base = 0;
-    for (int e = 0; e < d; ++e) base += S.ghist[p * 256 + e];
-    uint32_t *row = S.tile_hist + (size_t)d * S.max_tiles;
-    for (unsigned long long c = 0; c < tiles; c += blockDim.x) {
-        const unsigned long long t = c + threadIdx.x;
-        const uint32_t v = t < tiles ? row[t] : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_exscan(v, tot, sw);
-        if (t < tiles) row[t] = base + ex;
-        base += tot;
-    }
-}
-
-// Stable scatter of one tile.  Ranks come in (warp, round, lane) order, which
+// Tile of a radix pass in shared memory.  Ranks come in (warp, round, lane) order, which
 // is input order.  The tile is first rebuilt in shared memory in digit order,
 // then written out from there: consecutive threads write consecutive slots of
 // one digit's run, so the global stores coalesce (a direct store from the
@@ -187,7 +120,6 @@ struct ScatterStage {
     uint32_t vals[kTile];
     unsigned long long bar;  // mbarrier: the copy of the staged tile has landed
 };
-constexpr size_t kScatterSmem = sizeof(ScatterSmem);
 constexpr size_t kScatterSmemStaged = sizeof(ScatterSmem) + sizeof(ScatterStage);
 constexpr uint32_t kStageBytes = kTile * (sizeof(uint64_t) + sizeof(uint32_t));
 static_assert(sizeof(ScatterSmem) % 16 == 0, "staging buffer must start on a 16-byte boundary");
@@ -236,132 +168,6 @@ __device__ __forceinline__ void stage_issue(ScatterStage &sg, const uint64_t *ki
         : "memory");
 }
 
-template <bool kStaged>
-__global__ void __launch_bounds__(kSortThreads, 2) k_scatter(SortDev S, int p) {
-    if (!S.plan[p]) return;
-    extern __shared__ __align__(16) unsigned char scatter_raw[];
-    ScatterSmem &sm = *reinterpret_cast<ScatterSmem *>(scatter_raw);
-    ScatterStage &sg = *reinterpret_cast<ScatterStage *>(scatter_raw + sizeof(ScatterSmem));
-    const int src = S.plan[kPasses + p];
-    const unsigned long long n = sort_n(S);
-    const unsigned long long tiles = (n + kTile - 1) / kTile;
-    const unsigned long long full_tiles = n / kTile;  // tiles the copy engine stages
-    constexpr int kWarps = kSortThreads / 32;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    // selects, not an index: a dynamic index would copy the argument to the stack
-    const uint64_t *kin = src ? S.keys[1] : S.keys[0];
-    const uint32_t *vin = src ? S.vals[1] : S.vals[0];
-    uint64_t *kout = src ? S.keys[0] : S.keys[1];
-    uint32_t *vout = src ? S.vals[0] : S.vals[1];
-    uint32_t parity = 0;
-    if (kStaged) {
-        if (threadIdx.x == 0) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sg.bar)) : "memory");
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            if (blockIdx.x < full_tiles) stage_issue(sg, kin, vin, blockIdx.x);
-        }
-        __syncthreads();
-    }
-    for (unsigned long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        for (int i = threadIdx.x; i < kWarps * 256; i += blockDim.x) (&sm.wh[0][0])[i] = 0;
-        const unsigned long long wb = t * kTile + (unsigned long long)w * (32 * kSortItems);
-        // this tile's global start of digit threadIdx.x, fetched with the keys
-        const uint32_t gstart = S.tile_hist[(size_t)threadIdx.x * S.max_tiles + t];
-        uint64_t k[kSortItems];
-        uint32_t v[kSortItems];
-        uint32_t rank[kSortItems];
-        const bool staged = kStaged && t < full_tiles;
-        if (staged) {
-            // every thread sees the copy land; the CTA gives up together
-            const bool ok = stage_wait(smem_addr(&sg.bar), parity);
-            if (!__syncthreads_and(ok)) {
-                if (threadIdx.x == 0) {
-                    atomicOr(S.status, kStatusSortStall);
-                    stage_wait(smem_addr(&sg.bar), parity);  // let the copy in flight land
-                }
-                return;
-            }
-            parity ^= 1u;
-            const int lb = w * (32 * kSortItems) + lane;
-#pragma unroll
-            for (int j = 0; j < kSortItems; ++j) {
-                k[j] = sg.keys[lb + j * 32];
-                v[j] = sg.vals[lb + j * 32];
-            }
-            __syncthreads();  // the staging buffer is free: stream in the next tile
-            const unsigned long long nt = t + gridDim.x;
-            if (threadIdx.x == 0 && nt < full_tiles) stage_issue(sg, kin, vin, nt);
-        } else {
-            // Every load of the tile is in flight before the ranking starts:
-            // the ranking's shared-memory stores would otherwise order each
-            // item's load after the previous item's ranking.
-#pragma unroll
-            for (int j = 0; j < kSortItems; ++j) {
-                const unsigned long long i = wb + (unsigned long long)j * 32 + lane;
-                k[j] = i < n ? __ldg(kin + i) : 0ull;
-                v[j] = i < n ? __ldg(vin + i) : 0u;
-            }
-            __syncthreads();  // the warp histograms are cleared
-        }
-#pragma unroll
-        for (int j = 0; j < kSortItems; ++j) {
-            const unsigned long long i = wb + (unsigned long long)j * 32 + lane;
-            const bool ok = i < n;
-            const uint32_t d = ok ? (uint32_t)((k[j] >> (8 * p)) & 0xFF) : 256u;
-            // lanes with the same digit: intersect the eight bit-plane ballots
-            // (and the ninth bit that marks lanes past the end)
-            uint32_t peers = kFullMask;
-#pragma unroll
-            for (int bit = 0; bit < 9; ++bit) {
-                const uint32_t m = __ballot_sync(kFullMask, (d >> bit) & 1u);
-                peers &= ((d >> bit) & 1u) ? m : ~m;
-            }
-            const uint32_t before = (d < 256u) ? sm.wh[w][d] : 0u;
-            rank[j] = before + __popc(peers & lane_lt());
-            __syncwarp();
-            if (d < 256u && (peers & lane_lt()) == 0) sm.wh[w][d] = before + __popc(peers);
-            __syncwarp();
-        }
-        __syncthreads();
-        // thread d owns digit d: warp prefixes, local run start, global delta
-        {
-            const int d = threadIdx.x;  // kSortThreads == 256 digits
-            uint32_t c = 0;
-#pragma unroll
-            for (int ww = 0; ww < kWarps; ++ww) {
-                const uint32_t x = sm.wh[ww][d];
-                sm.wh[ww][d] = c;
-                c += x;
-            }
-            uint32_t tot;
-            const uint32_t lstart = block_exscan(c, tot, sm.sw);
-#pragma unroll
-            for (int ww = 0; ww < kWarps; ++ww) sm.wh[ww][d] += lstart;
-            sm.gdelta[d] = gstart - lstart;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < kSortItems; ++j) {
-            const unsigned long long i = wb + (unsigned long long)j * 32 + lane;
-            if (i < n) {
-                const uint32_t lp = sm.wh[w][(uint32_t)((k[j] >> (8 * p)) & 0xFF)] + rank[j];
-                sm.keys[lp] = k[j];
-                sm.vals[lp] = v[j];
-            }
-        }
-        __syncthreads();
-        const unsigned long long rem = n - t * kTile;
-        const int tn = rem < (unsigned long long)kTile ? (int)rem : kTile;
-        for (int i = threadIdx.x; i < tn; i += kSortThreads) {
-            const uint64_t key = sm.keys[i];
-            const uint32_t pos = sm.gdelta[(uint32_t)((key >> (8 * p)) & 0xFF)] + (uint32_t)i;
-            kout[pos] = key;
-            vout[pos] = sm.vals[i];
-        }
-        __syncthreads();
-    }
-}
-
 // Decoupled look-back words of the one-sweep passes: the kind in the top two
 // bits (a tile's own count of a digit, or the count of that digit over all
 // tiles up to and including it), the count below.  A word is written whole
@@ -385,9 +191,8 @@ __device__ __forceinline__ unsigned long long lb_load(const unsigned long long *
 // the counts of the tiles before it, found by looking back over their
 // published words until an inclusive count.  Every tile a CTA waits on was
 // claimed earlier by a running CTA, and waits only on tiles before it, so the
-// waits end.  The tile histogram and digit scan passes are not needed.  Tiles
-// are staged into shared memory one ahead by the bulk-copy engine, as in
-// k_scatter; the ranking and the write-out are those of k_scatter.
+// waits end.  Tiles are staged into shared memory one ahead by the bulk-copy
+// engine.
 __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(SortDev S, int p) {
     if (!S.plan[p]) return;
     extern __shared__ __align__(16) unsigned char scatter_raw[];
@@ -587,9 +392,6 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(SortDev S, int p) 
 }
 
 static cudaError_t scatter_smem_attr() {
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void *>(k_scatter<false>), kScatterSmem);
-    if (e == cudaSuccess) e = ensure_dynamic_smem(reinterpret_cast<const void *>(k_scatter<true>), kScatterSmemStaged);
-    if (e != cudaSuccess) return e;
     return ensure_dynamic_smem(reinterpret_cast<const void *>(k_onesweep), kScatterSmemStaged);
 }
 
@@ -950,20 +752,154 @@ cudaError_t launch_job_stats(const SinglesDev &s, const CoincDev &C, const JobSt
     return cudaGetLastError();
 }
 
-// Plan plus the eight radix passes over an already keyed working set (used by
-// the allocation-free sort entry point; the simulation path keeps its own
-// launcher below).
-cudaError_t launch_radix_passes(const SortDev &S, int sm_count, cudaStream_t st) {
-    cudaError_t e = scatter_smem_attr();
-    if (e != cudaSuccess) return e;
-    k_plan<<<1, kPasses * 32, 0, st>>>(S);
-    for (int p = 0; p < kPasses; ++p) {
-        const int tg = (int)(S.max_tiles < (unsigned long long)sm_count * 8 ? S.max_tiles
-                                                                              : (unsigned long long)sm_count * 8);
-        k_tile_hist<<<tg, kSortThreads, 0, st>>>(S, p);
-        k_digit_scan<<<256, 1024, 0, st>>>(S, p);
-        k_scatter<false><<<tg, kSortThreads, kScatterSmem, st>>>(S, p);
+// ---------------------------------------------------------------------------
+// Radix passes of the allocation-free sort (at most 2^20 keys, 256 tiles): one
+// kernel per digit as above, with what so few keys ask for.  A tile is sorted by
+// 512 threads with 8 keys each, since the pass is bound by the latency of its
+// ranking and look-back and not by bandwidth (every tile's CTA is resident at
+// once); look-back words are 32 bits and carry the pass they belong to, so that
+// one buffer in the scratch array serves all passes without being cleared
+// between them, and 16 of them are read per round trip.
+// 300007 keys with 46 varying bits: 12 kernels, where tile histogram, digit scan
+// and scatter as kernels of their own took 29.
+// ---------------------------------------------------------------------------
+constexpr int kPassThreads = 512, kPassItems = kTile / kPassThreads;
+constexpr uint32_t kWordAgg = 1u << 26, kWordIncl = 2u << 26, kWordCount = (1u << 26) - 1u;
+struct PassSmem {
+    uint64_t keys[kTile];
+    uint32_t vals[kTile];
+    uint32_t wh[kPassThreads / 32][256];
+    uint32_t gdelta[256], thist[256], sw[32];
+    uint32_t tile;
+};
+
+__global__ void __launch_bounds__(kPassThreads, 1) k_noalloc_pass(SortDev S, int p) {
+    if (!S.plan[p]) return;
+    extern __shared__ __align__(16) unsigned char pass_raw[];
+    PassSmem &sm = *reinterpret_cast<PassSmem *>(pass_raw);
+    const int src = S.plan[kPasses + p];
+    const uint32_t n = (uint32_t)sort_n(S), tiles = (n + kTile - 1) / kTile;
+    constexpr int kWarps = kPassThreads / 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint64_t *kin = src ? S.keys[1] : S.keys[0];
+    const uint32_t *vin = src ? S.vals[1] : S.vals[0];
+    uint64_t *kout = src ? S.keys[0] : S.keys[1];
+    uint32_t *vout = src ? S.vals[0] : S.vals[1];
+    if (threadIdx.x == 0) sm.tile = atomicAdd(S.tile_ctr + p, 1u);
+    for (int i = threadIdx.x; i < kWarps * 256; i += kPassThreads) (&sm.wh[0][0])[i] = 0;
+    if (threadIdx.x < 256) sm.thist[threadIdx.x] = 0;
+    __syncthreads();
+    const uint32_t t = sm.tile;   // tiles in the order of their start
+    if (t >= tiles) return;
+    // the digits' bases: exclusive scan of this pass's global histogram
+    uint32_t tot;
+    const uint32_t dbase = block_exscan(threadIdx.x < 256 ? S.ghist[p * 256 + threadIdx.x] : 0u, tot, sm.sw);
+    const uint32_t wb = t * kTile + (uint32_t)w * (32 * kPassItems) + (uint32_t)lane;
+    uint64_t k[kPassItems];
+    uint32_t v[kPassItems], rank[kPassItems];
+#pragma unroll
+    for (int j = 0; j < kPassItems; ++j) {
+        const uint32_t i = wb + 32 * j;
+        k[j] = i < n ? __ldg(kin + i) : 0ull;
+        v[j] = i < n ? __ldg(vin + i) : 0u;
     }
+    // the tile's digit counts, published before the ranking
+#pragma unroll
+    for (int j = 0; j < kPassItems; ++j)
+        if (wb + 32 * j < n) atomicAdd(&sm.thist[(uint32_t)((k[j] >> (8 * p)) & 0xFF)], 1u);
+    __syncthreads();
+    const uint32_t tag = (uint32_t)(p + 1) << 28;
+    volatile uint32_t *row = S.tile_words + (size_t)t * 256;
+    const uint32_t cnt = threadIdx.x < 256 ? sm.thist[threadIdx.x] : 0u;
+    if (threadIdx.x < 256) row[threadIdx.x] = tag | (t == 0 ? kWordIncl : kWordAgg) | cnt;
+#pragma unroll
+    for (int j = 0; j < kPassItems; ++j) {
+        const uint32_t d = wb + 32 * j < n ? (uint32_t)((k[j] >> (8 * p)) & 0xFF) : 256u;
+        uint32_t peers = kFullMask;
+#pragma unroll
+        for (int bit = 0; bit < 9; ++bit) {   // (the ninth separates the lanes past the end)
+            const uint32_t m = __ballot_sync(kFullMask, (d >> bit) & 1u);
+            peers &= ((d >> bit) & 1u) ? m : ~m;
+        }
+        const uint32_t before = d < 256u ? sm.wh[w][d] : 0u;
+        rank[j] = before + __popc(peers & lane_lt());
+        __syncwarp();
+        if (d < 256u && (peers & lane_lt()) == 0) sm.wh[w][d] = before + __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    uint32_t c = 0;
+    if (threadIdx.x < 256) {
+#pragma unroll
+        for (int ww = 0; ww < kWarps; ++ww) {
+            const uint32_t x = sm.wh[ww][threadIdx.x];
+            sm.wh[ww][threadIdx.x] = c;
+            c += x;
+        }
+    }
+    const uint32_t lstart = block_exscan(c, tot, sm.sw);
+    if (threadIdx.x < 256) {
+#pragma unroll
+        for (int ww = 0; ww < kWarps; ++ww) sm.wh[ww][threadIdx.x] += lstart;
+    }
+    __syncthreads();
+    // the tile in digit order in shared memory; its global offsets follow
+#pragma unroll
+    for (int j = 0; j < kPassItems; ++j)
+        if (wb + 32 * j < n) {
+            const uint32_t lp = sm.wh[w][(uint32_t)((k[j] >> (8 * p)) & 0xFF)] + rank[j];
+            sm.keys[lp] = k[j];
+            sm.vals[lp] = v[j];
+        }
+    int fail = 0;
+    if (threadIdx.x < 256) {
+        const uint32_t d = threadIdx.x;
+        uint32_t excl = 0;
+        constexpr int kWin = 16;
+        int polls = 0;
+        for (uint32_t j = t; j > 0 && !fail;) {   // tiles [0, j) not yet added
+            uint32_t wv[kWin];
+            const volatile uint32_t *q0 = S.tile_words + d;
+#pragma unroll
+            for (int q = 0; q < kWin; ++q) wv[q] = (uint32_t)q < j ? q0[(size_t)(j - 1 - q) * 256] : 0u;
+            bool found = false;
+#pragma unroll
+            for (int q = 0; q < kWin; ++q) {
+                if (found || fail || (uint32_t)q >= j) break;
+                uint32_t x = wv[q];
+                while ((x >> 28) != (uint32_t)(p + 1)) {
+                    if (++polls > kLookbackPolls) { fail = 1; break; }
+                    if (polls > 64) __nanosleep(64);
+                    x = q0[(size_t)(j - 1 - q) * 256];
+                }
+                if (fail) break;
+                excl += x & kWordCount;
+                found = (x & kWordIncl) != 0;
+            }
+            j = found ? 0u : (j > (uint32_t)kWin ? j - kWin : 0u);
+        }
+        if (!fail && t > 0) row[d] = tag | kWordIncl | (excl + cnt);
+        sm.gdelta[d] = dbase + excl - lstart;
+    }
+    // (a tile whose look-back gave up writes nothing; the call cannot report it,
+    // and its output is then incomplete)
+    if (__syncthreads_or(fail)) return;
+    const uint32_t tn = min(n - t * kTile, (uint32_t)kTile);
+    for (uint32_t i = threadIdx.x; i < tn; i += kPassThreads) {
+        const uint64_t key = sm.keys[i];
+        const uint32_t pos = sm.gdelta[(uint32_t)((key >> (8 * p)) & 0xFF)] + i;
+        if (pos < n) {
+            kout[pos] = key;
+            vout[pos] = sm.vals[i];
+        }
+    }
+}
+
+// the radix passes over a keyed and planned working set
+cudaError_t launch_noalloc_passes(const SortDev &S, unsigned tiles, cudaStream_t st) {
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void *>(k_noalloc_pass), sizeof(PassSmem));
+    if (e != cudaSuccess) return e;
+    for (int p = 0; p < kPasses; ++p) k_noalloc_pass<<<tiles, kPassThreads, sizeof(PassSmem), st>>>(S, p);
     return cudaGetLastError();
 }
 
@@ -1004,7 +940,6 @@ cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const Coi
 // load the digitizer's kernels and set their shared-memory limits (internal.h)
 cudaError_t preload_sort_kernels() {
     const void *fns[] = {reinterpret_cast<const void *>(k_make_keys), reinterpret_cast<const void *>(k_plan),
-                         reinterpret_cast<const void *>(k_tile_hist), reinterpret_cast<const void *>(k_digit_scan),
                          reinterpret_cast<const void *>(k_onesweep), reinterpret_cast<const void *>(k_bucket_count),
                          reinterpret_cast<const void *>(k_bucket_scan), reinterpret_cast<const void *>(k_bucket_place),
                          reinterpret_cast<const void *>(k_bucket_sort),

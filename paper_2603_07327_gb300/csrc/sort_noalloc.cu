@@ -11,6 +11,8 @@
 // The array is part of the library image: every GPU that loads the library
 // holds it until the process exits.  The caller still passes its inputs and
 // outputs.
+#include <algorithm>
+
 #include "gpet.h"
 #include "host.h"
 
@@ -21,18 +23,20 @@ constexpr unsigned long long kNoallocTiles = (kNoallocMaxKeys + 4095) / 4096;
 // layout of the scratch array (all offsets multiples of 256 bytes)
 constexpr size_t kOffN = 0;                                           // element count (8 bytes)
 constexpr size_t kOffHist = 256;                                      // [8][256] uint32 digit histograms
-constexpr size_t kOffPlan = kOffHist + 8 * 256 * 4;                   // 32 int plan words
+constexpr size_t kOffPlan = kOffHist + 8 * 256 * 4;                   // 32 int plan words, then 9 counters
+constexpr size_t kOffCounters = kOffPlan + 32 * 4;                    // tiles started per pass, blocks done
 constexpr size_t kOffKeys0 = kOffPlan + 256;
 constexpr size_t kOffKeys1 = kOffKeys0 + 8 * kNoallocMaxKeys;
 constexpr size_t kOffVals0 = kOffKeys1 + 8 * kNoallocMaxKeys;
 constexpr size_t kOffVals1 = kOffVals0 + 4 * kNoallocMaxKeys;
 constexpr size_t kOffTiles = kOffVals1 + 4 * kNoallocMaxKeys;
-constexpr size_t kScratchBytes = kOffTiles + 256 * 4 * kNoallocTiles;  // 24.26 MiB
+constexpr size_t kScratchBytes = kOffTiles + 256 * 4 * kNoallocTiles;  // look-back words; 24.26 MiB in all
 
 static __device__ __align__(256) unsigned char g_sort_scratch[kScratchBytes];
 
-// keys[0] = t, vals[0] = index, eight digit histograms
-__global__ void __launch_bounds__(256) k_noalloc_keys(const uint64_t *__restrict__ t_in, SortDev S) {
+// keys[0] = t, vals[0] = index, eight digit histograms, cleared look-back words;
+// the last block to finish plans the passes
+__global__ void __launch_bounds__(256) k_noalloc_keys(const uint64_t *__restrict__ t_in, SortDev S, unsigned *blocks_done) {
     __shared__ uint32_t h[8][256];
     for (int i = threadIdx.x; i < 8 * 256; i += blockDim.x) (&h[0][0])[i] = 0;
     __syncthreads();
@@ -45,14 +49,33 @@ __global__ void __launch_bounds__(256) k_noalloc_keys(const uint64_t *__restrict
 #pragma unroll
         for (int p = 0; p < 8; ++p) atomicAdd(&h[p][(key >> (8 * p)) & 0xFF], 1u);
     }
+    const unsigned long long words = (n + 4095) / 4096 * 256;
+    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < words;
+         i += (unsigned long long)gridDim.x * blockDim.x)
+        S.tile_words[i] = 0u;
     __syncthreads();
     for (int i = threadIdx.x; i < 8 * 256; i += blockDim.x) {
         const uint32_t v = (&h[0][0])[i];
         if (v) atomicAdd(S.ghist + i, v);
     }
+    __threadfence();
+    __syncthreads();
+    __shared__ bool last;
+    if (threadIdx.x == 0) last = atomicAdd(blocks_done, 1u) + 1u == gridDim.x;
+    __syncthreads();
+    if (last) {
+        __threadfence();
+        plan_passes(S, n);
+    }
 }
 
-__global__ void k_noalloc_set_n(unsigned long long *n_slot, unsigned long long n) { *n_slot = n; }
+// the element count, and the histograms and counters that the previous call left
+__global__ void __launch_bounds__(1024) k_noalloc_begin(unsigned long long *n_slot, unsigned long long n, SortDev S,
+                                                        unsigned *counters) {
+    for (int i = threadIdx.x; i < 8 * 256; i += 1024) S.ghist[i] = 0;
+    if (threadIdx.x < 9) counters[threadIdx.x] = 0;
+    if (threadIdx.x == 0) *n_slot = n;
+}
 
 __global__ void k_noalloc_out(SortDev S, uint64_t *__restrict__ t_out, uint32_t *__restrict__ perm_out) {
     const unsigned long long n = *S.n_in;
@@ -102,18 +125,18 @@ extern "C" int gpet_sort_times_noalloc(const uint64_t *d_t_in, uint64_t n, uint6
     S.keys[1] = reinterpret_cast<uint64_t *>(base + kOffKeys1);
     S.vals[0] = reinterpret_cast<uint32_t *>(base + kOffVals0);
     S.vals[1] = reinterpret_cast<uint32_t *>(base + kOffVals1);
-    S.tile_hist = reinterpret_cast<uint32_t *>(base + kOffTiles);
+    S.tile_words = reinterpret_cast<uint32_t *>(base + kOffTiles);
+    S.tile_ctr = reinterpret_cast<unsigned int *>(base + kOffCounters);
     S.max_tiles = kNoallocTiles;
     S.cap = kNoallocMaxKeys;
     S.job_shift = 64;  // the keys are the caller's time stamps alone
-    // the histograms keep the previous call's contents: clear them
-    e = cudaMemsetAsync(S.ghist, 0, 8 * 256 * 4, st);
-    if (e != cudaSuccess) return gpet_cuda_fail(e, "cudaMemsetAsync(sort scratch)");
-    k_noalloc_set_n<<<1, 1, 0, st>>>(reinterpret_cast<unsigned long long *>(base + kOffN), n);
-    k_noalloc_keys<<<sms * 4, 256, 0, st>>>(d_t_in, S);
-    e = launch_radix_passes(S, sms, st);
+    const unsigned tiles = (unsigned)((n + 4095) / 4096);
+    const unsigned blocks = std::min((unsigned)sms * 4, std::max(1u, tiles * 4));   // (1024 keys a block at least)
+    k_noalloc_begin<<<1, 1024, 0, st>>>(reinterpret_cast<unsigned long long *>(base + kOffN), n, S, S.tile_ctr);
+    k_noalloc_keys<<<blocks, 256, 0, st>>>(d_t_in, S, S.tile_ctr + 8);
+    e = launch_noalloc_passes(S, tiles, st);
     if (e != cudaSuccess) return gpet_cuda_fail(e, "radix passes");
-    k_noalloc_out<<<sms * 4, 256, 0, st>>>(S, d_t_out, d_perm_out);
+    k_noalloc_out<<<blocks, 256, 0, st>>>(S, d_t_out, d_perm_out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return gpet_cuda_fail(e, "gpet_sort_times_noalloc launch");
     return GPET_OK;
