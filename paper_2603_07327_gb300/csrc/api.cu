@@ -46,11 +46,20 @@ extern "C" const char *gpet_version(void) { return "gpet-gb300 0.1 (sm_103a)"; }
 namespace gpet {
 
 static std::mutex g_attr_mutex;
-static std::map<std::pair<int, const void *>, size_t> g_smem_limit;  // (device, kernel) -> limit set
+static std::map<std::pair<int, const void *>, size_t> g_smem_limit;
+static std::map<std::pair<int, const void *>, size_t> g_smem_asked;  // (device, kernel) -> limit set
 
 cudaError_t ensure_dynamic_smem(const void *fn, size_t bytes) {
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    {
+        // asked for before (the limit may be lower: the device's)
+        std::lock_guard<std::mutex> lk(g_attr_mutex);
+        size_t &asked = g_smem_asked[std::make_pair(dev, fn)];
+        if (bytes <= asked) return cudaSuccess;
+    }
+    const size_t wanted = bytes;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     // the limit covers the kernel's static shared memory as well
@@ -61,10 +70,14 @@ cudaError_t ensure_dynamic_smem(const void *fn, size_t bytes) {
     bytes = std::min(bytes, cap);
     std::lock_guard<std::mutex> lk(g_attr_mutex);
     size_t &have = g_smem_limit[std::make_pair(dev, fn)];
-    if (bytes <= have) return cudaSuccess;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) have = bytes;
-    return e;
+    if (bytes > have) {
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+        have = bytes;
+    }
+    size_t &asked = g_smem_asked[std::make_pair(dev, fn)];
+    asked = std::max(asked, wanted);
+    return cudaSuccess;
 }
 
 cudaError_t preload_kernels() {

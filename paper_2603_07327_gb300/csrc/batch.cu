@@ -46,7 +46,7 @@ int gpet_batch_build_run(Run &R, int32_t n_jobs, gpet_scanner *const *scanners, 
         R.windows.push_back((uint64_t)std::llround(digitizers[j].coinc_window_ns * 1000.0));
         total += n_decays[j];
     }
-    R.caps.singles = std::max<uint64_t>(65536, total * 6 / 10);
+    R.caps.singles = first_singles_guess(total);
     R.caps.hits = R.keep_hits ? std::max<uint64_t>(65536, total * 5 / 2) : 0;
     R.caps.ovf = std::max<uint64_t>(4096, total / 256);
     return GPET_OK;

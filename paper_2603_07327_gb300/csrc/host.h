@@ -108,6 +108,8 @@ struct Run {
     // per-job segments of the outputs (device, then host copies after collect)
     JobStatsDev JS{};
     std::vector<unsigned long long> s_off, c_off, job_hits;
+    std::vector<char> tables;            // host image of the uploaded descriptor tables
+    size_t readback_bytes = 0;           // header, job offsets, hits and window counts: one block from d_hdr on
     // energy windows counted in one pass over the sorted singles (sensitivity map)
     std::vector<float> win_lo, win_hi;
     unsigned long long *d_win_counts = nullptr;  // [job][window], cleared before every launch
@@ -193,5 +195,10 @@ int gpet_batch_build_run(gpet::Run &R, int32_t n_jobs, gpet_scanner *const *scan
 
 namespace gpet {
 void fill_counts(const Run &R, int job, uint64_t n_decays, int64_t n_crystals, gpet_counts *c);
+// Singles capacity of a run's first attempt: one per decay for runs of up to
+// 2^25 decays (4 GB of arena), 0.6 beyond.  A run that keeps more is repeated
+// whole with its exact count, so a guess that a wide ring's module-level
+// readout exceeds (0.62 per decay) costs such a run half of its time.
+uint64_t first_singles_guess(uint64_t n_decays);
 int run_with_retry(Run &R);            // plan + enqueue + collect, one exact-size re-run on overflow
 }

@@ -2,6 +2,10 @@
 // (device structs of the sort / coincidence stage and the host launchers).
 #pragma once
 
+#include <map>
+#include <mutex>
+#include <tuple>
+
 #include <cuda_runtime.h>
 
 #include "transport.cuh"
@@ -130,7 +134,26 @@ cudaError_t staged_geometry(Kernel k, int block, size_t pool_smem, int n_geoms, 
                             size_t *smem_out, int *occ_out) {
     int ng = n_geoms < max_geoms ? n_geoms : max_geoms;
     if (ng < 0) ng = 0;
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void *>(k),
+    // the answer depends on the kernel, the device and these counts alone: kept
+    // (a few entries per kernel), since a small run would spend 10 us asking
+    struct Known { int ng, occ; size_t smem; };
+    static std::mutex mu;
+    static std::map<std::tuple<const void *, int, int, int, size_t, int>, Known> known;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const auto key = std::make_tuple(reinterpret_cast<const void *>(k), dev, block, ng, pool_smem, max_geoms);
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        const auto it = known.find(key);
+        if (it != known.end()) {
+            *ng_out = it->second.ng;
+            *smem_out = it->second.smem;
+            *occ_out = it->second.occ;
+            return cudaSuccess;
+        }
+    }
+    e = ensure_dynamic_smem(reinterpret_cast<const void *>(k),
                                         pool_smem + (size_t)(max_geoms > 0 ? max_geoms : 0) * sizeof(GeomDev));
     if (e != cudaSuccess) return e;
     int occ0 = 0, occ = 0;
@@ -144,6 +167,8 @@ cudaError_t staged_geometry(Kernel k, int block, size_t pool_smem, int n_geoms, 
     *ng_out = ng;
     *smem_out = pool_smem + (size_t)ng * sizeof(GeomDev);
     *occ_out = occ;
+    std::lock_guard<std::mutex> lk(mu);
+    known[key] = {ng, occ, *smem_out};
     return cudaSuccess;
 }
 

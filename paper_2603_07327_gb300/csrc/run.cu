@@ -97,7 +97,11 @@ int run_default_cfg(Run &R, const gpet_options *opt_in, const gpet_scanner *sc) 
     return GPET_OK;
 }
 
-int run_plan(Run &R) {
+// Arenas up to this size are allocated without asking for the free memory
+// first (the query costs more than the allocation).
+constexpr size_t kSmallArena = (size_t)256 << 20;
+
+static int plan_once(Run &R, bool clamp) {
     const int nj = (int)R.jobs.size();
     // table sizes: the jobs themselves, or a live launch's capacities
     const int njc = R.live ? std::max(nj, R.live_cap.jobs) : nj;
@@ -169,12 +173,12 @@ int run_plan(Run &R) {
         }
     }
 
-    // The first guess of the singles capacity (0.6 per history) may exceed what
+    // The first guess of the singles capacity may exceed what
     // a long run needs by far (a narrow energy window keeps few singles): it
     // takes at most a quarter of the free device memory.  The device counts
     // past the capacity, so a run with more singles is detected and re-run once
     // with its exact count; so is a run with more than the launch limit.
-    if (R.caps.guess) {
+    if (R.caps.guess && clamp) {
         size_t free_b = 0, total_b = 0;
         if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
             // arena bytes per single of capacity: raw record, two key and index
@@ -192,12 +196,16 @@ int run_plan(Run &R) {
 
     Carver cv;
     // zeroed before every launch
-    cv.take(R.d_hdr, 1);
-    cv.take(R.S.ghist, 8 * 256);
-    cv.take(R.d_tally_count, (size_t)tcc);
-    cv.take(R.d_tally_efx, (size_t)tcc);
+    cv.take(R.d_hdr, 1);   // (first: the read-back block starts here)
+    // what is read back after the run, in one block with the header
+    JobStatsDev &JS = R.JS;
+    cv.take(JS.s_off, njc + 1); cv.take(JS.c_off, njc + 1); cv.take(JS.hits, njc);
     const size_t nwin = R.win_lo.size();
     if (nwin) cv.take(R.d_win_counts, (size_t)njc * nwin);
+    R.readback_bytes = cv.off;
+    cv.take(R.d_tally_count, (size_t)tcc);
+    cv.take(R.d_tally_efx, (size_t)tcc);
+    cv.take(R.S.ghist, 8 * 256);
     cv.take(R.C.scan, cap / kCoincScanTile + 2);
     if (n_buckets) {
         cv.take(R.S.bstart, n_buckets + 1);
@@ -222,6 +230,8 @@ int run_plan(Run &R) {
     cv.take(R.d_chunk_start, njc + 1);
     cv.take(R.d_window, njc);
     if (n_buckets) cv.take(R.d_buckets, njc);
+    cv.take(R.d_toff, njc); cv.take(R.d_tn, njc);
+    const size_t tables_end = cv.off;
     // raw singles
     OutDev &O = R.O;
     cv.take(O.s_raw, cap);
@@ -247,10 +257,6 @@ int run_plan(Run &R) {
     // coincidences
     CoincDev &C = R.C;
     cv.take(C.a, cap / 2 + 1); cv.take(C.b, cap / 2 + 1);
-    // per-job statistics
-    JobStatsDev &JS = R.JS;
-    cv.take(JS.s_off, njc + 1); cv.take(JS.c_off, njc + 1); cv.take(JS.hits, njc);
-    cv.take(R.d_toff, njc); cv.take(R.d_tn, njc);
     R.arena_bytes = align_up(cv.off, 256);
 
     // a live launch uploads (now and while it runs) on its own stream, which
@@ -262,6 +268,7 @@ int run_plan(Run &R) {
         return e == cudaErrorMemoryAllocation ? gpet_fail(GPET_ERR_OOM, "device arena of %zu bytes", R.arena_bytes)
                                               : gpet_cuda_fail(e, "cudaMallocAsync");
     }
+    const uintptr_t tables_off = reinterpret_cast<uintptr_t>(R.d_live);
     char *base = static_cast<char *>(R.arena);
     rebase(R.d_hdr, base);
     rebase(S.ghist, base);
@@ -349,26 +356,31 @@ int run_plan(Run &R) {
     C.n = &H->n_coinc;
     C.window_ps = R.d_window;
 
-    // upload descriptors (small; stream-ordered after the allocation)
-    e = cudaMemcpyAsync(R.d_jobs, R.jobs.data(), sizeof(JobDev) * nj, cudaMemcpyHostToDevice, up);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(R.d_geoms, R.geoms.data(), sizeof(GeomDev) * R.geoms.size(), cudaMemcpyHostToDevice, up);
+    // Upload the descriptors (stream-ordered after the allocation).  A live
+    // launch's tables have room for jobs to come, and it copies what there is,
+    // table by table; any other run's go in one copy.
+    std::vector<char> &tables = R.tables;   // (kept until the run is read back: a copy may still read it)
+    tables.assign(R.live ? 0 : tables_end - tables_off, 0);
+    auto put = [&](void *dst, const void *src, size_t bytes) {
+        if (R.live) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, up);
+        std::memcpy(tables.data() + (static_cast<char *>(dst) - base - tables_off), src, bytes);
+        return cudaSuccess;
+    };
+    const std::vector<long long> toff(R.tally_off.begin(), R.tally_off.end()), tn(R.job_crystals.begin(), R.job_crystals.end());
+    const unsigned long long live0[3] = {R.live_tail, 0ull, 0ull};  // published chunks, closed, claimed
+    e = put(R.d_live, live0, sizeof(live0));
+    if (e == cudaSuccess) e = put(R.d_jobs, R.jobs.data(), sizeof(JobDev) * nj);
+    if (e == cudaSuccess) e = put(R.d_geoms, R.geoms.data(), sizeof(GeomDev) * R.geoms.size());
     for (size_t i = 0; i < R.geoms.size() && e == cudaSuccess; ++i)
         if (i < R.geom_pose.size() && !R.geom_pose[i].empty())
-            e = cudaMemcpyAsync(R.d_pose + pose_off[i], R.geom_pose[i].data(), sizeof(float) * R.geom_pose[i].size(),
-                                cudaMemcpyHostToDevice, up);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(R.d_chunk_start, R.chunk_start.data(), sizeof(unsigned long long) * (njc + 1),
-                            cudaMemcpyHostToDevice, up);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(R.d_window, R.windows.data(), sizeof(uint64_t) * nj, cudaMemcpyHostToDevice, up);
-    if (e == cudaSuccess && n_buckets)
-        e = cudaMemcpyAsync(R.d_buckets, R.buckets.data(), sizeof(BucketJob) * nj, cudaMemcpyHostToDevice, up);
-    std::vector<long long> toff(R.tally_off.begin(), R.tally_off.end()), tn(R.job_crystals.begin(), R.job_crystals.end());
-    if (e == cudaSuccess) e = cudaMemcpyAsync(R.d_toff, toff.data(), sizeof(long long) * nj, cudaMemcpyHostToDevice, up);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(R.d_tn, tn.data(), sizeof(long long) * nj, cudaMemcpyHostToDevice, up);
-    const unsigned long long live0[3] = {R.live_tail, 0ull, 0ull};  // published chunks, closed, claimed
-    if (e == cudaSuccess) e = cudaMemcpyAsync(R.d_live, live0, sizeof(live0), cudaMemcpyHostToDevice, up);
+            e = put(R.d_pose + pose_off[i], R.geom_pose[i].data(), sizeof(float) * R.geom_pose[i].size());
+    if (e == cudaSuccess) e = put(R.d_chunk_start, R.chunk_start.data(), sizeof(unsigned long long) * (njc + 1));
+    if (e == cudaSuccess) e = put(R.d_window, R.windows.data(), sizeof(uint64_t) * nj);
+    if (e == cudaSuccess && n_buckets) e = put(R.d_buckets, R.buckets.data(), sizeof(BucketJob) * nj);
+    if (e == cudaSuccess) e = put(R.d_toff, toff.data(), sizeof(long long) * nj);
+    if (e == cudaSuccess) e = put(R.d_tn, tn.data(), sizeof(long long) * nj);
+    if (e == cudaSuccess && !R.live)
+        e = cudaMemcpyAsync(base + tables_off, tables.data(), tables.size(), cudaMemcpyHostToDevice, up);
     // a digitize-only run's singles and tallies are written by other launches'
     // kernels, possibly running now: the copy engine clears its zeroed region
     for (size_t off = 0; R.digitize_only && off < R.zero_bytes && e == cudaSuccess; off += R.zeros_bytes) {
@@ -376,13 +388,23 @@ int run_plan(Run &R) {
         e = cudaMemcpyAsync(base + off, R.zeros, std::min(R.zeros_bytes, R.zero_bytes - off), cudaMemcpyHostToDevice,
                             up);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(up);  // host vectors may change after return
+    // a run whose kernels go on another stream waits for the tables
+    if (e == cudaSuccess && up != R.stream) e = cudaStreamSynchronize(up);
     R.h2d_bytes = sizeof(JobDev) * nj + sizeof(GeomDev) * R.geoms.size() + sizeof(float) * pose_floats +
                   sizeof(unsigned long long) * (njc + 1) +
                   sizeof(uint64_t) * nj + 2 * sizeof(long long) * nj;
     if (e != cudaSuccess) return gpet_cuda_fail(e, "upload of the job descriptors");
     if (R.live) R.geom_keys.resize(R.geoms.size());
     return GPET_OK;
+}
+
+int run_plan(Run &R) {
+    // a small first guess is not worth the free-memory query, unless it fails
+    const uint64_t per_single = sizeof(RawSingle) + 2 * 8 + 2 * 4 + 8 + 8 + 6 * 4 + 4;
+    const bool small = R.caps.guess && R.caps.singles < kSmallArena / per_single;
+    int st = plan_once(R, !small);
+    if (st == GPET_ERR_OOM && small) st = plan_once(R, true);
+    return st;
 }
 
 static int stage_events(Run &R, unsigned *rec_flags) {
@@ -460,18 +482,22 @@ int run_collect(Run &R) {
     // stream, once the caller has seen its work complete: its own stream may
     // already hold the next launch.
     cudaStream_t rs = R.upload_stream ? R.upload_stream : R.stream;
-    cudaError_t e = cudaMemcpyAsync(&R.h_hdr, R.d_hdr, sizeof(RunHeader), cudaMemcpyDeviceToHost, rs);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(R.s_off.data(), R.JS.s_off, 8 * (nj + 1), cudaMemcpyDeviceToHost, rs);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(R.c_off.data(), R.JS.c_off, 8 * (nj + 1), cudaMemcpyDeviceToHost, rs);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(R.job_hits.data(), R.JS.hits, 8 * nj, cudaMemcpyDeviceToHost, rs);
-    if (e == cudaSuccess && R.d_win_counts) {
-        R.win_counts.resize(nj * R.win_lo.size());
-        e = cudaMemcpyAsync(R.win_counts.data(), R.d_win_counts, 8 * R.win_counts.size(), cudaMemcpyDeviceToHost,
-                            rs);
-    }
+    std::vector<char> block(R.readback_bytes);
+    cudaError_t e = cudaMemcpyAsync(block.data(), R.d_hdr, block.size(), cudaMemcpyDeviceToHost, rs);
     if (e == cudaSuccess) e = cudaStreamSynchronize(rs);
+    auto get = [&](void *dst, const void *src, size_t bytes) {
+        std::memcpy(dst, block.data() + (static_cast<const char *>(src) - reinterpret_cast<const char *>(R.d_hdr)), bytes);
+    };
+    if (e == cudaSuccess) {
+        get(&R.h_hdr, R.d_hdr, sizeof(RunHeader));
+        get(R.s_off.data(), R.JS.s_off, 8 * (nj + 1));
+        get(R.c_off.data(), R.JS.c_off, 8 * (nj + 1));
+        get(R.job_hits.data(), R.JS.hits, 8 * nj);
+        if (R.d_win_counts) {
+            R.win_counts.resize(nj * R.win_lo.size());
+            get(R.win_counts.data(), R.d_win_counts, 8 * R.win_counts.size());
+        }
+    }
     if (e != cudaSuccess) return gpet_cuda_fail(e, "run read-back");
     cta_counters(R.h_hdr.counters, R.h_hdr.counters + kCtaCounters);
     if (R.ev[0] && cudaEventElapsedTime(&R.transport_ms, R.ev[0], R.ev[1]) != cudaSuccess) {
@@ -573,8 +599,16 @@ int run_with_retry(Run &R) {
         }
         break;
     }
-    if (st != GPET_OK) run_release(R);
+    if (st != GPET_OK) {
+        cudaStreamSynchronize(R.stream);   // the tables' copy may not have run
+        run_release(R);
+    }
     return st;
+}
+
+uint64_t first_singles_guess(uint64_t n_decays) {
+    constexpr uint64_t kRoomy = 1ull << 25;
+    return std::max<uint64_t>(65536, n_decays <= kRoomy ? n_decays : std::max<uint64_t>(kRoomy, n_decays / 10 * 6));
 }
 
 void fill_counts(const Run &R, int job, uint64_t n_decays, int64_t n_crystals, gpet_counts *c) {
@@ -794,7 +828,7 @@ extern "C" int gpet_simulate(gpet_scanner *sc, const gpet_source *src, const gpe
     R.geom_pose = {sc->pose_dev};
     R.job_crystals = {sc->n_crystals};
     R.windows = {(uint64_t)std::llround(dg->coinc_window_ns * 1000.0)};
-    R.caps.singles = std::max<uint64_t>(65536, J.n_hist * 6 / 10);
+    R.caps.singles = first_singles_guess(J.n_hist);
     R.caps.hits = R.keep_hits ? std::max<uint64_t>(65536, J.n_hist * 5 / 2) : 0;
     R.caps.ovf = std::max<uint64_t>(4096, J.n_hist / 256);
     st = run_with_retry(R);
