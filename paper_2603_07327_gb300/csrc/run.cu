@@ -135,13 +135,22 @@ static int plan_once(Run &R, bool clamp) {
     }
     uint64_t cs = R.live_cap.chunk;
     if (!R.live && !R.digitize_only) {
-        // chunks: about 48 per resident warp, so that warps run out of work
-        // within a small fraction of the launch of one another (32..4096)
+        // Chunks: about 48 per resident warp, so that warps run out of work
+        // within a small fraction of the launch of one another (32..4096).  The
+        // warps of kernel 3 share their CTA's histories, so a CTA evens out the
+        // chunks of its 14 warps, and 8 chunks per warp of at least 256
+        // histories do (down to two per warp): a claim is then made once in
+        // several decay events (10 M pairs in ring A, whole launch: 1.22 ms with
+        // chunks of 288 against 1.27 ms with 48 of them; 3 M in the h2r ring:
+        // 0.81 ms with 256 against 0.87 ms with 32; a study of 24 designs 1.535
+        // against 1.575; 1 to 2 M pairs no different).
         long long warps = 0;
         cudaError_t we = transport_resident_warps((int)R.geoms.size(), R.cfg, &warps);
         if (we != cudaSuccess) return gpet_cuda_fail(we, "transport occupancy query");
-        cs = total / std::max<uint64_t>((uint64_t)warps * 48, 1);
-        cs = std::max<uint64_t>(32, std::min<uint64_t>(4096, cs / 32 * 32));
+        const bool shared = R.cfg.kernel == kKernelCta;
+        const uint64_t w = (uint64_t)std::max<long long>(warps, 1);
+        const uint64_t least = shared ? std::max<uint64_t>(32, std::min<uint64_t>(256, total / (2 * w) / 32 * 32)) : 32;
+        cs = std::max<uint64_t>(least, std::min<uint64_t>(4096, total / (w * (shared ? 8 : 48)) / 32 * 32));
     }
     R.chunk_size = (unsigned)cs;
     // a live launch's unpublished entries hold ~0: no chunk index reaches them
