@@ -157,10 +157,55 @@ __device__ __forceinline__ T table_load(const T *p) {
     return kLive ? __ldcg(p) : __ldg(p);
 }
 
+// The next chunk of a warp (lanes converged) whose last one is dealt out: its
+// histories become R.next..R.end.  Returns false if there is none: R.exhausted,
+// or R.waiting while a live launch may still publish one.  kLive: table reads
+// go to L2 (ld.cg), since a live launch appends to these tables.
+template <bool kLive>
+__device__ __forceinline__ bool next_chunk(const WorkDev &W, Refill &R) {
+    unsigned long long c = 0;
+    const int cl = claim_chunk<kLive>(W, R.pend, c);
+    R.exhausted = cl < 0;
+    R.waiting = cl == 0;  // try again at the next refill
+    if (cl <= 0) return false;
+    if (!kLive || c >= R.jend) {
+        // The job: the last chunk_start entry <= c.  A live launch's
+        // warp searches from its current job (its claims increase, so
+        // chunk_start[job] <= c), galloping forward, then bisects; a
+        // fixed launch bisects the whole table (cached in L1; measured
+        // faster there).
+        int lo = kLive ? R.job : 0, hi = W.n_jobs - 1, step = 1;
+#pragma unroll 1
+        while (kLive && lo < hi) {
+            const int probe = min(lo + step, hi);
+            if (table_load<kLive>(W.chunk_start + probe) <= c) {
+                lo = probe;
+                step <<= 1;
+            } else {
+                hi = probe - 1;
+                break;
+            }
+        }
+#pragma unroll 1
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (table_load<kLive>(W.chunk_start + mid) <= c) lo = mid; else hi = mid - 1;
+        }
+        // a published job's entries are final (its end is written with it)
+        R.job = lo;
+        R.jc0 = table_load<kLive>(W.chunk_start + lo);
+        R.jend = table_load<kLive>(W.chunk_start + lo + 1);
+        R.base = table_load<kLive>(reinterpret_cast<const unsigned long long *>(&W.jobs[lo].h_base));
+        R.nh = table_load<kLive>(reinterpret_cast<const unsigned long long *>(&W.jobs[lo].n_hist));
+    }
+    const uint64_t h0 = (uint64_t)(c - R.jc0) * W.chunk_size;
+    R.next = R.base + h0;
+    R.end = R.base + min(h0 + (uint64_t)W.chunk_size, R.nh);
+    return true;
+}
+
 // Warp-wide refill: lanes in `need` receive consecutive history ids from the
 // warp's current chunk, fetching new chunks (one atomic each) as needed.
-// kLive: table reads go to L2 (ld.cg), since a live launch appends to these
-// tables.
 template <bool kLive = true>
 __device__ __forceinline__ void warp_refill(const WorkDev &W, uint32_t need, Refill &R, bool &got, uint64_t &h,
                                             int &job) {
@@ -171,49 +216,7 @@ __device__ __forceinline__ void warp_refill(const WorkDev &W, uint32_t need, Ref
     while (need && !R.exhausted) {
         const uint64_t avail = R.end - R.next;
         if (avail == 0) {
-            unsigned long long c = 0;
-            const int cl = claim_chunk<kLive>(W, R.pend, c);
-            if (cl < 0) {
-                R.exhausted = true;
-                break;
-            }
-            if (cl == 0) {
-                R.waiting = true;  // try again at the next refill
-                break;
-            }
-            if (!kLive || c >= R.jend) {
-                // The job: the last chunk_start entry <= c.  A live launch's
-                // warp searches from its current job (its claims increase, so
-                // chunk_start[job] <= c), galloping forward, then bisects; a
-                // fixed launch bisects the whole table (cached in L1; measured
-                // faster there).
-                int lo = kLive ? R.job : 0, hi = W.n_jobs - 1, step = 1;
-#pragma unroll 1
-                while (kLive && lo < hi) {
-                    const int probe = min(lo + step, hi);
-                    if (table_load<kLive>(W.chunk_start + probe) <= c) {
-                        lo = probe;
-                        step <<= 1;
-                    } else {
-                        hi = probe - 1;
-                        break;
-                    }
-                }
-#pragma unroll 1
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (table_load<kLive>(W.chunk_start + mid) <= c) lo = mid; else hi = mid - 1;
-                }
-                // a published job's entries are final (its end is written with it)
-                R.job = lo;
-                R.jc0 = table_load<kLive>(W.chunk_start + lo);
-                R.jend = table_load<kLive>(W.chunk_start + lo + 1);
-                R.base = table_load<kLive>(reinterpret_cast<const unsigned long long *>(&W.jobs[lo].h_base));
-                R.nh = table_load<kLive>(reinterpret_cast<const unsigned long long *>(&W.jobs[lo].n_hist));
-            }
-            const uint64_t h0 = (uint64_t)(c - R.jc0) * W.chunk_size;
-            R.next = R.base + h0;
-            R.end = R.base + min(h0 + (uint64_t)W.chunk_size, R.nh);
+            if (!next_chunk<kLive>(W, R)) break;
             continue;
         }
         const uint32_t cnt = (uint32_t)__popc(need);
@@ -376,6 +379,10 @@ __device__ __forceinline__ uint64_t decay_time(const JobDev &J, const uint4 r) {
     return __umul64hi(J.t_span_ps, ((uint64_t)r.x << 32) | r.y);
 }
 
+// (vi / stride) % n, a voxel's index along an axis of a grid of 2^31 voxels or
+// more (out of line: 64-bit divisions are long, and such grids rare)
+static __device__ __noinline__ int axis_of_large(int64_t vi, int64_t stride, int n) { return (int)((vi / stride) % n); }
+
 // decay of history h (Sec. 2.3) from its first draw r and its azimuth (sine
 // sp, cosine cp of 2 pi u01(r.w)): annihilation point (x0, y0, z0), photon-0
 // direction (ox, oy, oz).  kMap: an activity map may be the source.
@@ -384,21 +391,23 @@ __device__ __forceinline__ void sample_decay(const JobDev &J, uint64_t h, const 
                                              float &y0, float &z0, float &ox, float &oy, float &oz) {
     if (kMap && J.src_kind == 1) {
         const uint4 q = draw(J.seed, h, kTagSource, 0u, 0u, 1u);
-        const uint4 zq = draw(J.seed, h, kTagSource, 0u, 0u, 2u);
+        const uint32_t z = draw(J.seed, h, kTagSource, 0u, 0u, 2u).x;
         const uint64_t r53 = ((uint64_t)q.x << 21) | (q.y >> 11);
         const double target = (double)r53 * 0x1p-53 * J.ph_total;
         const int64_t vi = pick_voxel(J, target);
-        int64_t ix, iy, iz;
+        int v3[3];
         if (J.ph_n <= 0x7FFFFFFFll) {   // 32-bit index arithmetic: a 64-bit division is ~5x dearer
             const uint32_t v = (uint32_t)vi, nx = (uint32_t)J.ph_nx, nxy = nx * (uint32_t)J.ph_ny;
             const uint32_t vz = v / nxy, r = v - vz * nxy, vy = r / nx;
-            ix = r - vy * nx; iy = vy; iz = vz;
+            v3[0] = (int)(r - vy * nx); v3[1] = (int)vy; v3[2] = (int)vz;
         } else {
-            ix = vi % J.ph_nx; iy = (vi / J.ph_nx) % J.ph_ny; iz = vi / ((int64_t)J.ph_nx * J.ph_ny);
+            v3[0] = axis_of_large(vi, 1, J.ph_nx);
+            v3[1] = axis_of_large(vi, J.ph_nx, J.ph_ny);
+            v3[2] = axis_of_large(vi, (int64_t)J.ph_nx * J.ph_ny, J.ph_nz);
         }
-        x0 = fmaf((float)ix + u01(q.z), J.ph_voxel[0], J.ph_origin[0]);
-        y0 = fmaf((float)iy + u01(q.w), J.ph_voxel[1], J.ph_origin[1]);
-        z0 = fmaf((float)iz + u01(zq.x), J.ph_voxel[2], J.ph_origin[2]);
+        x0 = fmaf((float)v3[0] + u01(q.z), J.ph_voxel[0], J.ph_origin[0]);
+        y0 = fmaf((float)v3[1] + u01(q.w), J.ph_voxel[1], J.ph_origin[1]);
+        z0 = fmaf((float)v3[2] + u01(z), J.ph_voxel[2], J.ph_origin[2]);
     } else {
         x0 = J.src_pos[0]; y0 = J.src_pos[1]; z0 = J.src_pos[2];
     }
@@ -428,36 +437,61 @@ __device__ __forceinline__ void ev_source(const JobDev &J, const GeomDev &g, PSt
 // photoelectric absorption or a Compton scatter
 enum : int { kStepExit = 0, kStepVirtual = 1, kStepPhoto = 2, kStepCompton = 3 };
 
-// one Woodcock step in the voxel phantom with draw r: moves the photon
-// (x, path) to its collision point or to the grid's exit
-__device__ __forceinline__ int phantom_step(const JobDev &J, const WorkDev &W, const uint4 r, PState &s) {
-    // distance to the grid box exit
-    float t_out = 3.0e38f;
-    if (s.dx != 0.f) t_out = fminf(t_out, ((s.dx > 0.f ? J.ph_hi[0] : J.ph_origin[0]) - s.x) / s.dx);
-    if (s.dy != 0.f) t_out = fminf(t_out, ((s.dy > 0.f ? J.ph_hi[1] : J.ph_origin[1]) - s.y) / s.dy);
-    if (s.dz != 0.f) t_out = fminf(t_out, ((s.dz > 0.f ? J.ph_hi[2] : J.ph_origin[2]) - s.z) / s.dz);
-    t_out = fmaxf(t_out, 0.0f);
+// One Woodcock step with draw r, in the current panel (kRegions & 1) or the
+// voxel phantom (kRegions & 2; both: where in_panel says): moves the photon
+// (x, path) to its collision point, or to the region's exit.  Panel: L is the
+// collision's place, and left_ring tells that the photon left through the
+// panel's back and can meet no other one.
+template <int kRegions, bool kPosed = true>
+__device__ __forceinline__ int woodcock_step(const JobDev &J, const GeomDev &g, const WorkDev &W, const uint4 r, PState &s,
+                                             bool in_panel, Loc &L, bool &left_ring) {
+    if (kRegions == 1) in_panel = true;
+    if (kRegions == 2) in_panel = false;
+    float t_lim = s.trem;
+    const float *mu_c = g.mu_c511, *mu_pe = g.mu_pe511;
+    int nmat = g.n_materials;
+    if (!in_panel) {
+        // distance to the grid box exit
+        t_lim = 3.0e38f;
+        if (s.dx != 0.f) t_lim = fminf(t_lim, ((s.dx > 0.f ? J.ph_hi[0] : J.ph_origin[0]) - s.x) / s.dx);
+        if (s.dy != 0.f) t_lim = fminf(t_lim, ((s.dy > 0.f ? J.ph_hi[1] : J.ph_origin[1]) - s.y) / s.dy);
+        if (s.dz != 0.f) t_lim = fminf(t_lim, ((s.dz > 0.f ? J.ph_hi[2] : J.ph_origin[2]) - s.z) / s.dz);
+        t_lim = fmaxf(t_lim, 0.0f);
+        mu_c = J.ph_mu_c511; mu_pe = J.ph_mu_pe511;
+        nmat = J.ph_nmat;
+    }
     const Xs xs = xs_at(s.E, W.gtab, W.ln_emin, W.inv_h);
     float mu_maj = 0.0f;
 #pragma unroll 1
-    for (int m = 0; m < J.ph_nmat; ++m) mu_maj = fmaxf(mu_maj, mu_total(J.ph_mu_c511[m], J.ph_mu_pe511[m], xs));
+    for (int m = 0; m < nmat; ++m) mu_maj = fmaxf(mu_maj, mu_total(mu_c[m], mu_pe[m], xs));
     // free path -ln(u) / mu: the fast log's absolute error (< 4e-7) moves a
     // step by < 5e-5 mm even in water, far below the position tolerance
     const float step = mu_maj > 0.0f ? -__logf(u01(r.x)) * (10.0f / mu_maj) : 3.0e38f;
-    if (step >= t_out) {
-        s.x = fmaf(t_out, s.dx, s.x); s.y = fmaf(t_out, s.dy, s.y); s.z = fmaf(t_out, s.dz, s.z);
-        s.path += t_out;
+    const bool out = step >= t_lim;
+    const float d = out ? t_lim : step;
+    s.x = fmaf(d, s.dx, s.x); s.y = fmaf(d, s.dy, s.y); s.z = fmaf(d, s.dz, s.z);
+    s.path += d;
+    if (out) {
+        if (in_panel) {                        // leaves the panel: back to flight
+            left_ring = s.x >= g.w_clear && s.dx >= 0.0f;
+            to_global<kPosed>(g, s);
+        }
         return kStepExit;
     }
-    s.x = fmaf(step, s.dx, s.x); s.y = fmaf(step, s.dy, s.y); s.z = fmaf(step, s.dz, s.z);
-    s.path += step;
-    int ix = (int)floorf((s.x - J.ph_origin[0]) * J.ph_inv_voxel[0]);
-    int iy = (int)floorf((s.y - J.ph_origin[1]) * J.ph_inv_voxel[1]);
-    int iz = (int)floorf((s.z - J.ph_origin[2]) * J.ph_inv_voxel[2]);
-    ix = min(max(ix, 0), J.ph_nx - 1); iy = min(max(iy, 0), J.ph_ny - 1); iz = min(max(iz, 0), J.ph_nz - 1);
-    const int m = __ldg(J.ph_mat + ((int64_t)iz * J.ph_ny + iy) * J.ph_nx + ix);
-    const float pe = J.ph_mu_pe511[m] * xs.r3;
-    const float mu_m = fmaf(J.ph_mu_c511[m], xs.g, pe);
+    int m;
+    if (in_panel) {
+        s.trem -= step;
+        L = locate(g, s.panel, s.x, s.y, s.z);
+        m = L.mat;
+    } else {
+        int ix = (int)floorf((s.x - J.ph_origin[0]) * J.ph_inv_voxel[0]);
+        int iy = (int)floorf((s.y - J.ph_origin[1]) * J.ph_inv_voxel[1]);
+        int iz = (int)floorf((s.z - J.ph_origin[2]) * J.ph_inv_voxel[2]);
+        ix = min(max(ix, 0), J.ph_nx - 1); iy = min(max(iy, 0), J.ph_ny - 1); iz = min(max(iz, 0), J.ph_nz - 1);
+        m = __ldg(J.ph_mat + ((int64_t)iz * J.ph_ny + iy) * J.ph_nx + ix);
+    }
+    const float pe = mu_pe[m] * xs.r3;
+    const float mu_m = fmaf(mu_c[m], xs.g, pe);
     if (u01(r.y) * mu_maj >= mu_m) return kStepVirtual;
     return u01(r.z) * mu_m < pe ? kStepPhoto : kStepCompton;
 }
@@ -468,7 +502,9 @@ __device__ __forceinline__ int ev_phantom(const JobDev &J, const GeomDev &g, con
     const uint4 r = draw(J.seed, s.h, kTagPhantom, s.gamma, s.sph, 0u);
     const uint32_t step_id = s.sph++;
     cnt.ph_steps++;
-    const int what = phantom_step(J, W, r, s);
+    Loc L;
+    bool left_ring;
+    const int what = woodcock_step<2>(J, g, W, r, s, false, L, left_ring);
     if (what == kStepExit) { s.phase = kPhFlight; return kStatusOk; }
     if (what == kStepVirtual) return kStatusOk;
     if (what == kStepPhoto) { photon_done(J, g, s, cnt); return kStatusOk; }
@@ -587,36 +623,6 @@ __device__ __forceinline__ void record_hit(const JobDev &J, const GeomDev &g, co
     add_single(g, s, SL, max_entries, crystal, module, dep, dtp, s.x);
 }
 
-// one Woodcock step inside the current panel with draw r: moves the photon
-// (x, path) to its collision point L or to the panel's exit
-// (left_ring: the photon left it through the back and can meet no other panel)
-template <bool kPosed = true>
-__device__ __forceinline__ int panel_step(const GeomDev &g, const WorkDev &W, const uint4 r, PState &s, Loc &L,
-                                          bool &left_ring) {
-    const Xs xs = xs_at(s.E, W.gtab, W.ln_emin, W.inv_h);
-    float mu_maj = 0.0f;
-#pragma unroll 1
-    for (int m = 0; m < g.n_materials; ++m) mu_maj = fmaxf(mu_maj, mu_total(g.mu_c511[m], g.mu_pe511[m], xs));
-    // free path -ln(u) / mu: the fast log's absolute error (< 4e-7) moves a
-    // step by < 5e-5 mm even in water, far below the position tolerance
-    const float step = mu_maj > 0.0f ? -__logf(u01(r.x)) * (10.0f / mu_maj) : 3.0e38f;
-    if (step >= s.trem) {                      // leaves the panel: back to flight
-        s.x = fmaf(s.trem, s.dx, s.x); s.y = fmaf(s.trem, s.dy, s.y); s.z = fmaf(s.trem, s.dz, s.z);
-        s.path += s.trem;
-        left_ring = s.x >= g.w_clear && s.dx >= 0.0f;
-        to_global<kPosed>(g, s);
-        return kStepExit;
-    }
-    s.x = fmaf(step, s.dx, s.x); s.y = fmaf(step, s.dy, s.y); s.z = fmaf(step, s.dz, s.z);
-    s.path += step;
-    s.trem -= step;
-    L = locate(g, s.panel, s.x, s.y, s.z);
-    const float pe = g.mu_pe511[L.mat] * xs.r3;
-    const float mu_m = fmaf(g.mu_c511[L.mat], xs.g, pe);
-    if (u01(r.y) * mu_maj >= mu_m) return kStepVirtual;
-    return u01(r.z) * mu_m < pe ? kStepPhoto : kStepCompton;
-}
-
 // one Woodcock step inside the current panel (layer selection, interaction, hit)
 template <bool kTallies>
 __device__ __forceinline__ int ev_panel(const JobDev &J, const GeomDev &g, const WorkDev &W, const OutDev &O,
@@ -627,7 +633,7 @@ __device__ __forceinline__ int ev_panel(const JobDev &J, const GeomDev &g, const
     cnt.det_steps++;
     Loc L;
     bool left_ring;
-    const int what = panel_step(g, W, r, s, L, left_ring);
+    const int what = woodcock_step<1>(J, g, W, r, s, true, L, left_ring);
     if (what == kStepExit) {
         s.last = s.panel;
         s.panel = -1;

@@ -136,6 +136,27 @@ __device__ __forceinline__ void count(uint32_t &acc, int i, uint32_t n) {
     if ((int)(threadIdx.x & 31) == i) acc += n;
 }
 
+// The warp's next chunk, for its refill state in shared memory (out of line: called once
+// in several decay events, and inline it took the step code's place
+// in the instruction cache; 60 M pairs in two ring geometries: 6.33 ms against 6.64)
+template <bool kLive>
+__device__ __noinline__ bool next_chunk_out(const WorkDev &W, Refill &R) {
+    Refill r;   // field by field: a copy of the whole would go through local memory
+    r.pend = R.pend; r.jc0 = R.jc0; r.jend = R.jend; r.base = R.base; r.nh = R.nh;
+    r.next = R.next; r.end = R.end;
+    r.job = R.job;
+    __syncwarp();
+    const bool got = next_chunk<kLive>(W, r);
+    if ((threadIdx.x & 31) == 0) {
+        R.next = r.next; R.end = r.end;
+        R.pend = r.pend; R.jc0 = r.jc0; R.jend = r.jend; R.base = r.base; R.nh = r.nh;
+        R.job = r.job;
+        R.exhausted = r.exhausted; R.waiting = r.waiting;
+    }
+    __syncwarp();
+    return got;
+}
+
 // a crystal interaction into the optional hit list (tests, depth studies)
 __device__ __noinline__ void keep_hit(const OutDev &O, const JobDev &J, const GeomDev &g, uint64_t h, int job,
                                       uint32_t gamma, uint32_t step, int crystal, float dep, uint32_t dtp, float x,
@@ -160,7 +181,8 @@ __device__ __noinline__ void keep_hit(const OutDev &O, const JobDev &J, const Ge
 // that a fixed launch without them carries none of their instructions,
 // registers and state words.
 template <int WARPS, int SLOTS, int CTAS, bool kPhantom, bool kPosed, bool kLive>
-__global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(WorkDev W, OutDev O, int ng_smem) {
+__global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid_constant__ WorkDev W,
+                                                                   const __grid_constant__ OutDev O, int ng_smem) {
     static_assert(SLOTS <= 32, "one mask bit per slot");
     using Pool = CtaPool<SLOTS, kPhantom>;
     constexpr int kN = Pool::kN;
@@ -256,15 +278,27 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(WorkDev W, O
         uint64_t h = 0;
         bool run = active;   // lanes with a history
         if (ph == kPhIdle) {
-            Refill rf = refills[wid];
-            __syncwarp();
-            int job = 0;
-            warp_refill<kLive>(W, am, rf, run, h, job);
-            if (lane == 0) refills[wid] = rf;
-            __syncwarp();
+            Refill &rf = refills[wid];
+            // consecutive histories of the warp's chunks to the claimed lanes
+            uint32_t need = am;
+            run = false;
+#pragma unroll 1
+            do {
+                const uint64_t next = rf.next, avail = rf.end - next;
+                const uint32_t rank = __popc(need & lanemask_lt());
+                const uint32_t take = (uint32_t)min(avail, (uint64_t)__popc(need));
+                if (((need >> lane) & 1u) && rank < take) {
+                    run = true;
+                    h = next + rank;
+                    jobw = (uint32_t)rf.job;
+                }
+                __syncwarp();
+                if (lane == 0) rf.next = next + take;
+                need &= ~__ballot_sync(kFullMask, run);
+                __syncwarp();
+            } while (need && next_chunk_out<kLive>(W, rf));
             done = rf.exhausted;
             waiting = rf.waiting;
-            jobw = (uint32_t)job;
         } else if (active) {
             jobw = ST(kSjob);
             pk = ST(kSpk);
@@ -357,13 +391,13 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(WorkDev W, O
                                           make_uint2((uint32_t)J.seed, (uint32_t)(J.seed >> 32)));
             if (ph == kPhPanel || (kPhantom && ph == kPhPhantom)) {
                 // one Woodcock step in the panel or the phantom
-                bool late = false;
                 uint32_t n_left = 0;
                 if (run) {
+                    const bool panel = !kPhantom || ph == kPhPanel;
                     PState s;
                     s.panel = (int)(pk & kPkPanel) - 1;
                     const uint32_t sph = kPhantom ? ST(kSph) : 0u;
-                    const bool fresh = ph == kPhPanel ? (pk & kPkFresh) != 0 : sph == 0;
+                    const bool fresh = panel ? (pk & kPkFresh) != 0 : sph == 0;
                     if (fresh) {   // starts at its decay point
                         s.x = kPhantom ? STF(kSx0) : J.src_pos[0];
                         s.y = kPhantom ? STF(kSy0) : J.src_pos[1];
@@ -379,53 +413,53 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(WorkDev W, O
                         s.E = STF(kSE);
                         s.path = STF(kSpath);
                     }
+                    bool moved = fresh;   // the direction is not the slot's
+                    s.trem = __uint_as_float(st[(fresh && gamma ? kSrem1 : kStrem) * kN + q]);
+                    if (panel && (pk & (kPkFresh | kPkLastMask))) {
+                        const int wi = !fresh ? kSrw : gamma ? kSin1 : kSpath;
+                        enter_panel<kPosed>(g, s.panel, __uint_as_float(st[wi * kN + q]), s);
+                        pk &= ~(kPkFresh | kPkLastMask);
+                        moved = true;
+                    }
+                    const bool late = (panel ? step : sph) >= (uint32_t)kMaxSteps;
+                    Loc L;
+                    L.crystal = -1;
+                    bool left_ring = false;
+                    // a branch each for panel and phantom (5 M pairs in the hot-rod phantom: 1.65 ms
+                    // against 1.71); a live launch, whose code is the longest, takes one for both
+                    // (a served burst: 2.89 ms against 3.03)
+                    int what;
+                    if (kLive) what = woodcock_step<3, kPosed>(J, g, W, r, s, panel, L, left_ring);
+                    else if (panel) what = woodcock_step<1, kPosed>(J, g, W, r, s, true, L, left_ring);
+                    else what = woodcock_step<2, kPosed>(J, g, W, r, s, false, L, left_ring);
+                    if (panel) pk += late ? 0u : 1u << kPkStep;
+                    else ST(kSph) = sph + 1u;
                     to = ph;
-                    if (!kPhantom || ph == kPhPanel) {
-                        const bool enter = pk & (kPkFresh | kPkLastMask);
-                        s.trem = __uint_as_float(st[(fresh && gamma ? kSrem1 : kStrem) * kN + q]);
-                        if (enter) {
-                            const int wi = !fresh ? kSrw : gamma ? kSin1 : kSpath;
-                            enter_panel<kPosed>(g, s.panel, __uint_as_float(st[wi * kN + q]), s);
-                            pk &= ~(kPkFresh | kPkLastMask);
-                        }
-                        late = step >= (uint32_t)kMaxSteps;
-                        Loc L;
-                        bool left_ring = false;
-                        const int what = panel_step<kPosed>(g, W, r, s, L, left_ring);
-                        pk += late ? 0u : 1u << kPkStep;
-                        ST(kStrem) = what >= kStepPhoto ? (uint32_t)L.crystal : __float_as_uint(s.trem);
-                        if (enter || what == kStepExit) STORE3(kSdx, s.dx, s.dy, s.dz);
-                        if (what == kStepExit) {
-                            if (left_ring) {
-                                // its flight would end it: counted as one, without the event
-                                n_left = 1;
-                                const float c0 = fmaf(s.x, s.x, s.y * s.y), a = fmaf(s.dx, s.dx, s.dy * s.dy);
-                                if (a > 0.0f && !(c0 < g.R2 * 0.9999f) && outside_screened(g, a, fmaf(s.x, s.dx, s.y * s.dy), c0))
-                                    n_left = 1u | 1u << 16;
-                                to = photon_end(pk, (jobw >> kJobPanel1) & 0x7Fu);
-                            } else {
-                                pk = (pk & ~kPkPanel) | ((pk & kPkPanel) << kPkLast);
-                                to = kPhFlightOut;
-                            }
-                        } else if (what != kStepVirtual) {
-                            ST(kSrw) = r.w & ~511u;
-                            pk = (pk & ~kPkPhoto) | (what == kStepPhoto ? kPkPhoto : 0u);
-                            to = kPhInteract;
-                        }
-                    } else {
-                        if (fresh) STORE3(kSdx, s.dx, s.dy, s.dz);
-                        late = sph >= (uint32_t)kMaxSteps;
-                        const int what = phantom_step(J, W, r, s);
-                        ST(kSph) = sph + 1u;
-                        if (what == kStepExit) {
+                    ST(kStrem) = what >= kStepPhoto ? (uint32_t)L.crystal : __float_as_uint(s.trem);
+                    if (moved || what == kStepExit) STORE3(kSdx, s.dx, s.dy, s.dz);
+                    bool ends = !panel && what == kStepPhoto;
+                    if (what == kStepExit) {
+                        if (!panel) {
                             to = kPhFlight;
-                        } else if (what == kStepPhoto) {
-                            to = photon_end(pk, 0);
-                            ST(kSph) = 0;
-                        } else if (what == kStepCompton) {
-                            ST(kSrw) = r.w & ~511u;
-                            to = kPhInteract;   // panel field 0: in the phantom
+                        } else if (left_ring) {
+                            // its flight would end it: counted as one, without the event
+                            ends = true;
+                            n_left = 1;
+                            const float c0 = fmaf(s.x, s.x, s.y * s.y), a = fmaf(s.dx, s.dx, s.dy * s.dy);
+                            if (a > 0.0f && !(c0 < g.R2 * 0.9999f) && outside_screened(g, a, fmaf(s.x, s.dx, s.y * s.dy), c0))
+                                n_left = 1u | 1u << 16;
+                        } else {
+                            pk = (pk & ~kPkPanel) | ((pk & kPkPanel) << kPkLast);
+                            to = kPhFlightOut;
                         }
+                    } else if (what != kStepVirtual) {
+                        ST(kSrw) = r.w & ~511u;
+                        pk = (pk & ~kPkPhoto) | (what == kStepPhoto ? kPkPhoto : 0u);
+                        to = kPhInteract;   // panel field 0: in the phantom
+                    }
+                    if (ends) {
+                        to = photon_end(pk, (jobw >> kJobPanel1) & 0x7Fu);
+                        if (kPhantom) ST(kSph) = 0;
                     }
                     STORE3(kSx, s.x, s.y, s.z);
                     ST(kSpath) = __float_as_uint(s.path);
