@@ -29,6 +29,12 @@
 //     directions), which keeps photon 1's panel and distances in the slot until
 //     its turn; a photon that leaves through a panel's back, where no other panel
 //     can be, ends without a flight event.
+//   - A history's singles are a chain of entries that the slots of a lane class
+//     share, so a list has no length of its own to overflow: only a class without
+//     a free entry leaves a history to the redo kernel.  With lists of six, that
+//     kernel's few serial histories took 30 us of every launch of 1e6 pairs and
+//     more (1e6 pairs in the 12-panel ring 207 us, now 175; 2e6 in four heads 235,
+//     now 213; 24 designs in one launch 1.44 ms, now 1.38).
 // Photons of a pair run one after the other, and events are those of
 // transport.cuh, so the histories equal the other kernels' bit for bit.
 //
@@ -45,12 +51,12 @@ namespace {
 // one more phase here than in transport.cuh: a collision to be sampled
 constexpr uint32_t kPhInteract = 7;
 constexpr int kPhCount = 8;
-constexpr int kCtaS = 6;      // singles of one history (more -> redo kernel)
 constexpr int kEntries = 48;  // singles entries of a lane class, for all of its slots
 
 // state words of a slot; the last four only where a job has a phantom
 enum : int { kSh0 = 0, kSh1,
-             kSjob,             // job; [16:23) photon 1's first panel + 1 (0: it enters none); [23:29) sixth entry
+             kSjob,             // job; [16:23) photon 1's first panel + 1 (0: it enters none);
+                                // [23:29) first entry + 1 of the history's singles list (0: empty)
              kSox, kSoy, kSoz,
              kSx, kSy, kSz, kSdx, kSdy, kSdz, kSE,
              kSpath,            // path; distance to the panel of a photon 0 that has not entered it yet
@@ -59,22 +65,21 @@ enum : int { kSh0 = 0, kSh1,
              kSrw,              // azimuth word (top 23 bits) of a collision and its Kahn trials (low 9 bits);
                                 // distance to the next panel of a photon between panels
              kSpk,
-             kSlist,            // the history's singles: six bits each, entries of the lane class
              kSx0, kSy0, kSz0, kSph };
 constexpr int kWordsPlain = kSx0, kWordsPhantom = kSph + 1;
-constexpr int kJobPanel1 = 16, kJobEntry = 23;
+constexpr int kJobPanel1 = 16, kJobList = 23;
 
-// packed word: [0:7) panel + 1 (finish event: next single), [7:14) last panel + 1
+// packed word: [0:7) panel + 1, [7:14) last panel + 1
 // (in a panel: not 0 where the photon has still to enter it; a collision: bit 7
-// counts 512 Kahn trials), [14] photon, [15:18) singles in the list, [18] list
+// counts 512 Kahn trials), [14] photon, [15] the list has singles, [18] list
 // overflowed, [19] photon 1 starts in the phantom, [20] photon not in its first
 // panel yet (its state is the decay's), [21:31) detector steps, [31]
 // photoelectric absorption
-constexpr int kPkLast = 7, kPkSing = 15, kPkStep = 21;
-constexpr uint32_t kPkPanel = 0x7Fu, kPkLastMask = 0x7Fu << kPkLast, kPkGamma = 1u << 14, kPkSingMask = 7u << kPkSing,
+constexpr int kPkLast = 7, kPkStep = 21;
+constexpr uint32_t kPkPanel = 0x7Fu, kPkLastMask = 0x7Fu << kPkLast, kPkGamma = 1u << 14, kPkSing = 1u << 15,
                    kPkOvf = 1u << 18, kPkPhantom1 = 1u << 19, kPkFresh = 1u << 20, kPkStepMask = 0x3FFu << kPkStep,
                    kPkPhoto = 1u << 31;
-static_assert(kMaxSteps < 1024 && kMaxPanels < 127 && kCtaS <= 6 && kMaxTrials <= 1024, "packed word fields");
+static_assert(kMaxSteps < 1024 && kMaxPanels < 127 && kMaxTrials <= 1024 && kEntries < 63, "packed word fields");
 
 // event counters: slots 0..7 count the events of each phase (decays in 0,
 // lanes fed in 1); lane i of a warp keeps counter i
@@ -92,13 +97,14 @@ struct CtaPool {
     float e_e[kEntries * 32];
     uint32_t e_dt[kEntries * 32];
     float e_ew[kEntries * 32];
+    uint8_t e_next[kEntries * 32];   // next entry + 1 of the history's list (0: the last); four of a lane in a word
 };
 
-// entries of a history's list, and the free entries of a lane class
-__device__ __forceinline__ uint32_t list_entry(uint32_t list, uint32_t jobw, uint32_t i) {
-    return i < 5u ? (list >> (6 * i)) & 63u : (jobw >> kJobEntry) & 63u;
-}
+// place of entry e in e_next
+__device__ __forceinline__ uint32_t next_at(uint32_t e, int lane) { return ((e >> 2) * 32u + lane) * 4u + (e & 3u); }
+// the free entries of a lane class (the entry's last reads come before)
 __device__ __forceinline__ void free_entry(uint32_t (*efree)[32], int lane, uint32_t e) {
+    asm volatile("" ::: "memory");
     atomicOr(&efree[e >> 5][lane], 1u << (e & 31u));
 }
 // a free entry, or kEntries
@@ -123,7 +129,7 @@ __device__ __forceinline__ uint32_t take_entry(uint32_t (*efree)[32], int lane) 
 // nothing to digitize, its slot is free.
 __device__ __forceinline__ uint32_t photon_end(uint32_t &pk, uint32_t panel1) {
     const bool first = !(pk & kPkGamma), ph1 = pk & kPkPhantom1;
-    pk &= kPkSingMask | kPkOvf;
+    pk &= kPkSing | kPkOvf;
     if (first && (ph1 || panel1)) {
         pk |= kPkGamma | (ph1 ? 0u : kPkFresh | panel1);
         return ph1 ? kPhPhantom : kPhPanel;
@@ -370,7 +376,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
         } else {
             // The other events begin with a draw, made here for all of them.
             const bool in_panel = !kPhantom || (pk & kPkPanel);
-            uint32_t c2 = kTagSource << 28, c3 = 0, rw = 0, list = 0, e = 0, unit = 0;
+            uint32_t c2 = kTagSource << 28, c3 = 0, rw = 0, e = 0, next = 0, unit = 0;
             const uint32_t step = (pk & kPkStepMask) >> kPkStep;
             if (ph == kPhPanel) {
                 c2 = (kTagDetector << 28) | (gamma << 27) | step;
@@ -381,9 +387,10 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                 c2 = (in_panel ? (kTagDetector << 28) | (step - 1u) : (kTagPhantom << 28) | (ST(kSph) - 1u)) | (gamma << 27);
                 c3 = 1u + (rw & 511u) + ((pk >> kPkLast) & 1u) * 512u;
             } else if (ph == kPhFinish) {
-                list = ST(kSlist);
-                e = list_entry(list, jobw, pk & kPkPanel) & 63u;
-                unit = P.e_unit[(run ? e : 0u) * 32 + lane];
+                e = ((jobw >> kJobList) & 63u) - 1u;
+                if (!run || !(pk & kPkSing)) e = 0;   // overflowed before its first single
+                unit = P.e_unit[e * 32 + lane];
+                next = P.e_next[next_at(e, lane)];
                 c2 = kTagDigi << 28;
                 c3 = unit;
             }
@@ -512,30 +519,33 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                                 unit = (uint32_t)crystal;
                                 if (g.readout_level == 0) unit = (pk & kPkPanel) - 1u;
                                 else if (g.readout_level == 1) unit = (uint32_t)crystal / (uint32_t)g.crystals_per_module;
-                                const uint32_t n = (pk & kPkSingMask) >> kPkSing;
-                                list = n ? ST(kSlist) : 0u;
-                                uint32_t ei = kEntries * 32;
+                                // the list's entry of this unit, or its last one
+                                uint32_t ei = kEntries * 32, last = 0;
+                                next = (jobw >> kJobList) & 63u;
 #pragma unroll 1
-                                for (uint32_t i = 0; i < n; ++i) {
-                                    const uint32_t ej = list_entry(list, jobw, i) * 32 + lane;
-                                    if (P.e_unit[ej] == unit) ei = ej;
+                                while (next) {
+                                    last = next--;
+                                    const uint32_t u = P.e_unit[next * 32 + lane];
+                                    if (u == unit) ei = next * 32 + lane;
+                                    next = P.e_next[next_at(next, lane)];
                                 }
                                 if (ei < kEntries * 32) {
                                     P.e_e[ei] += dep;
                                     P.e_ew[ei] += dep * x;
                                     P.e_dt[ei] = min(P.e_dt[ei], dtp);
                                 } else {
-                                    e = n < (uint32_t)kCtaS ? take_entry(efree, lane) : (uint32_t)kEntries;
+                                    e = take_entry(efree, lane);
                                     if (e < (uint32_t)kEntries) {
                                         ei = e * 32 + lane;
                                         P.e_unit[ei] = unit;
                                         P.e_e[ei] = dep;
                                         P.e_ew[ei] = dep * x;
                                         P.e_dt[ei] = dtp;
-                                        if (n < 5u) ST(kSlist) = list | (e << (6 * n));
-                                        else ST(kSjob) = jobw | (e << kJobEntry);
-                                        pk += 1u << kPkSing;
-                                    } else if (n < (uint32_t)kCtaS && *reinterpret_cast<volatile uint32_t *>(&mask[kPhFinish][lane])) {
+                                        P.e_next[next_at(e, lane)] = 0;
+                                        if (last) P.e_next[next_at(last - 1u, lane)] = (uint8_t)(e + 1u);
+                                        else ST(kSjob) = jobw | ((e + 1u) << kJobList);
+                                        pk |= kPkSing;
+                                    } else if (*reinterpret_cast<volatile uint32_t *>(&mask[kPhFinish][lane])) {
                                         held = true;     // entries come free: the same trial again then
                                     } else {
                                         pk |= kPkOvf;    // simulated again by the redo kernel
@@ -620,7 +630,6 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                     }
                 } else {
                     // digitizer: one single of the history's list, in list order
-                    const uint32_t n = (pk & kPkSingMask) >> kPkSing, j = pk & kPkPanel;
                     const bool ovf = run && (pk & kPkOvf), one = run && !ovf;
                     append_overflow(O, ovf, h, (int)(jobw & 0xFFFFu), kFullMask);
                     SingleOut so;
@@ -631,11 +640,17 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                         free_entry(efree, lane, e);
                     }
                     append_single<kLive, true>(W.geoms, O, J, (int)(jobw & 0xFFFFu), h, 0, so, kFullMask);
-                    if (ovf)
+                    if (ovf && (pk & kPkSing)) {
 #pragma unroll 1
-                        for (uint32_t i = 0; i < n; ++i) free_entry(efree, lane, list_entry(list, jobw, i));
-                    const bool last = ovf || j + 1u >= n;
-                    if (run && !last) ST(kSpk) = pk + 1u;
+                        for (;;) {
+                            free_entry(efree, lane, e);
+                            if (!next) break;
+                            e = next - 1u;
+                            next = P.e_next[next_at(e, lane)];
+                        }
+                    }
+                    const bool last = ovf || !next;
+                    if (run && !last) ST(kSjob) = (jobw & ~(63u << kJobList)) | (next << kJobList);
                     to = last ? kPhIdle : kPhFinish;
                     count(acc, kNFin, __popc(__ballot_sync(kFullMask, run && last)));
                     count(acc, kNSingles, __popc(__ballot_sync(kFullMask, one)));
