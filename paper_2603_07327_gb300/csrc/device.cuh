@@ -259,7 +259,21 @@ struct Loc {
     int32_t mat;
 };
 
-__device__ __forceinline__ Loc locate(const GeomDev &g, int k, float w, float u, float v) {
+// A geometry as one warp's lanes read it: fields that every lane reads alike, and
+// tables that a lane indexes by its panel, layer or material.  The same
+// descriptor serves both (GeomDev), or two copies of it do: kernel parameters,
+// which instructions take as operands, and shared memory (GeomOne).
+struct GeomOne {
+    const GeomDev &f, &t;
+};
+__device__ __forceinline__ const GeomDev &fields(const GeomDev &g) { return g; }
+__device__ __forceinline__ const GeomDev &tables(const GeomDev &g) { return g; }
+__device__ __forceinline__ const GeomDev &fields(const GeomOne &g) { return g.f; }
+__device__ __forceinline__ const GeomDev &tables(const GeomOne &g) { return g.t; }
+
+template <class Geom>
+__device__ __forceinline__ Loc locate(const Geom &geom, int k, float w, float u, float v) {
+    const GeomDev &g = fields(geom);
     Loc L;
     L.layer = -1; L.module = -1; L.crystal = -1;
     // layer-selection step: the layer whose depth range holds w
@@ -270,10 +284,10 @@ __device__ __forceinline__ Loc locate(const GeomDev &g, int k, float w, float u,
         if (w < g.layers[j].w1) { l = j; break; }
     }
     if (l < 0) {
-        L.mat = g.layers[owner].interval_mat;
+        L.mat = tables(geom).layers[owner].interval_mat;
         return L;
     }
-    const LayerDev &Ly = g.layers[l];
+    const LayerDev &Ly = tables(geom).layers[l];
     L.layer = l;
     L.mat = Ly.interval_mat;
     const float au = u + g.half_u, av = v + g.half_v;
@@ -305,10 +319,12 @@ __device__ __forceinline__ float panel_exit(const GeomDev &g, float w, float u, 
 
 // slab test of the ray against panel k's box in its own frame; keeps the
 // nearest entry (ties to the lower panel index)
-__device__ __forceinline__ void panel_slab(const GeomDev &g, int k, float x, float y, float z, float dx, float dy,
+template <class Geom>
+__device__ __forceinline__ void panel_slab(const Geom &geom, int k, float x, float y, float z, float dx, float dy,
                                            float dz, int &best, float &bi, float &bo) {
+    const GeomDev &g = fields(geom);
     {
-        const float c = g.pc[k], s = g.ps[k];
+        const float c = tables(geom).pc[k], s = tables(geom).ps[k];
         const float w0 = fmaf(x, c, y * s) - g.R;
         const float dw = fmaf(dx, c, dy * s);
         // behind the inner face and moving away: no entry
@@ -473,9 +489,10 @@ __device__ __forceinline__ bool outside_screened(const GeomDev &g, float a, floa
 // first and share one slab-test loop, so that a warp's lanes test together and
 // the test's code is there once.  kPosed = false: no geometry of the launch
 // has panel poses.
-template <bool kPosed = true>
-__device__ __forceinline__ int flight(const GeomDev &g, float x, float y, float z, float dx, float dy, float dz,
+template <bool kPosed = true, class Geom>
+__device__ __forceinline__ int flight(const Geom &geom, float x, float y, float z, float dx, float dy, float dz,
                                       int skip, float &t_in, float &t_out) {
+    const GeomDev &g = fields(geom);
     int best = -1;
     float bi = 3.0e38f, bo = 0.0f;
     if (kPosed && g.posed) {
@@ -537,7 +554,7 @@ __device__ __forceinline__ int flight(const GeomDev &g, float x, float y, float 
         if (!all) flight_sector(g, x, y, dx, dy, ta, tb, k, n);
 #pragma unroll 1
         for (; n > 0; --n) {
-            if (k != skip) panel_slab(g, k, x, y, z, dx, dy, dz, best, bi, bo);
+            if (k != skip) panel_slab(geom, k, x, y, z, dx, dy, dz, best, bi, bo);
             k = k + 1 == g.n_panels ? 0 : k + 1;
         }
         if (!two) break;

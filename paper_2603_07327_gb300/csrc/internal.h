@@ -25,6 +25,10 @@ struct LaunchCfg {
     bool phantom;        // a job of the launch has a phantom, or one may be appended
     bool posed;          // a geometry of the launch has panel poses, or one may be appended
     bool live;           // a live launch
+    // a launch of one job that is known when it is made: the job and its
+    // geometry, as they are in the device's tables (else NULL)
+    const struct JobDev *one_job;
+    const struct GeomDev *one_geom;
 };
 
 // one job's time buckets: a time t falls in bucket first + min(hi64(t * scale), n - 1)

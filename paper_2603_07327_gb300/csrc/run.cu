@@ -101,6 +101,15 @@ int run_default_cfg(Run &R, const gpet_options *opt_in, const gpet_scanner *sc) 
 // first (the query costs more than the allocation).
 constexpr size_t kSmallArena = (size_t)256 << 20;
 
+// the configuration of a run's transport launch
+static LaunchCfg launch_cfg(const Run &R) {
+    LaunchCfg cfg = R.cfg;
+    const bool one = !R.live && R.jobs.size() == 1;
+    cfg.one_job = one ? R.jobs.data() : nullptr;
+    cfg.one_geom = one ? &R.geoms[R.jobs[0].geom] : nullptr;
+    return cfg;
+}
+
 static int plan_once(Run &R, bool clamp) {
     const int nj = (int)R.jobs.size();
     // table sizes: the jobs themselves, or a live launch's capacities
@@ -145,7 +154,7 @@ static int plan_once(Run &R, bool clamp) {
         // 0.81 ms with 256 against 0.87 ms with 32; a study of 24 designs 1.535
         // against 1.575; 1 to 2 M pairs no different).
         long long warps = 0;
-        cudaError_t we = transport_resident_warps((int)R.geoms.size(), R.cfg, &warps);
+        cudaError_t we = transport_resident_warps((int)R.geoms.size(), launch_cfg(R), &warps);
         if (we != cudaSuccess) return gpet_cuda_fail(we, "transport occupancy query");
         const bool shared = R.cfg.kernel == kKernelCta;
         const uint64_t w = (uint64_t)std::max<long long>(warps, 1);
@@ -440,7 +449,7 @@ int run_enqueue_transport(Run &R) {
     e = cudaEventRecordWithFlags(R.ev[0], R.stream, rec_flags);
     // A live launch's kernel waits on the host: nothing else is launched while
     // it runs (the re-simulation of overflowed histories follows at its close).
-    if (e == cudaSuccess) e = launch_transport(R.W, R.O, R.cfg, R.stream, !R.live);
+    if (e == cudaSuccess) e = launch_transport(R.W, R.O, launch_cfg(R), R.stream, !R.live);
     if (e != cudaSuccess) return gpet_cuda_fail(e, "transport launch");
     if (!R.live) {
         e = cudaEventRecordWithFlags(R.ev[1], R.stream, rec_flags);

@@ -291,8 +291,9 @@ struct Counters {
     uint32_t src, fl_ev, fl_out, fin;
 };
 
-template <bool kPosed = true>
-__device__ __forceinline__ void to_global(const GeomDev &g, PState &s) {
+template <bool kPosed = true, class Geom>
+__device__ __forceinline__ void to_global(const Geom &geom, PState &s) {
+    const GeomDev &g = fields(geom);
     if (kPosed && g.posed) {
         const float4 aw = __ldg(g.pose + 4 * s.panel), au = __ldg(g.pose + 4 * s.panel + 1);
         const float4 av = __ldg(g.pose + 4 * s.panel + 2), o = __ldg(g.pose + 4 * s.panel + 3);
@@ -305,7 +306,7 @@ __device__ __forceinline__ void to_global(const GeomDev &g, PState &s) {
         s.dz = fmaf(dw, aw.z, fmaf(du, au.z, dv * av.z));
         return;
     }
-    const float c = g.pc[s.panel], sn = g.ps[s.panel];
+    const float c = tables(geom).pc[s.panel], sn = tables(geom).ps[s.panel];
     const float rw = g.R + s.x;
     const float gx = rw * c - s.y * sn, gy = rw * sn + s.y * c;
     const float gdx = s.dx * c - s.dy * sn, gdy = s.dx * sn + s.dy * c;
@@ -442,12 +443,13 @@ enum : int { kStepExit = 0, kStepVirtual = 1, kStepPhoto = 2, kStepCompton = 3 }
 // (x, path) to its collision point, or to the region's exit.  Panel: L is the
 // collision's place, and left_ring tells that the photon left through the
 // panel's back and can meet no other one.
-template <int kRegions, bool kPosed = true>
-__device__ __forceinline__ int woodcock_step(const JobDev &J, const GeomDev &g, const WorkDev &W, const uint4 r, PState &s,
+template <int kRegions, bool kPosed = true, class Geom>
+__device__ __forceinline__ int woodcock_step(const JobDev &J, const Geom &geom, const WorkDev &W, const uint4 r, PState &s,
                                              bool in_panel, Loc &L, bool &left_ring) {
     if (kRegions == 1) in_panel = true;
     if (kRegions == 2) in_panel = false;
     float t_lim = s.trem;
+    const GeomDev &g = fields(geom);
     const float *mu_c = g.mu_c511, *mu_pe = g.mu_pe511;
     int nmat = g.n_materials;
     if (!in_panel) {
@@ -474,15 +476,19 @@ __device__ __forceinline__ int woodcock_step(const JobDev &J, const GeomDev &g, 
     if (out) {
         if (in_panel) {                        // leaves the panel: back to flight
             left_ring = s.x >= g.w_clear && s.dx >= 0.0f;
-            to_global<kPosed>(g, s);
+            to_global<kPosed>(geom, s);
         }
         return kStepExit;
     }
     int m;
     if (in_panel) {
         s.trem -= step;
-        L = locate(g, s.panel, s.x, s.y, s.z);
+        L = locate(geom, s.panel, s.x, s.y, s.z);
         m = L.mat;
+        if (kRegions == 1) {
+            mu_c = tables(geom).mu_c511;
+            mu_pe = tables(geom).mu_pe511;
+        }
     } else {
         int ix = (int)floorf((s.x - J.ph_origin[0]) * J.ph_inv_voxel[0]);
         int iy = (int)floorf((s.y - J.ph_origin[1]) * J.ph_inv_voxel[1]);
@@ -524,8 +530,9 @@ __device__ __forceinline__ int ev_phantom(const JobDev &J, const GeomDev &g, con
 
 // the photon at panel k's box, t_in along its ray, in the panel-local frame
 // (w, u, v)
-template <bool kPosed = true>
-__device__ __forceinline__ void enter_panel(const GeomDev &g, int k, float t_in, PState &s) {
+template <bool kPosed = true, class Geom>
+__device__ __forceinline__ void enter_panel(const Geom &geom, int k, float t_in, PState &s) {
+    const GeomDev &g = fields(geom);
     const float ex = fmaf(t_in, s.dx, s.x), ey = fmaf(t_in, s.dy, s.y), ez = fmaf(t_in, s.dz, s.z);
     s.path += t_in;
     if (kPosed && g.posed) {
@@ -538,7 +545,7 @@ __device__ __forceinline__ void enter_panel(const GeomDev &g, int k, float t_in,
         s.z = fmaf(ex, av.x, fmaf(ey, av.y, fmaf(ez, av.z, -av.w)));
         s.dx = dw; s.dy = du; s.dz = dv;
     } else {
-        const float c = g.pc[k], sn = g.ps[k];
+        const float c = tables(geom).pc[k], sn = tables(geom).ps[k];
         const float w = fmaf(ex, c, ey * sn) - g.R;
         const float u = fmaf(-ex, sn, ey * c);
         const float dw = fmaf(s.dx, c, s.dy * sn), du = fmaf(-s.dx, sn, s.dy * c);

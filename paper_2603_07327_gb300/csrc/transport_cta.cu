@@ -186,9 +186,39 @@ __device__ __noinline__ void keep_hit(const OutDev &O, const JobDev &J, const Ge
 // bounded idle waits, per-job singles buffers).  Separate instantiations, so
 // that a fixed launch without them carries none of their instructions,
 // registers and state words.
-template <int WARPS, int SLOTS, int CTAS, bool kPhantom, bool kPosed, bool kLive>
+// kOne: the launch has one job, which with its geometry comes in the kernel's
+// parameters (CtaTables): what every lane reads alike is then an operand of the
+// instruction that uses it (the random draws' key schedule is the warp's, too),
+// where a launch of several jobs loads it lane by lane.  Tables that lanes index
+// by panel, layer or material stay in shared memory, since lanes that read
+// different constants read them one after the other.  10 M pairs in ring A
+// 1.127 ms without it, 1.080 with; 5 M in the hot-rod phantom 1.64, 1.51; 3 M in
+// the h2r ring 0.783, 0.743; 2e4 in the tiny ring 53 us, 51.
+template <bool kOne>
+struct CtaTables {
+    int ng_smem;   // geometries staged in shared memory
+};
+template <>
+struct CtaTables<true> {
+    JobDev J;
+    GeomDev g;
+};
+__device__ __forceinline__ int staged(const CtaTables<false> &T) { return T.ng_smem; }
+__device__ __forceinline__ int staged(const CtaTables<true> &) { return 1; }
+__device__ __forceinline__ const JobDev &job_of(const CtaTables<false> &, const WorkDev &W, uint32_t j) { return W.jobs[j]; }
+__device__ __forceinline__ const JobDev &job_of(const CtaTables<true> &T, const WorkDev &, uint32_t) { return T.J; }
+__device__ __forceinline__ const GeomDev &geom_of(const CtaTables<false> &T, const GeomDev *sgeom, const WorkDev &W, int i) {
+    return i < T.ng_smem ? sgeom[i] : W.geoms[i];
+}
+__device__ __forceinline__ GeomOne geom_of(const CtaTables<true> &T, const GeomDev *sgeom, const WorkDev &, int) {
+    return GeomOne{T.g, sgeom[0]};
+}
+
+template <int WARPS, int SLOTS, int CTAS, bool kPhantom, bool kPosed, bool kLive, bool kOne>
 __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid_constant__ WorkDev W,
-                                                                   const __grid_constant__ OutDev O, int ng_smem) {
+                                                                   const __grid_constant__ OutDev O,
+                                                                   const __grid_constant__ CtaTables<kOne> T) {
+    const int ng_smem = staged(T);
     static_assert(SLOTS <= 32, "one mask bit per slot");
     using Pool = CtaPool<SLOTS, kPhantom>;
     constexpr int kN = Pool::kN;
@@ -310,8 +340,9 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
             pk = ST(kSpk);
             h = ((uint64_t)ST(kSh1) << 32) | ST(kSh0);
         }
-        const JobDev &J = W.jobs[jobw & 0xFFFFu];
-        const GeomDev &g = J.geom < ng_smem ? sgeom[J.geom] : W.geoms[J.geom];
+        const JobDev &J = job_of(T, W, jobw & 0xFFFFu);
+        decltype(auto) geom = geom_of(T, sgeom, W, J.geom);
+        const GeomDev &g = fields(geom);
         const uint32_t gamma = (pk & kPkGamma) ? 1u : 0u;
         if (ph == kPhFlight || ph == kPhFlightOut) {
             // Flights to the next panel: the first ones of both photons from the
@@ -337,7 +368,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
 #pragma unroll 1
                 for (;;) {
                     float t_in, t_out;
-                    const int k = flight<kPosed>(g, x, y, z, dx, dy, dz, skip, t_in, t_out);
+                    const int k = flight<kPosed>(geom, x, y, z, dx, dy, dz, skip, t_in, t_out);
                     n_fl++;
                     n_scr += k == kFlightScreened ? 1u : 0u;
                     if (k >= 0) {
@@ -424,7 +455,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                     s.trem = __uint_as_float(st[(fresh && gamma ? kSrem1 : kStrem) * kN + q]);
                     if (panel && (pk & (kPkFresh | kPkLastMask))) {
                         const int wi = !fresh ? kSrw : gamma ? kSin1 : kSpath;
-                        enter_panel<kPosed>(g, s.panel, __uint_as_float(st[wi * kN + q]), s);
+                        enter_panel<kPosed>(geom, s.panel, __uint_as_float(st[wi * kN + q]), s);
                         pk &= ~(kPkFresh | kPkLastMask);
                         moved = true;
                     }
@@ -436,9 +467,9 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                     // against 1.71); a live launch, whose code is the longest, takes one for both
                     // (a served burst: 2.89 ms against 3.03)
                     int what;
-                    if (kLive) what = woodcock_step<3, kPosed>(J, g, W, r, s, panel, L, left_ring);
-                    else if (panel) what = woodcock_step<1, kPosed>(J, g, W, r, s, true, L, left_ring);
-                    else what = woodcock_step<2, kPosed>(J, g, W, r, s, false, L, left_ring);
+                    if (kLive) what = woodcock_step<3, kPosed>(J, geom, W, r, s, panel, L, left_ring);
+                    else if (panel) what = woodcock_step<1, kPosed>(J, geom, W, r, s, true, L, left_ring);
+                    else what = woodcock_step<2, kPosed>(J, geom, W, r, s, false, L, left_ring);
                     if (panel) pk += late ? 0u : 1u << kPkStep;
                     else ST(kSph) = sph + 1u;
                     to = ph;
@@ -681,31 +712,33 @@ template <> struct Shape<8> { static constexpr int kPlain = 18, kPhantom = 16, k
 template <> struct Shape<14> { static constexpr int kPlain = 32, kPhantom = 28, kCtas = 2; };
 template <> struct Shape<16> { static constexpr int kPlain = 32, kPhantom = 28, kCtas = 2; };
 
-using CtaKernel = void (*)(WorkDev, OutDev, int);
-
-template <int WARPS>
-static CtaKernel cta_kernel(const LaunchCfg &cfg, size_t *pool) {
+// the kernel that cfg selects, and the size of its pool
+template <int WARPS, bool kOne>
+static const void *cta_kernel(const LaunchCfg &cfg, size_t *pool) {
     using S = Shape<WARPS>;
     *pool = cfg.phantom ? sizeof(CtaPool<S::kPhantom, true>) : sizeof(CtaPool<S::kPlain, false>);
-    if (cfg.live) return k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, true>;
+    if constexpr (!kOne)
+        if (cfg.live) return (const void *)k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, true, false>;
     if (cfg.phantom)
-        return cfg.posed ? k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, false>
-                         : k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, false, false>;
-    return cfg.posed ? k_transport_cta<WARPS, S::kPlain, S::kCtas, false, true, false>
-                     : k_transport_cta<WARPS, S::kPlain, S::kCtas, false, false, false>;
+        return cfg.posed ? (const void *)k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, false, kOne>
+                         : (const void *)k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, false, false, kOne>;
+    return cfg.posed ? (const void *)k_transport_cta<WARPS, S::kPlain, S::kCtas, false, true, false, kOne>
+                     : (const void *)k_transport_cta<WARPS, S::kPlain, S::kCtas, false, false, false, kOne>;
 }
 
-static CtaKernel cta_kernel(const LaunchCfg &cfg, int *threads, size_t *pool) {
+static const void *cta_kernel(const LaunchCfg &cfg, int *threads, size_t *pool) {
     switch (cfg.block_size) {
-        case 128: *threads = 128; return cta_kernel<4>(cfg, pool);
-        case 256: *threads = 256; return cta_kernel<8>(cfg, pool);
-        case 512: *threads = 512; return cta_kernel<16>(cfg, pool);
-        default: *threads = kCtaThreads; return cta_kernel<kCtaThreads / 32>(cfg, pool);
+        case 128: *threads = 128; return cta_kernel<4, false>(cfg, pool);
+        case 256: *threads = 256; return cta_kernel<8, false>(cfg, pool);
+        case 512: *threads = 512; return cta_kernel<16, false>(cfg, pool);
+        default: *threads = kCtaThreads;
     }
+    if (cfg.one_job && !cfg.live) return cta_kernel<kCtaThreads / 32, true>(cfg, pool);
+    return cta_kernel<kCtaThreads / 32, false>(cfg, pool);
 }
 
 // kernel, threads, dynamic shared memory and resident CTAs of the launch that cfg selects
-static cudaError_t cta_shape(int n_geoms, const LaunchCfg &cfg, CtaKernel *k, int *threads, size_t *smem, int *ctas,
+static cudaError_t cta_shape(int n_geoms, const LaunchCfg &cfg, const void **k, int *threads, size_t *smem, int *ctas,
                              int *ng) {
     size_t pool = 0;
     int occ = 0;
@@ -719,7 +752,7 @@ static cudaError_t cta_shape(int n_geoms, const LaunchCfg &cfg, CtaKernel *k, in
 
 // resident warps of the launch that launch_transport_cta makes
 cudaError_t cta_resident_warps(int n_geoms, const LaunchCfg &cfg, long long *warps) {
-    CtaKernel k;
+    const void *k;
     size_t smem = 0;
     int threads = 0, ctas = 0, ng = 0;
     cudaError_t e = cta_shape(n_geoms, cfg, &k, &threads, &smem, &ctas, &ng);
@@ -728,13 +761,21 @@ cudaError_t cta_resident_warps(int n_geoms, const LaunchCfg &cfg, long long *war
 }
 
 cudaError_t launch_transport_cta(const WorkDev &W, const OutDev &O, const LaunchCfg &cfg, cudaStream_t st) {
-    CtaKernel k;
+    const void *k;
     size_t smem = 0;
     int threads = 0, ctas = 0, ng = 0;
     cudaError_t e = cta_shape(W.n_geoms, cfg, &k, &threads, &smem, &ctas, &ng);
     if (e != cudaSuccess) return e;
-    k<<<ctas, threads, smem, st>>>(W, O, ng);
-    return cudaGetLastError();
+    CtaTables<false> many{ng};
+    CtaTables<true> one;
+    void *tables = &many;
+    if (cfg.one_job && !cfg.live && threads == kCtaThreads) {
+        if (ng < 1) return cudaErrorInvalidConfiguration;   // (its pool leaves room for one geometry)
+        one = {*cfg.one_job, *cfg.one_geom};
+        tables = &one;
+    }
+    void *args[] = {const_cast<WorkDev *>(&W), const_cast<OutDev *>(&O), tables};
+    return cudaLaunchKernel(k, dim3(ctas), dim3(threads), args, smem, st);
 }
 
 void cta_counters(unsigned long long *c, const unsigned long long *raw) {
@@ -762,16 +803,17 @@ void cta_counters(unsigned long long *c, const unsigned long long *raw) {
 cudaError_t preload_cta_kernels() {
     LaunchCfg cfg{};
     for (int block : {128, 256, kCtaThreads, 512})
-        for (int form = 0; form < 5; ++form) {
+        for (int form = 0; form < 9; ++form) {
             cfg.block_size = block;
-            cfg.phantom = form >= 2;
-            cfg.posed = form == 1 || form >= 3;
-            cfg.live = form == 4;
+            const JobDev any{};
+            cfg.phantom = form & 1;
+            cfg.posed = form & 2;
+            cfg.one_job = form & 4 ? &any : nullptr;
+            cfg.live = form == 8;
             int threads = 0;
             size_t pool = 0;
-            CtaKernel k = cta_kernel(cfg, &threads, &pool);
-            cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void *>(k),
-                                                pool + (size_t)kMaxStagedGeoms * sizeof(GeomDev));
+            const void *k = cta_kernel(cfg, &threads, &pool);
+            cudaError_t e = ensure_dynamic_smem(k, pool + (size_t)kMaxStagedGeoms * sizeof(GeomDev));
             if (e != cudaSuccess) return e;
         }
     return cudaSuccess;
