@@ -406,6 +406,7 @@ int gpet_delta_sym(int64_t n, const double *s_a, const double *s_b, double *out)
  *              the sort is stable (equal keys keep their input order)
  *   n          <= 1048576 (2^20); larger n returns GPET_ERR_INVALID_ARG
  *   stream     cudaStream_t; the call is asynchronous on it
+ * One cooperative kernel (a block per multiprocessor at most) does the sort.
  * The first call on a device, made with that device current, is its set-up:
  * CUDA loads a library's kernels and device arrays lazily, so that call loads
  * the code it runs and the 24.3 MiB array, which takes device memory then.

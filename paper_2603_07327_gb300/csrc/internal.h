@@ -43,7 +43,6 @@ struct SortDev {
     uint32_t *vals[2];
     uint32_t *ghist;                 // [8][256]
     int *plan;                       // [8] active, [8] source buffer, [1] final buffer
-    uint32_t *tile_words;            // allocation-free sort: look-back words [tiles][256]
     unsigned long long max_tiles;
     unsigned long long cap;
     const unsigned long long *n_in;  // device count of unsorted singles
@@ -195,7 +194,44 @@ constexpr int kCtaCounters = 20, kCtaCounterSlots = 16;
 void cta_counters(unsigned long long *counters, const unsigned long long *raw);
 cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const CoincDev &C, int sm_count,
                               cudaStream_t st);
-cudaError_t launch_noalloc_passes(const SortDev &S, unsigned tiles, cudaStream_t st);
+
+// polls of a look-back word before the pass gives up (with 64 ns sleeps after
+// the first 64 polls: about a second); a tile whose owner never publishes is
+// reported, not waited for forever
+constexpr int kLookbackPolls = 1 << 24;
+
+__device__ __forceinline__ uint32_t lane_lt() {
+    uint32_t m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
+
+// block-wide exclusive scan of one value per thread (blockDim a multiple of 32, at most 1024)
+__device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t &total, uint32_t *sw) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFullMask, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) sw[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        uint32_t w = lane < (int)(blockDim.x >> 5) ? sw[lane] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFullMask, w, o);
+            if (lane >= o) w += y;
+        }
+        sw[lane] = w;  // inclusive warp prefix
+    }
+    __syncthreads();
+    const uint32_t warp_base = wid ? sw[wid - 1] : 0;
+    total = sw[(blockDim.x >> 5) - 1];
+    __syncthreads();
+    return warp_base + x - v;
+}
 
 // Pass plan of a radix sort from the digit histograms S.ghist, by a block of
 // eight warps: which passes run, and which buffer each one reads.

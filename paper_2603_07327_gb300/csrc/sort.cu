@@ -16,8 +16,9 @@
 // same digit (the intersection of bit-plane ballots), in input order.  A pass's
 // input tiles are streamed into shared memory by the bulk-copy engine
 // (cp.async.bulk completing on an mbarrier), one tile ahead of the tile being
-// ranked.  The allocation-free sort has passes of its own (k_noalloc_pass).  The
-// element count is read on the device, so the whole chain is enqueued without a
+// ranked.  (The
+// allocation-free sort is a kernel of its own, sort_noalloc.cu.)  The element
+// count is read on the device, so the whole chain is enqueued without a
 // host round trip.
 #include "internal.h"
 
@@ -28,12 +29,6 @@ constexpr int kSortItems = 16;
 constexpr int kTile = kSortThreads * kSortItems;  // 4096 keys per tile
 constexpr int kPasses = 8;
 static_assert(kSortThreads == 256, "one thread per 8-bit digit in the pass's prefix step");
-
-__device__ __forceinline__ uint32_t lane_lt() {
-    uint32_t m;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-    return m;
-}
 
 __device__ __forceinline__ unsigned long long sort_n(const SortDev &S) {
     const unsigned long long n = *S.n_in;
@@ -71,33 +66,6 @@ __global__ void __launch_bounds__(kSortThreads) k_make_keys(SortDev S) {
 
 // which passes run, and which buffer each one reads (one warp per pass)
 __global__ void __launch_bounds__(kPasses * 32) k_plan(SortDev S) { plan_passes(S, sort_n(S)); }
-
-// block-wide exclusive scan of one value per thread (blockDim a multiple of 32, at most 1024)
-__device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t &total, uint32_t *sw) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFullMask, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) sw[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        uint32_t w = lane < (int)(blockDim.x >> 5) ? sw[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(kFullMask, w, o);
-            if (lane >= o) w += y;
-        }
-        sw[lane] = w;  // inclusive warp prefix
-    }
-    __syncthreads();
-    const uint32_t warp_base = wid ? sw[wid - 1] : 0;
-    total = sw[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return warp_base + x - v;
-}
 
 // Tile of a radix pass in shared memory.  Ranks come in (warp, round, lane) order, which
 // is input order.  The tile is first rebuilt in shared memory in digit order,
@@ -173,11 +141,6 @@ __device__ __forceinline__ void stage_issue(ScatterStage &sg, const uint64_t *ki
 // tiles up to and including it), the count below.  A word is written whole
 // (one aligned 64-bit store), so a reader sees 0 or a complete word.
 constexpr unsigned long long kLbAgg = 1ull << 62, kLbIncl = 2ull << 62, kLbCount = (1ull << 62) - 1ull;
-// polls of a look-back word before the pass gives up (with 64 ns sleeps after
-// the first 64 polls: about a second); a tile whose owner never publishes is
-// reported, not waited for forever
-constexpr int kLookbackPolls = 1 << 24;
-
 __device__ __forceinline__ void lb_store(unsigned long long *p, unsigned long long v) {
     *reinterpret_cast<volatile unsigned long long *>(p) = v;
 }
@@ -749,157 +712,6 @@ __global__ void __launch_bounds__(1024) k_job_stats(SinglesDev s, CoincDev C, Jo
 
 cudaError_t launch_job_stats(const SinglesDev &s, const CoincDev &C, const JobStatsDev &J, cudaStream_t st) {
     k_job_stats<<<J.n_jobs, 1024, 0, st>>>(s, C, J);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// Radix passes of the allocation-free sort (at most 2^20 keys, 256 tiles): one
-// kernel per digit as above, with what so few keys ask for.  A tile is sorted by
-// 512 threads with 8 keys each, since the pass is bound by the latency of its
-// ranking and look-back and not by bandwidth (every tile's CTA is resident at
-// once); look-back words are 32 bits and carry the pass they belong to, so that
-// one buffer in the scratch array serves all passes without being cleared
-// between them, and 16 of them are read per round trip.
-// 300007 keys with 46 varying bits: 12 kernels, where tile histogram, digit scan
-// and scatter as kernels of their own took 29.
-// ---------------------------------------------------------------------------
-constexpr int kPassThreads = 512, kPassItems = kTile / kPassThreads;
-constexpr uint32_t kWordAgg = 1u << 26, kWordIncl = 2u << 26, kWordCount = (1u << 26) - 1u;
-struct PassSmem {
-    uint64_t keys[kTile];
-    uint32_t vals[kTile];
-    uint32_t wh[kPassThreads / 32][256];
-    uint32_t gdelta[256], thist[256], sw[32];
-    uint32_t tile;
-};
-
-__global__ void __launch_bounds__(kPassThreads, 1) k_noalloc_pass(SortDev S, int p) {
-    if (!S.plan[p]) return;
-    extern __shared__ __align__(16) unsigned char pass_raw[];
-    PassSmem &sm = *reinterpret_cast<PassSmem *>(pass_raw);
-    const int src = S.plan[kPasses + p];
-    const uint32_t n = (uint32_t)sort_n(S), tiles = (n + kTile - 1) / kTile;
-    constexpr int kWarps = kPassThreads / 32;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint64_t *kin = src ? S.keys[1] : S.keys[0];
-    const uint32_t *vin = src ? S.vals[1] : S.vals[0];
-    uint64_t *kout = src ? S.keys[0] : S.keys[1];
-    uint32_t *vout = src ? S.vals[0] : S.vals[1];
-    if (threadIdx.x == 0) sm.tile = atomicAdd(S.tile_ctr + p, 1u);
-    for (int i = threadIdx.x; i < kWarps * 256; i += kPassThreads) (&sm.wh[0][0])[i] = 0;
-    if (threadIdx.x < 256) sm.thist[threadIdx.x] = 0;
-    __syncthreads();
-    const uint32_t t = sm.tile;   // tiles in the order of their start
-    if (t >= tiles) return;
-    // the digits' bases: exclusive scan of this pass's global histogram
-    uint32_t tot;
-    const uint32_t dbase = block_exscan(threadIdx.x < 256 ? S.ghist[p * 256 + threadIdx.x] : 0u, tot, sm.sw);
-    const uint32_t wb = t * kTile + (uint32_t)w * (32 * kPassItems) + (uint32_t)lane;
-    uint64_t k[kPassItems];
-    uint32_t v[kPassItems], rank[kPassItems];
-#pragma unroll
-    for (int j = 0; j < kPassItems; ++j) {
-        const uint32_t i = wb + 32 * j;
-        k[j] = i < n ? __ldg(kin + i) : 0ull;
-        v[j] = i < n ? __ldg(vin + i) : 0u;
-    }
-    // the tile's digit counts, published before the ranking
-#pragma unroll
-    for (int j = 0; j < kPassItems; ++j)
-        if (wb + 32 * j < n) atomicAdd(&sm.thist[(uint32_t)((k[j] >> (8 * p)) & 0xFF)], 1u);
-    __syncthreads();
-    const uint32_t tag = (uint32_t)(p + 1) << 28;
-    volatile uint32_t *row = S.tile_words + (size_t)t * 256;
-    const uint32_t cnt = threadIdx.x < 256 ? sm.thist[threadIdx.x] : 0u;
-    if (threadIdx.x < 256) row[threadIdx.x] = tag | (t == 0 ? kWordIncl : kWordAgg) | cnt;
-#pragma unroll
-    for (int j = 0; j < kPassItems; ++j) {
-        const uint32_t d = wb + 32 * j < n ? (uint32_t)((k[j] >> (8 * p)) & 0xFF) : 256u;
-        uint32_t peers = kFullMask;
-#pragma unroll
-        for (int bit = 0; bit < 9; ++bit) {   // (the ninth separates the lanes past the end)
-            const uint32_t m = __ballot_sync(kFullMask, (d >> bit) & 1u);
-            peers &= ((d >> bit) & 1u) ? m : ~m;
-        }
-        const uint32_t before = d < 256u ? sm.wh[w][d] : 0u;
-        rank[j] = before + __popc(peers & lane_lt());
-        __syncwarp();
-        if (d < 256u && (peers & lane_lt()) == 0) sm.wh[w][d] = before + __popc(peers);
-        __syncwarp();
-    }
-    __syncthreads();
-    uint32_t c = 0;
-    if (threadIdx.x < 256) {
-#pragma unroll
-        for (int ww = 0; ww < kWarps; ++ww) {
-            const uint32_t x = sm.wh[ww][threadIdx.x];
-            sm.wh[ww][threadIdx.x] = c;
-            c += x;
-        }
-    }
-    const uint32_t lstart = block_exscan(c, tot, sm.sw);
-    if (threadIdx.x < 256) {
-#pragma unroll
-        for (int ww = 0; ww < kWarps; ++ww) sm.wh[ww][threadIdx.x] += lstart;
-    }
-    __syncthreads();
-    // the tile in digit order in shared memory; its global offsets follow
-#pragma unroll
-    for (int j = 0; j < kPassItems; ++j)
-        if (wb + 32 * j < n) {
-            const uint32_t lp = sm.wh[w][(uint32_t)((k[j] >> (8 * p)) & 0xFF)] + rank[j];
-            sm.keys[lp] = k[j];
-            sm.vals[lp] = v[j];
-        }
-    int fail = 0;
-    if (threadIdx.x < 256) {
-        const uint32_t d = threadIdx.x;
-        uint32_t excl = 0;
-        constexpr int kWin = 16;
-        int polls = 0;
-        for (uint32_t j = t; j > 0 && !fail;) {   // tiles [0, j) not yet added
-            uint32_t wv[kWin];
-            const volatile uint32_t *q0 = S.tile_words + d;
-#pragma unroll
-            for (int q = 0; q < kWin; ++q) wv[q] = (uint32_t)q < j ? q0[(size_t)(j - 1 - q) * 256] : 0u;
-            bool found = false;
-#pragma unroll
-            for (int q = 0; q < kWin; ++q) {
-                if (found || fail || (uint32_t)q >= j) break;
-                uint32_t x = wv[q];
-                while ((x >> 28) != (uint32_t)(p + 1)) {
-                    if (++polls > kLookbackPolls) { fail = 1; break; }
-                    if (polls > 64) __nanosleep(64);
-                    x = q0[(size_t)(j - 1 - q) * 256];
-                }
-                if (fail) break;
-                excl += x & kWordCount;
-                found = (x & kWordIncl) != 0;
-            }
-            j = found ? 0u : (j > (uint32_t)kWin ? j - kWin : 0u);
-        }
-        if (!fail && t > 0) row[d] = tag | kWordIncl | (excl + cnt);
-        sm.gdelta[d] = dbase + excl - lstart;
-    }
-    // (a tile whose look-back gave up writes nothing; the call cannot report it,
-    // and its output is then incomplete)
-    if (__syncthreads_or(fail)) return;
-    const uint32_t tn = min(n - t * kTile, (uint32_t)kTile);
-    for (uint32_t i = threadIdx.x; i < tn; i += kPassThreads) {
-        const uint64_t key = sm.keys[i];
-        const uint32_t pos = sm.gdelta[(uint32_t)((key >> (8 * p)) & 0xFF)] + i;
-        if (pos < n) {
-            kout[pos] = key;
-            vout[pos] = sm.vals[i];
-        }
-    }
-}
-
-// the radix passes over a keyed and planned working set
-cudaError_t launch_noalloc_passes(const SortDev &S, unsigned tiles, cudaStream_t st) {
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void *>(k_noalloc_pass), sizeof(PassSmem));
-    if (e != cudaSuccess) return e;
-    for (int p = 0; p < kPasses; ++p) k_noalloc_pass<<<tiles, kPassThreads, sizeof(PassSmem), st>>>(S, p);
     return cudaGetLastError();
 }
 
