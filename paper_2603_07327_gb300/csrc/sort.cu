@@ -676,42 +676,48 @@ __device__ __forceinline__ unsigned long long warp_lower_bound(unsigned long lon
     return lo;
 }
 
+// (the tallies in slices: one block per job took 11 us for 67 k crystals, eight
+// and a ninth for the segments take 4)
+constexpr int kStatsSlices = 8;
 __global__ void __launch_bounds__(1024) k_job_stats(SinglesDev s, CoincDev C, JobStatsDev J) {
     const int j = blockIdx.x;
-    const unsigned long long ns = *s.n, nc = *C.n;
-    const int wid = threadIdx.x >> 5;
-    if (wid == 0) {   // first coincidence whose first single has job >= j
-        const unsigned long long lo = j == 0 ? 0 : warp_lower_bound(nc, j, [&](unsigned long long i) { return s.job[C.a[i]]; });
-        if (threadIdx.x == 0) J.c_off[j] = lo;
-    } else if (wid == 1) {   // first single with job >= j
-        const unsigned long long lo = j == 0 ? 0
-                                      : J.bjobs ? J.bstart[J.bjobs[j].first]
-                                                : warp_lower_bound(ns, j, [&](unsigned long long i) { return s.job[i]; });
-        if (threadIdx.x == 32) J.s_off[j] = lo;
+    if (blockIdx.y == kStatsSlices) {
+        const unsigned long long ns = *s.n, nc = *C.n;
+        const int wid = threadIdx.x >> 5;
+        if (wid == 0) {   // first coincidence whose first single has job >= j
+            const unsigned long long lo = j == 0 ? 0 : warp_lower_bound(nc, j, [&](unsigned long long i) { return s.job[C.a[i]]; });
+            if (threadIdx.x == 0) J.c_off[j] = lo;
+        } else if (wid == 1) {   // first single with job >= j
+            const unsigned long long lo = j == 0 ? 0
+                                          : J.bjobs ? J.bstart[J.bjobs[j].first]
+                                                    : warp_lower_bound(ns, j, [&](unsigned long long i) { return s.job[i]; });
+            if (threadIdx.x == 32) J.s_off[j] = lo;
+        }
+        if (threadIdx.x == 0 && j == J.n_jobs - 1) {
+            J.s_off[J.n_jobs] = ns;
+            J.c_off[J.n_jobs] = nc;
+        }
+        return;
     }
-    if (threadIdx.x == 0 && j == J.n_jobs - 1) {
-        J.s_off[J.n_jobs] = ns;
-        J.c_off[J.n_jobs] = nc;
-    }
-    // hits of job j = sum of its per-crystal counts
+    // hits of job j = sum of its per-crystal counts (hits is cleared before a run)
     unsigned long long acc = 0;
     const unsigned long long *t = J.tally_count + J.tally_off[j];
     const long long nt = J.tally_n[j];
-#pragma unroll 16
-    for (long long i = threadIdx.x; i < nt; i += 1024) acc += t[i];
+#pragma unroll 8
+    for (long long i = (long long)blockIdx.y * 1024 + threadIdx.x; i < nt; i += 1024 * kStatsSlices) acc += t[i];
     __shared__ unsigned long long red[32];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFullMask, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long tot = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-        J.hits[j] = tot;
+    if (threadIdx.x < 32) {
+        acc = red[threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFullMask, acc, o);
+        if (threadIdx.x == 0 && acc) atomicAdd(J.hits + j, acc);
     }
 }
 
 cudaError_t launch_job_stats(const SinglesDev &s, const CoincDev &C, const JobStatsDev &J, cudaStream_t st) {
-    k_job_stats<<<J.n_jobs, 1024, 0, st>>>(s, C, J);
+    k_job_stats<<<dim3(J.n_jobs, kStatsSlices + 1), 1024, 0, st>>>(s, C, J);
     return cudaGetLastError();
 }
 
