@@ -935,6 +935,7 @@ static int copy_run(const gpet_result *r, int32_t which, void *dst, size_t cap_b
 // device, where these stores kept the link's rate.
 __global__ void k_store_to_host(const uint4 *__restrict__ src, uint4 *dst, size_t n16,
                                 const uint32_t *__restrict__ src4, uint32_t *dst4, unsigned n4) {
+    after_previous();
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x)
         dst[i] = __ldcs(src + i);
     if (blockIdx.x == 0 && threadIdx.x < n4) dst4[threadIdx.x] = src4[threadIdx.x];
@@ -969,10 +970,9 @@ static cudaError_t store_to_host(void *dst_dev, const void *src, size_t bytes, c
     const unsigned n4 = (unsigned)((bytes - 16 * n16) / 4);
     const size_t want = (n16 + 511) / 512;
     const int grid = (int)std::max<size_t>(1, std::min<size_t>(want, (size_t)sms * 4));
-    k_store_to_host<<<grid, 512, 0, st>>>(static_cast<const uint4 *>(src), static_cast<uint4 *>(dst_dev), n16,
-                                          reinterpret_cast<const uint32_t *>(static_cast<const char *>(src) + 16 * n16),
-                                          reinterpret_cast<uint32_t *>(static_cast<char *>(dst_dev) + 16 * n16), n4);
-    return cudaGetLastError();
+    return launch_next(k_store_to_host, grid, 512, 0, st, static_cast<const uint4 *>(src), static_cast<uint4 *>(dst_dev), n16,
+                       reinterpret_cast<const uint32_t *>(static_cast<const char *>(src) + 16 * n16),
+                       reinterpret_cast<uint32_t *>(static_cast<char *>(dst_dev) + 16 * n16), n4);
 }
 
 extern "C" int gpet_result_copy_run(const gpet_result *r, int32_t which, void *dst, size_t cap_bytes,

@@ -30,6 +30,7 @@ constexpr int kWinLocalJobs = 32;          // jobs a block counts in shared memo
 
 __global__ void __launch_bounds__(kWinThreads) k_coinc_windows(SinglesDev s, const uint64_t *__restrict__ window_ps,
                                                                WinDev win, unsigned long long *counts) {
+    after_previous();
     __shared__ unsigned int cnt[kWinLocalJobs * kMaxWindows];
     const unsigned long long n = *s.n;
     const unsigned long long first = (unsigned long long)blockIdx.x * kWinTile;
@@ -85,8 +86,7 @@ __global__ void __launch_bounds__(kWinThreads) k_coinc_windows(SinglesDev s, con
 cudaError_t launch_coinc_windows(const SinglesDev &s, const CoincDev &C, const WinDev &win,
                                  unsigned long long *counts, unsigned long long cap, cudaStream_t st) {
     const unsigned long long blocks = (cap + kWinTile - 1) / kWinTile;
-    k_coinc_windows<<<(unsigned int)(blocks ? blocks : 1), kWinThreads, 0, st>>>(s, C.window_ps, win, counts);
-    return cudaGetLastError();
+    return launch_next(k_coinc_windows, (unsigned int)(blocks ? blocks : 1), kWinThreads, 0, st, s, C.window_ps, win, counts);
 }
 
 // load the window-count kernel (internal.h)

@@ -39,6 +39,7 @@ __device__ __forceinline__ unsigned long long sort_n(const SortDev &S) {
 // keys (smem, then global atomics).  The keys themselves were written by the
 // transport's finish event, next to each single's record.
 __global__ void __launch_bounds__(kSortThreads) k_make_keys(SortDev S) {
+    after_previous();
     __shared__ uint32_t h[kPasses][256];
     for (int i = threadIdx.x; i < kPasses * 256; i += blockDim.x) (&h[0][0])[i] = 0;
     __syncthreads();
@@ -65,7 +66,7 @@ __global__ void __launch_bounds__(kSortThreads) k_make_keys(SortDev S) {
 }
 
 // which passes run, and which buffer each one reads (one warp per pass)
-__global__ void __launch_bounds__(kPasses * 32) k_plan(SortDev S) { plan_passes(S, sort_n(S)); }
+__global__ void __launch_bounds__(kPasses * 32) k_plan(SortDev S) { after_previous(); plan_passes(S, sort_n(S)); }
 
 // Tile of a radix pass in shared memory.  Ranks come in (warp, round, lane) order, which
 // is input order.  The tile is first rebuilt in shared memory in digit order,
@@ -157,6 +158,7 @@ __device__ __forceinline__ unsigned long long lb_load(const unsigned long long *
 // waits end.  Tiles are staged into shared memory one ahead by the bulk-copy
 // engine.
 __global__ void __launch_bounds__(kSortThreads, 2) k_onesweep(SortDev S, int p) {
+    after_previous();
     if (!S.plan[p]) return;
     extern __shared__ __align__(16) unsigned char scatter_raw[];
     ScatterSmem &sm = *reinterpret_cast<ScatterSmem *>(scatter_raw);
@@ -384,6 +386,7 @@ __device__ __forceinline__ uint32_t bucket_of(const SortDev &S, uint64_t key) {
 }
 
 __global__ void __launch_bounds__(256) k_bucket_count(SortDev S) {
+    after_previous();
     const unsigned long long n = sort_n(S), step = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long i0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * step) {
         uint32_t r[4];
@@ -433,6 +436,7 @@ __device__ __forceinline__ bool warp_lookback(unsigned long long *words, uint32_
 // bucket counts to first positions, in place (n_buckets + 1 of them): one pass,
 // tiles in the order of a ticket, each tile's base by looking back
 __global__ void __launch_bounds__(1024) k_bucket_scan(SortDev S) {
+    after_previous();
     __shared__ uint32_t sw[32];
     __shared__ uint32_t tile_sh, base_sh;
     __shared__ int fail_sh;
@@ -471,6 +475,7 @@ __global__ void __launch_bounds__(1024) k_bucket_scan(SortDev S) {
 
 // each single's index to its bucket's next place, in order of arrival
 __global__ void __launch_bounds__(256) k_bucket_place(SortDev S) {
+    after_previous();
     const unsigned long long n = sort_n(S);
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
@@ -508,6 +513,7 @@ __device__ __forceinline__ uint32_t bucket_edge(const SortDev &S, unsigned long 
 }
 
 __global__ void __launch_bounds__(256) k_bucket_sort(SortDev S, SinglesDev out) {
+    after_previous();
     __shared__ uint64_t key[kBucketRoom];
     __shared__ uint32_t idx[kBucketRoom];
     __shared__ uint32_t edge[2];
@@ -563,6 +569,7 @@ __global__ void __launch_bounds__(256) k_bucket_sort(SortDev S, SinglesDev out) 
 
 // singles into time order, after the radix passes
 __global__ void k_gather(SortDev S, SinglesDev out) {
+    after_previous();
     const unsigned long long n = sort_n(S);
     const int fin = S.plan[2 * kPasses];
     const uint32_t *perm = fin ? S.vals[1] : S.vals[0];
@@ -588,6 +595,7 @@ constexpr int kCoincThreads = 256, kCoincPer = 4, kCoincTile = kCoincThreads * k
 static_assert(kCoincTile == (int)kCoincScanTile, "look-back words are allocated per tile");
 
 __global__ void __launch_bounds__(kCoincThreads) k_coinc(SinglesDev s, CoincDev C, int *status) {
+    after_previous();
     __shared__ uint64_t st[kCoincTile + 2];   // times and jobs of the tile, one single more at either end
     __shared__ int32_t sj[kCoincTile + 2];
     __shared__ uint32_t flag[kCoincTile / 32];
@@ -680,6 +688,7 @@ __device__ __forceinline__ unsigned long long warp_lower_bound(unsigned long lon
 // and a ninth for the segments take 4)
 constexpr int kStatsSlices = 8;
 __global__ void __launch_bounds__(1024) k_job_stats(SinglesDev s, CoincDev C, JobStatsDev J) {
+    after_previous();
     const int j = blockIdx.x;
     if (blockIdx.y == kStatsSlices) {
         const unsigned long long ns = *s.n, nc = *C.n;
@@ -717,8 +726,7 @@ __global__ void __launch_bounds__(1024) k_job_stats(SinglesDev s, CoincDev C, Jo
 }
 
 cudaError_t launch_job_stats(const SinglesDev &s, const CoincDev &C, const JobStatsDev &J, cudaStream_t st) {
-    k_job_stats<<<dim3(J.n_jobs, kStatsSlices + 1), 1024, 0, st>>>(s, C, J);
-    return cudaGetLastError();
+    return launch_next(k_job_stats, dim3(J.n_jobs, kStatsSlices + 1), 1024, 0, st, s, C, J);
 }
 
 cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const CoincDev &C, int sm_count,
@@ -731,28 +739,27 @@ cudaError_t launch_sort_coinc(const SortDev &S, const SinglesDev &out, const Coi
     if (S.n_buckets) {
         const unsigned long long want = (S.cap + kBucketCta - 1) / kBucketCta;
         const int bg = (int)(want < (unsigned long long)sm_count * 8 ? want : (unsigned long long)sm_count * 8);
-        k_bucket_count<<<bg, 256, 0, st>>>(S);
-        k_bucket_scan<<<(S.n_buckets + kBucketScanTile) / kBucketScanTile, 1024, 0, st>>>(S);
-        k_bucket_place<<<bg, 256, 0, st>>>(S);
-        k_bucket_sort<<<bg, 256, 0, st>>>(S, out);
+        e = launch_next(k_bucket_count, bg, 256, 0, st, S);
+        if (e == cudaSuccess) e = launch_next(k_bucket_scan, (S.n_buckets + kBucketScanTile) / kBucketScanTile, 1024, 0, st, S);
+        if (e == cudaSuccess) e = launch_next(k_bucket_place, bg, 256, 0, st, S);
+        if (e == cudaSuccess) e = launch_next(k_bucket_sort, bg, 256, 0, st, S, out);
     } else {
         e = cudaMemsetAsync(S.ghist, 0, sizeof(uint32_t) * kPasses * 256, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(S.tile_ctr, 0, sizeof(unsigned int) * kPasses, st);
         if (e != cudaSuccess) return e;
-        k_make_keys<<<sm_count * 4, kSortThreads, 0, st>>>(S);
-        k_plan<<<1, kPasses * 32, 0, st>>>(S);
+        e = launch_next(k_make_keys, sm_count * 4, kSortThreads, 0, st, S);
+        if (e == cudaSuccess) e = launch_next(k_plan, 1, kPasses * 32, 0, st, S);
         // two CTAs per SM are resident; more would only claim tiles later
         const int tg = (int)(S.max_tiles < (unsigned long long)sm_count * 2 ? (S.max_tiles ? S.max_tiles : 1)
                                                                             : (unsigned long long)sm_count * 2);
-        for (int p = 0; p < kPasses; ++p) k_onesweep<<<tg, kSortThreads, kScatterSmemStaged, st>>>(S, p);
-        k_gather<<<grid, 256, 0, st>>>(S, out);
+        for (int p = 0; p < kPasses && e == cudaSuccess; ++p)
+            e = launch_next(k_onesweep, tg, kSortThreads, kScatterSmemStaged, st, S, p);
+        if (e == cudaSuccess) e = launch_next(k_gather, grid, 256, 0, st, S, out);
     }
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const unsigned long long ct = (S.cap + kCoincTile - 1) / kCoincTile;
     const int cg = (int)(ct < (unsigned long long)sm_count * 8 ? ct : (unsigned long long)sm_count * 8);
-    k_coinc<<<cg, kCoincThreads, 0, st>>>(out, C, S.status);
-    return cudaGetLastError();
+    return launch_next(k_coinc, cg, kCoincThreads, 0, st, out, C, S.status);
 }
 
 // load the digitizer's kernels and set their shared-memory limits (internal.h)

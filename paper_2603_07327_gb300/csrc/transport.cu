@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(256) k_transport_loop(WorkDev W, OutDev O, int
 // local memory.  Tallies and hits were already counted by the main kernel, so
 // only the singles are emitted here.
 __global__ void __launch_bounds__(128) k_transport_redo(WorkDev W, OutDev O) {
+    after_previous();
     constexpr int S = 64;
     uint32_t l_unit[S];
     float l_e[S];
@@ -179,8 +180,7 @@ cudaError_t transport_resident_warps(int n_geoms, const LaunchCfg &cfg, long lon
 }
 
 cudaError_t launch_transport_redo(const WorkDev &W, const OutDev &O, const LaunchCfg &cfg, cudaStream_t st) {
-    k_transport_redo<<<cfg.sm_count, 128, 0, st>>>(W, O);
-    return cudaGetLastError();
+    return launch_next(k_transport_redo, cfg.sm_count, 128, 0, st, W, O);
 }
 
 cudaError_t launch_transport(const WorkDev &W, const OutDev &O, const LaunchCfg &cfg, cudaStream_t st,
