@@ -490,18 +490,21 @@ __global__ void __launch_bounds__(256) k_bucket_place(SortDev S) {
 constexpr int kBucketCta = 512;
 constexpr int kBucketRoom = kBucketCta + (int)kBucketMax;
 
-// a single's record from the transport to place i of the time-ordered arrays
-__device__ __forceinline__ void gather_one(const RawSingle *src, const SinglesDev &out, unsigned long long i) {
-    const uint4 *r = reinterpret_cast<const uint4 *>(src);
-    const uint4 a = __ldg(r), b = __ldg(r + 1), c = __ldg(r + 2);
-    out.t[i] = ((uint64_t)a.y << 32) | a.x;
-    out.h[i] = ((uint64_t)a.w << 32) | a.z;
-    out.unit[i] = (int32_t)b.x;
-    out.panel[i] = (int32_t)b.y;
-    out.job[i] = (int32_t)b.z;
-    out.e[i] = __uint_as_float(b.w);
-    out.eraw[i] = __uint_as_float(c.x);
-    out.doi[i] = __uint_as_float(c.y);
+// a single, its sort key and its record from the transport, to place i of the
+// time-ordered arrays
+__device__ __forceinline__ void gather_one(const SortDev &S, uint64_t key, uint32_t slot, const SinglesDev &out,
+                                           unsigned long long i) {
+    const uint4 *r = reinterpret_cast<const uint4 *>(S.in_raw + slot);
+    const uint4 a = __ldg(r), b = __ldg(r + 1);
+    const bool jobs = S.job_shift < 64;
+    out.t[i] = jobs ? key & ((1ull << S.job_shift) - 1ull) : key;
+    out.job[i] = jobs ? (int32_t)(key >> S.job_shift) : 0;
+    out.h[i] = ((uint64_t)a.y << 32) | a.x;
+    out.unit[i] = (int32_t)a.z;
+    out.panel[i] = (int32_t)a.w;
+    out.e[i] = __uint_as_float(b.x);
+    out.eraw[i] = __uint_as_float(b.y);
+    out.doi[i] = __uint_as_float(b.z);
 }
 
 // first place at or after x where a bucket starts
@@ -561,7 +564,7 @@ __global__ void __launch_bounds__(256) k_bucket_sort(SortDev S, SinglesDev out) 
             }
 #pragma unroll
             for (int q = 0; q < 2; ++q)
-                if (i0 + 256 * q < m) gather_one(S.in_raw + v[q], out, p0 + lo[q]);
+                if (i0 + 256 * q < m) gather_one(S, k[q], v[q], out, p0 + lo[q]);
         }
         __syncthreads();
     }
@@ -573,9 +576,10 @@ __global__ void k_gather(SortDev S, SinglesDev out) {
     const unsigned long long n = sort_n(S);
     const int fin = S.plan[2 * kPasses];
     const uint32_t *perm = fin ? S.vals[1] : S.vals[0];
+    const uint64_t *key = fin ? S.keys[1] : S.keys[0];
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
-        gather_one(S.in_raw + perm[i], out, i);
+        gather_one(S, key[i], perm[i], out, i);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) *out.n = n;
 }

@@ -713,16 +713,14 @@ __device__ __forceinline__ void blur_single(const JobDev &J, const uint4 q, floa
 }
 
 // a kept single's record
-__device__ __forceinline__ void write_single(const GeomDev &g, RawSingle *dst, int job, uint64_t h, uint64_t t,
-                                             const SingleOut &o) {
+__device__ __forceinline__ void write_single(const GeomDev &g, RawSingle *dst, uint64_t h, const SingleOut &o) {
     // units per panel: 1, its modules, or its crystals
     const uint32_t per = g.readout_level == 0 ? 1u : (uint32_t)(g.modules_u * g.modules_v) *
                                                          (g.readout_level == 1 ? 1u : (uint32_t)g.crystals_per_module);
     const int panel = (int)(o.unit / per);
     uint4 *r = reinterpret_cast<uint4 *>(dst);
-    r[0] = make_uint4((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)h, (uint32_t)(h >> 32));
-    r[1] = make_uint4(o.unit, (uint32_t)panel, (uint32_t)job, __float_as_uint(o.eb));
-    r[2] = make_uint4(__float_as_uint(o.e), __float_as_uint(o.db), 0u, 0u);
+    r[0] = make_uint4((uint32_t)h, (uint32_t)(h >> 32), o.unit, (uint32_t)panel);
+    r[1] = make_uint4(__float_as_uint(o.eb), __float_as_uint(o.e), __float_as_uint(o.db), 0u);
 }
 
 // a kept single at slot `slot` of the launch's buffer: record and sort key
@@ -730,7 +728,7 @@ __device__ __forceinline__ void store_single(const GeomDev *__restrict__ geoms, 
                                              uint64_t h, uint64_t t, const SingleOut &o, unsigned long long slot) {
     if (slot >= O.s_cap) return;
     O.s_keys[slot] = O.key_shift < 64 ? ((uint64_t)job << O.key_shift) | t : t;
-    write_single(geoms[J.geom], O.s_raw + slot, job, h, t, o);
+    write_single(geoms[J.geom], O.s_raw + slot, h, o);
 }
 
 // Append the kept singles of a warp (call with the lanes of `mask` converged):
@@ -776,7 +774,7 @@ __device__ __forceinline__ void append_single(const GeomDev *__restrict__ geoms,
     if (kJobDest && J.s_raw) {
         // a job with its own buffer is job 0 of the one-job run that buffer belongs to
         J.s_keys[slot] = t;
-        write_single(geoms[J.geom], dst + slot, 0, h, t, o);
+        write_single(geoms[J.geom], dst + slot, h, o);
     } else {
         store_single(geoms, O, J, job, h, t, o, slot);
     }
