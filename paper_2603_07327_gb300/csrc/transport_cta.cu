@@ -726,6 +726,11 @@ static const void *cta_kernel(const LaunchCfg &cfg, size_t *pool) {
                      : (const void *)k_transport_cta<WARPS, S::kPlain, S::kCtas, false, false, false, kOne>;
 }
 
+// A launch of one job in the default shape takes its tables as parameters: the
+// kernel and its arguments are both chosen by this.
+static bool takes_one(const LaunchCfg &cfg) { return cfg.one_job && !cfg.live && cfg.block_size == kCtaThreads; }
+static_assert(kCtaThreads != 128 && kCtaThreads != 256 && kCtaThreads != 512, "the other shapes take the job table");
+
 static const void *cta_kernel(const LaunchCfg &cfg, int *threads, size_t *pool) {
     switch (cfg.block_size) {
         case 128: *threads = 128; return cta_kernel<4, false>(cfg, pool);
@@ -733,7 +738,7 @@ static const void *cta_kernel(const LaunchCfg &cfg, int *threads, size_t *pool) 
         case 512: *threads = 512; return cta_kernel<16, false>(cfg, pool);
         default: *threads = kCtaThreads;
     }
-    if (cfg.one_job && !cfg.live) return cta_kernel<kCtaThreads / 32, true>(cfg, pool);
+    if (takes_one(cfg)) return cta_kernel<kCtaThreads / 32, true>(cfg, pool);
     return cta_kernel<kCtaThreads / 32, false>(cfg, pool);
 }
 
@@ -769,7 +774,7 @@ cudaError_t launch_transport_cta(const WorkDev &W, const OutDev &O, const Launch
     CtaTables<false> many{ng};
     CtaTables<true> one;
     void *tables = &many;
-    if (cfg.one_job && !cfg.live && threads == kCtaThreads) {
+    if (takes_one(cfg)) {
         if (ng < 1) return cudaErrorInvalidConfiguration;   // (its pool leaves room for one geometry)
         one = {*cfg.one_job, *cfg.one_geom};
         tables = &one;
