@@ -65,7 +65,7 @@ struct SortDev {
 
 // singles per time bucket at one single per history, most singles of one
 // bucket, and the narrowest bucket (ps): see sort.cu
-constexpr uint32_t kBucketHistories = 32, kBucketMax = 1024;
+constexpr uint32_t kBucketHistories = 16, kBucketMax = 1024;
 constexpr uint64_t kBucketMinPs = 10000;
 constexpr uint32_t kBucketScanTile = 4096, kCoincScanTile = 1024;
 
