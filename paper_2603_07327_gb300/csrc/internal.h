@@ -281,6 +281,67 @@ __device__ __forceinline__ void plan_passes(const SortDev &S, unsigned long long
     }
 }
 
+// A tile of time-ordered singles in shared memory for cluster-by-cluster work: one
+// single more at either end, whether each is linked to the one before it (same
+// job, gap within the window; one bit more than the tile has singles), and the
+// singles where a cluster of several begins, packed for the block's threads.
+// Most singles are alone, and a thread per single waits for its warp's clusters:
+// with a thread per cluster, 5.6 M singles take 79 us for coincidences (104) and
+// 106 us for the counts of four energy windows (149).
+template <int kThreads, int kTile>
+struct ClusterTile {
+    uint64_t t[kTile + 2];
+    int32_t job[kTile + 2];
+    uint32_t link[kTile / 32 + 1];
+    uint16_t start[kTile];
+    uint32_t n_start;
+
+    __device__ __forceinline__ uint64_t time(const SinglesDev &s, uint32_t lo, uint32_t i) const {
+        return i + 1u - lo < (uint32_t)(kTile + 2) ? t[i + 1u - lo] : s.t[i];
+    }
+    __device__ __forceinline__ bool linked(const SinglesDev &s, const uint64_t *window_ps, uint32_t lo, uint32_t n,
+                                           uint32_t i) const {
+        const uint32_t l = i - lo;
+        if (l <= (uint32_t)kTile) return (link[l >> 5] >> (l & 31u)) & 1u;
+        return i > 0u && i < n && s.job[i - 1u] == s.job[i] && s.t[i] - s.t[i - 1u] <= window_ps[s.job[i]];
+    }
+    // tile lo.. of n singles (all of the block's threads)
+    __device__ __forceinline__ void load(const SinglesDev &s, const uint64_t *window_ps, uint32_t lo, uint32_t n) {
+        if (threadIdx.x == 0) n_start = 0;
+        for (int k = threadIdx.x; k < kTile + 2; k += kThreads) {
+            const uint32_t i = lo + k - 1u;   // (wraps below 0: not < n)
+            t[k] = i < n ? s.t[i] : 0ull;
+            job[k] = i < n ? s.job[i] : -1;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int l0 = 0; l0 <= kTile; l0 += kThreads) {
+            const int l = l0 + threadIdx.x;
+            bool on = false;
+            if (l <= kTile) {
+                const int j = job[l + 1];
+                on = j >= 0 && j == job[l] && t[l + 1] - t[l] <= __ldg(window_ps + j);
+            }
+            const uint32_t w = __ballot_sync(kFullMask, on);
+            if ((threadIdx.x & 31) == 0 && l <= kTile) link[l >> 5] = w;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int l0 = 0; l0 < kTile; l0 += kThreads) {
+            const int l = l0 + threadIdx.x;
+            const uint32_t w = link[l >> 5], next = (l & 31) == 31 ? link[(l >> 5) + 1] & 1u : (w >> ((l & 31) + 1)) & 1u;
+            const bool begins = next && !((w >> (l & 31)) & 1u);
+            const uint32_t m = __ballot_sync(kFullMask, begins);
+            if (m == 0) continue;
+            uint32_t at = 0;
+            if ((threadIdx.x & 31) == 0) at = atomicAdd(&n_start, (uint32_t)__popc(m));
+            at = __shfl_sync(kFullMask, at, 0);
+            if (begins) start[at + __popc(m & lane_lt())] = (uint16_t)l;
+        }
+        __syncthreads();
+    }
+};
+
 // energy windows of one pass over the time-sorted singles
 constexpr int kMaxWindows = 16;
 struct WinDev {

@@ -32,46 +32,51 @@ __global__ void __launch_bounds__(kWinThreads) k_coinc_windows(SinglesDev s, con
                                                                WinDev win, unsigned long long *counts) {
     after_previous();
     __shared__ unsigned int cnt[kWinLocalJobs * kMaxWindows];
-    const unsigned long long n = *s.n;
-    const unsigned long long first = (unsigned long long)blockIdx.x * kWinTile;
-    if (first >= n) return;
-    const unsigned long long last = (first + kWinTile < n ? first + kWinTile : n) - 1;
+    __shared__ ClusterTile<kWinThreads, kWinTile> tl;
+    const uint32_t n = (uint32_t)*s.n;
+    if ((unsigned long long)blockIdx.x * kWinTile >= n) return;
+    const uint32_t first = blockIdx.x * kWinTile, last = min(n - first, (uint32_t)kWinTile) + first - 1u;
     const int nw = win.n;
     // singles are ordered by job: the block's jobs are [j0, j1]
     const int j0 = s.job[first], j1 = s.job[last];
     const bool local = j1 - j0 < kWinLocalJobs;
     for (int i = threadIdx.x; i < kWinLocalJobs * nw; i += kWinThreads) cnt[i] = 0u;
-    __syncthreads();
-    for (unsigned long long i = first + threadIdx.x; i <= last; i += kWinThreads) {
-        const int ji = s.job[i];
-        const uint64_t ti = s.t[i];
-        const uint64_t W = window_ps[ji];
-        if (!(i == 0 || s.job[i - 1] != ji || ti - s.t[i - 1] > W)) continue;
-        // end of this cluster of the widest window
-        unsigned long long e = i;
-        while (e + 1 < n && s.job[e + 1] == ji && s.t[e + 1] - s.t[e] <= W) ++e;
-        for (int w = 0; w < nw; ++w) {
-            const float lo = win.lo[w], hi = win.hi[w];
-            unsigned int c = 0;
-            unsigned long long k = i;
-            while (k <= e && !(s.e[k] >= lo && s.e[k] <= hi)) ++k;
-            while (k <= e) {
-                const unsigned long long a = k;
-                const uint64_t ta = s.t[a];
-                unsigned long long second = a;
-                int in_window = 1;
-                for (k = a + 1; k <= e && s.t[k] - ta <= W; ++k) {
-                    if (s.e[k] >= lo && s.e[k] <= hi) {
-                        if (++in_window == 2) second = k;
-                    }
-                }
-                if (in_window == 2 && s.panel[a] != s.panel[second]) ++c;
-                while (k <= e && !(s.e[k] >= lo && s.e[k] <= hi)) ++k;
+    tl.load(s, window_ps, first, n);
+    // a thread per window and cluster of several singles (of the widest window):
+    // most singles are alone, and their threads used to wait for the others
+    for (uint32_t q = threadIdx.x; q < tl.n_start * nw; q += kWinThreads) {
+        const uint32_t at = q / nw;
+        const int w = (int)(q - at * nw);
+        const uint32_t i = first + tl.start[at];
+        const int ji = tl.job[tl.start[at] + 1];
+        const uint64_t W = __ldg(window_ps + ji);
+        const float lo = win.lo[w], hi = win.hi[w];
+        auto linked = [&](uint32_t k) { return tl.linked(s, window_ps, first, n, k); };
+        auto kept = [&](uint32_t k) { const float e = s.e[k]; return e >= lo && e <= hi; };
+        unsigned int c = 0;
+        uint32_t k = i;
+        for (bool more = true; more;) {
+            // the first single of the window's own at or after k
+            while (!kept(k) && more) {
+                more = linked(k + 1u);
+                if (more) ++k;
             }
-            if (c) {
-                if (local) atomicAdd(&cnt[(ji - j0) * nw + w], c);
-                else atomicAdd(counts + (unsigned long long)ji * nw + w, (unsigned long long)c);
+            if (!more) break;
+            const uint32_t a = k;
+            const uint64_t ta = tl.time(s, first, a);
+            uint32_t second = a;
+            int in_window = 1;
+            for (;;) {
+                more = linked(k + 1u);
+                if (more) ++k;
+                if (!more || tl.time(s, first, k) - ta > W) break;
+                if (kept(k) && ++in_window == 2) second = k;
             }
+            if (in_window == 2 && s.panel[a] != s.panel[second]) ++c;
+        }
+        if (c) {
+            if (local) atomicAdd(&cnt[(ji - j0) * nw + w], c);
+            else atomicAdd(counts + (unsigned long long)ji * nw + w, (unsigned long long)c);
         }
     }
     if (!local) return;

@@ -603,48 +603,35 @@ static_assert(kCoincTile == (int)kCoincScanTile, "look-back words are allocated 
 
 __global__ void __launch_bounds__(kCoincThreads) k_coinc(SinglesDev s, CoincDev C, int *status) {
     after_previous();
-    __shared__ uint64_t st[kCoincTile + 2];   // times and jobs of the tile, one single more at either end
-    __shared__ int32_t sj[kCoincTile + 2];
+    __shared__ ClusterTile<kCoincThreads, kCoincTile> tl;
     __shared__ uint32_t flag[kCoincTile / 32];
     __shared__ uint32_t sw[32], tile_sh, base_sh;
     __shared__ int fail_sh;
-    const unsigned long long n = *s.n, tiles = (n + kCoincTile - 1) / kCoincTile;
+    const uint32_t n = (uint32_t)*s.n, tiles = (n + kCoincTile - 1) / kCoincTile;
     for (;;) {
         if (threadIdx.x == 0) tile_sh = (uint32_t)atomicAdd(C.scan, 1ull);
         if (threadIdx.x < kCoincTile / 32) flag[threadIdx.x] = 0;
         __syncthreads();
         const uint32_t tile = tile_sh;
         if (tile >= tiles) break;
-        const unsigned long long lo = (unsigned long long)tile * kCoincTile;
-        const unsigned long long hi = lo + kCoincTile < n ? lo + kCoincTile : n;
-        for (int k = threadIdx.x; k < kCoincTile + 2; k += kCoincThreads) {
-            const unsigned long long i = lo + k - 1;   // (wraps below 0: not < n)
-            st[k] = i < n ? s.t[i] : 0ull;
-            sj[k] = i < n ? s.job[i] : -1;
-        }
-        __syncthreads();
-        auto T = [&](unsigned long long i) { return i + 1 - lo < kCoincTile + 2 ? st[i + 1 - lo] : s.t[i]; };
-        auto JOB = [&](unsigned long long i) { return i + 1 - lo < kCoincTile + 2 ? sj[i + 1 - lo] : s.job[i]; };
-#pragma unroll 1
-        for (int q = 0; q < kCoincPer; ++q) {
-            const unsigned long long i = lo + q * kCoincThreads + threadIdx.x;
-            if (i >= hi) break;
-            const int ji = JOB(i);
-            const uint64_t W = C.window_ps[ji];
-            unsigned long long a = i;
-            if (i > 0 && JOB(i - 1) == ji && T(i) - T(i - 1) <= W) {
-                if (i != lo) continue;   // inside a cluster
-                do --a; while (a > 0 && JOB(a - 1) == ji && T(a) - T(a - 1) <= W);
-            }
+        const uint32_t lo = tile * kCoincTile, hi = min(lo + kCoincTile, n);
+        tl.load(s, C.window_ps, lo, n);
+        auto linked = [&](uint32_t i) { return tl.linked(s, C.window_ps, lo, n, i); };
+        // the clusters that begin in the tile, and the one that reaches into it
+        const uint32_t before = linked(lo) ? 1u : 0u;
+        for (uint32_t c = threadIdx.x; c < tl.n_start + before; c += kCoincThreads) {
+            uint32_t a = lo;
+            if (c < tl.n_start) a += tl.start[c];
+            else do --a; while (linked(a));
+            const uint64_t W = __ldg(C.window_ps + (a + 1u - lo < kCoincTile + 2u ? tl.job[a + 1u - lo] : s.job[a]));
             while (a < hi) {
-                unsigned long long b = a;
-                const uint64_t ta = T(a);
-                while (b + 1 < n && JOB(b + 1) == ji && T(b + 1) - ta <= W) ++b;
-                if (b == a + 1 && a >= lo && s.panel[a] != s.panel[b])
+                uint32_t b = a;
+                const uint64_t ta = tl.time(s, lo, a);
+                while (linked(b + 1u) && tl.time(s, lo, b + 1u) - ta <= W) ++b;
+                if (b == a + 1u && a >= lo && s.panel[a] != s.panel[b])
                     atomicOr(&flag[(a - lo) >> 5], 1u << ((a - lo) & 31));
-                // the cluster ends where the next gap exceeds the window
-                if (b + 1 >= n || JOB(b + 1) != ji || T(b + 1) - T(b) > W) break;
-                a = b + 1;
+                if (!linked(b + 1u)) break;   // the cluster's end
+                a = b + 1u;
             }
         }
         __syncthreads();
