@@ -84,7 +84,11 @@ static_assert(kMaxSteps < 1024 && kMaxPanels < 127 && kMaxTrials <= 1024 && kEnt
 // event counters: slots 0..7 count the events of each phase (decays in 0,
 // lanes fed in 1); lane i of a warp keeps counter i
 enum : int { kNLanes = 1, kNScrStart = 8, kNScrFlight, kNEntered, kNHits, kNTrials, kNSingles, kNFin, kNIter, kNCount };
-constexpr int kSticky = 22;    // lanes with a slot in a warp's last phase for which it stays with that phase
+// Lanes with a slot in a warp's last phase for which it stays with that phase.  Where
+// the code is longer than the instruction cache likes, fewer lanes are the better
+// price: 5 M pairs in the hot-rod phantom with 10, 14, 18, 22, 26 of them 1.477,
+// 1.479, 1.499, 1.533, 1.582 ms; 10 M in ring A 1.107, 1.071, 1.052, 1.045, 1.056.
+constexpr int sticky_lanes(bool phantom) { return phantom ? 14 : 22; }
 constexpr uint32_t kMaxSpins = 1u << 24;  // waits for a slot (over a second) before a warp gives up
 constexpr unsigned kFlushEvery = 1u << 20;  // events; below 2^32 counts in as many of any kind
 
@@ -254,7 +258,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
         // else the one with the most lanes (ties to the later one, so that
         // histories end before others begin)
         uint32_t m = *reinterpret_cast<volatile uint32_t *>(&mask[ph][lane]);
-        if ((ph == kPhIdle && (done || (kLive && waiting))) || __popc(__ballot_sync(kFullMask, m != 0)) < kSticky) {
+        if ((ph == kPhIdle && (done || (kLive && waiting))) || __popc(__ballot_sync(kFullMask, m != 0)) < sticky_lanes(kPhantom)) {
             uint32_t best = 0;
             alone = true;
 #pragma unroll
