@@ -118,19 +118,19 @@ class Clocks:
 # Entries are named by capture id (the summary of each capture under that id
 # gives its command).
 TRANSPORT_SOURCES = ("device.cuh", "transport.cuh", "transport.cu", "transport_cta.cu")
-TRANSPORT_CAPTURE = dict(id="k_transport_cta_sweep_122x1e7", sha1="f4a6704d15a30fafa6a2dd16570072434011662a",
-                         warp_inst_per_pair=143.306, dram_bytes_per_pair=9.798)
+TRANSPORT_CAPTURE = dict(id="k_transport_cta_sweep_122x1e7", sha1="5b074788c7289f1438ef1aa864d6673a07cc68c8",
+                         warp_inst_per_pair=89.854, dram_bytes_per_pair=7.012)
 # Issue detail of the same kernel from one ncu --set full capture of a
 # 2e6-pair sweep position: issue-active fraction of the schedulers and SIMT
 # efficiency (thread instructions per warp instruction / 32).
-TRANSPORT_DETAIL = dict(id="k_transport_cta_sweep_position_2e6", sha1="f4a6704d15a30fafa6a2dd16570072434011662a",
-                        issue_active=0.494, simt_efficiency=0.583)
+TRANSPORT_DETAIL = dict(id="k_transport_cta_sweep_position_2e6", sha1="5b074788c7289f1438ef1aa864d6673a07cc68c8",
+                        issue_active=0.723, simt_efficiency=0.667)
 # algorithmic bytes of the digitizer back end per single (the model in run_ours)
-DIGITIZER_BYTES_PER_SINGLE = 330
-# DRAM bytes of the digitizer back end (make_keys .. job_stats of one step), per single.
-DIGITIZER_SOURCES = ("device.cuh", "sort.cu")
-DIGITIZER_TRAFFIC = dict(id="traffic_digitizer_sweep_8x1e7", sha1="6fd97e665d63322ce912e6a20bee0aebc691fc9c",
-                         bytes_per_single=361.6)
+DIGITIZER_BYTES_PER_SINGLE = 130
+# DRAM bytes of the digitizer back end (bucket_count .. job_stats of one step), per single.
+DIGITIZER_SOURCES = ("device.cuh", "internal.h", "sort.cu")
+DIGITIZER_TRAFFIC = dict(id="traffic_digitizer_sweep_8x1e7", sha1="4103ded240543c12805a6a4c209ef3edf3b724c4",
+                         bytes_per_single=239.4)
 
 
 def _current(entry, sources):
@@ -586,10 +586,10 @@ def run_ours(args):
             roof["event_isolated"] = dict(error=f"{type(exc).__name__}: {exc}")
 
     # digitizer back end (time sort + coincidences), HBM-bound: algorithmic bytes
-    # per single = key pass 12 (the key the transport wrote read, the index
-    # written) + 8 one-sweep radix passes x 25 (key and index read 12 and
-    # written 12, look-back words 1) + gather 84 (index 4, 8 fields read 40 +
-    # written 40) + coincidence pass 34 = 330
+    # per single = bucket counts 12 (key read, rank written) + places 20 (key and
+    # rank read, start of the bucket read, index written) + order and gather 84
+    # (index 4, key 8, record 32 read, 40 written) + coincidences 14 (time and job
+    # read, a seventh of a pair written) = 130
     singles_step = sum(c["singles"] for c in counts) / args.steps
     dig_bytes = DIGITIZER_BYTES_PER_SINGLE * singles_step
     dig_gbs = dig_bytes / (dg_ms / args.steps / 1000.0) / 1e9 if dg_ms > 0 else None
@@ -697,9 +697,9 @@ def run_ours(args):
                 per_step_counts=dict(hits=sum(c["hits"] for c in counts) // args.steps,
                                      singles=sum(c["singles"] for c in counts) // args.steps,
                                      coincidences=sum(c["coincidences"] for c in counts) // args.steps))
-    # kernels per launch: transport + redo, key pass, plan, 8 one-sweep radix passes, gather,
-    # 4 coincidence kernels, job statistics
-    per_launch = 2 + 2 + 8 + 1 + 4 + 1
+    # kernels per launch: transport + redo, time buckets (count, scan, place, order and gather),
+    # coincidences, job statistics
+    per_launch = 2 + 4 + 1 + 1
     line["gpu_launches"] = per_launch * args.steps * (1 if args.form == "batched" else len(jobs))
     if args.form == "batched" and args.compare_plain:
         # the plain per-position form on the same sweep, for the batched-vs-plain metric

@@ -395,7 +395,7 @@ int gpet_delta_sym(int64_t n, const double *s_a, const double *s_b, double *out)
  * up front by another allocator (for example a caching allocator that has
  * reserved the pool, or a server with a fixed memory budget), or a
  * latency-critical loop that cannot take an allocation's implicit device
- * synchronisation.  It runs the digitizer's radix time sort on n 64-bit keys
+ * synchronisation.  It sorts n 64-bit keys
  * (the singles' time stamps in ps) with its whole working set in a fixed
  * 24.3 MiB array that is part of the library image, held on every GPU that
  * loads the library until the process exits; it calls no cudaMalloc, no

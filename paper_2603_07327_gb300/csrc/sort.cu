@@ -16,10 +16,9 @@
 // same digit (the intersection of bit-plane ballots), in input order.  A pass's
 // input tiles are streamed into shared memory by the bulk-copy engine
 // (cp.async.bulk completing on an mbarrier), one tile ahead of the tile being
-// ranked.  (The
-// allocation-free sort is a kernel of its own, sort_noalloc.cu.)  The element
-// count is read on the device, so the whole chain is enqueued without a
-// host round trip.
+// ranked.  (The allocation-free sort is a kernel of its own, sort_noalloc.cu.)
+// The element count is read on the device, so the whole chain is enqueued
+// without a host round trip.
 #include "internal.h"
 
 namespace gpet {

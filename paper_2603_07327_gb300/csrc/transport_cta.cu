@@ -18,7 +18,7 @@
 //     event of its own with its lanes packed, and a rejected trial waits for the
 //     next one.  The finish event digitizes one single per lane, where a loop
 //     over a history's singles waits for the warp's longest list.
-//   - The code of all events together is small (45 KB, the hot part less), since
+//   - The code of all events together is small (46 KB, the hot part less), since
 //     the warps of an SM are in different phases at once: one flight routine with
 //     one slab-test loop for every kind of flight, one Philox draw and one sine
 //     and cosine for all events that need them, cold paths out of line.  At 74 KB
@@ -40,7 +40,7 @@
 //
 // Measured on a GB300, transport of one sweep position of 1e7 pairs: 2.52 ms
 // with the phase chosen per CTA behind a barrier and per-warp pools, 1.28 ms
-// here.
+// with this scheme alone, 1.04 ms with what the comments below add.
 #include "internal.h"
 #include "transport.cuh"
 
@@ -706,7 +706,8 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
 // The launch shapes: 448 threads by default, or 128, 256 or 512
 // (gpet_options.block_size); slots of a lane class without and with the
 // phantom's state words, and CTAs an SM.  Measured on a sweep position (1e7
-// pairs, transport ms) and on the hot-rod phantom (5e6 pairs): 12 warps 1.31 and
+// pairs, transport ms) and on the hot-rod phantom (5e6 pairs) when the scheme was
+// new, and again at 1.04 ms with the same order (15 warps 1.09): 12 warps 1.31 and
 // 1.97, 14 warps 1.28 and 1.89, 15 warps 1.27 and 1.88 (two CTAs an SM each);
 // 8 warps 1.66 (two CTAs) and 1.57 (three); 20 warps (one CTA) 1.68.
 template <int WARPS>
