@@ -190,38 +190,48 @@ __device__ __noinline__ void keep_hit(const OutDev &O, const JobDev &J, const Ge
 // bounded idle waits, per-job singles buffers).  Separate instantiations, so
 // that a fixed launch without them carries none of their instructions,
 // registers and state words.
-// kOne: the launch has one job, which with its geometry comes in the kernel's
-// parameters (CtaTables): what every lane reads alike is then an operand of the
-// instruction that uses it (the random draws' key schedule is the warp's, too),
-// where a launch of several jobs loads it lane by lane.  Tables that lanes index
-// by panel, layer or material stay in shared memory, since lanes that read
-// different constants read them one after the other.  10 M pairs in ring A
-// 1.127 ms without it, 1.080 with; 5 M in the hot-rod phantom 1.64, 1.51; 3 M in
-// the h2r ring 0.783, 0.743; 2e4 in the tiny ring 53 us, 51.
-template <bool kOne>
+// kTab: where an event finds its job and geometry.
+// - kTabOne: the launch has one job, which with its geometry comes in the kernel's
+//   parameters: what every lane reads alike is then an operand of the instruction
+//   that uses it (the random draws' key schedule is the warp's, too), where a
+//   launch of several jobs loads it lane by lane.  Tables that lanes index by
+//   panel, layer or material stay in shared memory, since lanes that read
+//   different constants read them one after the other.  10 M pairs in ring A
+//   1.127 ms without it, 1.080 with; 5 M in the hot-rod phantom 1.64, 1.51; 3 M in
+//   the h2r ring 0.783, 0.743; 2e4 in the tiny ring 53 us, 51.
+// - kTabStaged: several jobs, and all of the launch's geometries are staged in
+//   shared memory: read there, where the general form reads through a pointer to
+//   either memory.  60 M pairs in two rings 6.25 ms without it, 6.03 with; a map of
+//   6.4 M pairs in two rings 2.04, 1.98.  (The jobs staged as well: 6.13.)
+// - kTabJobs: any launch.
+enum : int { kTabJobs = 0, kTabOne = 1, kTabStaged = 2 };
+template <int kTab>
 struct CtaTables {
     int ng_smem;   // geometries staged in shared memory
 };
 template <>
-struct CtaTables<true> {
+struct CtaTables<kTabOne> {
     JobDev J;
     GeomDev g;
 };
-__device__ __forceinline__ int staged(const CtaTables<false> &T) { return T.ng_smem; }
-__device__ __forceinline__ int staged(const CtaTables<true> &) { return 1; }
-__device__ __forceinline__ const JobDev &job_of(const CtaTables<false> &, const WorkDev &W, uint32_t j) { return W.jobs[j]; }
-__device__ __forceinline__ const JobDev &job_of(const CtaTables<true> &T, const WorkDev &, uint32_t) { return T.J; }
-__device__ __forceinline__ const GeomDev &geom_of(const CtaTables<false> &T, const GeomDev *sgeom, const WorkDev &W, int i) {
-    return i < T.ng_smem ? sgeom[i] : W.geoms[i];
+template <int kTab>
+__device__ __forceinline__ int staged(const CtaTables<kTab> &T) { return T.ng_smem; }
+__device__ __forceinline__ int staged(const CtaTables<kTabOne> &) { return 1; }
+template <int kTab>
+__device__ __forceinline__ const JobDev &job_of(const CtaTables<kTab> &, const WorkDev &W, uint32_t j) { return W.jobs[j]; }
+__device__ __forceinline__ const JobDev &job_of(const CtaTables<kTabOne> &T, const WorkDev &, uint32_t) { return T.J; }
+template <int kTab>
+__device__ __forceinline__ const GeomDev &geom_of(const CtaTables<kTab> &T, const GeomDev *sgeom, const WorkDev &W, int i) {
+    return kTab == kTabStaged || i < T.ng_smem ? sgeom[i] : W.geoms[i];
 }
-__device__ __forceinline__ GeomOne geom_of(const CtaTables<true> &T, const GeomDev *sgeom, const WorkDev &, int) {
+__device__ __forceinline__ GeomOne geom_of(const CtaTables<kTabOne> &T, const GeomDev *sgeom, const WorkDev &, int) {
     return GeomOne{T.g, sgeom[0]};
 }
 
-template <int WARPS, int SLOTS, int CTAS, bool kPhantom, bool kPosed, bool kLive, bool kOne>
+template <int WARPS, int SLOTS, int CTAS, bool kPhantom, bool kPosed, bool kLive, int kTab>
 __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid_constant__ WorkDev W,
                                                                    const __grid_constant__ OutDev O,
-                                                                   const __grid_constant__ CtaTables<kOne> T) {
+                                                                   const __grid_constant__ CtaTables<kTab> T) {
     const int ng_smem = staged(T);
     static_assert(SLOTS <= 32, "one mask bit per slot");
     using Pool = CtaPool<SLOTS, kPhantom>;
@@ -717,75 +727,78 @@ template <> struct Shape<8> { static constexpr int kPlain = 18, kPhantom = 16, k
 template <> struct Shape<14> { static constexpr int kPlain = 32, kPhantom = 28, kCtas = 2; };
 template <> struct Shape<16> { static constexpr int kPlain = 32, kPhantom = 28, kCtas = 2; };
 
-// the kernel that cfg selects, and the size of its pool
-template <int WARPS, bool kOne>
+// the kernel that cfg and kTab select, and the size of its pool
+template <int WARPS, int kTab>
 static const void *cta_kernel(const LaunchCfg &cfg, size_t *pool) {
     using S = Shape<WARPS>;
     *pool = cfg.phantom ? sizeof(CtaPool<S::kPhantom, true>) : sizeof(CtaPool<S::kPlain, false>);
-    if constexpr (!kOne)
-        if (cfg.live) return (const void *)k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, true, false>;
+    if constexpr (kTab == kTabJobs)
+        if (cfg.live) return (const void *)k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, true, kTab>;
     if (cfg.phantom)
-        return cfg.posed ? (const void *)k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, false, kOne>
-                         : (const void *)k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, false, false, kOne>;
-    return cfg.posed ? (const void *)k_transport_cta<WARPS, S::kPlain, S::kCtas, false, true, false, kOne>
-                     : (const void *)k_transport_cta<WARPS, S::kPlain, S::kCtas, false, false, false, kOne>;
+        return cfg.posed ? (const void *)k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, true, false, kTab>
+                         : (const void *)k_transport_cta<WARPS, S::kPhantom, S::kCtas, true, false, false, kTab>;
+    return cfg.posed ? (const void *)k_transport_cta<WARPS, S::kPlain, S::kCtas, false, true, false, kTab>
+                     : (const void *)k_transport_cta<WARPS, S::kPlain, S::kCtas, false, false, false, kTab>;
 }
 
-// A launch of one job in the default shape takes its tables as parameters: the
-// kernel and its arguments are both chosen by this.
-static bool takes_one(const LaunchCfg &cfg) { return cfg.one_job && !cfg.live && cfg.block_size == kCtaThreads; }
+// (the other shapes and live launches have the general form alone)
+static bool has_tab(const LaunchCfg &cfg) { return !cfg.live && cfg.block_size == kCtaThreads; }
 static_assert(kCtaThreads != 128 && kCtaThreads != 256 && kCtaThreads != 512, "the other shapes take the job table");
 
-static const void *cta_kernel(const LaunchCfg &cfg, int *threads, size_t *pool) {
+static const void *cta_kernel(const LaunchCfg &cfg, int tab, int *threads, size_t *pool) {
     switch (cfg.block_size) {
-        case 128: *threads = 128; return cta_kernel<4, false>(cfg, pool);
-        case 256: *threads = 256; return cta_kernel<8, false>(cfg, pool);
-        case 512: *threads = 512; return cta_kernel<16, false>(cfg, pool);
+        case 128: *threads = 128; return cta_kernel<4, kTabJobs>(cfg, pool);
+        case 256: *threads = 256; return cta_kernel<8, kTabJobs>(cfg, pool);
+        case 512: *threads = 512; return cta_kernel<16, kTabJobs>(cfg, pool);
         default: *threads = kCtaThreads;
     }
-    if (takes_one(cfg)) return cta_kernel<kCtaThreads / 32, true>(cfg, pool);
-    return cta_kernel<kCtaThreads / 32, false>(cfg, pool);
+    constexpr int kW = kCtaThreads / 32;
+    return tab == kTabOne ? cta_kernel<kW, kTabOne>(cfg, pool) : tab == kTabStaged ? cta_kernel<kW, kTabStaged>(cfg, pool)
+                                                                                  : cta_kernel<kW, kTabJobs>(cfg, pool);
 }
 
-// kernel, threads, dynamic shared memory and resident CTAs of the launch that cfg selects
-static cudaError_t cta_shape(int n_geoms, const LaunchCfg &cfg, const void **k, int *threads, size_t *smem, int *ctas,
-                             int *ng) {
-    size_t pool = 0;
+// A launch's kernel, its form of the tables, threads, dynamic shared memory,
+// CTAs and staged geometries
+struct CtaLaunch {
+    const void *k;
+    int tab, threads, ctas, ng;
+    size_t smem;
+};
+static cudaError_t cta_shape(int n_geoms, const LaunchCfg &cfg, CtaLaunch &L) {
+    L.tab = !has_tab(cfg) ? kTabJobs : cfg.one_job ? kTabOne : kTabStaged;
     int occ = 0;
-    *k = cta_kernel(cfg, threads, &pool);
-    cudaError_t e = staged_geometry(*k, *threads, pool, n_geoms, cfg.max_smem_geoms, ng, smem, &occ);
-    if (e != cudaSuccess) return e;
+    for (;; L.tab = kTabJobs) {
+        size_t pool = 0;
+        L.k = cta_kernel(cfg, L.tab, &L.threads, &pool);
+        cudaError_t e = staged_geometry(L.k, L.threads, pool, n_geoms, cfg.max_smem_geoms, &L.ng, &L.smem, &occ);
+        if (e != cudaSuccess) return e;
+        // (all geometries fit beside the pool, one of them always does)
+        if (L.tab == kTabJobs || (L.ng >= n_geoms && occ >= 1)) break;
+    }
     if (occ < 1) return cudaErrorInvalidConfiguration;
-    *ctas = cfg.sm_count * occ;
+    L.ctas = cfg.sm_count * occ;
     return cudaSuccess;
 }
 
 // resident warps of the launch that launch_transport_cta makes
 cudaError_t cta_resident_warps(int n_geoms, const LaunchCfg &cfg, long long *warps) {
-    const void *k;
-    size_t smem = 0;
-    int threads = 0, ctas = 0, ng = 0;
-    cudaError_t e = cta_shape(n_geoms, cfg, &k, &threads, &smem, &ctas, &ng);
-    *warps = (long long)ctas * (threads / 32);
+    CtaLaunch L{};
+    cudaError_t e = cta_shape(n_geoms, cfg, L);
+    *warps = (long long)L.ctas * (L.threads / 32);
     return e;
 }
 
 cudaError_t launch_transport_cta(const WorkDev &W, const OutDev &O, const LaunchCfg &cfg, cudaStream_t st) {
-    const void *k;
-    size_t smem = 0;
-    int threads = 0, ctas = 0, ng = 0;
-    cudaError_t e = cta_shape(W.n_geoms, cfg, &k, &threads, &smem, &ctas, &ng);
+    CtaLaunch L{};
+    cudaError_t e = cta_shape(W.n_geoms, cfg, L);
     if (e != cudaSuccess) return e;
-    CtaTables<false> many{ng};
-    CtaTables<true> one;
-    void *tables = &many;
-    if (takes_one(cfg)) {
-        if (ng < 1) return cudaErrorInvalidConfiguration;   // (its pool leaves room for one geometry)
-        one = {*cfg.one_job, *cfg.one_geom};
-        tables = &one;
-    }
+    CtaTables<kTabJobs> many{L.ng};
+    CtaTables<kTabStaged> all{L.ng};
+    CtaTables<kTabOne> one;
+    if (L.tab == kTabOne) one = {*cfg.one_job, *cfg.one_geom};
+    void *tables = L.tab == kTabOne ? (void *)&one : L.tab == kTabStaged ? (void *)&all : (void *)&many;
     void *args[] = {const_cast<WorkDev *>(&W), const_cast<OutDev *>(&O), tables};
-    return cudaLaunchKernel(k, dim3(ctas), dim3(threads), args, smem, st);
+    return cudaLaunchKernel(L.k, dim3(L.ctas), dim3(L.threads), args, L.smem, st);
 }
 
 void cta_counters(unsigned long long *c, const unsigned long long *raw) {
@@ -811,20 +824,20 @@ void cta_counters(unsigned long long *c, const unsigned long long *raw) {
 
 // load every instantiation and set its shared-memory limit (internal.h)
 cudaError_t preload_cta_kernels() {
-    LaunchCfg cfg{};
     for (int block : {128, 256, kCtaThreads, 512})
-        for (int form = 0; form < 9; ++form) {
+        for (int form = 0; form < 5; ++form) {
+            LaunchCfg cfg{};
             cfg.block_size = block;
-            const JobDev any{};
             cfg.phantom = form & 1;
             cfg.posed = form & 2;
-            cfg.one_job = form & 4 ? &any : nullptr;
-            cfg.live = form == 8;
-            int threads = 0;
-            size_t pool = 0;
-            const void *k = cta_kernel(cfg, &threads, &pool);
-            cudaError_t e = ensure_dynamic_smem(k, pool + (size_t)kMaxStagedGeoms * sizeof(GeomDev));
-            if (e != cudaSuccess) return e;
+            cfg.live = form == 4;
+            for (int tab = 0; tab < (has_tab(cfg) ? 3 : 1); ++tab) {
+                int threads = 0;
+                size_t pool = 0;
+                const void *k = cta_kernel(cfg, tab, &threads, &pool);
+                cudaError_t e = ensure_dynamic_smem(k, pool + (size_t)kMaxStagedGeoms * sizeof(GeomDev));
+                if (e != cudaSuccess) return e;
+            }
         }
     return cudaSuccess;
 }
