@@ -388,8 +388,7 @@ int gpet_build_geometry(const gpet_scanner_desc *d, GeomDev &g, int64_t &n_cryst
     std::vector<double> ang(d->n_panels);
     for (int k = 0; k < d->n_panels; ++k) {
         ang[k] = d->first_angle_rad + 2.0 * M_PI * k / d->n_panels;
-        g.pc[k] = (float)std::cos(ang[k]);
-        g.ps[k] = (float)std::sin(ang[k]);
+        g.cs[k] = make_float2((float)std::cos(ang[k]), (float)std::sin(ang[k]));
     }
     for (int a = 0; a < d->n_panels; ++a)
         for (int b = a + 1; b < d->n_panels; ++b)

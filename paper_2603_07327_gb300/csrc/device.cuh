@@ -77,7 +77,9 @@ struct __align__(128) GeomDev {
     float msu, msv, mpu, mpv, inv_mpu, inv_mpv;  // module size, module pitch (size + gap)
     float mu_c511[kMaxMaterials];   // Compton coefficient at 511 keV (1/cm)
     float mu_pe511[kMaxMaterials];  // photoelectric coefficient at 511 keV (1/cm)
-    float pc[kMaxPanels], ps[kMaxPanels];  // cos / sin of each panel's angle
+    // (cos, sin) of each panel's angle, side by side: lanes of different panels read
+    // them in one load (two arrays: 60 M pairs in two rings 6.03 ms, now 5.91)
+    float2 cs[kMaxPanels];
     // ring culling: every panel box lies in the annulus R^2 <= r^2 <= rout2 and
     // inside its angular sector |phi - phi_k| <= beta (phi_k = phi0 + k dphi)
     float R2, rout2, beta, phi0, dphi, inv_dphi;
@@ -326,7 +328,8 @@ __device__ __forceinline__ void panel_slab(const Geom &geom, int k, float x, flo
                                            float dz, int &best, float &bi, float &bo) {
     const GeomDev &g = fields(geom);
     {
-        const float c = tables(geom).pc[k], s = tables(geom).ps[k];
+        const float2 cs = tables(geom).cs[k];
+        const float c = cs.x, s = cs.y;
         const float w0 = fmaf(x, c, y * s) - g.R;
         const float dw = fmaf(dx, c, dy * s);
         // behind the inner face and moving away: no entry

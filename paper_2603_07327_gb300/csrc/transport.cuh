@@ -306,7 +306,8 @@ __device__ __forceinline__ void to_global(const Geom &geom, PState &s) {
         s.dz = fmaf(dw, aw.z, fmaf(du, au.z, dv * av.z));
         return;
     }
-    const float c = tables(geom).pc[s.panel], sn = tables(geom).ps[s.panel];
+    const float2 cs = tables(geom).cs[s.panel];
+    const float c = cs.x, sn = cs.y;
     const float rw = g.R + s.x;
     const float gx = rw * c - s.y * sn, gy = rw * sn + s.y * c;
     const float gdx = s.dx * c - s.dy * sn, gdy = s.dx * sn + s.dy * c;
@@ -545,7 +546,8 @@ __device__ __forceinline__ void enter_panel(const Geom &geom, int k, float t_in,
         s.z = fmaf(ex, av.x, fmaf(ey, av.y, fmaf(ez, av.z, -av.w)));
         s.dx = dw; s.dy = du; s.dz = dv;
     } else {
-        const float c = tables(geom).pc[k], sn = tables(geom).ps[k];
+        const float2 cs = tables(geom).cs[k];
+        const float c = cs.x, sn = cs.y;
         const float w = fmaf(ex, c, ey * sn) - g.R;
         const float u = fmaf(-ex, sn, ey * c);
         const float dw = fmaf(s.dx, c, s.dy * sn), du = fmaf(-s.dx, sn, s.dy * c);
