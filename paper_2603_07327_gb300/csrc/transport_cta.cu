@@ -40,7 +40,7 @@
 //
 // Measured on a GB300, transport of one sweep position of 1e7 pairs: 2.52 ms
 // with the phase chosen per CTA behind a barrier and per-warp pools, 1.28 ms
-// with this scheme alone, 1.04 ms with what the comments below add.
+// with this scheme alone, 1.03 ms with what the comments below add.
 #include "internal.h"
 #include "transport.cuh"
 
