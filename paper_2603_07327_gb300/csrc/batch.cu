@@ -48,7 +48,7 @@ int gpet_batch_build_run(Run &R, int32_t n_jobs, gpet_scanner *const *scanners, 
     }
     R.caps.singles = first_singles_guess(total);
     R.caps.hits = R.keep_hits ? std::max<uint64_t>(65536, total * 5 / 2) : 0;
-    R.caps.ovf = std::max<uint64_t>(4096, total / 256);
+    R.caps.ovf = overflow_room(total);
     return GPET_OK;
 }
 

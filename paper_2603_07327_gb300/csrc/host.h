@@ -2,6 +2,7 @@
 // the run machinery shared by the plain, batched and served entry points.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <functional>
 #include <memory>
@@ -200,5 +201,9 @@ void fill_counts(const Run &R, int job, uint64_t n_decays, int64_t n_crystals, g
 // whole with its exact count, so a guess that a wide ring's module-level
 // readout exceeds (0.62 per decay) costs such a run half of its time.
 uint64_t first_singles_guess(uint64_t n_decays);
+// Histories a run's overflow list first holds (12 bytes each): a launch's first
+// histories start in all slots at once, and 3 % of 1e6 pairs overflow in a long LYSO
+// ring of 2.6 hits per pair, 0.6 % of 1.5e7.  A run with more is repeated whole.
+inline uint64_t overflow_room(uint64_t n_decays) { return std::max<uint64_t>(4096, n_decays / 16); }
 int run_with_retry(Run &R);            // plan + enqueue + collect, one exact-size re-run on overflow
 }

@@ -848,7 +848,7 @@ extern "C" int gpet_simulate(gpet_scanner *sc, const gpet_source *src, const gpe
     R.windows = {(uint64_t)std::llround(dg->coinc_window_ns * 1000.0)};
     R.caps.singles = first_singles_guess(J.n_hist);
     R.caps.hits = R.keep_hits ? std::max<uint64_t>(65536, J.n_hist * 5 / 2) : 0;
-    R.caps.ovf = std::max<uint64_t>(4096, J.n_hist / 256);
+    R.caps.ovf = overflow_room(J.n_hist);
     st = run_with_retry(R);
     if (st != GPET_OK) {
         delete res;

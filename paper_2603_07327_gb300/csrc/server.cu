@@ -183,7 +183,7 @@ int run_whole(gpet_server *S, Pipe &P, Req *r, std::shared_ptr<Run> &out) {
     R->job_crystals = {r->sc->n_crystals};
     R->windows = {r->window_ps};
     R->caps.singles = std::max<uint64_t>(65536, (uint64_t)(r->n * kGuessPerDecay));
-    R->caps.ovf = std::max<uint64_t>(4096, r->n / 256);
+    R->caps.ovf = overflow_room(r->n);
     st = run_with_retry(*R);
     if (st != GPET_OK) return st;
     charge(S, *R, R->arena_bytes);
@@ -248,7 +248,8 @@ std::unique_ptr<Launch> open_launch(gpet_server *S, Pipe &P, const JobDev &J, co
     R.windows = {window_ps};
     R.caps.singles = S->launch_singles;
     R.caps.guess = false;
-    R.caps.ovf = std::max<uint64_t>(4096, S->launch_singles / 64);
+    // (the share of a plain run's list while that is small beside the arena, whose bytes admission counts without it)
+    R.caps.ovf = std::max<uint64_t>(std::min<uint64_t>(overflow_room(S->launch_singles), 1u << 18), S->launch_singles / 64);
     st = run_plan(R);
     if (st == GPET_OK) st = run_enqueue_transport(R);
     if (st != GPET_OK) return nullptr;

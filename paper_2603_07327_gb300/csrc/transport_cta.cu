@@ -31,10 +31,11 @@
 //     can be, ends without a flight event.
 //   - A history's singles are a chain of entries that the slots of a lane class
 //     share, so a list has no length of its own to overflow: only a class without
-//     a free entry leaves a history to the redo kernel.  With lists of six, that
-//     kernel's few serial histories took 30 us of every launch of 1e6 pairs and
-//     more (1e6 pairs in the 12-panel ring 207 us, now 175; 2e6 in four heads 235,
-//     now 213; 24 designs in one launch 1.44 ms, now 1.38).
+//     a free entry leaves a history to the redo kernel, which simulates it again,
+//     and has a slot less from then on.  Nothing waits for an entry.  With lists of
+//     six, that kernel's few serial histories took 30 us of every launch of 1e6
+//     pairs and more (1e6 pairs in the 12-panel ring 207 us, now 175; 2e6 in four
+//     heads 235, now 213; 24 designs in one launch 1.44 ms, now 1.38).
 // Photons of a pair run one after the other, and events are those of
 // transport.cuh, so the histories equal the other kernels' bit for bit.
 //
@@ -51,7 +52,9 @@ namespace {
 // one more phase here than in transport.cuh: a collision to be sampled
 constexpr uint32_t kPhInteract = 7;
 constexpr int kPhCount = 8;
+constexpr uint32_t kPhGivenUp = kPhSource;  // (the decay is the idle phase's event here)
 constexpr int kEntries = 48;  // singles entries of a lane class, for all of its slots
+constexpr int kKeptSlots = 8;  // slots of a lane class that are never given up
 
 // state words of a slot; the last four only where a job has a phantom
 enum : int { kSh0 = 0, kSh1,
@@ -125,6 +128,17 @@ __device__ __forceinline__ uint32_t take_entry(uint32_t (*efree)[32], int lane) 
         }
     }
     return (uint32_t)kEntries;
+}
+
+// frees a history's whole list, whose first entry + 1 is in jobw (out of line: rarely run,
+// and its code in the collision's place made 10 M pairs in ring A 1.061 ms, not 1.028)
+__device__ __noinline__ uint32_t free_list(uint32_t (*efree)[32], const uint8_t *e_next, int lane, uint32_t jobw) {
+    for (uint32_t next = (jobw >> kJobList) & 63u; next;) {
+        const uint32_t e = next - 1u;
+        next = e_next[next_at(e, lane)];
+        free_entry(efree, lane, e);
+    }
+    return jobw & ~(63u << kJobList);
 }
 
 // Photon of packed word pk is done: the slot's next phase.  Photon 0 hands
@@ -273,7 +287,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
             alone = true;
 #pragma unroll
             for (int p = 0; p < kPhCount; ++p) {
-                if (p == 1 || (p == 2 && !kPhantom)) continue;
+                if (p == (int)kPhGivenUp || (p == 2 && !kPhantom)) continue;
                 const uint32_t v = *reinterpret_cast<volatile uint32_t *>(&mask[p][lane]);
                 uint32_t n = (p == kPhIdle && done) ? 0u : (uint32_t)__popc(__ballot_sync(kFullMask, v != 0));
                 // a live launch's warp whose next chunk is not published yet asks for
@@ -433,7 +447,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                 c3 = 1u + (rw & 511u) + ((pk >> kPkLast) & 1u) * 512u;
             } else if (ph == kPhFinish) {
                 e = ((jobw >> kJobList) & 63u) - 1u;
-                if (!run || !(pk & kPkSing)) e = 0;   // overflowed before its first single
+                if (!run || !(pk & kPkSing)) e = 0;   // overflowed: it has no list
                 unit = P.e_unit[e * 32 + lane];
                 next = P.e_next[next_at(e, lane)];
                 c2 = kTagDigi << 28;
@@ -557,7 +571,6 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                             const bool dead = photo || Ep < J.e_cut;
                             const float dep = dead ? E : E * xm1 / (1.0f + xm1);
                             const int crystal = in_panel ? (int)ST(kStrem) : -1;
-                            bool held = false;
                             if (crystal >= 0) {
                                 // a crystal interaction: the history's singles, tallies, optional hit list
                                 const uint32_t dtp = (uint32_t)floorf(STF(kSpath) * kInvCmmPerPs);
@@ -578,7 +591,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                                     P.e_e[ei] += dep;
                                     P.e_ew[ei] += dep * x;
                                     P.e_dt[ei] = min(P.e_dt[ei], dtp);
-                                } else {
+                                } else if (!(pk & kPkOvf)) {
                                     e = take_entry(efree, lane);
                                     if (e < (uint32_t)kEntries) {
                                         ei = e * 32 + lane;
@@ -590,38 +603,32 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                                         if (last) P.e_next[next_at(last - 1u, lane)] = (uint8_t)(e + 1u);
                                         else ST(kSjob) = jobw | ((e + 1u) << kJobList);
                                         pk |= kPkSing;
-                                    } else if (*reinterpret_cast<volatile uint32_t *>(&mask[kPhFinish][lane])) {
-                                        held = true;     // entries come free: the same trial again then
                                     } else {
-                                        pk |= kPkOvf;    // simulated again by the redo kernel
+                                        // simulated again by the redo kernel; its entries are the others' now
+                                        pk = (pk & ~kPkSing) | kPkOvf;
+                                        ST(kSjob) = free_list(efree, P.e_next, lane, jobw);
                                     }
                                 }
-                                if (!held) {
-                                    n_hits = 1;
-                                    atomicAdd(J.tally_count + crystal, 1ull);
-                                    atomicAdd(J.tally_efx + crystal, (unsigned long long)__float2ull_rn(dep * kEfxScale));
-                                    if (O.hit_cap)
-                                        keep_hit(O, J, g, h, (int)(jobw & 0xFFFFu), gamma, step - 1u, crystal, dep, dtp, x, y, z);
-                                }
+                                n_hits = 1;
+                                atomicAdd(J.tally_count + crystal, 1ull);
+                                atomicAdd(J.tally_efx + crystal, (unsigned long long)__float2ull_rn(dep * kEfxScale));
+                                if (O.hit_cap)
+                                    keep_hit(O, J, g, h, (int)(jobw & 0xFFFFu), gamma, step - 1u, crystal, dep, dtp, x, y, z);
                             }
-                            if (held) {
-                                n_trials = 0;
+                            pk &= ~kPkLastMask;
+                            if (dead) {
+                                to = photon_end(pk, (jobw >> kJobPanel1) & 0x7Fu);
+                                if (kPhantom) ST(kSph) = 0;
                             } else {
-                                pk &= ~kPkLastMask;
-                                if (dead) {
-                                    to = photon_end(pk, (jobw >> kJobPanel1) & 0x7Fu);
-                                    if (kPhantom) ST(kSph) = 0;
-                                } else {
-                                    // rotation in the panel frame with v as polar reference: for the ring
-                                    // (w, u, v) is a rotation of (x, y, z) about the axis, so this equals the
-                                    // global rotation; a posed panel takes its own v axis
-                                    float dx = STF(kSdx), dy = STF(kSdy), dz = STF(kSdz);
-                                    rotate_dir(dx, dy, dz, xm1 / (E * kInvMec2), sp, cp);
-                                    STORE3(kSdx, dx, dy, dz);
-                                    ST(kSE) = __float_as_uint(Ep);
-                                    if (in_panel) ST(kStrem) = __float_as_uint(panel_exit(g, x, y, z, dx, dy, dz));
-                                    to = in_panel ? kPhPanel : kPhPhantom;
-                                }
+                                // rotation in the panel frame with v as polar reference: for the ring
+                                // (w, u, v) is a rotation of (x, y, z) about the axis, so this equals the
+                                // global rotation; a posed panel takes its own v axis
+                                float dx = STF(kSdx), dy = STF(kSdy), dz = STF(kSdz);
+                                rotate_dir(dx, dy, dz, xm1 / (E * kInvMec2), sp, cp);
+                                STORE3(kSdx, dx, dy, dz);
+                                ST(kSE) = __float_as_uint(Ep);
+                                if (in_panel) ST(kStrem) = __float_as_uint(panel_exit(g, x, y, z, dx, dy, dz));
+                                to = in_panel ? kPhPanel : kPhPhantom;
                             }
                         }
                         ST(kSpk) = pk;
@@ -685,18 +692,15 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                         free_entry(efree, lane, e);
                     }
                     append_single<kLive, true>(W.geoms, O, J, (int)(jobw & 0xFFFFu), h, 0, so, kFullMask);
-                    if (ovf && (pk & kPkSing)) {
-#pragma unroll 1
-                        for (;;) {
-                            free_entry(efree, lane, e);
-                            if (!next) break;
-                            e = next - 1u;
-                            next = P.e_next[next_at(e, lane)];
-                        }
-                    }
                     const bool last = ovf || !next;
                     if (run && !last) ST(kSjob) = (jobw & ~(63u << kJobList)) | (next << kJobList);
                     to = last ? kPhIdle : kPhFinish;
+                    // An overflow tells that the class has more histories in flight than entries
+                    // for them: the slot is given up (no event serves the phase it goes to), but
+                    // for the class's first ones.  Overflows at 2.6 hits per pair, without and with
+                    // the rule: 2.0 and 0.6 % of 15 M histories; at 3.8 hits 21 and 1.9 %, at 11 hits
+                    // 75 and 26 %; at one hit none.
+                    if (ovf && (bit >> kKeptSlots)) to = kPhGivenUp;
                     count(acc, kNFin, __popc(__ballot_sync(kFullMask, run && last)));
                     count(acc, kNSingles, __popc(__ballot_sync(kFullMask, one)));
                 }
