@@ -205,5 +205,5 @@ uint64_t first_singles_guess(uint64_t n_decays);
 // histories start in all slots at once, and 3 % of 1e6 pairs overflow in a long LYSO
 // ring of 2.6 hits per pair, 0.6 % of 1.5e7.  A run with more is repeated whole.
 inline uint64_t overflow_room(uint64_t n_decays) { return std::max<uint64_t>(4096, n_decays / 16); }
-int run_with_retry(Run &R);            // plan + enqueue + collect, one exact-size re-run on overflow
+int run_with_retry(Run &R);            // plan + enqueue + collect, re-runs with exact sizes on overflow
 }

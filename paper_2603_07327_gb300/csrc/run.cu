@@ -588,8 +588,11 @@ size_t run_footprint(uint64_t total_decays, int64_t total_crystals, int n_jobs, 
 
 int run_with_retry(Run &R) {
     int st = GPET_OK;
-    bool resized = false;
-    for (int attempt = 0; attempt < 3; ++attempt) {
+    // Up to three sizes after the first: a run whose overflow list was full does
+    // not count the singles of the histories that had no place there, so the next
+    // one may fill the singles' buffer, and which histories overflow depends on
+    // the launch's schedule.
+    for (int resized = 0;;) {
         st = run_plan(R);
         if (st == GPET_OK) st = run_enqueue(R);
         if (st == GPET_OK) st = run_collect(R);
@@ -604,13 +607,13 @@ int run_with_retry(Run &R) {
             run_release(R);
             continue;
         }
-        if (st == GPET_ERR_OVERFLOW && !resized && !(R.h_hdr.status & kStatusOverflow)) {
-            resized = true;
+        if (st == GPET_ERR_OVERFLOW && resized < 3 && !(R.h_hdr.status & kStatusOverflow)) {
+            ++resized;
             // the device counters kept counting past the capacities: re-run with exact sizes
             R.caps.guess = false;
             R.caps.singles = std::max<uint64_t>(R.caps.singles, R.h_hdr.n_singles + 1024);
             R.caps.hits = std::max<uint64_t>(R.caps.hits, R.h_hdr.n_hits + 1024);
-            // (which lists overflow can depend on the launch's schedule: with room to spare)
+            // (with room to spare, as the next run's number may be another)
             R.caps.ovf = std::max<uint64_t>(R.caps.ovf, R.h_hdr.n_ovf + R.h_hdr.n_ovf / 4 + 4096);
             run_release(R);
             continue;

@@ -11,7 +11,9 @@ import workloads as W
 pytestmark = pytest.mark.gpu
 
 # Compton and photoelectric coefficient (1/cm), depth, pitch, half-length (mm), cutoff (keV), pairs
-DESIGNS = {"long_lyso": (0.5742, 0.2958, 20.0, 1.0, 150.0, 10.0, 1_000_003)}
+DESIGNS = {"long_lyso": (0.5742, 0.2958, 20.0, 1.0, 150.0, 10.0, 1_000_003),
+           "scatterer": (0.8, 0.07, 20.0, 1.0, 150.0, 10.0, 1_000_003),
+           "compton_only": (1.5, 0.0, 25.0, 0.5, 150.0, 80.0, 300_007)}
 COUNTS = ("hits", "singles", "coincidences", "det_steps", "flights", "compton_trials", "entered", "singles_formed")
 
 
