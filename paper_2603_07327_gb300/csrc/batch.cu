@@ -52,6 +52,31 @@ int gpet_batch_build_run(Run &R, int32_t n_jobs, gpet_scanner *const *scanners, 
     return GPET_OK;
 }
 
+// the whole hot path into the graph that gpet_batch_run replays
+static int capture(gpet_batch *b) {
+    Run &R = *b->run;
+    cudaError_t e = cudaStreamBeginCapture(R.stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return gpet_cuda_fail(e, "cudaStreamBeginCapture");
+    const int st = run_enqueue(R);
+    cudaGraph_t g = nullptr;
+    e = cudaStreamEndCapture(R.stream, &g);
+    cudaGraphExec_t x = nullptr;
+    if (st == GPET_OK && e == cudaSuccess) e = cudaGraphInstantiate(&x, g, 0);
+    if (st != GPET_OK || e != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        return st != GPET_OK ? st : gpet_cuda_fail(e, "capture of the batch");
+    }
+    if (b->exec) cudaGraphExecDestroy(b->exec);
+    if (b->graph) cudaGraphDestroy(b->graph);
+    b->graph = g;
+    b->exec = x;
+    return GPET_OK;
+}
+
+// Room in the overflow list of a batch after a run with n overflowed histories:
+// how many overflow depends on the launch's schedule.
+static uint64_t replay_room(uint64_t n) { return 2 * n + 4096; }
+
 extern "C" int gpet_batch_create(int32_t n_jobs, gpet_scanner *const *scanners, const gpet_source *sources,
                                  const gpet_digitizer *digitizers, const uint64_t *n_decays, const uint64_t *seeds,
                                  const gpet_options *opt, gpet_batch **out) {
@@ -73,18 +98,10 @@ extern "C" int gpet_batch_create(int32_t n_jobs, gpet_scanner *const *scanners, 
     }
     // first run sizes the buffers (exact re-run on overflow) and gives results
     st = run_with_retry(R);
-    if (st != GPET_OK) { delete b; return st; }
+    if (st == GPET_OK && R.h_hdr.n_ovf > R.O.ovf_cap / 2) st = run_grow_overflow(R, replay_room(R.h_hdr.n_ovf));
     // capture the whole hot path once; replays reuse the same arena
-    cudaError_t e = cudaStreamBeginCapture(R.stream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) { delete b; return gpet_cuda_fail(e, "cudaStreamBeginCapture"); }
-    st = run_enqueue(R);
-    cudaGraph_t g = nullptr;
-    e = cudaStreamEndCapture(R.stream, &g);
-    if (st != GPET_OK) { if (g) cudaGraphDestroy(g); delete b; return st; }
-    if (e != cudaSuccess) { delete b; return gpet_cuda_fail(e, "cudaStreamEndCapture"); }
-    b->graph = g;
-    e = cudaGraphInstantiate(&b->exec, g, 0);
-    if (e != cudaSuccess) { delete b; return gpet_cuda_fail(e, "cudaGraphInstantiate"); }
+    if (st == GPET_OK) st = capture(b);
+    if (st != GPET_OK) { delete b; return st; }
     *out = b;
     return GPET_OK;
 }
@@ -92,9 +109,17 @@ extern "C" int gpet_batch_create(int32_t n_jobs, gpet_scanner *const *scanners, 
 extern "C" int gpet_batch_run(gpet_batch *b) {
     if (!b || !b->exec) return gpet_fail(GPET_ERR_INVALID_ARG, "batch is NULL");
     Run &R = *b->run;
-    cudaError_t e = cudaGraphLaunch(b->exec, R.stream);
-    if (e != cudaSuccess) return gpet_cuda_fail(e, "cudaGraphLaunch");
-    return run_collect(R);
+    for (int grown = 0;; ++grown) {
+        cudaError_t e = cudaGraphLaunch(b->exec, R.stream);
+        if (e != cudaSuccess) return gpet_cuda_fail(e, "cudaGraphLaunch");
+        int st = run_collect(R);
+        // (the graph's run sized everything else: only the overflow list can be too small)
+        if (st != GPET_ERR_OVERFLOW || R.h_hdr.n_ovf <= R.O.ovf_cap || (R.h_hdr.status & kStatusOverflow) || grown == 3)
+            return st;
+        st = run_grow_overflow(R, replay_room(R.h_hdr.n_ovf));
+        if (st == GPET_OK) st = capture(b);
+        if (st != GPET_OK) return st;
+    }
 }
 
 extern "C" int gpet_batch_jobs(const gpet_batch *b, int32_t *n_jobs) {

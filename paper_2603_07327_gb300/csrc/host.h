@@ -89,6 +89,7 @@ struct Run {
     BucketJob *d_buckets = nullptr;
     bool keep_hits = false;
     LaunchCfg cfg{};
+    void *ovf_list = nullptr;            // overflow list of its own, outside the arena (run_grow_overflow)
     // arena
     void *arena = nullptr;
     size_t arena_bytes = 0;
@@ -205,5 +206,8 @@ uint64_t first_singles_guess(uint64_t n_decays);
 // histories start in all slots at once, and 3 % of 1e6 pairs overflow in a long LYSO
 // ring of 2.6 hits per pair, 0.6 % of 1.5e7.  A run with more is repeated whole.
 inline uint64_t overflow_room(uint64_t n_decays) { return std::max<uint64_t>(4096, n_decays / 16); }
+// An overflow list of cap histories in memory of its own, the other arrays
+// where they are; launches enqueued from now on fill it.
+int run_grow_overflow(Run &R, uint64_t cap);
 int run_with_retry(Run &R);            // plan + enqueue + collect, re-runs with exact sizes on overflow
 }

@@ -554,7 +554,8 @@ void run_release(Run &R) {
     // and a run may outlive the stream it ran on (a server worker's, a
     // caller's): free in the order of the legacy stream, never the run's own.
     if (R.arena) cudaFreeAsync(R.arena, cudaStreamLegacy);
-    R.arena = nullptr;
+    if (R.ovf_list) cudaFreeAsync(R.ovf_list, cudaStreamLegacy);
+    R.arena = R.ovf_list = nullptr;
     for (auto &e : R.ev)
         if (e) { cudaEventDestroy(e); e = nullptr; }
 }
@@ -625,6 +626,19 @@ int run_with_retry(Run &R) {
         run_release(R);
     }
     return st;
+}
+
+int run_grow_overflow(Run &R, uint64_t cap) {
+    void *list = nullptr;
+    cudaError_t e = cudaMallocAsync(&list, cap * (sizeof(*R.O.ovf_h) + sizeof(*R.O.ovf_job)), R.stream);
+    if (e == cudaErrorMemoryAllocation) return gpet_fail(GPET_ERR_OOM, "overflow list of %llu histories", (unsigned long long)cap);
+    if (e != cudaSuccess) return gpet_cuda_fail(e, "cudaMallocAsync");
+    if (R.ovf_list) cudaFreeAsync(R.ovf_list, R.stream);
+    R.ovf_list = list;
+    R.O.ovf_h = static_cast<decltype(R.O.ovf_h)>(list);
+    R.O.ovf_job = reinterpret_cast<decltype(R.O.ovf_job)>(R.O.ovf_h + cap);
+    R.O.ovf_cap = cap;
+    return GPET_OK;
 }
 
 uint64_t first_singles_guess(uint64_t n_decays) {

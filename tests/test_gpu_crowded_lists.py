@@ -65,3 +65,23 @@ def test_live_launch(G):
     for i, j in zip(ids, jobs):
         same(server.wait(i), plain(j, 1), ("hits", "singles", "coincidences"))
     server.close()
+
+
+@pytest.mark.parametrize("n", range(3_420_000, 3_560_000, 20_000))
+def test_batch_replays(G, n):
+    """Which histories overflow depends on the schedule: sizes whose overflow list of one history in 16
+    is just large enough, or just too small, for one run are replayed without an error all the same."""
+    j = dict(job(G, "scatterer"), n_decays=n, digitizer=W.digitizer())
+    b = G.Batch([j])
+    first = b.result(0)
+    c, t, ptr = first.counts(), first.tallies(), first.device_ptr(G.SINGLES_H)
+    for _ in range(12):
+        b.run()
+    r = b.result(0)
+    assert {k: r.counts()[k] for k in COUNTS} == {k: c[k] for k in COUNTS}
+    assert all(np.array_equal(x, y) for x, y in zip(r.tallies(), t))
+    # a view made before the replays shows them
+    assert first.device_ptr(G.SINGLES_H) == ptr
+    s, u = first.singles(), r.singles()
+    assert all(np.array_equal(np.sort(s[k]), np.sort(u[k])) for k in s)
+    b.close()
