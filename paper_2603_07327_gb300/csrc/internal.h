@@ -92,6 +92,7 @@ struct SinglesDev {
 
 struct CoincDev {
     unsigned long long *scan;        // tile ticket, then a look-back word per tile
+    uint32_t *open;                  // per tile: first single + 1 of a window that reaches the next tile's cluster
     int32_t *a, *b;
     unsigned long long *n;
     const uint64_t *window_ps;       // per job
@@ -298,6 +299,9 @@ struct ClusterTile {
 
     __device__ __forceinline__ uint64_t time(const SinglesDev &s, uint32_t lo, uint32_t i) const {
         return i + 1u - lo < (uint32_t)(kTile + 2) ? t[i + 1u - lo] : s.t[i];
+    }
+    __device__ __forceinline__ int32_t job_of(const SinglesDev &s, uint32_t lo, uint32_t n, uint32_t i) const {
+        return i + 1u - lo < (uint32_t)(kTile + 2) ? job[i + 1u - lo] : i < n ? s.job[i] : -1;
     }
     __device__ __forceinline__ bool linked(const SinglesDev &s, const uint64_t *window_ps, uint32_t lo, uint32_t n,
                                            uint32_t i) const {

@@ -225,6 +225,7 @@ static int plan_once(Run &R, bool clamp) {
     cv.take(R.d_tally_efx, (size_t)tcc);
     cv.take(R.S.ghist, 8 * 256);
     cv.take(R.C.scan, cap / kCoincScanTile + 2);
+    cv.take(R.C.open, cap / kCoincScanTile + 1);
     if (n_buckets) {
         cv.take(R.S.bstart, n_buckets + 1);
         cv.take(R.S.bscan, n_buckets / kBucketScanTile + 3);
@@ -323,7 +324,7 @@ static int plan_once(Run &R, bool clamp) {
     rebase(S.plan, base); rebase(S.lb[0], base); rebase(S.lb[1], base); rebase(S.tile_ctr, base);
     rebase(SD.t, base); rebase(SD.h, base); rebase(SD.unit, base); rebase(SD.panel, base); rebase(SD.job, base);
     rebase(SD.e, base); rebase(SD.eraw, base); rebase(SD.doi, base);
-    rebase(C.scan, base); rebase(C.a, base); rebase(C.b, base);
+    rebase(C.scan, base); rebase(C.open, base); rebase(C.a, base); rebase(C.b, base);
     rebase(JS.s_off, base); rebase(JS.c_off, base); rebase(JS.hits, base); rebase(R.d_toff, base);
     rebase(R.d_tn, base);
     JS.n_jobs = nj;
@@ -582,7 +583,7 @@ size_t run_footprint(uint64_t total_decays, int64_t total_crystals, int n_jobs, 
     b += ocap * 12;                              // overflow list
     b += cap * (2 * 8 + 2 * 4) + 2 * 256 * 8 * tiles + 8 * 4 + 128;  // sort (look-back words, tile counters)
     b += cap * (8 + 8 + 4 * 6);                  // sorted singles
-    b += 8 * (cap / kCoincScanTile + 2) + 2 * 4 * (cap / 2 + 1); // coincidences
+    b += 12 * (cap / kCoincScanTile + 2) + 2 * 4 * (cap / 2 + 1); // coincidences
     b += 8 * (n_jobs + 1) * 2 + 8 * n_jobs * 3;  // per-job statistics
     return b + 64 * 256;                         // alignment slack
 }

@@ -591,14 +591,32 @@ __global__ void k_gather(SortDev S, SinglesDev out) {
 // ends, so each cluster is processed alone: the earliest unconsumed single opens
 // [t0, t0 + window]; exactly two singles in different panels make a coincidence;
 // all singles in the window are consumed.
-// One pass over tiles of singles: the thread at a cluster's start replays it,
-// and the one at the tile's first single also the cluster that began before the
-// tile (walking back to its start), each up to the tile's end; the pairs found
+// One pass over tiles of singles: a thread per cluster that begins in the tile
+// replays it up to the tile's end, and one goes on with the cluster that reaches
+// into the tile from the window that the tile before left open.  The work is then
+// that of one walk over the singles however long a cluster is, and a tile waits
+// for those before it only through the words that they leave it.  (Walking back to
+// the cluster's start took 392 ms for one cluster of 9.5e5 singles, and with the
+// square of the tiles more for larger ones; now 2.1 ms.)  The pairs found
 // in the tile are written after those of the tiles before it, whose number comes
 // by look-back.  (Flags, counts, a scan and the writes as kernels of their own
 // took 41 us for 1.6e6 singles and 18 us for any small number.)
 constexpr int kCoincThreads = 256, kCoincPer = 4, kCoincTile = kCoincThreads * kCoincPer;
 static_assert(kCoincTile == (int)kCoincScanTile, "look-back words are allocated per tile");
+
+// The first single of the window that the tile before left open (its word is that
+// single's index + 1), or false when the word did not come within the wait limit.
+// That tile is done or being worked on, and leaves the word after at most a walk
+// over its singles and the same wait: tiles are claimed in order.
+__device__ __forceinline__ bool wait_open(const uint32_t *word, uint32_t &a) {
+    uint32_t w = *reinterpret_cast<const volatile uint32_t *>(word);
+    for (int polls = 0; w == 0u && polls < kLookbackPolls; ++polls) {
+        if (polls > 64) __nanosleep(64);
+        w = *reinterpret_cast<const volatile uint32_t *>(word);
+    }
+    a = w - 1u;
+    return w != 0u;
+}
 
 __global__ void __launch_bounds__(kCoincThreads) k_coinc(SinglesDev s, CoincDev C, int *status) {
     after_previous();
@@ -608,7 +626,10 @@ __global__ void __launch_bounds__(kCoincThreads) k_coinc(SinglesDev s, CoincDev 
     __shared__ int fail_sh;
     const uint32_t n = (uint32_t)*s.n, tiles = (n + kCoincTile - 1) / kCoincTile;
     for (;;) {
-        if (threadIdx.x == 0) tile_sh = (uint32_t)atomicAdd(C.scan, 1ull);
+        if (threadIdx.x == 0) {
+            tile_sh = (uint32_t)atomicAdd(C.scan, 1ull);
+            fail_sh = 0;
+        }
         if (threadIdx.x < kCoincTile / 32) flag[threadIdx.x] = 0;
         __syncthreads();
         const uint32_t tile = tile_sh;
@@ -619,21 +640,44 @@ __global__ void __launch_bounds__(kCoincThreads) k_coinc(SinglesDev s, CoincDev 
         // the clusters that begin in the tile, and the one that reaches into it
         const uint32_t before = linked(lo) ? 1u : 0u;
         for (uint32_t c = threadIdx.x; c < tl.n_start + before; c += kCoincThreads) {
-            uint32_t a = lo;
-            if (c < tl.n_start) a += tl.start[c];
-            else do --a; while (linked(a));
-            const uint64_t W = __ldg(C.window_ps + (a + 1u - lo < kCoincTile + 2u ? tl.job[a + 1u - lo] : s.job[a]));
-            while (a < hi) {
-                uint32_t b = a;
+            // the window's first single, and the first one of the tile that may lie beyond the window
+            uint32_t a = lo, b = lo;
+            if (c < tl.n_start) {
+                a += tl.start[c];
+                b = a + 1u;
+            } else if (!wait_open(C.open + tile - 1u, a)) {
+                fail_sh = 1;
+                break;
+            }
+            const int job = tl.job[b - lo];
+            const uint64_t W = __ldg(C.window_ps + job);
+            for (;;) {
+                // (the singles of one job within W of a are those that follow it up to some place)
                 const uint64_t ta = tl.time(s, lo, a);
-                while (linked(b + 1u) && tl.time(s, lo, b + 1u) - ta <= W) ++b;
-                if (b == a + 1u && a >= lo && s.panel[a] != s.panel[b])
+                auto within = [&](uint32_t i) { return tl.job_of(s, lo, n, i) == job && tl.time(s, lo, i) - ta <= W; };
+                if (a >= lo && within(a + 1u) && !within(a + 2u) && s.panel[a] != s.panel[a + 1u])
                     atomicOr(&flag[(a - lo) >> 5], 1u << ((a - lo) & 31));
-                if (!linked(b + 1u)) break;   // the cluster's end
-                a = b + 1u;
+                // the place by steps that double, then halve: most windows hold two singles, some a thousand
+                uint32_t step = 1;
+                while (b + step <= hi && within(b + step - 1u)) {
+                    b += step;
+                    step *= 2u;
+                }
+                while (step /= 2u)
+                    if (b + step <= hi && within(b + step - 1u)) b += step;
+                if (!linked(b)) break;   // the cluster's end
+                if (b == hi) {           // the tile's: the window is the next one's to go on with
+                    *reinterpret_cast<volatile uint32_t *>(C.open + tile) = a + 1u;
+                    break;
+                }
+                a = b++;
             }
         }
         __syncthreads();
+        if (fail_sh) {
+            if (threadIdx.x == 0) atomicOr(status, kStatusSortStall);
+            break;
+        }
         uint32_t f = (flag[threadIdx.x * kCoincPer >> 5] >> (threadIdx.x * kCoincPer & 31)) & ((1u << kCoincPer) - 1u);
         uint32_t tot;
         uint32_t at = block_exscan(__popc(f), tot, sw);
