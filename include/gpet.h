@@ -419,6 +419,13 @@ int gpet_delta_sym(int64_t n, const double *s_a, const double *s_b, double *out)
  * serialise them. */
 int gpet_sort_times_noalloc(const uint64_t *d_t_in, uint64_t n, uint64_t *d_t_out, uint32_t *d_perm_out,
                             void *stream);
+/* Waits for `stream` and tells whether every sort enqueued before has written
+ * its whole output: GPET_OK, or GPET_ERR_CUDA once after a sort whose blocks
+ * waited for one another longer than their limit (seconds; the blocks of a
+ * cooperative kernel run together, so none does in ordinary use).  Such a sort
+ * ends, but leaves d_t_out and d_perm_out incomplete, and the asynchronous call
+ * itself cannot report it. */
+int gpet_sort_times_noalloc_status(void *stream);
 
 /* ------------------------------------------------------------------------ */
 /* autotuner                                                                 */

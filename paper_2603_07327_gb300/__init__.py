@@ -143,6 +143,7 @@ SIGNATURES = {
     "gpet_server_stats_get": (C.c_int, [_P, C.POINTER(ServerStats)]),
     "gpet_server_destroy": (None, [_P]),
     "gpet_sort_times_noalloc": (C.c_int, [_P, C.c_uint64, _P, _P, _P]),
+    "gpet_sort_times_noalloc_status": (C.c_int, [_P]),
     "gpet_event_costs": (C.c_int, [_P, C.POINTER(Source), C.POINTER(Digitizer), C.c_uint64, C.c_uint64,
                                    C.POINTER(C.c_double), C.POINTER(C.c_uint64)]),
     "gpet_sensitivity_map": (C.c_int, [C.c_int32, C.POINTER(_P), C.c_int32, C.POINTER(C.c_double), C.c_double,

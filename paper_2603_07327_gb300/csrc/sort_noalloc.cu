@@ -22,6 +22,7 @@ constexpr int kNoallocTile = 4096;                                    // keys of
 constexpr unsigned long long kNoallocTiles = (kNoallocMaxKeys + kNoallocTile - 1) / kNoallocTile;
 // layout of the scratch array (all offsets multiples of 256 bytes)
 constexpr size_t kOffCtl = 0;                                         // NoallocCtl
+constexpr size_t kOffFailed = 128;                                    // not 0: a sort gave up since the last query
 constexpr size_t kOffHist = 256;                                      // [8][256] uint32 digit histograms
 constexpr size_t kOffKeys = kOffHist + 8 * 256 * 4 + 256;             // two buffers, or the buckets' keys
 constexpr size_t kOffVals = kOffKeys + 2 * 8 * kNoallocMaxKeys;       // and their indices
@@ -61,17 +62,26 @@ static_assert(kMaxBuckets * 4 <= 256 * 4 * kNoallocTiles, "the bucket counts lie
 static_assert(kMaxBuckets * kBucketMean <= 2 * kNoallocMaxKeys && kMaxBuckets * kBucketMean >= kNoallocMaxKeys,
               "room for twice the mean, and a mean no larger than meant");
 
+// polls of a wait of the whole grid before it gives up (several seconds; a test
+// makes it none)
+#ifndef GPET_GRID_WAIT_POLLS
+#define GPET_GRID_WAIT_POLLS kLookbackPolls
+#endif
+constexpr int kGridWaitPolls = GPET_GRID_WAIT_POLLS;
+
 struct NoallocCtl {
     unsigned long long nmin, max;   // of the keys: ~min, max
     unsigned int arrived;           // blocks, over all waits of the grid
     unsigned int crowded;           // a bucket is full
 };
+static_assert(sizeof(NoallocCtl) <= kOffFailed, "a call clears the control block, not the word behind it");
 struct NoallocArgs {
     const uint64_t *t_in;
     uint64_t *t_out;
     uint32_t *perm;                 // or NULL
     uint32_t n;
     NoallocCtl *ctl;
+    unsigned int *failed;
     uint32_t *ghist, *words;
     uint64_t *keys;
     uint32_t *vals;
@@ -90,16 +100,18 @@ struct BucketSmem {
 constexpr size_t kNoallocSmem = sizeof(TileSmem) > sizeof(BucketSmem) ? sizeof(TileSmem) : sizeof(BucketSmem);
 
 // All blocks have come here `turn` times (they are resident together: the launch
-// is cooperative).  False if the wait ran out, after which the block gives up.
-__device__ __forceinline__ bool grid_wait(NoallocCtl *ctl, unsigned turn) {
+// is cooperative).  False if the wait ran out, after which the block gives up; the
+// caller learns of it from gpet_sort_times_noalloc_status.
+__device__ __forceinline__ bool grid_wait(const NoallocArgs &A, unsigned turn) {
     __syncthreads();
     int fail = 0;
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(&ctl->arrived, 1u);
+        atomicAdd(&A.ctl->arrived, 1u);
         int polls = 0;
-        while (*reinterpret_cast<volatile unsigned *>(&ctl->arrived) < turn * gridDim.x)
-            if (++polls > kLookbackPolls) { fail = 1; break; }
+        while (*reinterpret_cast<volatile unsigned *>(&A.ctl->arrived) < turn * gridDim.x)
+            if (++polls > kGridWaitPolls) { fail = 1; break; }
+        if (fail) atomicOr(A.failed, 1u);
         __threadfence();
     }
     return !__syncthreads_or(fail);
@@ -209,9 +221,11 @@ __device__ __forceinline__ bool sort_tile(const NoallocArgs &A, TileSmem &sm, ui
         if (!fail && t > 0) row[d] = tag | kWordIncl | (excl + cnt);
         sm.gdelta[d] = dbase + excl - lstart;
     }
-    // (a tile whose look-back gave up writes nothing; the call cannot report it,
-    // and its output is then incomplete)
-    if (__syncthreads_or(fail)) return false;
+    // (a tile whose look-back gave up writes nothing: the output is then incomplete)
+    if (__syncthreads_or(fail)) {
+        if (threadIdx.x == 0) atomicOr(A.failed, 1u);
+        return false;
+    }
     const uint32_t tn = min(n - t * kNoallocTile, (uint32_t)kNoallocTile);
     for (uint32_t i = threadIdx.x; i < tn; i += kSortBlock) {
         const uint64_t key = sm.keys[i];
@@ -243,7 +257,7 @@ __device__ __noinline__ void radix_sort(const NoallocArgs &A, TileSmem &sm, uint
     __syncthreads();
     for (int i = threadIdx.x; i < 8 * 256; i += kSortBlock)
         if (h[i]) atomicAdd(A.ghist + i, h[i]);
-    if (!grid_wait(A.ctl, ++turn)) return;
+    if (!grid_wait(A, ++turn)) return;
     // the digits that vary (every block finds the same ones)
     __shared__ int varies[8];
     if (threadIdx.x < 256) {
@@ -260,7 +274,7 @@ __device__ __noinline__ void radix_sort(const NoallocArgs &A, TileSmem &sm, uint
         for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x)
             if (!sort_tile(A, sm, sw, p, src, t)) return;
         src ^= 1;
-        if (!grid_wait(A.ctl, ++turn)) return;
+        if (!grid_wait(A, ++turn)) return;
     }
     for (uint32_t i = first; i < n; i += stride) {
         A.t_out[i] = __ldcg(A.keys + (src ? kNoallocMaxKeys : 0) + i);
@@ -310,7 +324,7 @@ __global__ void __launch_bounds__(kSortBlock, 1) k_noalloc_sort(const __grid_con
     // (a sample over the whole input, the same for every block)
     const bool sampled = n > kSampleFrom;
     const unsigned long long sample = A.t_in[sampled ? (uint32_t)((unsigned long long)threadIdx.x * n / kSortBlock) : 0u];
-    if (!grid_wait(A.ctl, 1)) return;
+    if (!grid_wait(A, 1)) return;
     // 2. each key to its bucket: hi64((key - min) * scale), or key - min where
     // there are no more values than buckets (scale 0)
     const unsigned long long mn = ~__ldcg(&A.ctl->nmin);
@@ -355,7 +369,7 @@ __global__ void __launch_bounds__(kSortBlock, 1) k_noalloc_sort(const __grid_con
         }
     }
     if (__syncthreads_or(crowded) && threadIdx.x == 0) atomicOr(&A.ctl->crowded, 1u);
-    if (!grid_wait(A.ctl, 2)) return;
+    if (!grid_wait(A, 2)) return;
     if (__ldcg(&A.ctl->crowded)) {
         radix_sort(A, *reinterpret_cast<TileSmem *>(raw), sw, 2);
         return;
@@ -437,6 +451,7 @@ extern "C" int gpet_sort_times_noalloc(const uint64_t *d_t_in, uint64_t n, uint6
     A.perm = d_perm_out;
     A.n = (uint32_t)n;
     A.ctl = reinterpret_cast<NoallocCtl *>(base + kOffCtl);
+    A.failed = reinterpret_cast<unsigned int *>(base + kOffFailed);
     A.ghist = reinterpret_cast<uint32_t *>(base + kOffHist);
     A.keys = reinterpret_cast<uint64_t *>(base + kOffKeys);
     A.vals = reinterpret_cast<uint32_t *>(base + kOffVals);
@@ -449,5 +464,20 @@ extern "C" int gpet_sort_times_noalloc(const uint64_t *d_t_in, uint64_t n, uint6
     void *args[] = {&A};
     if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kSortBlock), args, kNoallocSmem, st);
     if (e != cudaSuccess) return gpet_cuda_fail(e, "gpet_sort_times_noalloc launch");
+    return GPET_OK;
+}
+
+extern "C" int gpet_sort_times_noalloc_status(void *stream) {
+    void *sym = nullptr;
+    cudaError_t e = cudaGetSymbolAddress(&sym, g_sort_scratch);
+    if (e != cudaSuccess) return gpet_cuda_fail(e, "cudaGetSymbolAddress(sort scratch)");
+    unsigned char *word = static_cast<unsigned char *>(sym) + kOffFailed;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    unsigned int failed = 0;
+    e = cudaMemcpyAsync(&failed, word, sizeof(failed), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && failed) e = cudaMemsetAsync(word, 0, sizeof(failed), st);
+    if (e != cudaSuccess) return gpet_cuda_fail(e, "gpet_sort_times_noalloc_status");
+    if (failed) return gpet_fail(GPET_ERR_CUDA, "a wait of gpet_sort_times_noalloc ran out: its output is incomplete");
     return GPET_OK;
 }
