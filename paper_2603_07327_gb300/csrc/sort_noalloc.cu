@@ -459,10 +459,17 @@ extern "C" int gpet_sort_times_noalloc(const uint64_t *d_t_in, uint64_t n, uint6
     const void *fn = reinterpret_cast<const void *>(k_noalloc_sort);
     e = ensure_dynamic_smem(fn, kNoallocSmem);
     if (e == cudaSuccess) e = cudaMemsetAsync(A.ctl, 0, sizeof(NoallocCtl), st);
-    // one block per multiprocessor at most (all of them run at once), 512 keys a block at least
-    const unsigned blocks = (unsigned)std::min<uint64_t>((uint64_t)sms, (n + 511) / 512);
+    // one block per multiprocessor at most (all of them run at once), 512 keys a block at least; fewer where the
+    // stream has a part of the device's multiprocessors
+    unsigned blocks = (unsigned)std::min<uint64_t>((uint64_t)sms, (n + 511) / 512);
     void *args[] = {&A};
-    if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kSortBlock), args, kNoallocSmem, st);
+    while (e == cudaSuccess) {
+        e = cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kSortBlock), args, kNoallocSmem, st);
+        if (e != cudaErrorCooperativeLaunchTooLarge || blocks == 1) break;
+        cudaGetLastError();
+        e = cudaSuccess;
+        blocks /= 2;
+    }
     if (e != cudaSuccess) return gpet_cuda_fail(e, "gpet_sort_times_noalloc launch");
     return GPET_OK;
 }
