@@ -164,19 +164,20 @@ def _digitizer_traffic(singles_per_step):
     return t["bytes_per_single"] * singles_per_step if t else None
 
 
-def event_isolated(scanners, dg, counts, tr_ms, n_sample=1_000_000):
-    """Event-isolated fraction of the transport: each phase's events of the
-    timed launches (counted by the kernel) times that event's GPU time when it
-    runs alone at full width (gpet_event_costs, on states of geometry A and B
-    with the source at the centre, averaged: the sweep is half of each), over
-    the measured transport time."""
+def event_costs(scanners, dg, counts, tr_ms, n_sample=1_000_000):
+    """Each phase's events of the timed launches (counted by the kernel) times
+    that event's GPU time when its per-lane form runs alone at full width
+    (gpet_event_costs, on states of geometry A and B with the source at the
+    centre, averaged: the sweep is half of each), against the measured transport
+    time.  No bound: the kernel cuts events where lanes diverge and repacks
+    them, so it takes less than the sum."""
     costs = [scanners[g].event_costs(W.point_source((0.0, 0.0, 0.0)), dg, n_sample=n_sample, seed=2)[0]
              for g in ("A", "B")]
     ns = [0.5 * (a + b) for a, b in zip(*costs)]
     events = [sum(c["phase_events"][p] for c in counts) for p in range(len(PHASES))]
     pairs = sum(c["n_decays"] for c in counts)
-    ideal_ms = sum(events[p] * ns[p] for p in range(1, len(PHASES))) * 1e-6
-    return dict(frac=ideal_ms / tr_ms, ideal_transport_ms=ideal_ms, transport_ms=tr_ms,
+    alone_ms = sum(events[p] * ns[p] for p in range(1, len(PHASES))) * 1e-6
+    return dict(events_alone_over_transport=alone_ms / tr_ms, events_alone_ms=alone_ms, transport_ms=tr_ms,
                 ns_per_event={PHASES[p]: ns[p] for p in range(1, len(PHASES))},
                 events_per_pair={PHASES[p]: events[p] / pairs for p in range(1, len(PHASES))},
                 sample=f"{n_sample} histories of geometry A and of B, source at the centre")
@@ -576,14 +577,13 @@ def run_ours(args):
                 issue_detail=dict(issue_active=detail["issue_active"], simt_efficiency=detail["simt_efficiency"],
                                   capture=detail["id"]) if detail else None,
                 transport_share=tr_ms / (tr_ms + dg_ms))
-    # beside it: the transport time the launch's events would take if each ran
-    # alone at full width (per-event costs from micro-kernels on this GPU, on
-    # states of this workload), over the measured transport time
+    # the time the launch's events take as micro-kernels of their own (no roofline)
+    costs = None
     if default_kernel:
         try:
-            roof["event_isolated"] = event_isolated(scanners, dg, counts, tr_ms)
+            costs = event_costs(scanners, dg, counts, tr_ms)
         except Exception as exc:  # noqa: BLE001
-            roof["event_isolated"] = dict(error=f"{type(exc).__name__}: {exc}")
+            costs = dict(error=f"{type(exc).__name__}: {exc}")
 
     # digitizer back end (time sort + coincidences), HBM-bound: algorithmic bytes
     # per single = bucket counts 12 (key read, rank written) + places 20 (key and
@@ -685,7 +685,7 @@ def run_ours(args):
                             pairs_per_step=pairs_per_step,
                             l2="flushed between steps (256 MB write)", kernel=args.kernel or "default",
                             parallelism=f"replicas x{world}" if world > 1 else "1 GPU"),
-                wall_s=wall, gpu_launches=None, roofline=roof, roofline_digitizer=roof_dig, clocks=clk,
+                wall_s=wall, gpu_launches=None, roofline=roof, roofline_digitizer=roof_dig, event_costs=costs, clocks=clk,
                 e2e=dict(value=pairs_per_step * world / e2e_dt, unit="pairs/s", h2d_bytes_per_step=h2d,
                          d2h_bytes_per_step=d2h, ms_per_step=1000 * e2e_dt, simulate_ms_per_step=1000 * e2e_sim_s,
                          copy_ms_per_step=1000 * (e2e_dt - e2e_sim_s), copy_ms_steps=[round(c, 2) for c in copy_ms],

@@ -46,8 +46,8 @@ extern "C" const char *gpet_version(void) { return "gpet-gb300 0.1 (sm_103a)"; }
 namespace gpet {
 
 static std::mutex g_attr_mutex;
-static std::map<std::pair<int, const void *>, size_t> g_smem_limit;
-static std::map<std::pair<int, const void *>, size_t> g_smem_asked;  // (device, kernel) -> limit set
+static std::map<std::pair<int, const void *>, size_t> g_smem_limit;  // (device, kernel) -> limit set
+static std::map<std::pair<int, const void *>, size_t> g_smem_asked;  // (device, kernel) -> most bytes asked for
 
 cudaError_t ensure_dynamic_smem(const void *fn, size_t bytes) {
     int dev = 0, optin = 0;

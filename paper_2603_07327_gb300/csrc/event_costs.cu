@@ -8,9 +8,10 @@
 // which every lane of every warp runs that phase's event on pool states, over
 // and over, is timed with CUDA events.  Its time per event is what the event
 // costs when the whole GPU runs nothing else at full SIMT width -- without the
-// regrouping, barriers and refills of a wavefront kernel.  The sum over a
-// launch's events of these costs, over the launch's transport time, is the
-// transport's event-isolated roofline fraction.
+// regrouping and refills of a wavefront kernel.  The events are the per-lane
+// ones of transport.cuh, with lists of six singles.  The slot-pool kernel cuts
+// them where lanes diverge and repacks the lanes, so the sum of a launch's
+// events at these costs is no bound of its time: it takes less.
 #include <algorithm>
 #include <cstring>
 #include <vector>

@@ -8,11 +8,11 @@
 // maximal run of one job's time-sorted singles whose consecutive gaps are at
 // most the coincidence window -- can therefore only split when singles are
 // removed, never grow into its neighbour (the gap to the neighbour is already
-// wider than the window and removing singles only widens it).  The thread at
-// the start of each cluster of the widest window replays the coincidence
-// policy (earliest unconsumed single opens [t, t + window]; exactly two
-// singles in different panels count; everything in the window is consumed)
-// on the cluster's singles inside each energy window in turn.  The blurred
+// wider than the window and removing singles only widens it).  For each cluster of
+// several singles of the widest window and each energy window, a thread replays
+// the coincidence policy (earliest unconsumed single opens [t, t + window];
+// exactly two singles in different panels count; everything in the window is
+// consumed) on the cluster's singles inside that energy window.  The blurred
 // energies and the window edges are the same FP32 values a run with that
 // window alone compares, so the counts equal those runs' counts exactly.
 #include <cmath>

@@ -615,7 +615,7 @@ extern "C" int gpet_server_create(const gpet_server_config *cfg, gpet_server **o
     S->max_launch_ms = cfg->max_launch_ms > 0.0 ? cfg->max_launch_ms : 20.0;
     // One launch's arena takes at most a quarter of the budget (the open launch,
     // the one finishing and split requests' buffers share it), and at most
-    // 2^26 singles (7.9 GB); a piece's first guess of singles fits half of it.
+    // 2^26 singles (6.7 GB); a piece's first guess of singles fits half of it.
     const size_t per_single = sizeof(RawSingle) + 2 * 8 + 2 * 4 + 8 + 8 + 6 * 4 + 4;
     S->launch_crystals = (int64_t)std::min<size_t>(1 << 22, std::max<size_t>(1 << 18, cfg->hbm_budget_bytes / 400));
     const size_t fixed = run_footprint(0, S->launch_crystals, S->max_jobs, 64, false);

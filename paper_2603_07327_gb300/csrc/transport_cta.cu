@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                     STORE3(kSx, s.x, s.y, s.z);
                     ST(kSpath) = __float_as_uint(s.path);
                     ST(kSpk) = pk;
-                    if (late) {   // step cap hit: abandon the history, flag the run
+                    if (late) {   // step cap hit: abandon the history (and its entries), flag the run
                         atomicOr(O.status, kStatusTimeout);
                         to = kPhIdle;
                     }
