@@ -118,18 +118,18 @@ class Clocks:
 # Entries are named by capture id (the summary of each capture under that id
 # gives its command).
 TRANSPORT_SOURCES = ("device.cuh", "transport.cuh", "transport.cu", "transport_cta.cu")
-TRANSPORT_CAPTURE = dict(id="k_transport_cta_sweep_122x1e7", sha1="bbb093e4a789da5513ca6e3dfa759997a91a189c",
-                         warp_inst_per_pair=87.692, dram_bytes_per_pair=7.015)
+TRANSPORT_CAPTURE = dict(id="k_transport_cta_sweep_122x1e7", sha1="5d44f212b6bb47717363cb045eb783658d386280",
+                         warp_inst_per_pair=86.466, dram_bytes_per_pair=7.015)
 # Issue detail of the same kernel from one ncu --set full capture of a
 # 2e6-pair sweep position: issue-active fraction of the schedulers and SIMT
 # efficiency (thread instructions per warp instruction / 32).
-TRANSPORT_DETAIL = dict(id="k_transport_cta_sweep_position_2e6", sha1="bbb093e4a789da5513ca6e3dfa759997a91a189c",
-                        issue_active=0.726, simt_efficiency=0.669)
+TRANSPORT_DETAIL = dict(id="k_transport_cta_sweep_position_2e6", sha1="5d44f212b6bb47717363cb045eb783658d386280",
+                        issue_active=0.731, simt_efficiency=0.671)
 # algorithmic bytes of the digitizer back end per single (the model in run_ours)
 DIGITIZER_BYTES_PER_SINGLE = 130
 # DRAM bytes of the digitizer back end (bucket_count .. job_stats of one step), per single.
 DIGITIZER_SOURCES = ("device.cuh", "internal.h", "sort.cu")
-DIGITIZER_TRAFFIC = dict(id="traffic_digitizer_sweep_8x1e7", sha1="cf81f50a403bc839fd8ae9f207a7f63b93469281",
+DIGITIZER_TRAFFIC = dict(id="traffic_digitizer_sweep_8x1e7", sha1="1e1470cc73c0460dbcd71d9720230ba66f9b8c02",
                          bytes_per_single=239.0)
 
 

@@ -203,8 +203,8 @@ void fill_counts(const Run &R, int job, uint64_t n_decays, int64_t n_crystals, g
 // readout exceeds (0.62 per decay) costs such a run half of its time.
 uint64_t first_singles_guess(uint64_t n_decays);
 // Histories a run's overflow list first holds (12 bytes each): a launch's first
-// histories start in all slots at once, and 3 % of 1e6 pairs overflow in a long LYSO
-// ring of 2.6 hits per pair, 0.6 % of 1.5e7.  A run with more is repeated whole.
+// histories start in all slots at once, and 4.2 % of 1e6 pairs overflow in a long LYSO
+// ring of 2.6 hits per pair, 0.8 % of 1e7.  A run with more is repeated whole.
 inline uint64_t overflow_room(uint64_t n_decays) { return std::max<uint64_t>(4096, n_decays / 16); }
 // An overflow list of cap histories in memory of its own, the other arrays
 // where they are; launches enqueued from now on fill it.

@@ -12,7 +12,8 @@
 // same for every key (high time bytes, unused job bits), and every remaining
 // pass is one kernel (k_onesweep: tiles claimed in order, each tile's digit
 // offsets from the global histogram and a decoupled look-back over the tiles
-// before it).  Stable ranks inside a tile come from the lanes of a warp with the
+// before it: the published one-sweep radix sort of Adinets and Merrill, 2022, on
+// the single-pass scan of Merrill and Garland, 2016).  Stable ranks inside a tile come from the lanes of a warp with the
 // same digit (the intersection of bit-plane ballots), in input order.  A pass's
 // input tiles are streamed into shared memory by the bulk-copy engine
 // (cp.async.bulk completing on an mbarrier), one tile ahead of the tile being

@@ -45,7 +45,7 @@ static __device__ __align__(256) unsigned char g_sort_scratch[kScratchBytes];
 // digits of eight bits at most, those that vary, a wait of the grid after each.
 // A tile is ranked by the lanes of a warp with the same digit (the intersection
 // of bit-plane ballots), in input order, so the passes are stable; a tile's
-// offsets come by look-back over the tiles before it.  The look-back words carry
+// offsets come by look-back over the tiles before it (Merrill and Garland, 2016).  The look-back words carry
 // the pass they belong to, so one buffer serves all passes without being cleared
 // between them, and 16 of them are read per round trip.
 // Both ways give the one stable order, keys by value and equal ones by index.

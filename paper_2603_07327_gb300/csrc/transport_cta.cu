@@ -23,7 +23,7 @@
 //     one slab-test loop for every kind of flight, one Philox draw and one sine
 //     and cosine for all events that need them, cold paths out of line.  At 74 KB
 //     the same scheme lost half of its issue slots to instruction fetch (7.6 of
-//     14 warp-cycles per issue; now 1.9 of 9), and events that a whole CTA runs
+//     14 warp-cycles per issue; now 1.4 of 9), and events that a whole CTA runs
 //     together behind a barrier lost them to the barrier (6.0 of 13.5).
 //   - First flights of a pair's two photons are one event (the same ray in both
 //     directions), which keeps photon 1's panel and distances in the slot until
@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) k_transport_cta(const __grid
                     to = last ? kPhIdle : kPhFinish;
                     // An overflow tells that the class has more histories in flight than entries
                     // for them: the slot is given up (no event serves the phase it goes to), but
-                    // for the class's first ones.  Overflows at 2.6 hits per pair, without and with
+                    // for the class's first ones.  Overflows (on the CPU) at 2.6 hits per pair, without and with
                     // the rule: 2.0 and 0.6 % of 15 M histories; at 3.8 hits 21 and 1.9 %, at 11 hits
                     // 75 and 26 %; at one hit none.
                     if (ovf && (bit >> kKeptSlots)) to = kPhGivenUp;
